@@ -224,6 +224,23 @@ struct bse_dotfuse {
 // A[p][k][n] = dv sum_x conj(f_p(x)) e^{ik.x} u_nk(x) on device arrays (k_local.cu)
 bse_status bse_local_projection_device(const double2* u, const int* nk, const int* nx, int nb, const double* kshift,
                                        const double2* f, int np, double dv, double2* a, cudaStream_t st);
+// FP64 products on the FP16 tensor cores by exact splitting (k_oz.cu): an
+// operand's digits [batches][7][rows][kp] and row scales [batches][rows]
+struct bse_oz_operand {
+  void* digits = nullptr;
+  double* scale = nullptr;
+  int batches = 1, rows = 0, kp = 0;
+};
+size_t bse_oz_digit_bytes(int batches, int rows, int kp);
+int bse_oz_kp(int k);   // K padded to whole blocks
+// digits of complex rows x [rows][n], entries times d[batch][n] if given; pair = 1 writes two
+// real rows per complex row so that a product with pair = 0 rows is sum a conj(x)
+bse_status bse_oz_split_rows(const double2* x, int rows, int n, const double2* d, int batches, int pair,
+                             const bse_oz_operand& o, int* bad, cudaStream_t st);
+// out = alpha A_b B_b^T for every batch (an operand with one batch serves all);
+// element (b, row, col) at out + b sb + (row/2) sr2 + (row%2) sr1 + col sc
+bse_status bse_oz_gemm(const bse_oz_operand& a, const bse_oz_operand& b, int batches, double alpha, double* out,
+                       long long sb, long long sr2, long long sr1, long long sc, int* err, cudaStream_t st);
 // screening: G_j = psi diag(1/(mu + i t_j - eps)) psi^H for all j, chi0 from them (k_screen.cu)
 bse_status bse_screening_device(const double2* psi, const double* eps, int nr, int nkk, double mu, const double* t,
                                 const double* w, int nt, double2* G, double2* chi, cudaStream_t st);

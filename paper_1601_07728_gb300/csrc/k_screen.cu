@@ -82,12 +82,94 @@ __global__ void chi0_kernel(const double2* __restrict__ G, const double* __restr
   chi[e] = make_double2(sr * s, si * s);
 }
 
+// d_j(K) = 1 / (mu - eps_K + i t_j)
+__global__ void green_weights(const double* __restrict__ eps, int nkk, double mu, const double* __restrict__ t,
+                              double2* __restrict__ d) {
+  const int K = blockIdx.x * blockDim.x + threadIdx.x;
+  if (K >= nkk) return;
+  const double tj = t[blockIdx.y];
+  const double x = mu - eps[K], den = x * x + tj * tj;
+  d[(size_t)blockIdx.y * nkk + K] = make_double2(x / den, -tj / den);
+}
+
+struct Scratch {
+  void* p = nullptr;
+  ~Scratch() {
+    if (p) cudaFree(p);
+  }
+};
+
+// G_j on the tensor cores (k_oz.cu): the rows psi(r, :) d_j against the row
+// pairs of psi(r', :), as many frequencies per pass as the scratch holds.
+// *done = false (and nothing but G written) where the scratch cannot be had or
+// psi d_j holds Inf/NaN or a magnitude outside 2^+-400.
+bse_status green_tensor(const double2* psi, const double* eps, int nr, int nkk, double mu, const double* t, int nt,
+                        double2* G, cudaStream_t st, bool* done) {
+  *done = false;
+  const int kp = bse_oz_kp(2 * nkk);
+  const size_t per = bse_oz_digit_bytes(1, nr, kp), fixed = bse_oz_digit_bytes(1, 2 * nr, kp);
+  const size_t budget = (size_t)512 << 20;
+  int nj = (int)(budget / per);
+  nj = nj < 1 ? 1 : (nj > nt ? nt : nj);
+  const size_t bd = bse_oz_digit_bytes(nj, nr, kp);
+  const size_t tab = ((size_t)nt * nkk * sizeof(double2) + 255) / 256 * 256;
+  const size_t sca = ((size_t)nj * nr * sizeof(double) + 255) / 256 * 256;
+  const size_t scb = ((size_t)2 * nr * sizeof(double) + 255) / 256 * 256;
+  Scratch sc;
+  if (cudaMalloc(&sc.p, bd + fixed + tab + sca + scb + 256) != cudaSuccess) {
+    cudaGetLastError();
+    sc.p = nullptr;
+    return BSE_OK;
+  }
+  char* q = (char*)sc.p;
+  bse_oz_operand a, b;
+  a.digits = q, q += bd;
+  b.digits = q, q += fixed;
+  double2* d = (double2*)q;
+  q += tab;
+  a.scale = (double*)q, q += sca;
+  b.scale = (double*)q, q += scb;
+  int* word = (int*)q;   // {wait gave up, out of range}
+  a.rows = nr, b.rows = 2 * nr;
+  a.kp = b.kp = kp;
+  cudaMemsetAsync(word, 0, 2 * sizeof(int), st);
+  green_weights<<<dim3((unsigned)((nkk + 255) / 256), (unsigned)nt), 256, 0, st>>>(eps, nkk, mu, t, d);
+  bse_status s = bse_oz_split_rows(psi, nr, nkk, nullptr, 1, 1, b, word + 1, st);
+  for (int j = 0; j < nt && s == BSE_OK; j += nj) {
+    const int n = nt - j < nj ? nt - j : nj;
+    a.batches = n;
+    s = bse_oz_split_rows(psi, nr, nkk, d + (size_t)j * nkk, n, 0, a, word + 1, st);
+    if (s == BSE_OK)
+      s = bse_oz_gemm(a, b, n, 1.0, (double*)(G + (size_t)j * nr * nr), 2ll * nr * nr, 4ll * nr, 2ll * nr, 1, word, st);
+  }
+  int hw[2] = {0, 0};
+  if (s == BSE_OK && (cudaMemcpyAsync(hw, word, sizeof(hw), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+                      cudaStreamSynchronize(st) != cudaSuccess))
+    s = BSE_ERR_CUDA;
+  if (s != BSE_OK) {
+    cudaStreamSynchronize(st);   // before the scratch goes
+    return s;
+  }
+  if (hw[0]) return BSE_ERR_TIMEOUT;
+  *done = hw[1] == 0;
+  return BSE_OK;
+}
+
 }  // namespace
 
 bse_status bse_screening_device(const double2* psi, const double* eps, int nr, int nkk, double mu, const double* t,
                                 const double* w, int nt, double2* G, double2* chi, cudaStream_t st) {
-  const dim3 g((unsigned)((nr + GT - 1) / GT), (unsigned)((nr + GT - 1) / GT), (unsigned)nt);
-  green_kernel<<<g, 256, 0, st>>>(psi, eps, nr, nkk, mu, t, G);
+  // from 2^22 complex products on (FP64 kernel: about 0.1 ms) the tensor-core
+  // form; K is bounded by its 64-bit partial sums
+  bool done = false;
+  if ((double)nr * nr * nkk * nt >= 4194304.0 && nkk <= (1 << 20)) {
+    const bse_status s = green_tensor(psi, eps, nr, nkk, mu, t, nt, G, st, &done);
+    if (s != BSE_OK) return s;
+  }
+  if (!done) {
+    const dim3 g((unsigned)((nr + GT - 1) / GT), (unsigned)((nr + GT - 1) / GT), (unsigned)nt);
+    green_kernel<<<g, 256, 0, st>>>(psi, eps, nr, nkk, mu, t, G);
+  }
   const size_t n = (size_t)nr * nr;
   chi0_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(G, w, nr, nt, chi);
   return cudaGetLastError() == cudaSuccess ? BSE_OK : BSE_ERR_CUDA;
