@@ -1,13 +1,17 @@
 // FP64 matrix products D_b[m][n] = alpha sum_K A_b[m][K] B_b[n][K] on the FP16
 // tensor cores by exact splitting (oz_dev.cuh), and the kernels that write the
-// operands' digits.  User: the screening stage's Green's functions (Sec. 3.3).
+// operands' digits.  Users: the screening stage's Green's functions (Sec. 3.3)
+// and the set-up projection onto the local basis (Sec. 3.2.2).
 //
 // Why: GB300 retires 2 FP64 FMAs per SM and clock and about 2000 times as many
 // FP16 products, so that the 19 products of 128 x 128 x 16 which replace one
 // FP64 product of 128 x 64 x 16 still run some 50 times faster.  Measured:
 // Green's functions of 900 points, 4096 states and 16 frequencies 682 ms
-// (FP64 kernel) -> 14.0 ms (this one 12.9, writing the digits 0.97).  The error
-// against 64 bits fell from 1.9e-15 to 1.3e-15.  What bounds it now: operand tiles from L2 (35 bytes per SM and clock) beside the
+// (FP64 kernel) -> 14.0 ms (this one 12.9, writing the digits 0.97); the
+// projection of 8^3 k x 16^3 points x 64 bands onto 64 functions 102.6 ms ->
+// 4.4 ms (this one 2.0, digits 2.07, row scales 0.32).  The error against 64
+// bits fell from 1.9e-15 to 1.3e-15 and from 1.3e-15 to 0.9e-15.  What bounds
+// it now: operand tiles from L2 (35 bytes per SM and clock) beside the
 // products' 64 clocks each.
 #include "bse_internal.cuh"
 #include "oz_dev.cuh"
@@ -27,6 +31,11 @@ constexpr int OZ_THREADS = 320;
 constexpr int OZ_BAREA = OZ_BS * (OZ_B + OZ_BD) + OZ_BD;
 constexpr size_t OZ_SMEM = 1024 + (size_t)OZ_AS * OZ_A + OZ_BAREA + 512;
 constexpr unsigned long long OZ_WAIT_NS = 2000000000ull;
+
+struct oz_mesh {
+  int nk[3], nx[3];
+  double s[3];
+};
 
 struct OzParams {
   int mt, nt, ntiles, kb;       // M tiles, N tiles, tiles over all batches, K blocks
@@ -320,6 +329,84 @@ __global__ void __launch_bounds__(256) oz_split_rows(const double2* __restrict__
   }
 }
 
+// Largest magnitude key of u[k][x][n] over x for every (k, n): blocks of 32
+// bands x 8 rows walk a part of the grid (coalesced along n).
+__global__ void __launch_bounds__(256) oz_col_keys(const double2* __restrict__ u, int nx, int nb, int per,
+                                                   unsigned* __restrict__ keys) {
+  __shared__ unsigned sk[8][32];
+  const int n = blockIdx.y * 32 + (threadIdx.x & 31), g = threadIdx.x >> 5, k = blockIdx.z;
+  const int x0 = blockIdx.x * per, x1 = min(nx, x0 + per);
+  unsigned key = 0;
+  if (n < nb) {
+    const double2* p = u + (size_t)k * nx * nb + n;
+#pragma unroll 4
+    for (int x = x0 + g; x < x1; x += 8) {
+      const double2 v = p[(size_t)x * nb];
+      key = max(key, max(oz_key(v.x), oz_key(v.y)));
+    }
+  }
+  sk[g][threadIdx.x & 31] = key;
+  __syncthreads();
+  if (g == 0 && n < nb) {
+#pragma unroll
+    for (int i = 1; i < 8; ++i) key = max(key, sk[i][threadIdx.x]);
+    atomicMax(keys + (size_t)k * nb + n, key);
+  }
+}
+
+// Digits of the rows (n) of e^{ik.x} u_nk(x), K = 2x interleaved (re, im):
+// u [k][x][n] is read coalesced along n and written transposed.  One block:
+// 32 grid points of one k, every band; a warp holds 4 bands x 8 groups of 4
+// points, so that both the 64-byte reads and the 128-byte digit rows fill
+// their sectors.  |e^{ik.x} u| components are at most sqrt 2 times those of u:
+// the row scale has one more bit.
+__global__ void __launch_bounds__(256) oz_split_bloch(const double2* __restrict__ u, oz_mesh ms, int k0, int nb, int kp,
+                                                      const unsigned* __restrict__ keys, __half* __restrict__ dig,
+                                                      double* __restrict__ scale, int* __restrict__ bad) {
+  __shared__ double2 ph[32];
+  const int nx = ms.nx[0] * ms.nx[1] * ms.nx[2];
+  const int kl = blockIdx.y, k = k0 + kl, x0 = blockIdx.x * 32;
+  if (threadIdx.x < 32) {
+    const int x = x0 + threadIdx.x;
+    double sn = 0.0, cs = 1.0;
+    if (x < nx) {
+      const int m2 = k % ms.nk[2], m1 = (k / ms.nk[2]) % ms.nk[1], m0 = k / (ms.nk[1] * ms.nk[2]);
+      const int j2 = x % ms.nx[2], j1 = (x / ms.nx[2]) % ms.nx[1], j0 = x / (ms.nx[1] * ms.nx[2]);
+      double fr = (m0 + ms.s[0]) * j0 / ((double)ms.nk[0] * ms.nx[0]) + (m1 + ms.s[1]) * j1 / ((double)ms.nk[1] * ms.nx[1]) +
+                  (m2 + ms.s[2]) * j2 / ((double)ms.nk[2] * ms.nx[2]);
+      fr -= floor(fr);
+      sincospi(2.0 * fr, &sn, &cs);
+    }
+    ph[threadIdx.x] = make_double2(cs, sn);
+  }
+  __syncthreads();
+  const int xg = threadIdx.x & 7, x = x0 + 4 * xg;
+  double2 c[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) c[i] = ph[4 * xg + i];
+  for (int n = threadIdx.x >> 3; n < nb; n += 32) {
+    int flag = 0;
+    const int e = oz_exponent(keys[(size_t)kl * nb + n], &flag) + 1;
+    if (xg == 0 && blockIdx.x == 0) {
+      scale[(size_t)kl * nb + n] = scalbn(1.0, e);
+      if (flag) atomicOr(bad, 1);
+    }
+    unsigned long long f[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const double2 w = x + i < nx ? u[((size_t)k * nx + x + i) * nb + n] : make_double2(0.0, 0.0);
+      f[2 * i] = oz_fixed(w.x * c[i].x - w.y * c[i].y, e);
+      f[2 * i + 1] = oz_fixed(w.x * c[i].y + w.y * c[i].x, e);
+    }
+    __half* o = dig + ((size_t)kl * OZ_S * nb + n) * kp + 2 * x;
+#pragma unroll
+    for (int i = 0; i < OZ_S; ++i)
+      *reinterpret_cast<uint4*>(o + (size_t)i * nb * kp) =
+          make_uint4(oz_digit2(f[0], f[1], i), oz_digit2(f[2], f[3], i), oz_digit2(f[4], f[5], i),
+                     oz_digit2(f[6], f[7], i));
+  }
+}
+
 typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -347,12 +434,31 @@ bool digit_map(CUtensorMap* m, const __half* base, int kp, int rows, int z, int 
 size_t bse_oz_digit_bytes(int batches, int rows, int kp) {
   return (((size_t)batches * OZ_S * rows * kp * sizeof(__half)) + 255) / 256 * 256;
 }
+int bse_oz_tiles(int rows_a, int rows_b) { return (rows_a + OZ_M - 1) / OZ_M * ((rows_b + OZ_N - 1) / OZ_N); }
 int bse_oz_kp(int k) { return (k + OZ_KB - 1) / OZ_KB * OZ_KB; }
 
 bse_status bse_oz_split_rows(const double2* x, int rows, int n, const double2* d, int batches, int pair,
                              const bse_oz_operand& o, int* bad, cudaStream_t st) {
   oz_split_rows<<<dim3((unsigned)rows, (unsigned)batches), 256, 0, st>>>(x, n, d, rows, o.kp, pair, (__half*)o.digits,
                                                                           o.scale, bad);
+  return cudaGetLastError() == cudaSuccess ? BSE_OK : BSE_ERR_CUDA;
+}
+
+bse_status bse_oz_split_bloch(const double2* u, const int* nk, const int* nx, const double* kshift, int nb, int k0,
+                              int nkc, const bse_oz_operand& o, unsigned* keys, int* bad, cudaStream_t st) {
+  oz_mesh ms;
+  for (int i = 0; i < 3; ++i) {
+    ms.nk[i] = nk[i];
+    ms.nx[i] = nx[i];
+    ms.s[i] = kshift ? kshift[i] : 0.0;
+  }
+  const int nxt = nx[0] * nx[1] * nx[2];
+  const int per = nxt > 8192 ? 1024 : 512;
+  cudaMemsetAsync(keys, 0, (size_t)nkc * nb * sizeof(unsigned), st);
+  oz_col_keys<<<dim3((unsigned)((nxt + per - 1) / per), (unsigned)((nb + 31) / 32), (unsigned)nkc), 256, 0, st>>>(
+      u + (size_t)k0 * nxt * nb, nxt, nb, per, keys);
+  oz_split_bloch<<<dim3((unsigned)(o.kp / OZ_KB), (unsigned)nkc), 256, 0, st>>>(u, ms, k0, nb, o.kp, keys,
+                                                                                (__half*)o.digits, o.scale, bad);
   return cudaGetLastError() == cudaSuccess ? BSE_OK : BSE_ERR_CUDA;
 }
 

@@ -87,3 +87,37 @@ def test_values_outside_the_scheme_take_the_fp64_kernel(value):
         assert np.abs(g[0][hit]).max() > 1e200
     else:
         assert not np.any(np.isfinite(g[0][hit]))
+
+
+# bands around the 64-column tile, projectors around the 128-row tile (two rows
+# each), grids that do not fill a K block, a shifted and a non-cubic mesh
+@pytest.mark.parametrize("shape", [((2, 2, 2), (9, 9, 9), 64, 64, (0.0, 0.0, 0.0)),
+                                   ((3, 1, 2), (11, 8, 7), 65, 65, (0.25, 0.5, 0.0)),
+                                   ((5, 4, 4), (5, 7, 6), 33, 16, (0.0, 0.0, 0.25)),
+                                   ((1, 1, 1), (16, 16, 16), 130, 9, (0.0, 0.0, 0.0)),
+                                   ((8, 8, 8), (5, 5, 5), 9, 9, (0.0, 0.5, 0.0))])
+def test_projection_within_the_bound(shape):
+    nk, nx, nb, npj, ks = shape
+    assert np.prod(nk) * np.prod(nx) * nb * npj >= 1 << 22
+    rng = np.random.default_rng(npj * nb)
+    u = S.orthonormal_bloch(rng, int(np.prod(nk)), int(np.prod(nx)), nb)
+    f = S.complex_normal(rng, (npj, int(np.prod(nx))))
+    a = bse.local_projection(u, nk, nx, f, 0.37, ks)
+    ref = O.local_projection(u, nk, nx, f, 0.37, ks)
+    um = np.maximum(np.abs(u.real), np.abs(u.imag)).max(axis=1)   # [k][n]
+    bound = 4 * 2 * np.prod(nx) * 2.0 ** -51 * 0.37 * _row_max(f)[:, None, None] * um[None]
+    assert np.all(np.abs(a - ref) <= bound)
+    assert np.linalg.norm(a - ref) <= 1e-14 * np.sqrt(np.prod(nx)) * np.linalg.norm(ref)
+
+
+def test_projection_with_nan_takes_the_fp64_kernel():
+    nk, nx, nb, npj = (2, 2, 2), (9, 9, 9), 40, 20
+    rng = np.random.default_rng(8)
+    u = S.complex_normal(rng, (8, 729, nb))
+    f = S.complex_normal(rng, (npj, 729))
+    ref = O.local_projection(u, nk, nx, f, 1.0)
+    u[3, 100, 7] = np.nan
+    a = bse.local_projection(u, nk, nx, f, 1.0)
+    assert not np.any(np.isfinite(a[:, 3, 7]))
+    a[:, 3, 7] = ref[:, 3, 7]
+    assert np.abs(a - ref).max() <= 1e-12 * np.abs(ref).max()
