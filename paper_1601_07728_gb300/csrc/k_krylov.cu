@@ -84,6 +84,23 @@ __device__ double2 sum_partials(const double2* partial, int v, int nblk) {
   return block_sum2(acc);
 }
 
+// sum_partials(...).x by one warp: the same pairs in the same order
+__device__ double warp_partials_x(const double2* __restrict__ p, int n) {
+  const int lane = threadIdx.x & 31;
+  double x[RB / 32];
+#pragma unroll
+  for (int i = 0; i < RB / 32; ++i) {
+    x[i] = 0.0;
+    for (int t = lane + 32 * i; t < n; t += RB) x[i] += p[t].x;
+  }
+#pragma unroll
+  for (int h = RB / 64; h >= 1; h >>= 1)
+#pragma unroll
+    for (int i = 0; i < h; ++i) x[i] += x[i + h];
+  for (int off = 16; off > 0; off >>= 1) x[0] += __shfl_xor_sync(0xffffffffu, x[0], off);
+  return x[0];
+}
+
 // ---------------------------------------------------------------------------
 // Haydock
 // ---------------------------------------------------------------------------
@@ -174,20 +191,28 @@ __global__ void __launch_bounds__(RB) hay_b_finalize(const double2* partial, int
   }
 }
 
-// coef[v][j] = sum of partials (grid (nj, nv)); optionally accumulated into hacc
-__global__ void __launch_bounds__(RB) gs_dot_finalize(const double2* partial, int nblk, double2* coef,
-                                                      int coef_stride, double2* hacc, int hacc_stride) {
-  const int j = blockIdx.x, v = blockIdx.y;
-  double2 acc = make_double2(0, 0);
-  const double2* p = partial + ((size_t)v * gridDim.x + j) * nblk;
-  for (int i = threadIdx.x; i < nblk; i += RB) acc = cadd(acc, p[i]);
-  double2 s = block_sum2(acc);
-  if (threadIdx.x == 0) {
-    coef[(size_t)v * coef_stride + j] = s;
-    if (hacc) {
-      double2 o = hacc[(size_t)v * hacc_stride + j];
-      hacc[(size_t)v * hacc_stride + j] = cadd(o, s);
-    }
+// The Gram-Schmidt kernels keep one order for every sum -- 64 blocks of 256
+// threads stride over a vector, warps reduce by halves, warps and blocks in
+// index order -- whatever the launch shape: GMRES on the reduced-precision
+// operators repeats a solve bit for bit only if these sums do.
+
+// coef[v][j] = sum of the 64 partials (one warp per j; grid (ceil(nj/8), nv)),
+// only where mask[v] != 0 (mask may be null); optionally accumulated into hacc
+constexpr int GS_BLK = 64;   // blocks per vector of the multi-dot
+__global__ void __launch_bounds__(256) gs_dot_finalize(const double2* __restrict__ partial, int nj, double2* coef,
+                                                       long long coef_vs, long long coef_js, double2* hacc,
+                                                       int hacc_stride, const int* __restrict__ mask) {
+  const int j = blockIdx.x * 8 + (threadIdx.x >> 5), v = blockIdx.y, lane = threadIdx.x & 31;
+  if (j >= nj || (mask && !mask[v])) return;
+  const double2* p = partial + ((size_t)v * nj + j) * GS_BLK;
+  double2 s = cadd(p[lane], p[lane + 32]);
+  for (int off = 16; off > 0; off >>= 1) {
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+  }
+  if (lane == 0) {
+    coef[(size_t)v * coef_vs + (size_t)j * coef_js] = s;
+    if (hacc) hacc[(size_t)v * hacc_stride + j] = cadd(hacc[(size_t)v * hacc_stride + j], s);
   }
 }
 
@@ -257,63 +282,83 @@ bse_status apply_chunked(bse_handle* h, const double2* in, double2* out, int n_v
   return BSE_OK;
 }
 
-// CGS2: for pass in 0,1: coef = basis^H w; w -= basis coef; hacc += coef.
-// Gram-Schmidt projections <basis_j|w> for JB basis vectors at a time: w is
-// read once per group of JB (not once per basis vector).  partial[v][j][blk].
+// Gram-Schmidt projections <basis_j|w> of GS_JB basis vectors per block (w is
+// read once per group of GS_JB).  partial[v][j][blk]; grid (GS_BLK, groups, nv).
+// The 16 sums of a warp are reduced by exchanging halves: the same pairs as a
+// butterfly per sum, at 16 FP64 additions per lane instead of 80, which at two
+// FP64 operations per SM and clock were most of the kernel on short vectors,
+// and the groups of a long basis run beside one another.  Mean over j = 1..12:
+// 16 systems of 12,288 rows 86 -> 35 us, 32 systems of 196,608 rows 850 -> 746
+// (FP64 pipe: 6 operations per entry, 2 per SM and clock, 460 us).
 constexpr int GS_JB = 8;
-constexpr int GS_BLK = 64;   // blocks per vector of the multi-dot: long loops, few partials to reduce
 __global__ void __launch_bounds__(RB) gs_dot_multi(const double2* __restrict__ basis, long long bstride,
-                                                   const double2* __restrict__ w, long long N, int nj,
+                                                   long long jstride, const double2* __restrict__ w,
+                                                   long long wstride, long long N, int nj,
                                                    double2* __restrict__ partial, const int* __restrict__ mask) {
-  const int v = blockIdx.y;
-  const bool on = !mask || mask[v];
-  const double2* bv = basis + (size_t)v * bstride;
-  const double2* wv = w + (size_t)v * N;
-  __shared__ double2 sred[RB / 32][GS_JB];
-  for (int j0 = 0; j0 < nj; j0 += GS_JB) {
-    double2 acc[GS_JB];
+  const int v = blockIdx.z, j0 = blockIdx.y * GS_JB;
+  if (mask && !mask[v]) return;
+  const double2* bv = basis + (size_t)v * bstride + (size_t)j0 * jstride;
+  const double2* wv = w + (size_t)v * wstride;
+  const int njg = nj - j0 < GS_JB ? nj - j0 : GS_JB;
+  double acc[2 * GS_JB];
 #pragma unroll
-    for (int q = 0; q < GS_JB; ++q) acc[q] = make_double2(0, 0);
-    if (on) {
-      for (long long e = (long long)blockIdx.x * RB + threadIdx.x; e < N; e += (long long)gridDim.x * RB) {
-        const double2 b = wv[e];
+  for (int q = 0; q < 2 * GS_JB; ++q) acc[q] = 0.0;
+  for (long long e = (long long)blockIdx.x * RB + threadIdx.x; e < N; e += (long long)GS_BLK * RB) {
+    const double2 b = wv[e];
+    double2 a[GS_JB];
 #pragma unroll
-        for (int q = 0; q < GS_JB; ++q) {
-          if (j0 + q < nj) {
-            const double2 a = bv[(size_t)(j0 + q) * N + e];
-            acc[q].x += a.x * b.x + a.y * b.y;
-            acc[q].y += a.x * b.y - a.y * b.x;
-          }
-        }
-      }
-    }
+    for (int q = 0; q < GS_JB; ++q)
+      if (q < njg) a[q] = bv[(size_t)q * jstride + e];
 #pragma unroll
     for (int q = 0; q < GS_JB; ++q) {
-      for (int off = 16; off > 0; off >>= 1) {
-        acc[q].x += __shfl_xor_sync(0xffffffffu, acc[q].x, off);
-        acc[q].y += __shfl_xor_sync(0xffffffffu, acc[q].y, off);
+      if (q < njg) {
+        acc[2 * q] += a[q].x * b.x + a[q].y * b.y;
+        acc[2 * q + 1] += a[q].x * b.y - a[q].y * b.x;
       }
-      if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5][q] = acc[q];
     }
-    __syncthreads();
-    if (threadIdx.x < GS_JB && j0 + threadIdx.x < nj) {
-      double2 s = make_double2(0, 0);
-      for (int wq = 0; wq < RB / 32; ++wq) s = cadd(s, sred[wq][threadIdx.x]);
-      partial[((size_t)v * nj + j0 + threadIdx.x) * gridDim.x + blockIdx.x] = s;
+  }
+  // lane L ends with sum L >> 1
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int h = GS_JB; h >= 1; h >>= 1) {
+    const bool up = (lane & (2 * h)) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double mine = up ? acc[h + i] : acc[i], other = up ? acc[i] : acc[h + i];
+      acc[i] = mine + __shfl_xor_sync(0xffffffffu, other, 2 * h);
     }
-    __syncthreads();
+  }
+  acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+  __shared__ double sred[RB / 32][2 * GS_JB];
+  if ((lane & 1) == 0) sred[threadIdx.x >> 5][lane >> 1] = acc[0];
+  __syncthreads();
+  if ((int)threadIdx.x < 2 * njg) {
+    double t = 0.0;
+    for (int i = 0; i < RB / 32; ++i) t += sred[i][threadIdx.x];
+    double* o = reinterpret_cast<double*>(partial + ((size_t)v * nj + j0 + (threadIdx.x >> 1)) * GS_BLK + blockIdx.x);
+    o[threadIdx.x & 1] = t;
   }
 }
 
+// coef[v][j] = <basis_j|w> (and += into hacc) for the systems of `mask`
+void gs_project(bse_handle* h, const double2* basis, long long bstride, const double2* w, int nv, int nj,
+                double2* partial, double2* coef, int coef_stride, double2* hacc, int hacc_stride, const int* mask) {
+  BSE_PROF(h, BSE_K_RECURSION,
+           gs_dot_multi<<<dim3(GS_BLK, (nj + GS_JB - 1) / GS_JB, nv), RB, 0, h->stream>>>(
+               basis, bstride, h->N, w, h->N, h->N, nj, partial, mask));
+  BSE_PROF(h, BSE_K_RECURSION,
+           gs_dot_finalize<<<dim3((nj + 7) / 8, nv), 256, 0, h->stream>>>(partial, nj, coef, coef_stride, 1, hacc,
+                                                                           hacc_stride, mask));
+}
+
+// CGS2: for pass in 0,1: coef = basis^H w; w -= basis coef; hacc += coef.
 bse_status cgs2(bse_handle* h, const double2* basis, long long bstride, double2* w, int nv, int nj,
                 double2* partial, double2* coef, int coef_stride, double2* hacc, int hacc_stride,
                 const int* mask) {
-  cudaStream_t st = h->stream;
-  const long long N = h->N;
   for (int pass = 0; pass < 2; ++pass) {
-    BSE_PROF(h, BSE_K_RECURSION, gs_dot_multi<<<dim3(GS_BLK, nv), RB, 0, st>>>(basis, bstride, w, N, nj, partial, mask));
-    BSE_PROF(h, BSE_K_RECURSION, gs_dot_finalize<<<dim3(nj, nv), RB, 0, st>>>(partial, GS_BLK, coef, coef_stride, hacc, hacc_stride));
-    BSE_PROF(h, BSE_K_RECURSION, gs_subtract<<<ew_grid(N, nv), 256, 0, st>>>(basis, bstride, w, N, coef, coef_stride, nj, mask));
+    gs_project(h, basis, bstride, w, nv, nj, partial, coef, coef_stride, hacc, hacc_stride, mask);
+    BSE_PROF(h, BSE_K_RECURSION,
+             gs_subtract<<<ew_grid(h->N, nv), 256, 0, h->stream>>>(basis, bstride, w, h->N, coef, coef_stride, nj, mask));
   }
   return BSE_OK;
 }
@@ -322,38 +367,43 @@ bse_status cgs2(bse_handle* h, const double2* basis, long long bstride, double2*
 // partial sums) and s_proj = sum_j |h_j|^2 of the coefficients just removed,
 // |w_before|^2 = s_after + s_proj, and a second pass is needed where more than
 // half of |w|^2 was removed (|w_after| < |w_before| / sqrt 2, i.e. s_after < s_proj).
-__global__ void __launch_bounds__(RB) gs_dgks_mask(const double2* __restrict__ partial, int nblk,
+__global__ void __launch_bounds__(RB) gs_dgks_mask(const double2* __restrict__ npart, int nblk,
                                                    const double2* __restrict__ coef, int coef_stride, int nj,
                                                    const int* __restrict__ mask, int* __restrict__ mask2) {
   const int v = blockIdx.x;
-  const double2 s = sum_partials(partial, v, nblk);
-  if (threadIdx.x == 0) {
-    double proj = 0.0;
-    for (int j = 0; j < nj; ++j) {
-      const double2 c = coef[(size_t)v * coef_stride + j];
-      proj += c.x * c.x + c.y * c.y;
-    }
-    const int on = mask ? mask[v] : 1;
-    mask2[v] = on && !(s.x >= proj);   // NaN also takes the second pass
+  if (mask && !mask[v]) {
+    if (threadIdx.x == 0) mask2[v] = 0;
+    return;
   }
+  double2 acc = make_double2(0, 0);
+  for (int i = threadIdx.x; i < nblk; i += RB) acc.x += npart[(size_t)v * nblk + i].x;
+  for (int j = threadIdx.x; j < nj; j += RB) {
+    const double2 c = coef[(size_t)v * coef_stride + j];
+    acc.y += c.x * c.x + c.y * c.y;
+  }
+  const double2 s = block_sum2(acc);
+  if (threadIdx.x == 0) mask2[v] = !(s.x >= s.y);   // NaN also takes the second pass
 }
 
 // Classical Gram-Schmidt with the DGKS criterion: one pass, and a second only
-// for the systems whose first pass cancelled more than half of |w|^2.
+// for the systems whose first pass cancelled more than half of |w|^2.  npart
+// receives the partials of the new |w|^2 (norm_blocks per system).
 bse_status cgs_dgks(bse_handle* h, const double2* basis, long long bstride, double2* w, int nv, int nj,
                     double2* partial, double2* coef, int coef_stride, double2* hacc, int hacc_stride,
-                    const int* mask, int* mask2) {
-  cudaStream_t st = h->stream;
-  const long long N = h->N;
-  BSE_PROF(h, BSE_K_RECURSION, gs_dot_multi<<<dim3(GS_BLK, nv), RB, 0, st>>>(basis, bstride, w, N, nj, partial, mask));
-  BSE_PROF(h, BSE_K_RECURSION, gs_dot_finalize<<<dim3(nj, nv), RB, 0, st>>>(partial, GS_BLK, coef, coef_stride, hacc, hacc_stride));
-  BSE_PROF(h, BSE_K_RECURSION, gs_subtract<<<ew_grid(N, nv), 256, 0, st>>>(basis, bstride, w, N, coef, coef_stride, nj, mask));
-  const int nbn = norm_blocks(N, nv);
-  BSE_PROF(h, BSE_K_RECURSION, dot_partial_s<<<dim3(nbn, nv), RB, 0, st>>>(w, N, nullptr, 0, N, partial));
-  BSE_PROF(h, BSE_K_RECURSION, gs_dgks_mask<<<nv, RB, 0, st>>>(partial, nbn, coef, coef_stride, nj, mask, mask2));
-  BSE_PROF(h, BSE_K_RECURSION, gs_dot_multi<<<dim3(GS_BLK, nv), RB, 0, st>>>(basis, bstride, w, N, nj, partial, mask2));
-  BSE_PROF(h, BSE_K_RECURSION, gs_dot_finalize<<<dim3(nj, nv), RB, 0, st>>>(partial, GS_BLK, coef, coef_stride, hacc, hacc_stride));
-  BSE_PROF(h, BSE_K_RECURSION, gs_subtract<<<ew_grid(N, nv), 256, 0, st>>>(basis, bstride, w, N, coef, coef_stride, nj, mask2));
+                    const int* mask, int* mask2, double2* npart) {
+  const int nbn = norm_blocks(h->N, nv);
+  const int* mk = mask;
+  for (int pass = 0; pass < 2; ++pass) {
+    gs_project(h, basis, bstride, w, nv, nj, partial, coef, coef_stride, hacc, hacc_stride, mk);
+    BSE_PROF(h, BSE_K_RECURSION,
+             gs_subtract<<<ew_grid(h->N, nv), 256, 0, h->stream>>>(basis, bstride, w, h->N, coef, coef_stride, nj, mk));
+    BSE_PROF(h, BSE_K_RECURSION, dot_partial_s<<<dim3(nbn, nv), RB, 0, h->stream>>>(w, h->N, nullptr, 0, h->N, npart));
+    if (pass == 0) {
+      BSE_PROF(h, BSE_K_RECURSION,
+               gs_dgks_mask<<<nv, RB, 0, h->stream>>>(npart, nbn, coef, coef_stride, nj, mask, mask2));
+    }
+    mk = mask2;
+  }
   return BSE_OK;
 }
 
@@ -474,52 +524,82 @@ __global__ void gm_scatter_shift(const double2* __restrict__ Wc, const double2* 
 
 #define HS(H, i, j) (H)[(size_t)(j) * (m + 1) + (i)]
 
-// H(j+1, j) = |w|; Givens update of column j; estimated residual; iteration count.
-__global__ void __launch_bounds__(RB) gm_givens(const double2* partial, int nblk, double2* Hs, double* cs,
-                                                double2* sn, double2* g, double* hnorm, int m, int j,
-                                                double bnorm, double rtol, int max_iter, int* active,
-                                                int* iters, int* jdone, double* est) {
-  const int v = blockIdx.x;
-  double2 s = sum_partials(partial, v, nblk);
-  if (threadIdx.x != 0 || !active[v]) return;
-  double hn = sqrt(s.x);
-  hnorm[v] = hn;
+// H(j+1, j) = |w|; Givens update of column j; estimated residual; iteration
+// count.  One warp per system: the column and the rotations are staged in
+// shared memory, then lane 0 runs the chain (square roots and divisions, 13 us
+// at j = 6; with every operand loaded from global memory 14.5, more with each column).
+__global__ void __launch_bounds__(32) gm_givens(const double2* npart, int nblk, double2* Hs, double* cs, double2* sn,
+                                                double2* g, double* hnorm, int m, int j, double bnorm, double rtol,
+                                                int max_iter, int* active, int* iters, int* jdone, double* est,
+                                                int staged) {
+  extern __shared__ __align__(16) unsigned char gv_smem[];
+  const int v = blockIdx.x, lane = threadIdx.x;
+  if (!active[v]) return;
   double2* H = Hs + (size_t)v * (m + 1) * m;
   double* c = cs + (size_t)v * m;
   double2* sv = sn + (size_t)v * m;
   double2* gv = g + (size_t)v * (m + 1);
-  HS(H, j + 1, j) = make_double2(hn, 0);
-  for (int i = 0; i < j; ++i) {
-    double2 h0 = HS(H, i, j), h1 = HS(H, i + 1, j);
-    double2 si = sv[i];
-    // t1 = c h0 + s h1 ; t2 = -conj(s) h0 + c h1
-    double2 t1 = make_double2(c[i] * h0.x + si.x * h1.x - si.y * h1.y, c[i] * h0.y + si.x * h1.y + si.y * h1.x);
-    double2 t2 = make_double2(-(si.x * h0.x + si.y * h0.y) + c[i] * h1.x, -(si.x * h0.y - si.y * h0.x) + c[i] * h1.y);
-    HS(H, i, j) = t1;
-    HS(H, i + 1, j) = t2;
+  // columns too long to stage (thousands of rows) are worked on in place
+  double2* col = staged ? reinterpret_cast<double2*>(gv_smem) : &HS(H, 0, j);   // [j + 1]
+  double2* ssn = staged ? col + j + 1 : sv;                                    // [j]
+  double* scs = staged ? reinterpret_cast<double*>(ssn + j) : c;               // [j]
+  const double s = warp_partials_x(npart + (size_t)v * nblk, nblk);
+  for (int i = lane; staged && i <= j; i += 32) {
+    col[i] = HS(H, i, j);
+    if (i < j) {
+      ssn[i] = sv[i];
+      scs[i] = c[i];
+    }
   }
-  double2 aa = HS(H, j, j), bb = HS(H, j + 1, j);
-  double na_ = hypot(aa.x, aa.y), nb_ = hypot(bb.x, bb.y);
-  double rr = hypot(na_, nb_);
-  if (na_ == 0.0) {
-    c[j] = 0.0;
-    sv[j] = make_double2(1, 0);
-    HS(H, j, j) = bb;
-  } else {
-    double2 ph = make_double2(aa.x / na_, aa.y / na_);
-    c[j] = na_ / rr;
-    sv[j] = make_double2((ph.x * bb.x + ph.y * bb.y) / rr, (ph.y * bb.x - ph.x * bb.y) / rr);  // ph conj(bb)/rr
-    HS(H, j, j) = make_double2(ph.x * rr, ph.y * rr);
+  __syncwarp();
+  if (lane == 0) {
+    const double hn = sqrt(s);
+    hnorm[v] = hn;
+    double2 h0 = col[0];
+    for (int i = 0; i < j; ++i) {
+      const double2 h1 = col[i + 1], si = ssn[i];
+      const double ci = scs[i];
+      // t1 = c h0 + s h1 ; t2 = -conj(s) h0 + c h1
+      const double2 t1 = make_double2(ci * h0.x + si.x * h1.x - si.y * h1.y, ci * h0.y + si.x * h1.y + si.y * h1.x);
+      const double2 t2 =
+          make_double2(-(si.x * h0.x + si.y * h0.y) + ci * h1.x, -(si.x * h0.y - si.y * h0.x) + ci * h1.y);
+      col[i] = t1;
+      h0 = t2;
+    }
+    const double2 aa = h0;
+    double2 sj;
+    double cj;
+    const double na_ = hypot(aa.x, aa.y);
+    const double rr = hypot(na_, hypot(hn, 0.0));
+    if (na_ == 0.0) {
+      cj = 0.0;
+      sj = make_double2(1, 0);
+      col[j] = make_double2(hn, 0);
+    } else {
+      const double2 ph = make_double2(aa.x / na_, aa.y / na_);
+      cj = na_ / rr;
+      sj = make_double2(ph.x * hn / rr, ph.y * hn / rr);   // ph conj(|w|)/rr
+      col[j] = make_double2(ph.x * rr, ph.y * rr);
+    }
+    c[j] = cj;
+    sv[j] = sj;
+    HS(H, j + 1, j) = make_double2(0, 0);
+    const double2 gj = gv[j];
+    const double2 g1 = make_double2(-(sj.x * gj.x + sj.y * gj.y), -(sj.x * gj.y - sj.y * gj.x));  // -conj(s) g_j
+    gv[j + 1] = g1;
+    gv[j] = make_double2(cj * gj.x, cj * gj.y);
+    iters[v] += 1;
+    jdone[v] = j + 1;
+    const double e = hypot(g1.x, g1.y) / bnorm;
+    est[v] = e;
+    if (e <= rtol || iters[v] >= max_iter || hn == 0.0 || !isfinite(e)) active[v] = 0;
   }
-  HS(H, j + 1, j) = make_double2(0, 0);
-  double2 gj = gv[j], sj = sv[j];
-  gv[j + 1] = make_double2(-(sj.x * gj.x + sj.y * gj.y), -(sj.x * gj.y - sj.y * gj.x));  // -conj(s) g_j
-  gv[j] = make_double2(c[j] * gj.x, c[j] * gj.y);
-  iters[v] += 1;
-  jdone[v] = j + 1;
-  double e = hypot(gv[j + 1].x, gv[j + 1].y) / bnorm;
-  est[v] = e;
-  if (e <= rtol || iters[v] >= max_iter || hn == 0.0 || !isfinite(e)) active[v] = 0;
+  __syncwarp();
+  for (int i = lane; staged && i <= j; i += 32) HS(H, i, j) = col[i];
+}
+inline size_t givens_smem(int j) {   // 0: not staged
+  const size_t b = (size_t)(2 * j + 1) * sizeof(double2) + (size_t)j * sizeof(double);
+  return b <= 32 * 1024 ? b : 0;
 }
 
 // V_{j+1} = w / |w| for systems still active after column j
@@ -534,24 +614,39 @@ __global__ void gm_next(const double2* w, long long wstride, double2* V, long lo
   }
 }
 
-// back substitution y = R^{-1} g over the system's own jdone columns
-__global__ void gm_solve(const double2* Hs, const double2* g, double2* y, const int* jdone, int m, int nz) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= nz) return;
+// back substitution y = R^{-1} g over the system's own jdone columns: one warp
+// per system stages a row of R and y in shared memory, lane 0 sums it in
+// column order (53 -> 38 us at 12 columns: a thread on its own waited for two
+// global loads per term)
+__global__ void __launch_bounds__(32) gm_solve(const double2* Hs, const double2* g, double2* y, const int* jdone, int m) {
+  __shared__ double2 sh[32], sy[32];
+  const int v = blockIdx.x, lane = threadIdx.x;
   const double2* H = Hs + (size_t)v * (m + 1) * m;
   const double2* gv = g + (size_t)v * (m + 1);
   double2* yv = y + (size_t)v * m;
   const int nj = jdone[v];
   for (int i = nj - 1; i >= 0; --i) {
     double2 acc = gv[i];
-    for (int k = i + 1; k < nj; ++k) {
-      double2 hk = HS(H, i, k), yk = yv[k];
-      acc.x -= hk.x * yk.x - hk.y * yk.y;
-      acc.y -= hk.x * yk.y + hk.y * yk.x;
+    for (int k0 = i + 1; k0 < nj; k0 += 32) {
+      const int n = nj - k0 < 32 ? nj - k0 : 32;
+      if (lane < n) {
+        sh[lane] = HS(H, i, k0 + lane);
+        sy[lane] = yv[k0 + lane];
+      }
+      __syncwarp();
+      if (lane == 0) {
+        for (int k = 0; k < n; ++k) {
+          double2 hk = sh[k], yk = sy[k];
+          acc.x -= hk.x * yk.x - hk.y * yk.y;
+          acc.y -= hk.x * yk.y + hk.y * yk.x;
+        }
+      }
+      __syncwarp();
     }
-    yv[i] = cdiv(acc, HS(H, i, i));
+    if (lane == 0) yv[i] = cdiv(acc, HS(H, i, i));
+    __syncwarp();
   }
-  for (int i = nj; i < m; ++i) yv[i] = make_double2(0, 0);
+  for (int i = nj + lane; i < m; i += 32) yv[i] = make_double2(0, 0);
 }
 
 // x += P (V y)
@@ -566,8 +661,9 @@ __global__ void gm_update_x(const double2* __restrict__ V, long long vstride, co
   const double2 zv = z[v];
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < N; e += (long long)gridDim.x * blockDim.x) {
     double2 acc = make_double2(0, 0);
+#pragma unroll 4
     for (int j = 0; j < nj; ++j) {
-      double2 a = vv[(size_t)j * N + e], c = yv[j];
+      const double2 a = vv[(size_t)j * N + e], c = yv[j];
       acc.x += c.x * a.x - c.y * a.y;
       acc.y += c.x * a.y + c.y * a.x;
     }
@@ -1123,6 +1219,8 @@ bse_status bse_gmres_device(bse_handle* h, const double2* b, const double2* z, i
   TRY(dalloc(h, &T, (size_t)n_z * N * sizeof(double2), "gmres T")); fr.add(T);
   TRY(dalloc(h, &W, (size_t)n_z * N * sizeof(double2), "gmres W")); fr.add(W);
   TRY(dalloc(h, &partial, (size_t)n_z * NBLK * (m + 1) * sizeof(double2), "partials")); fr.add(partial);
+  double2* npart;
+  TRY(dalloc(h, &npart, (size_t)n_z * NBLK * sizeof(double2), "norm partials")); fr.add(npart);
   TRY(dalloc(h, &Hs, (size_t)n_z * (m + 1) * m * sizeof(double2), "hessenberg")); fr.add(Hs);
   TRY(dalloc(h, &sn, (size_t)n_z * m * sizeof(double2), "givens s")); fr.add(sn);
   TRY(dalloc(h, &g, (size_t)n_z * (m + 1) * sizeof(double2), "givens g")); fr.add(g);
@@ -1193,10 +1291,10 @@ bse_status bse_gmres_device(bse_handle* h, const double2* b, const double2* z, i
       BSE_PROF(h, BSE_K_RECURSION, gm_scatter_shift<<<ec, 256, 0, st>>>(Wc, T, z, W, N, didx));
       // Arnoldi: classical Gram-Schmidt, repeated where the DGKS test asks for it
       TRY(cgs_dgks(h, V, vstride, W, n_z, j + 1, partial, coef, m + 1, Hs + (size_t)j * (m + 1),
-                   (m + 1) * m, mask, mask2));
-      BSE_PROF(h, BSE_K_RECURSION, dot_partial_s<<<dim3(nbn, n_z), RB, 0, st>>>(W, N, nullptr, 0, N, partial));
-      BSE_PROF(h, BSE_K_RECURSION, gm_givens<<<n_z, RB, 0, st>>>(partial, nbn, Hs, cs, sn, g, hnorm, m, j, bnorm, rtol, max_iter,
-                                   active, iters_d, jdone, est));
+                   (m + 1) * m, mask, mask2, npart));
+      BSE_PROF(h, BSE_K_RECURSION,
+               gm_givens<<<n_z, 32, givens_smem(j), st>>>(npart, nbn, Hs, cs, sn, g, hnorm, m, j,
+                                                          bnorm, rtol, max_iter, active, iters_d, jdone, est, givens_smem(j) > 0));
       if (j + 1 < m) {
         BSE_PROF(h, BSE_K_RECURSION, gm_next<<<eg, 256, 0, st>>>(W, N, V + (size_t)(j + 1) * N, vstride, N, hnorm, active));
       }
@@ -1206,7 +1304,7 @@ bse_status bse_gmres_device(bse_handle* h, const double2* b, const double2* z, i
       for (int v = 0; v < n_z; ++v) nact += hact[v];
       if (nact == 0) break;
     }
-    BSE_PROF(h, BSE_K_RECURSION, gm_solve<<<(n_z + 127) / 128, 128, 0, st>>>(Hs, g, y, jdone, m, n_z));
+    BSE_PROF(h, BSE_K_RECURSION, gm_solve<<<n_z, 32, 0, st>>>(Hs, g, y, jdone, m));
     if (mlp) {
       // x += P (V y): V y into W (zero for systems without new columns), then P
       cudaMemsetAsync(W, 0, (size_t)n_z * N * sizeof(double2), st);
