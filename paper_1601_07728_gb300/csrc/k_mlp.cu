@@ -407,11 +407,43 @@ __global__ void to_half(const float* __restrict__ w, __half* __restrict__ w16, i
 }
 
 // ---- GMRES application of P = diag(p) + U V^H / N to packed vectors ----
-// part[s][blk][q] = sum_j conj(V_s,jq) x_s,j   (system of slot s = idx[s])
+// sums over a warp of v[0..15] by exchanging halves: lane L ends with sum
+// L >> 1 (the pairs of a butterfly per sum, at 16 additions per lane
+// instead of 80; an FP64 addition of a warp holds the pipe for 16 clocks)
+__device__ __forceinline__ double warp_sum16(double* v, int lane) {
+#pragma unroll
+  for (int h = 8; h >= 1; h >>= 1) {
+    const bool up = (lane & (2 * h)) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double mine = up ? v[h + i] : v[i], other = up ? v[i] : v[h + i];
+      v[i] = mine + __shfl_xor_sync(0xffffffffu, other, 2 * h);
+    }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+__device__ __forceinline__ void load_rank(const float2* __restrict__ p, float2* f) {   // RANK entries, 64-byte aligned
+#pragma unroll
+  for (int q = 0; q < RANK / 2; ++q) {
+    const float4 t = reinterpret_cast<const float4*>(p)[q];
+    f[2 * q] = make_float2(t.x, t.y);
+    f[2 * q + 1] = make_float2(t.z, t.w);
+  }
+}
+
+// part[s][blk][q] = sum_j conj(V_s,jq) x_s,j   (system of slot s = idx[s]); the
+// rows are dealt to NRED blocks of 256 threads whatever N is (the sums, and
+// with them a GMRES solve, keep their bits), blocks beyond the rows write zeros.
+// 16 systems of 12,288 rows: 100 -> 20 us, nearly all of it the warp sums' FP64 additions before.
 __global__ void __launch_bounds__(256) pc_apply_red(const double2* __restrict__ x, long long xstride,
                                                     const float2* __restrict__ V, long long fstride, long long N,
                                                     const int* __restrict__ idx, double2* __restrict__ part) {
   const int s = blockIdx.y, sys = idx ? idx[s] : s;
+  double* po = reinterpret_cast<double*>(part + ((size_t)s * gridDim.x + blockIdx.x) * RANK);
+  if ((long long)blockIdx.x * blockDim.x >= N) {
+    if (threadIdx.x < 2 * RANK) po[threadIdx.x] = 0.0;
+    return;
+  }
   const double2* xs = x + (size_t)(idx ? sys : s) * xstride;
   const float2* vs = V + (size_t)sys * fstride * N * RANK;
   // FP32 products and per-thread sums (V is FP32; FP64 here would make this
@@ -422,59 +454,57 @@ __global__ void __launch_bounds__(256) pc_apply_red(const double2* __restrict__ 
   for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (long long)gridDim.x * blockDim.x) {
     const double2 xd = xs[j];
     const float2 xx = make_float2((float)xd.x, (float)xd.y);
+    float2 vq[RANK];
+    load_rank(vs + j * RANK, vq);
 #pragma unroll
     for (int q = 0; q < RANK; ++q) {
-      const float2 vv = vs[j * RANK + q];
+      const float2 vv = vq[q];
       fr[q] += vv.x * xx.x + vv.y * xx.y;
       fi[q] += vv.x * xx.y - vv.y * xx.x;
     }
   }
-  double cr[RANK], ci[RANK];
+  double c[2 * RANK];
 #pragma unroll
   for (int q = 0; q < RANK; ++q) {
-    cr[q] = fr[q];
-    ci[q] = fi[q];
+    c[2 * q] = fr[q];
+    c[2 * q + 1] = fi[q];
   }
-  __shared__ double sr[8][RANK], si[8][RANK];
-#pragma unroll
-  for (int q = 0; q < RANK; ++q) {
-    for (int off = 16; off > 0; off >>= 1) {
-      cr[q] += __shfl_xor_sync(0xffffffffu, cr[q], off);
-      ci[q] += __shfl_xor_sync(0xffffffffu, ci[q], off);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      sr[threadIdx.x >> 5][q] = cr[q];
-      si[threadIdx.x >> 5][q] = ci[q];
-    }
-  }
+  __shared__ double sr[8][2 * RANK];
+  const int lane = threadIdx.x & 31;
+  const double w = warp_sum16(c, lane);
+  if ((lane & 1) == 0) sr[threadIdx.x >> 5][lane >> 1] = w;
   __syncthreads();
-  if (threadIdx.x < RANK) {
-    double a = 0, b = 0;
-    for (int w = 0; w < 8; ++w) {
-      a += sr[w][threadIdx.x];
-      b += si[w][threadIdx.x];
-    }
-    part[((size_t)s * gridDim.x + blockIdx.x) * RANK + threadIdx.x] = make_double2(a, b);
+  if (threadIdx.x < 2 * RANK) {
+    double t = 0;
+    for (int i = 0; i < 8; ++i) t += sr[i][threadIdx.x];
+    po[threadIdx.x] = t;
   }
 }
 
-// y_s = p (.) x_s + U c_s / N with c_s = sum_blk part[s][blk]; add != 0: y += (...)
-__global__ void pc_apply(const double2* __restrict__ x, long long xstride, long long fstride,
-                         const float2* __restrict__ pv,
-                         const float2* __restrict__ U, const double2* __restrict__ part, int nblk, long long N,
-                         const int* __restrict__ idx, double2* __restrict__ y, long long ystride, int add) {
-  const int s = blockIdx.y, sys = idx ? idx[s] : s;
-  __shared__ float2 c[RANK];
-  if (threadIdx.x < RANK) {
-    double a = 0, b = 0;
-    for (int blk = 0; blk < nblk; ++blk) {
-      const double2 v = part[((size_t)s * nblk + blk) * RANK + threadIdx.x];
-      a += v.x;
-      b += v.y;
-    }
-    c[threadIdx.x] = make_float2((float)(a / N), (float)(b / N));
-  }
+// c[s][q] = sum_blk part[s][blk][q] / N in block order, once per system (every
+// block of pc_apply used to run this chain on global loads: 78 -> 9 us there)
+__global__ void __launch_bounds__(256) pc_coef(const double2* __restrict__ part, long long N, float2* __restrict__ c) {
+  __shared__ double sp[NRED * 2 * RANK];
+  const double* p = reinterpret_cast<const double*>(part + (size_t)blockIdx.x * NRED * RANK);
+  for (int i = threadIdx.x; i < NRED * 2 * RANK; i += blockDim.x) sp[i] = p[i];
   __syncthreads();
+  if (threadIdx.x < 2 * RANK) {
+    double a = 0;
+#pragma unroll 8
+    for (int blk = 0; blk < NRED; ++blk) a += sp[blk * 2 * RANK + threadIdx.x];
+    reinterpret_cast<float*>(c + (size_t)blockIdx.x * RANK)[threadIdx.x] = (float)(a / N);
+  }
+}
+
+// y_s = p (.) x_s + U c_s / N; add != 0: y += (...)
+__global__ void __launch_bounds__(256) pc_apply(const double2* __restrict__ x, long long xstride, long long fstride,
+                                                const float2* __restrict__ pv, const float2* __restrict__ U,
+                                                const float2* __restrict__ coef, long long N,
+                                                const int* __restrict__ idx, double2* __restrict__ y,
+                                                long long ystride, int add) {
+  const int s = blockIdx.y, sys = idx ? idx[s] : s;
+  float2 c[RANK];
+  load_rank(coef + (size_t)s * RANK, c);
   const double2* xs = x + (size_t)(idx ? sys : s) * xstride;
   double2* ys = y + (size_t)s * ystride;
   const float2* ps = pv + (size_t)sys * fstride * N;
@@ -482,11 +512,13 @@ __global__ void pc_apply(const double2* __restrict__ x, long long xstride, long 
   for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (long long)gridDim.x * blockDim.x) {
     const double2 xx = xs[j];
     const float2 pp = ps[j];
+    float2 uq[RANK];
+    load_rank(us + j * RANK, uq);
     double rx = pp.x * xx.x - pp.y * xx.y, ry = pp.x * xx.y + pp.y * xx.x;
     float lx = 0.f, ly = 0.f;
 #pragma unroll
     for (int q = 0; q < RANK; ++q) {
-      const float2 uu = us[j * RANK + q];
+      const float2 uu = uq[q];
       lx += uu.x * c[q].x - uu.y * c[q].y;
       ly += uu.x * c[q].y + uu.y * c[q].x;
     }
@@ -1053,15 +1085,18 @@ bse_status bse_mlp_apply(bse_handle* h, const float2* p, const float2* u, const 
                          double2* part, long long fstride) {
   if (ns <= 0) return BSE_OK;
   const long long N = h->N;
+  float2* coef = reinterpret_cast<float2*>(part + (size_t)ns * NRED * RANK);   // [ns][RANK]
+  const long long nb = (N + 255) / 256;
   BSE_PROF(h, BSE_K_RECURSION,
            pc_apply_red<<<dim3(NRED, ns), 256, 0, h->stream>>>(x, xstride, v, fstride, N, idx, part));
+  BSE_PROF(h, BSE_K_RECURSION, pc_coef<<<ns, 256, 0, h->stream>>>(part, N, coef));
   BSE_PROF(h, BSE_K_RECURSION,
-           pc_apply<<<dim3(NRED, ns), 256, 0, h->stream>>>(x, xstride, fstride, p, u, part, NRED, N, idx, y, ystride,
-                                                           add));
+           pc_apply<<<dim3((unsigned)std::min<long long>(nb, 1184), ns), 256, 0, h->stream>>>(
+               x, xstride, fstride, p, u, coef, N, idx, y, ystride, add));
   return bse_cuda_check(h, cudaGetLastError(), "mlp apply");
 }
 
-size_t bse_mlp_apply_scratch(int ns) { return (size_t)ns * NRED * RANK * sizeof(double2); }
+size_t bse_mlp_apply_scratch(int ns) { return (size_t)ns * (NRED * RANK * sizeof(double2) + RANK * sizeof(float2)); }
 
 extern "C" {
 
