@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(RB) gs_dot_multi(const double2* __restrict__ b
   double acc[2 * GS_JB];
 #pragma unroll
   for (int q = 0; q < 2 * GS_JB; ++q) acc[q] = 0.0;
-  for (long long e = (long long)blockIdx.x * RB + threadIdx.x; e < N; e += (long long)GS_BLK * RB) {
+  for (long long e = (long long)blockIdx.x * RB + threadIdx.x; e < N; e += (long long)gridDim.x * RB) {
     const double2 b = wv[e];
     double2 a[GS_JB];
 #pragma unroll
@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(RB) gs_dot_multi(const double2* __restrict__ b
   if ((int)threadIdx.x < 2 * njg) {
     double t = 0.0;
     for (int i = 0; i < RB / 32; ++i) t += sred[i][threadIdx.x];
-    double* o = reinterpret_cast<double*>(partial + ((size_t)v * nj + j0 + (threadIdx.x >> 1)) * GS_BLK + blockIdx.x);
+    double* o = reinterpret_cast<double*>(partial + ((size_t)v * nj + j0 + (threadIdx.x >> 1)) * gridDim.x + blockIdx.x);
     o[threadIdx.x & 1] = t;
   }
 }
@@ -677,7 +677,35 @@ __global__ void gm_update_x(const double2* __restrict__ V, long long vstride, co
   }
 }
 
+// Inner products of several vectors with several bases for the k-step loss
+// (k_mlp.cu): MD_BLK blocks per vector whatever its length, block sums added in
+// order -- the loss solves a Gram system of condition 1e8, in which another
+// order of these sums shows in the sixth digit of the gradient.
+constexpr int MD_BLK = 128;
+__global__ void __launch_bounds__(256) multi_dot_finalize(const double2* __restrict__ partial, int nj,
+                                                          double2* __restrict__ out, long long ovs, long long ojs) {
+  __shared__ double sp[8][2 * MD_BLK];
+  const int v = blockIdx.y, w = threadIdx.x >> 5, lane = threadIdx.x & 31, j = blockIdx.x * 8 + w;
+  if (j >= nj) return;
+  const double* p = reinterpret_cast<const double*>(partial + ((size_t)v * nj + j) * MD_BLK);
+  for (int i = lane; i < 2 * MD_BLK; i += 32) sp[w][i] = p[i];
+  __syncwarp();
+  if (lane < 2) {
+    double t = 0.0;
+#pragma unroll 8
+    for (int i = 0; i < MD_BLK; ++i) t += sp[w][2 * i + lane];
+    reinterpret_cast<double*>(out + v * ovs + j * ojs)[lane] = t;
+  }
+}
 }  // namespace
+void bse_multi_dot(bse_handle* h, const double2* basis, long long vstride, long long jstride, const double2* w,
+                   long long wstride, int nv, int nj, double2* partial, double2* out, long long ovs, long long ojs) {
+  BSE_PROF(h, BSE_K_PREP,
+           gs_dot_multi<<<dim3(MD_BLK, (nj + GS_JB - 1) / GS_JB, nv), RB, 0, h->stream>>>(
+               basis, vstride, jstride, w, wstride, h->N, nj, partial, nullptr));
+  BSE_PROF(h, BSE_K_PREP,
+           multi_dot_finalize<<<dim3((nj + 7) / 8, nv), 256, 0, h->stream>>>(partial, nj, out, ovs, ojs));
+}
 
 // learned preconditioner (k_mlp.cu)
 bse_status bse_mlp_factors(bse_handle* h, bse_mlp* m, const double2* z_host, int n_z, float2* p, float2* u, float2* v);

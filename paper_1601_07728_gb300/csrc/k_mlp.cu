@@ -31,7 +31,7 @@ constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + F_IN * WID, OFF_W2 = OFF_B1 + WID, O
               OFF_W3 = OFF_B2 + WID, OFF_B3 = OFF_W3 + WID * F_OUT, NPARAM = OFF_B3 + F_OUT;
 constexpr int RB = 64;        // rows per dense-layer block
 constexpr int NRED = 128;     // blocks of the row reductions
-constexpr int WG_BLOCKS = 64; // blocks of the weight-gradient reduction
+constexpr int WG_BLOCKS = 152; // blocks of the weight-gradient reduction (one per SM)
 
 __device__ __forceinline__ float silu_f(float x) { return x / (1.f + __expf(-x)); }
 __device__ __forceinline__ float dsilu_f(float x) {
@@ -68,134 +68,181 @@ __global__ void mlp_features(const double* __restrict__ jdiag, const double* __r
   for (int q = 0; q < 6; ++q) x[6 + q] = (q == (a < 5 ? a : 5)) ? 1.f : 0.f;
 }
 
-// Z = X W + b (W [in][out] FP16), H = silu(Z) when H != nullptr.  64 rows per block.
-__global__ void __launch_bounds__(256) mlp_dense(const float* __restrict__ X, int in, const __half* __restrict__ W,
-                                                 const __half* __restrict__ b, int out, float* __restrict__ Z,
-                                                 float* __restrict__ H, int rows) {
+// Dense layers on tiles of 64 rows, weights staged in shared memory as FP32
+// once per block (a block walks several tiles), R rows x 4 columns per
+// thread: FP32-pipe bound, 16 FMAs per shared-memory load instead of 3, every
+// sum over k in ascending order.
+//   forward:  Z = X W + b (W [K][OUT] FP16), H = silu(Z) when H != nullptr
+//   backward: Z = (X W^T) * silu'(Zprev)     (X = dZ, W [OUT][K] FP16)
+// 12,288 rows, 128 x 128: forward 54 -> 24 us, backward 57 -> 32 us (192 tiles
+// on 152 SMs: loading the weights is half of it; it is spread over more tiles
+// on longer vectors).
+template <int OUT, bool BWD>
+constexpr int dense_ldw() {   // row length of the staged weights (backward: padded, they are written transposed)
+  return (OUT + 3) / 4 * 4 + (BWD ? 4 : 0);
+}
+template <int K, int OUT, int R, int NT, bool BWD>
+__global__ void __launch_bounds__(NT) mlp_dense(const float* __restrict__ X, const __half* __restrict__ W,
+                                                const __half* __restrict__ b, const float* __restrict__ Zprev,
+                                                float* __restrict__ Z, float* __restrict__ H, int rows) {
+  constexpr int KP = (K + 3) / 4 * 4, LD = KP + 4, NG = (OUT + 3) / 4, NRG = RB / R;
+  constexpr int OUTP = dense_ldw<OUT, BWD>();
+  static_assert(NG * NRG <= NT, "one thread per tile of R x 4 outputs");
   extern __shared__ __align__(16) float dsm[];
-  const int outp = (out + 3) & ~3;
-  float* Xs = dsm;             // [RB][in]
-  float* Ws = dsm + RB * in;   // [in][outp]
-  const int r0 = blockIdx.x * RB;
-  for (int e = threadIdx.x; e < RB * in; e += blockDim.x) {
-    const int r = e / in, k = e % in;
-    Xs[e] = (r0 + r < rows) ? X[(size_t)(r0 + r) * in + k] : 0.f;
-  }
-  for (int e = threadIdx.x; e < in * outp; e += blockDim.x) {
-    const int k = e / outp, o = e % outp;
-    Ws[e] = o < out ? __half2float(W[k * out + o]) : 0.f;
-  }
-  __syncthreads();
-  const int ng = outp / 4;
-  for (int idx = threadIdx.x; idx < RB * ng; idx += blockDim.x) {
-    const int r = idx / ng, cg = idx % ng;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    for (int k = 0; k < in; ++k) {
-      const float xv = Xs[r * in + k];
-      const float4 w4 = *reinterpret_cast<const float4*>(&Ws[k * outp + 4 * cg]);
-      a0 = fmaf(xv, w4.x, a0);
-      a1 = fmaf(xv, w4.y, a1);
-      a2 = fmaf(xv, w4.z, a2);
-      a3 = fmaf(xv, w4.w, a3);
+  float* Ws = dsm;               // [KP][OUTP], zero-padded
+  float* Xs = dsm + KP * OUTP;   // [RB][LD]
+  if constexpr (K % 8 == 0 && OUT % 8 == 0) {   // eight weights per load (rows of W are 16-byte aligned)
+    constexpr int IN8 = (BWD ? K : OUT) / 8, NROW = BWD ? OUT : K;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < NROW * IN8; e += NT) {
+      const int r = e / IN8, c = e % IN8 * 8;
+      const uint4 t = reinterpret_cast<const uint4*>(W)[e];
+      const __half2* hp = reinterpret_cast<const __half2*>(&t);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 f = __half22float2(hp[q]);
+        Ws[BWD ? (c + 2 * q) * OUTP + r : r * OUTP + c + 2 * q] = f.x;
+        Ws[BWD ? (c + 2 * q + 1) * OUTP + r : r * OUTP + c + 2 * q + 1] = f.y;
+      }
     }
-    const float acc[4] = {a0, a1, a2, a3};
-    if (r0 + r < rows) {
+  } else {
+    for (int e = threadIdx.x; e < KP * OUTP; e += NT) {
+      const int k = BWD ? e % KP : e / OUTP, o = BWD ? e / KP : e % OUTP;
+      Ws[k * OUTP + o] = k < K && o < OUT ? __half2float(BWD ? W[o * K + k] : W[k * OUT + o]) : 0.f;
+    }
+  }
+  const int cg = threadIdx.x % NG, rg = threadIdx.x / NG;
+  const bool on = rg < NRG;
+  for (int r0 = blockIdx.x * RB; r0 < rows; r0 += gridDim.x * RB) {
+    __syncthreads();
+    if constexpr (K % 4 == 0) {
+#pragma unroll 4
+      for (int e = threadIdx.x; e < RB * (K / 4); e += NT) {
+        const int r = e / (K / 4), k = e % (K / 4) * 4;
+        *reinterpret_cast<float4*>(&Xs[r * LD + k]) =
+            r0 + r < rows ? *reinterpret_cast<const float4*>(&X[(size_t)(r0 + r) * K + k]) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    } else {
+      for (int e = threadIdx.x; e < RB * KP; e += NT) {
+        const int r = e / KP, k = e % KP;
+        Xs[r * LD + k] = k < K && r0 + r < rows ? X[(size_t)(r0 + r) * K + k] : 0.f;
+      }
+    }
+    __syncthreads();
+    if (!on) continue;
+    float acc[R][4];
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[i][q] = 0.f;
+#pragma unroll 2
+    for (int k = 0; k < KP; k += 4) {
+      float4 w[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) w[t] = *reinterpret_cast<const float4*>(&Ws[(k + t) * OUTP + 4 * cg]);
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const float4 x = *reinterpret_cast<const float4*>(&Xs[(rg * R + i) * LD + k]);
+        const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          acc[i][0] = fmaf(xv[t], w[t].x, acc[i][0]);
+          acc[i][1] = fmaf(xv[t], w[t].y, acc[i][1]);
+          acc[i][2] = fmaf(xv[t], w[t].z, acc[i][2]);
+          acc[i][3] = fmaf(xv[t], w[t].w, acc[i][3]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = r0 + rg * R + i;
+      if (r >= rows) continue;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int col = 4 * cg + q;
-        if (col < out) {
-          const float zv = acc[q] + __half2float(b[col]);
-          Z[(size_t)(r0 + r) * out + col] = zv;
-          if (H) H[(size_t)(r0 + r) * out + col] = silu_f(zv);
+        if (col < OUT) {
+          const size_t o = (size_t)r * OUT + col;
+          if constexpr (BWD) {
+            Z[o] = acc[i][q] * dsilu_f(Zprev[o]);
+          } else {
+            const float zv = acc[i][q] + __half2float(b[col]);
+            Z[o] = zv;
+            if (H) H[o] = silu_f(zv);
+          }
         }
       }
     }
   }
 }
-
-// dX = dZ W^T, then dZprev = dX * silu'(Zprev):  dZ [rows][out], W [in][out] -> dZprev [rows][in]
-__global__ void __launch_bounds__(256) mlp_dense_bwd(const float* __restrict__ dZ, int out,
-                                                     const __half* __restrict__ W, int in,
-                                                     const float* __restrict__ Zprev, float* __restrict__ dZprev,
-                                                     int rows) {
-  extern __shared__ __align__(16) float dsm[];
-  const int inp = (in + 3) & ~3;
-  float* Ds = dsm;              // [RB][out]
-  float* Wt = dsm + RB * out;   // [out][inp] = W^T
-  const int r0 = blockIdx.x * RB;
-  for (int e = threadIdx.x; e < RB * out; e += blockDim.x) {
-    const int r = e / out, o = e % out;
-    Ds[e] = (r0 + r < rows) ? dZ[(size_t)(r0 + r) * out + o] : 0.f;
-  }
-  for (int e = threadIdx.x; e < out * inp; e += blockDim.x) {
-    const int o = e / inp, i = e % inp;
-    Wt[e] = i < in ? __half2float(W[i * out + o]) : 0.f;
-  }
-  __syncthreads();
-  const int ng = inp / 4;
-  for (int idx = threadIdx.x; idx < RB * ng; idx += blockDim.x) {
-    const int r = idx / ng, cg = idx % ng;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    for (int o = 0; o < out; ++o) {
-      const float dv = Ds[r * out + o];
-      const float4 w4 = *reinterpret_cast<const float4*>(&Wt[o * inp + 4 * cg]);
-      a0 = fmaf(dv, w4.x, a0);
-      a1 = fmaf(dv, w4.y, a1);
-      a2 = fmaf(dv, w4.z, a2);
-      a3 = fmaf(dv, w4.w, a3);
-    }
-    const float acc[4] = {a0, a1, a2, a3};
-    if (r0 + r < rows) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int col = 4 * cg + q;
-        if (col < in) {
-          const size_t o = (size_t)(r0 + r) * in + col;
-          dZprev[o] = acc[q] * dsilu_f(Zprev[o]);
-        }
-      }
-    }
-  }
+template <int K, int OUT, int R, int NT, bool BWD>
+void launch_dense(const float* X, const __half* W, const __half* b, const float* Zprev, float* Z, float* H, int rows,
+                  cudaStream_t st) {
+  constexpr int KP = (K + 3) / 4 * 4, OUTP = dense_ldw<OUT, BWD>();
+  constexpr size_t smem = (size_t)(KP * OUTP + RB * (KP + 4)) * sizeof(float);
+  cudaFuncSetAttribute(mlp_dense<K, OUT, R, NT, BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int tiles = (rows + RB - 1) / RB;   // two blocks per SM of 152 hold the widest layer
+  mlp_dense<K, OUT, R, NT, BWD><<<std::min(tiles, 304), NT, smem, st>>>(X, W, b, Zprev, Z, H, rows);
 }
 
-// part[blk][(in+1)*out]: sum over this block's rows of X[r][i] dZ[r][o] (i = in: bias, X = 1)
-constexpr int WG_PER = 65;   // outputs per thread (>= ceil(129*128/256))
-__global__ void __launch_bounds__(256) mlp_wgrad(const float* __restrict__ X, int in, const float* __restrict__ dZ,
-                                                 int out, int rows, float* __restrict__ part) {
-  __shared__ float Xs[32][WID + 1];
-  __shared__ float Ds[32][WID];
-  const int nout = (in + 1) * out;
-  float acc[WG_PER];
+// part[blk][(IN+1)*OUT]: sum over this block's rows of X[r][i] dZ[r][o] (i = IN:
+// bias, X = 1).  TI x TO outputs per thread from 32 staged rows at a time;
+// one block per SM.  12,288 rows, 128 x 128: 166 -> 34 us (one output per
+// thread and row took two shared-memory loads per FMA, on 64 blocks).
+template <int IN, int OUT, int TI, int TO>
+__global__ void __launch_bounds__(256) mlp_wgrad(const float* __restrict__ X, const float* __restrict__ dZ, int rows,
+                                                 float* __restrict__ part) {
+  constexpr int OUTP = (OUT + TO - 1) / TO * TO, GO = OUTP / TO, GI = IN / TI;
+  static_assert(IN % TI == 0 && GI * GO <= 256, "one thread per tile of outputs");
+  __shared__ __align__(16) float Xs[32][IN];
+  __shared__ __align__(16) float Ds[32][OUTP];
+  const int to = threadIdx.x % GO, ti = threadIdx.x / GO;
+  const bool on = ti < GI;
+  float acc[TI][TO], bias[TO];
 #pragma unroll
-  for (int j = 0; j < WG_PER; ++j) acc[j] = 0.f;
+  for (int j = 0; j < TO; ++j) {
+    bias[j] = 0.f;
+#pragma unroll
+    for (int i = 0; i < TI; ++i) acc[i][j] = 0.f;
+  }
   const int per = (rows + gridDim.x - 1) / gridDim.x;
   const int rbeg = blockIdx.x * per, rend = min(rows, rbeg + per);
   for (int c0 = rbeg; c0 < rend; c0 += 32) {
-    for (int e = threadIdx.x; e < 32 * (in + 1); e += blockDim.x) {
-      const int r = e / (in + 1), i = e % (in + 1);
-      Xs[r][i] = (c0 + r < rend) ? (i < in ? X[(size_t)(c0 + r) * in + i] : 1.f) : 0.f;
+    for (int e = threadIdx.x; e < 32 * IN; e += 256) {
+      const int r = e / IN;
+      Xs[r][e % IN] = c0 + r < rend ? X[(size_t)c0 * IN + e] : 0.f;
     }
-    for (int e = threadIdx.x; e < 32 * out; e += blockDim.x) {
-      const int r = e / out, o = e % out;
-      Ds[r][o] = (c0 + r < rend) ? dZ[(size_t)(c0 + r) * out + o] : 0.f;
+    for (int e = threadIdx.x; e < 32 * OUTP; e += 256) {
+      const int r = e / OUTP, o = e % OUTP;
+      Ds[r][o] = c0 + r < rend && o < OUT ? dZ[(size_t)(c0 + r) * OUT + o] : 0.f;
     }
     __syncthreads();
+    if (on) {
+#pragma unroll 2
+      for (int r = 0; r < 32; ++r) {
+        float x[TI], d[TO];
 #pragma unroll
-    for (int j = 0; j < WG_PER; ++j) {
-      const int e = threadIdx.x + 256 * j;
-      if (e < nout) {
-        const int i = e / out, o = e % out;
-        float s = acc[j];
-        for (int r = 0; r < 32; ++r) s = fmaf(Xs[r][i], Ds[r][o], s);
-        acc[j] = s;
+        for (int i = 0; i < TI; ++i) x[i] = Xs[r][ti * TI + i];
+#pragma unroll
+        for (int j = 0; j < TO; ++j) d[j] = Ds[r][to * TO + j];
+#pragma unroll
+        for (int j = 0; j < TO; ++j) {
+          bias[j] += d[j];
+#pragma unroll
+          for (int i = 0; i < TI; ++i) acc[i][j] = fmaf(x[i], d[j], acc[i][j]);
+        }
       }
     }
     __syncthreads();
   }
+  if (!on) return;
+  float* o = part + (size_t)blockIdx.x * (IN + 1) * OUT;
 #pragma unroll
-  for (int j = 0; j < WG_PER; ++j) {
-    const int e = threadIdx.x + 256 * j;
-    if (e < nout) part[(size_t)blockIdx.x * nout + e] = acc[j];
+  for (int j = 0; j < TO; ++j) {
+    const int col = to * TO + j;
+    if (col >= OUT) continue;
+#pragma unroll
+    for (int i = 0; i < TI; ++i) o[(ti * TI + i) * OUT + col] = acc[i][j];
+    if (ti == 0) o[IN * OUT + col] = bias[j];
   }
 }
 
@@ -206,6 +253,7 @@ __global__ void mlp_wgrad_reduce(const float* __restrict__ part, int nblk, int i
   const int nout = (in + 1) * out;
   if (e >= nout) return;
   float s = 0.f;
+#pragma unroll 8
   for (int b = 0; b < nblk; ++b) s += part[(size_t)b * nout + e];
   const int i = e / out, o = e % out;
   if (i < in)
@@ -231,128 +279,123 @@ __global__ void pc_assemble(const float* __restrict__ O, const double* __restric
   }
 }
 
-// block partials over rows of (sum_j conj(V_jq) r_tj  [q < 8],  sum_j |e_tj|^2): part[blk][t][9]
-__global__ void __launch_bounds__(256) pc_red_c(const float2* __restrict__ v, const double2* __restrict__ r,
-                                                const double2* __restrict__ e, int N, double2* __restrict__ part) {
-  const int t = blockIdx.y;
-  double cr[RANK + 1], ci[RANK + 1];
+// sums over a warp of v[0..15] by exchanging halves: lane L ends with sum
+// L >> 1 (the pairs of a butterfly per sum, at 16 additions per lane
+// instead of 80; an FP64 addition of a warp holds the pipe for 16 clocks)
+__device__ __forceinline__ double warp_sum16(double* v, int lane) {
 #pragma unroll
-  for (int q = 0; q <= RANK; ++q) cr[q] = ci[q] = 0.0;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
-    const double2 rr = r[(size_t)t * N + j], ee = e[(size_t)t * N + j];
+  for (int h = 8; h >= 1; h >>= 1) {
+    const bool up = (lane & (2 * h)) != 0;
 #pragma unroll
-    for (int q = 0; q < RANK; ++q) {
-      const float2 vv = v[(size_t)j * RANK + q];
-      cr[q] += vv.x * rr.x + vv.y * rr.y;
-      ci[q] += vv.x * rr.y - vv.y * rr.x;
-    }
-    cr[RANK] += ee.x * ee.x + ee.y * ee.y;
-  }
-  __shared__ double sr[8][RANK + 1], si[8][RANK + 1];
-#pragma unroll
-  for (int q = 0; q <= RANK; ++q) {
-    for (int off = 16; off > 0; off >>= 1) {
-      cr[q] += __shfl_xor_sync(0xffffffffu, cr[q], off);
-      ci[q] += __shfl_xor_sync(0xffffffffu, ci[q], off);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      sr[threadIdx.x >> 5][q] = cr[q];
-      si[threadIdx.x >> 5][q] = ci[q];
+    for (int i = 0; i < h; ++i) {
+      const double mine = up ? v[h + i] : v[i], other = up ? v[i] : v[h + i];
+      v[i] = mine + __shfl_xor_sync(0xffffffffu, other, 2 * h);
     }
   }
-  __syncthreads();
-  if (threadIdx.x <= RANK) {
-    double a = 0, b = 0;
-    for (int w = 0; w < 8; ++w) {
-      a += sr[w][threadIdx.x];
-      b += si[w][threadIdx.x];
-    }
-    part[((size_t)blockIdx.x * gridDim.y + t) * (RANK + 1) + threadIdx.x] = make_double2(a, b);
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+__device__ __forceinline__ void load_rank(const float2* __restrict__ p, float2* f) {   // RANK entries, 64-byte aligned
+#pragma unroll
+  for (int q = 0; q < RANK / 2; ++q) {
+    const float4 t = reinterpret_cast<const float4*>(p)[q];
+    f[2 * q] = make_float2(t.x, t.y);
+    f[2 * q + 1] = make_float2(t.z, t.w);
   }
 }
 
-// out[t][q] = sum_blk part[blk][t][q]
-__global__ void pc_red_finish(const double2* __restrict__ part, int nblk, int T, double2* __restrict__ out) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= T * (RANK + 1)) return;
+// Statistics of T vectors against the factor F (V or U): block partials over
+// rows of (sum_j conj(F_jq) x_tj [q < 8], sum_j |e_tj|^2), part[t][9][blk].
+// FP64-pipe bound (50 operations per row and vector); blocks cover at least
+// 1024 rows so that the block sums stay small beside it.  40 vectors of 12,288
+// rows: 300 -> 65 us.
+__global__ void __launch_bounds__(256) pc_red(const float2* __restrict__ F, const double2* __restrict__ x,
+                                              const double2* __restrict__ e, int N, double2* __restrict__ part) {
+  const int t = blockIdx.y;
+  double c[2 * RANK], e2 = 0.0;
+#pragma unroll
+  for (int q = 0; q < 2 * RANK; ++q) c[q] = 0.0;
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
+    const double2 rr = x[(size_t)t * N + j], ee = e[(size_t)t * N + j];
+    float2 f[RANK];
+    load_rank(F + (size_t)j * RANK, f);
+#pragma unroll
+    for (int q = 0; q < RANK; ++q) {
+      const double fx = f[q].x, fy = f[q].y;
+      c[2 * q] = fma(fx, rr.x, fma(fy, rr.y, c[2 * q]));
+      c[2 * q + 1] = fma(fx, rr.y, fma(-fy, rr.x, c[2 * q + 1]));
+    }
+    e2 = fma(ee.x, ee.x, fma(ee.y, ee.y, e2));
+  }
+  __shared__ double sr[8][2 * RANK + 1];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const double s = warp_sum16(c, lane);
+  for (int off = 16; off > 0; off >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, off);
+  if ((lane & 1) == 0) sr[w][lane >> 1] = s;
+  if (lane == 0) sr[w][2 * RANK] = e2;
+  __syncthreads();
+  if (threadIdx.x < 2 * (RANK + 1)) {
+    double a = 0;
+    if (threadIdx.x <= 2 * RANK)
+      for (int i = 0; i < 8; ++i) a += sr[i][threadIdx.x];
+    reinterpret_cast<double*>(part + ((size_t)t * (RANK + 1) + (threadIdx.x >> 1)) * gridDim.x +
+                              blockIdx.x)[threadIdx.x & 1] = a;
+  }
+}
+inline int pc_red_blocks(int N) { return std::min(NRED, (N + 1023) / 1024); }
+
+// out[e] = sum_blk part[e][blk], one warp per entry
+__global__ void __launch_bounds__(256) pc_red_finish(const double2* __restrict__ part, int nblk, int n,
+                                                     double2* __restrict__ out) {
+  const int e = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (e >= n) return;
   double a = 0, b = 0;
-  for (int blk = 0; blk < nblk; ++blk) {
-    const double2 v = part[(size_t)blk * T * (RANK + 1) + e];
+  for (int blk = lane; blk < nblk; blk += 32) {
+    const double2 v = part[(size_t)e * nblk + blk];
     a += v.x;
     b += v.y;
   }
-  out[e] = make_double2(a, b);
-}
-
-// partials of (lambda_tq = sum_j conj(U_jq) g_tj,  sum_j |q_tj|^2)
-__global__ void __launch_bounds__(256) pc_red_spai(const float2* __restrict__ u, const double2* __restrict__ G,
-                                                   const double2* __restrict__ Q, int N, double2* __restrict__ part) {
-  const int t = blockIdx.y;
-  double lr[RANK + 1], li[RANK + 1];
-#pragma unroll
-  for (int q = 0; q <= RANK; ++q) lr[q] = li[q] = 0.0;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N; j += gridDim.x * blockDim.x) {
-    const double2 gg = G[(size_t)t * N + j], qq = Q[(size_t)t * N + j];
-#pragma unroll
-    for (int q = 0; q < RANK; ++q) {
-      const float2 uu = u[(size_t)j * RANK + q];
-      lr[q] += uu.x * gg.x + uu.y * gg.y;   // conj(u) g
-      li[q] += uu.x * gg.y - uu.y * gg.x;
-    }
-    lr[RANK] += qq.x * qq.x + qq.y * qq.y;
+  for (int off = 16; off > 0; off >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, off);
+    b += __shfl_xor_sync(0xffffffffu, b, off);
   }
-  __shared__ double sr[8][RANK + 1], si[8][RANK + 1];
-#pragma unroll
-  for (int q = 0; q <= RANK; ++q) {
-    for (int off = 16; off > 0; off >>= 1) {
-      lr[q] += __shfl_xor_sync(0xffffffffu, lr[q], off);
-      li[q] += __shfl_xor_sync(0xffffffffu, li[q], off);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      sr[threadIdx.x >> 5][q] = lr[q];
-      si[threadIdx.x >> 5][q] = li[q];
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x <= RANK) {
-    double a = 0, b = 0;
-    for (int w = 0; w < 8; ++w) {
-      a += sr[w][threadIdx.x];
-      b += si[w][threadIdx.x];
-    }
-    part[((size_t)blockIdx.x * gridDim.y + t) * (RANK + 1) + threadIdx.x] = make_double2(a, b);
-  }
+  if (lane == 0) out[e] = make_double2(a, b);
 }
 
 // dO per row from T (vector r_t, adjoint g_t) pairs and their statistics (C:
 // V^H r and |r|^2, L: U^H g): g_p = sum_t w_t g_t conj(r_t), g_U = sum_t w_t
 // g_t c_t^H, g_V = sum_t w_t r_t lambda_t^H / N.  Weights: wts[t] when given,
 // else w_t = 2/|r_t|^2 (0 for |r_t|^2 <= r2_min).
-__global__ void pc_dout(const float2* __restrict__ p, const float2* __restrict__ u, const double2* __restrict__ C,
-                        const double2* __restrict__ L, const double2* __restrict__ r, const double2* __restrict__ G,
-                        int T, int N, double r2_min, const double* __restrict__ wts, float* __restrict__ dO) {
+// The statistics are brought to FP32 once per block (each thread used to
+// convert and divide them again for every t: 496 -> 39 us for 40 pairs of
+// 12,288 rows); 1/N of g_V is applied to the sum.
+constexpr int PC_TMAX = 64;   // pairs
+__global__ void __launch_bounds__(64) pc_dout(const float2* __restrict__ p, const double2* __restrict__ C,
+                                              const double2* __restrict__ L, const double2* __restrict__ r,
+                                              const double2* __restrict__ G, int T, int N, double r2_min,
+                                              const double* __restrict__ wts, float* __restrict__ dO) {
+  __shared__ float sw[PC_TMAX];
+  __shared__ float2 sc[PC_TMAX * RANK], sl[PC_TMAX * RANK];
+  for (int i = threadIdx.x; i < T * RANK; i += blockDim.x) {
+    const double2 cc = C[i / RANK * (RANK + 1) + i % RANK], ll = L[i / RANK * (RANK + 1) + i % RANK];
+    sc[i] = make_float2((float)(cc.x / N), (float)(cc.y / N));
+    sl[i] = make_float2((float)ll.x, (float)ll.y);
+  }
+  for (int t = threadIdx.x; t < T; t += blockDim.x) {
+    const double r2 = C[t * (RANK + 1) + RANK].x;
+    // residuals of an already converged solve carry no information
+    sw[t] = wts ? (float)wts[t] : r2 > r2_min ? (float)(2.0 / r2) : 0.f;
+  }
+  __syncthreads();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= N) return;
   const float2 pp = p[j];
   float gpx = 0.f, gpy = 0.f;
   float gux[RANK] = {0}, guy[RANK] = {0}, gvx[RANK] = {0}, gvy[RANK] = {0};
+#pragma unroll 2
   for (int t = 0; t < T; ++t) {
-    float w;
-    if (wts) {
-      w = (float)wts[t];
-      if (w == 0.f) continue;
-    } else {
-      const double r2 = C[t * (RANK + 1) + RANK].x;
-      if (!(r2 > r2_min)) continue;   // residuals of an already converged solve carry no information
-      w = (float)(2.0 / r2);
-    }
-    float2 c[RANK];
-#pragma unroll
-    for (int q = 0; q < RANK; ++q) {
-      const double2 cc = C[t * (RANK + 1) + q];
-      c[q] = make_float2((float)(cc.x / N), (float)(cc.y / N));
-    }
+    const float w = sw[t];
     const double2 rr = r[(size_t)t * N + j], gg = G[(size_t)t * N + j];
+    if (w == 0.f) continue;
     const float rx = (float)rr.x, ry = (float)rr.y;
     const float dx = (float)gg.x, dy = (float)gg.y;
     // g_p += w delta conj(r)
@@ -360,14 +403,13 @@ __global__ void pc_dout(const float2* __restrict__ p, const float2* __restrict__
     gpy += w * (dy * rx - dx * ry);
 #pragma unroll
     for (int q = 0; q < RANK; ++q) {
+      const float2 c = sc[t * RANK + q], l = sl[t * RANK + q];
       // g_u += w delta conj(c)
-      gux[q] += w * (dx * c[q].x + dy * c[q].y);
-      guy[q] += w * (dy * c[q].x - dx * c[q].y);
+      gux[q] += w * (dx * c.x + dy * c.y);
+      guy[q] += w * (dy * c.x - dx * c.y);
       // g_v += w r conj(lambda) / N
-      const double2 ll = L[t * (RANK + 1) + q];
-      const float lx = (float)ll.x, ly = (float)ll.y;
-      gvx[q] += w * (rx * lx + ry * ly) / N;
-      gvy[q] += w * (ry * lx - rx * ly) / N;
+      gvx[q] += w * (rx * l.x + ry * l.y);
+      gvy[q] += w * (ry * l.x - rx * l.y);
     }
   }
   // gs = conj(g_p) p^2
@@ -380,8 +422,8 @@ __global__ void pc_dout(const float2* __restrict__ p, const float2* __restrict__
   for (int q = 0; q < RANK; ++q) {
     d[2 + q] = gux[q];
     d[2 + RANK + q] = guy[q];
-    d[2 + 2 * RANK + q] = gvx[q];
-    d[2 + 3 * RANK + q] = gvy[q];
+    d[2 + 2 * RANK + q] = gvx[q] / N;
+    d[2 + 3 * RANK + q] = gvy[q] / N;
   }
 }
 
@@ -407,34 +449,10 @@ __global__ void to_half(const float* __restrict__ w, __half* __restrict__ w16, i
 }
 
 // ---- GMRES application of P = diag(p) + U V^H / N to packed vectors ----
-// sums over a warp of v[0..15] by exchanging halves: lane L ends with sum
-// L >> 1 (the pairs of a butterfly per sum, at 16 additions per lane
-// instead of 80; an FP64 addition of a warp holds the pipe for 16 clocks)
-__device__ __forceinline__ double warp_sum16(double* v, int lane) {
-#pragma unroll
-  for (int h = 8; h >= 1; h >>= 1) {
-    const bool up = (lane & (2 * h)) != 0;
-#pragma unroll
-    for (int i = 0; i < h; ++i) {
-      const double mine = up ? v[h + i] : v[i], other = up ? v[i] : v[h + i];
-      v[i] = mine + __shfl_xor_sync(0xffffffffu, other, 2 * h);
-    }
-  }
-  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
-}
-__device__ __forceinline__ void load_rank(const float2* __restrict__ p, float2* f) {   // RANK entries, 64-byte aligned
-#pragma unroll
-  for (int q = 0; q < RANK / 2; ++q) {
-    const float4 t = reinterpret_cast<const float4*>(p)[q];
-    f[2 * q] = make_float2(t.x, t.y);
-    f[2 * q + 1] = make_float2(t.z, t.w);
-  }
-}
-
 // part[s][blk][q] = sum_j conj(V_s,jq) x_s,j   (system of slot s = idx[s]); the
 // rows are dealt to NRED blocks of 256 threads whatever N is (the sums, and
 // with them a GMRES solve, keep their bits), blocks beyond the rows write zeros.
-// 16 systems of 12,288 rows: 100 -> 20 us, nearly all of it the warp sums' FP64 additions before.
+// 16 systems of 12,288 rows: 100 -> 19 us, nearly all of it the warp sums' FP64 additions before.
 __global__ void __launch_bounds__(256) pc_apply_red(const double2* __restrict__ x, long long xstride,
                                                     const float2* __restrict__ V, long long fstride, long long N,
                                                     const int* __restrict__ idx, double2* __restrict__ part) {
@@ -482,7 +500,7 @@ __global__ void __launch_bounds__(256) pc_apply_red(const double2* __restrict__ 
 }
 
 // c[s][q] = sum_blk part[s][blk][q] / N in block order, once per system (every
-// block of pc_apply used to run this chain on global loads: 78 -> 9 us there)
+// block of pc_apply used to run this chain on global loads: 78 us there, 8 now)
 __global__ void __launch_bounds__(256) pc_coef(const double2* __restrict__ part, long long N, float2* __restrict__ c) {
   __shared__ double sp[NRED * 2 * RANK];
   const double* p = reinterpret_cast<const double*>(part + (size_t)blockIdx.x * NRED * RANK);
@@ -556,6 +574,9 @@ struct bse_mlp {
 bse_status bse_mlp_apply(bse_handle* h, const float2* p, const float2* u, const float2* v, const double2* x,
                          long long xstride, int ns, const int* idx, double2* y, long long ystride, int add,
                          double2* part, long long fstride);
+// out[v ovs + j ojs] = <basis_v,j | w_v> for j < nj (k_krylov.cu); partial holds nv * nj * 128 entries
+void bse_multi_dot(bse_handle* h, const double2* basis, long long vstride, long long jstride, const double2* w,
+                   long long wstride, int nv, int nj, double2* partial, double2* out, long long ovs, long long ojs);
 
 namespace {
 
@@ -611,8 +632,6 @@ bse_status ensure_rows(bse_handle* h, bse_mlp* m, size_t rows, Act* a) {
   return BSE_OK;
 }
 
-size_t dense_smem(int in, int out) { return (size_t)(RB * in + in * ((out + 3) & ~3)) * sizeof(float); }
-
 bse_status ensure_anorm(bse_handle* h) {
   if (h->mlp_anorm || h->np == 0) return BSE_OK;
   const int nkb = h->nk * h->nb;
@@ -630,22 +649,13 @@ bse_status forward(bse_handle* h, bse_mlp* m, double omega, double gamma, Act* a
   BSE_PROF(h, BSE_K_PREP,
            mlp_features<<<(N + 255) / 256, 256, 0, st>>>(h->jdiag, h->e_nk, h->chi, h->mlp_anorm, h->na,
                                                          h->nk * h->nb, omega, gamma, a->X));
-  const int g = (N + RB - 1) / RB;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(mlp_dense, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dense_smem(WID, WID));
-    cudaFuncSetAttribute(mlp_dense_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dense_smem(WID, WID));
-    attr = true;
-  }
   BSE_PROF(h, BSE_K_PREP,
-           mlp_dense<<<g, 256, dense_smem(F_IN, WID), st>>>(a->X, F_IN, m->w16 + OFF_W1, m->w16 + OFF_B1, WID, a->Z1,
-                                                            a->H1, N));
+           (launch_dense<F_IN, WID, 8, 256, false>(a->X, m->w16 + OFF_W1, m->w16 + OFF_B1, nullptr, a->Z1, a->H1, N, st)));
   BSE_PROF(h, BSE_K_PREP,
-           mlp_dense<<<g, 256, dense_smem(WID, WID), st>>>(a->H1, WID, m->w16 + OFF_W2, m->w16 + OFF_B2, WID, a->Z2,
-                                                           a->H2, N));
+           (launch_dense<WID, WID, 8, 256, false>(a->H1, m->w16 + OFF_W2, m->w16 + OFF_B2, nullptr, a->Z2, a->H2, N, st)));
   BSE_PROF(h, BSE_K_PREP,
-           mlp_dense<<<g, 256, dense_smem(WID, F_OUT), st>>>(a->H2, WID, m->w16 + OFF_W3, m->w16 + OFF_B3, F_OUT,
-                                                             a->O, nullptr, N));
+           (launch_dense<WID, F_OUT, 4, 160, false>(a->H2, m->w16 + OFF_W3, m->w16 + OFF_B3, nullptr, a->O, nullptr, N,
+                                                    st)));
   return bse_cuda_check(h, cudaGetLastError(), "mlp forward");
 }
 
@@ -669,66 +679,6 @@ __global__ void spai_g(double2* __restrict__ G, const double2* __restrict__ Q, d
 
 // ---- k-step minimal-residual loss ----
 constexpr int KMAX = 16;   // largest number of Krylov steps of the loss
-
-// partials of <Y_i, Y_j> (i = 0..j) per probe t for one j: part[blk][t][i][j], Y [(k+1)][T][N]
-template <int NI>
-__global__ void __launch_bounds__(256) ks_dots(const double2* __restrict__ Y, int T, int N, int j, int k,
-                                               double2* __restrict__ part) {
-  const int t = blockIdx.y;
-  double ar[NI], ai[NI];
-#pragma unroll
-  for (int i = 0; i < NI; ++i) ar[i] = ai[i] = 0.0;
-  const size_t tn = (size_t)T * N;
-  const double2* yj = Y + (size_t)j * tn + (size_t)t * N;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < N; e += gridDim.x * blockDim.x) {
-    const double2 b = yj[e];
-#pragma unroll
-    for (int i = 0; i < NI; ++i) {
-      if (i <= j) {
-        const double2 a = Y[(size_t)i * tn + (size_t)t * N + e];
-        ar[i] += a.x * b.x + a.y * b.y;   // conj(a) b
-        ai[i] += a.x * b.y - a.y * b.x;
-      }
-    }
-  }
-  __shared__ double sr[8][NI], si[8][NI];
-#pragma unroll
-  for (int i = 0; i < NI; ++i) {
-    for (int off = 16; off > 0; off >>= 1) {
-      ar[i] += __shfl_xor_sync(0xffffffffu, ar[i], off);
-      ai[i] += __shfl_xor_sync(0xffffffffu, ai[i], off);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      sr[threadIdx.x >> 5][i] = ar[i];
-      si[threadIdx.x >> 5][i] = ai[i];
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x <= j && threadIdx.x < NI) {
-    double a = 0, b = 0;
-    for (int w = 0; w < 8; ++w) {
-      a += sr[w][threadIdx.x];
-      b += si[w][threadIdx.x];
-    }
-    part[(((size_t)blockIdx.x * T + t) * (k + 1) + threadIdx.x) * (k + 1) + j] = make_double2(a, b);
-  }
-}
-
-// gram[t][i][j] = sum_blk part[blk][t][i][j] for i <= j (fixed order)
-__global__ void ks_dots_finish(const double2* __restrict__ part, int nblk, int T, int k, double2* __restrict__ gram) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  const int per = (k + 1) * (k + 1);
-  if (e >= T * per) return;
-  const int i = (e % per) / (k + 1), j = e % (k + 1);
-  if (i > j) return;
-  double a = 0, b = 0;
-  for (int blk = 0; blk < nblk; ++blk) {
-    const double2 v = part[(size_t)blk * T * per + e];
-    a += v.x;
-    b += v.y;
-  }
-  gram[e] = make_double2(a, b);
-}
 
 // out_t = (x0 ? x0_t : 0) + sum_{i < n} coef[t][i] X_i,t   (X_i,t = X + i*xs + t*N; coef [T][KMAX])
 __global__ void ks_lincomb(double2* __restrict__ out, const double2* __restrict__ x0, const double2* __restrict__ X,
@@ -774,20 +724,19 @@ bse_status apply_h_chunks(bse_handle* h, const double2* in, double2* out, int n)
 bse_status backward(bse_handle* h, bse_mlp* m, const Act& a) {
   cudaStream_t st = h->stream;
   const int N = (int)h->N;
-  const int g = (N + RB - 1) / RB;
-  BSE_PROF(h, BSE_K_PREP, mlp_wgrad<<<WG_BLOCKS, 256, 0, st>>>(a.H2, WID, a.dO, F_OUT, N, m->wpart));
+  BSE_PROF(h, BSE_K_PREP, (mlp_wgrad<WID, F_OUT, 8, 4><<<WG_BLOCKS, 256, 0, st>>>(a.H2, a.dO, N, m->wpart)));
   BSE_PROF(h, BSE_K_PREP,
            mlp_wgrad_reduce<<<((WID + 1) * F_OUT + 255) / 256, 256, 0, st>>>(m->wpart, WG_BLOCKS, WID, F_OUT, m->g,
                                                                               OFF_W3, OFF_B3));
   BSE_PROF(h, BSE_K_PREP,
-           mlp_dense_bwd<<<g, 256, dense_smem(F_OUT, WID), st>>>(a.dO, F_OUT, m->w16 + OFF_W3, WID, a.Z2, a.dA, N));
-  BSE_PROF(h, BSE_K_PREP, mlp_wgrad<<<WG_BLOCKS, 256, 0, st>>>(a.H1, WID, a.dA, WID, N, m->wpart));
+           (launch_dense<F_OUT, WID, 8, 256, true>(a.dO, m->w16 + OFF_W3, nullptr, a.Z2, a.dA, nullptr, N, st)));
+  BSE_PROF(h, BSE_K_PREP, (mlp_wgrad<WID, WID, 8, 8><<<WG_BLOCKS, 256, 0, st>>>(a.H1, a.dA, N, m->wpart)));
   BSE_PROF(h, BSE_K_PREP,
            mlp_wgrad_reduce<<<((WID + 1) * WID + 255) / 256, 256, 0, st>>>(m->wpart, WG_BLOCKS, WID, WID, m->g,
                                                                             OFF_W2, OFF_B2));
   BSE_PROF(h, BSE_K_PREP,
-           mlp_dense_bwd<<<g, 256, dense_smem(WID, WID), st>>>(a.dA, WID, m->w16 + OFF_W2, WID, a.Z1, a.dB, N));
-  BSE_PROF(h, BSE_K_PREP, mlp_wgrad<<<WG_BLOCKS, 256, 0, st>>>(a.X, F_IN, a.dB, WID, N, m->wpart));
+           (launch_dense<WID, WID, 8, 256, true>(a.dA, m->w16 + OFF_W2, nullptr, a.Z1, a.dB, nullptr, N, st)));
+  BSE_PROF(h, BSE_K_PREP, (mlp_wgrad<F_IN, WID, 6, 1><<<WG_BLOCKS, 256, 0, st>>>(a.X, a.dB, N, m->wpart)));
   BSE_PROF(h, BSE_K_PREP,
            mlp_wgrad_reduce<<<((F_IN + 1) * WID + 255) / 256, 256, 0, st>>>(m->wpart, WG_BLOCKS, F_IN, WID, m->g,
                                                                              OFF_W1, OFF_B1));
@@ -839,12 +788,13 @@ bse_status loss_grad_spai(bse_handle* h, bse_mlp* m, double omega, double gamma,
   BSE_PROF(h, BSE_K_PREP, spai_g<<<ge, 256, 0, st>>>(G, Q, omega, gamma, tn));
   double2* C = m->stats;
   double2* L = m->stats + T * (RANK + 1);
-  BSE_PROF(h, BSE_K_PREP, pc_red_c<<<dim3(NRED, T), 256, 0, st>>>(v, r, r, N, part));
-  BSE_PROF(h, BSE_K_PREP, pc_red_finish<<<1, 256, 0, st>>>(part, NRED, T, C));
-  BSE_PROF(h, BSE_K_PREP, pc_red_spai<<<dim3(NRED, T), 256, 0, st>>>(u, G, Q, N, part));
-  BSE_PROF(h, BSE_K_PREP, pc_red_finish<<<1, 256, 0, st>>>(part, NRED, T, L));
+  const int nrb = pc_red_blocks(N), ns = T * (RANK + 1);
+  BSE_PROF(h, BSE_K_PREP, pc_red<<<dim3(nrb, T), 256, 0, st>>>(v, r, r, N, part));
+  BSE_PROF(h, BSE_K_PREP, pc_red_finish<<<(ns + 7) / 8, 256, 0, st>>>(part, nrb, ns, C));
+  BSE_PROF(h, BSE_K_PREP, pc_red<<<dim3(nrb, T), 256, 0, st>>>(u, G, Q, N, part));
+  BSE_PROF(h, BSE_K_PREP, pc_red_finish<<<(ns + 7) / 8, 256, 0, st>>>(part, nrb, ns, L));
   BSE_PROF(h, BSE_K_PREP,
-           pc_dout<<<(N + 255) / 256, 256, 0, st>>>(p, u, C, L, r, G, T, N, r2_min, nullptr, a.dO));
+           pc_dout<<<(N + 63) / 64, 64, 0, st>>>(p, C, L, r, G, T, N, r2_min, nullptr, a.dO));
   if ((s = backward(h, m, a)) != BSE_OK) return s;
   if (loss_out) {
     std::vector<double2> hs(2 * T * (RANK + 1));
@@ -963,10 +913,9 @@ bse_status loss_grad_krylov(bse_handle* h, bse_mlp* m, double omega, double gamm
     BSE_PROF(h, BSE_K_PREP, ks_shift<<<ge, 256, 0, st>>>(Y + (size_t)i * tn, Tt, omega, gamma, tn));
   }
   // Gram matrix <Y_i, Y_j>, 0 <= i <= j <= k
-  for (int j = 0; j <= k; ++j)
-    BSE_PROF(h, BSE_K_PREP, ks_dots<KMAX + 1><<<dim3(NRED, T), 256, 0, st>>>(Y, T, N, j, k, part));
   double2* gram = m->stats;   // [T][k+1][k+1]
-  BSE_PROF(h, BSE_K_PREP, ks_dots_finish<<<(T * per + 255) / 256, 256, 0, st>>>(part, NRED, T, k, gram));
+  for (int j = 0; j <= k; ++j)
+    bse_multi_dot(h, Y, N, (long long)tn, Y + (size_t)j * tn, N, T, j + 1, part, gram + j, per, k + 1);
   std::vector<double2> hg((size_t)T * per);
   s = bse_cuda_check(h, cudaMemcpyAsync(hg.data(), gram, hg.size() * sizeof(double2), cudaMemcpyDeviceToHost, st),
                      "gram");
@@ -1041,12 +990,13 @@ bse_status loss_grad_krylov(bse_handle* h, bse_mlp* m, double omega, double gamm
   if (s != BSE_OK) return s;
   double2* C = m->stats + (size_t)T * per + (size_t)T * KMAX + TT;   // after the weights (TT doubles)
   double2* L = C + (size_t)TT * (RANK + 1);
-  BSE_PROF(h, BSE_K_PREP, pc_red_c<<<dim3(NRED, TT), 256, 0, st>>>(v, Y, Y, N, part));
-  BSE_PROF(h, BSE_K_PREP, pc_red_finish<<<(TT * (RANK + 1) + 255) / 256, 256, 0, st>>>(part, NRED, TT, C));
-  BSE_PROF(h, BSE_K_PREP, pc_red_spai<<<dim3(NRED, TT), 256, 0, st>>>(u, GJ, GJ, N, part));
-  BSE_PROF(h, BSE_K_PREP, pc_red_finish<<<(TT * (RANK + 1) + 255) / 256, 256, 0, st>>>(part, NRED, TT, L));
+  const int nrb = pc_red_blocks(N), ns = TT * (RANK + 1);
+  BSE_PROF(h, BSE_K_PREP, pc_red<<<dim3(nrb, TT), 256, 0, st>>>(v, Y, Y, N, part));
+  BSE_PROF(h, BSE_K_PREP, pc_red_finish<<<(ns + 7) / 8, 256, 0, st>>>(part, nrb, ns, C));
+  BSE_PROF(h, BSE_K_PREP, pc_red<<<dim3(nrb, TT), 256, 0, st>>>(u, GJ, GJ, N, part));
+  BSE_PROF(h, BSE_K_PREP, pc_red_finish<<<(ns + 7) / 8, 256, 0, st>>>(part, nrb, ns, L));
   BSE_PROF(h, BSE_K_PREP,
-           pc_dout<<<(N + 255) / 256, 256, 0, st>>>(p, u, C, L, Y, GJ, TT, N, 0.0, dwts, a.dO));
+           pc_dout<<<(N + 63) / 64, 64, 0, st>>>(p, C, L, Y, GJ, TT, N, 0.0, dwts, a.dO));
   if ((s = backward(h, m, a)) != BSE_OK) return s;
   s = bse_cuda_check(h, cudaStreamSynchronize(st), "loss/grad sync");
   if (s != BSE_OK) return s;
