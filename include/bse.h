@@ -66,7 +66,8 @@ typedef enum {
  * lines).  The Haydock / GMRES recursion, inner products, diagonal, spin-orbit
  * and short-range terms are FP64 in every mode. */
 typedef enum {
-  BSE_PREC_FP64 = 0,        /* u complex128, FP64 FMA: the plain form                 */
+  BSE_PREC_FP64 = 0,        /* u complex128, sums to FP64 accuracy: FP64 FMAs, or exactly
+                               split FP16 tensor-core products where they are faster  */
   BSE_PREC_FP32 = 1,        /* u complex64, FP32 FMA, FP32 k-transforms               */
   BSE_PREC_SPLIT_BF16 = 2   /* u split into bf16 hi+lo, tcgen05 tensor-core MMAs with
                                3 products (hi*hi + hi*lo + lo*hi), FP32 accumulation */

@@ -117,6 +117,7 @@ void free_handle(bse_handle* h) {
   for (void* p : ptrs)
     if (p) cudaFree(p);
   bse_tc_free(h);
+  bse_ozh_free(h);
   if (h->io_in) cudaFree(h->io_in);
   if (h->io_out) cudaFree(h->io_out);
   if (h->ws) cudaFree(h->ws);

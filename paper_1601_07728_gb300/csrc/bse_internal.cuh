@@ -105,6 +105,9 @@ struct bse_handle {
   int op_max_vec = 0;          // one pass: largest n_vec it takes (0: none)
   bool concurrent = false;     // kernels of other handles may run beside this one's (many-site graph)
 
+  // tensor-core form of the FP64 contractions (k_ozh.cu), nullptr where not used
+  void* ozh = nullptr;
+
   // grow-only device workspace of the Haydock driver (kept between calls)
   void* ws = nullptr;
   size_t ws_cap = 0;
@@ -258,6 +261,14 @@ bse_operand_out bse_tc_operand(const bse_handle* h);
 bse_status bse_apply_device(bse_handle* h, const double2* psi, double2* hpsi, int n_vec,
                             const bse_dotfuse* fuse = nullptr);
 bool bse_apply_fuses_dot(const bse_handle* h);
+
+// FP64 form on the tensor cores by exact splitting (k_ozh.cu)
+void bse_ozh_prepare(bse_handle* h);   // sets h->ozh where it applies
+bool bse_ozh_takes(const bse_handle* h, int nc);   // nc columns are worth its launches
+void bse_ozh_free(bse_handle* h);
+bse_status bse_ozh_band_to_grid(bse_handle* h, const double2* psi, int nc);
+bse_status bse_ozh_grid_to_band(bse_handle* h, const double2* psi, double2* hpsi, int nc);
+bse_status bse_ozh_status(bse_handle* h);
 
 // tensor-core band<->grid path (k_tc.cu)
 bse_status bse_tc_prepare(bse_handle* h);

@@ -1,5 +1,5 @@
-// H psi on the device: SIMT band<->grid contractions (FP64 and FP32 forms)
-// and the short-range projector terms.
+// H psi on the device: the band<->grid contractions of the FP32 form and of
+// small FP64 problems, and the short-range projector terms.
 //
 // Algorithm 1 (Sec. 3.2.1), with the loop over x and alpha turned inside out:
 //   band->grid  phi[k][c][x]  = sum_n  U[k][x][n] psi[c][k][n]   (U = e^{ik.x} u)
@@ -159,6 +159,104 @@ __global__ void __launch_bounds__(256) g2b_simt(
 }
 
 // ---------------------------------------------------------------------------
+// FP64 contractions on the FP64 pipe: small problems, where the tensor-core
+// form's six launches cost more than the sums, and handles without that form.
+// CC columns per pass (the smallest of 1, 2, 4, 6, 8 that holds them: a column
+// that is not there costs as much as one that is).
+// band -> grid: four lanes per grid row, 32 rows per block
+// ---------------------------------------------------------------------------
+constexpr int D_N = 64;   // bands staged at a time
+template <int CC>
+__global__ void __launch_bounds__(128) b2g_fp64(const double2* __restrict__ U, const double2* __restrict__ psi,
+                                                double2* __restrict__ phi, int nk, int nx, int nb, int c0, int ncc,
+                                                int nc_total) {
+  __shared__ double2 Ps[CC][D_N];
+  const int row = threadIdx.x >> 2, l = threadIdx.x & 3, k = blockIdx.y, x = blockIdx.x * 32 + row;
+  const double2* Ux = U + ((size_t)k * nx + (x < nx ? x : 0)) * nb;
+  double2 acc[CC];
+#pragma unroll
+  for (int c = 0; c < CC; ++c) acc[c] = make_double2(0.0, 0.0);
+  for (int n0 = 0; n0 < nb; n0 += D_N) {
+    const int nn = nb - n0 < D_N ? nb - n0 : D_N;
+    __syncthreads();
+    for (int e = threadIdx.x; e < CC * D_N; e += 128) {
+      const int c = e / D_N, j = e % D_N;
+      Ps[c][j] = c < ncc && j < nn ? psi[((size_t)(c0 + c) * nk + k) * nb + n0 + j] : make_double2(0.0, 0.0);
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int j = l; j < nn; j += 4) {
+      const double2 u = Ux[n0 + j];
+#pragma unroll
+      for (int c = 0; c < CC; ++c) cmac(acc[c], u, Ps[c][j]);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < CC; ++c)
+#pragma unroll
+    for (int off = 1; off < 4; off <<= 1) {
+      acc[c].x += __shfl_xor_sync(0xffffffffu, acc[c].x, off);
+      acc[c].y += __shfl_xor_sync(0xffffffffu, acc[c].y, off);
+    }
+  if (x >= nx) return;
+#pragma unroll
+  for (int c = 0; c < CC; ++c)
+    if ((c & 3) == l && c < ncc) phi[((size_t)k * nc_total + c0 + c) * nx + x] = acc[c];
+}
+
+// grid -> band and the diagonal, spin-orbit and short-range terms: sixteen
+// bands x sixteen shares of the grid per block
+template <int CC>
+__global__ void __launch_bounds__(256) g2b_fp64(const double2* __restrict__ U, const double2* __restrict__ phi,
+                                                const double2* __restrict__ psi, double2* __restrict__ out,
+                                                const double* __restrict__ e_nk, const double2* __restrict__ chi,
+                                                const double2* __restrict__ a_proj, const double2* __restrict__ srcp,
+                                                int nk, int nx, int nb, int na, int np, int c0, int ncc, int nc_total) {
+  __shared__ double2 red[16][16][CC];
+  const int nl = threadIdx.x & 15, g = threadIdx.x >> 4, k = blockIdx.y, n = blockIdx.x * 16 + nl;
+  const double2* Un = U + (size_t)k * nx * nb + (n < nb ? n : 0);
+  const double2* f = phi + ((size_t)k * nc_total + c0) * nx;
+  double2 acc[CC];
+#pragma unroll
+  for (int c = 0; c < CC; ++c) acc[c] = make_double2(0.0, 0.0);
+#pragma unroll 4
+  for (int x = g; x < nx; x += 16) {
+    const double2 u = Un[(size_t)x * nb];
+#pragma unroll
+    for (int c = 0; c < CC; ++c) cmac_conj(acc[c], u, f[(size_t)(c < ncc ? c : 0) * nx + x]);
+  }
+#pragma unroll
+  for (int c = 0; c < CC; ++c) red[g][nl][c] = acc[c];
+  __syncthreads();
+  const int cc = threadIdx.x >> 4;
+  if (cc >= ncc || cc >= CC || n >= nb) return;
+  double2 lr = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    lr.x += red[i][nl][cc].x;
+    lr.y += red[i][nl][cc].y;
+  }
+  const size_t nkb = (size_t)nk * nb, kn = (size_t)k * nb + n;
+  const int c = c0 + cc, v = c / na, a = c % na;
+  double2 rest = make_double2(0.0, 0.0);   // -chi psi + short-range out
+  for (int b = 0; b < na; ++b) {
+    const double2 ch = chi[a * na + b], pb = psi[(size_t)(v * na + b) * nkb + kn];
+    rest.x -= ch.x * pb.x - ch.y * pb.y;
+    rest.y -= ch.x * pb.y + ch.y * pb.x;
+  }
+  const double2* cp = srcp + (size_t)v * na * np + (size_t)a * np;
+#pragma unroll 4
+  for (int p = 0; p < np; ++p) {
+    const double2 ap = a_proj[(size_t)p * nkb + kn], q = cp[p];
+    rest.x += ap.x * q.x + ap.y * q.y;
+    rest.y += ap.x * q.y - ap.y * q.x;
+  }
+  const double2 ps = psi[(size_t)c * nkb + kn];
+  const double e = e_nk[kn];
+  out[(size_t)c * nkb + kn] = make_double2(lr.x + rest.x + e * ps.x, lr.y + rest.y + e * ps.y);
+}
+
+// ---------------------------------------------------------------------------
 // short range (Sec. 3.2.2): c[c][p] = sum_{kn} A[p][kn] psi[c][kn];  c' = M c
 // Split-K projection: block b sums kn in [b*SRK*srt, (b+1)*SRK*srt) in srt
 // shared-memory tiles of SRK for up to SRC columns and all Np functions,
@@ -286,6 +384,48 @@ bse_status apply_simt(bse_handle* h, const double2* psi, double2* hpsi, int n_ve
   return bse_cuda_check(h, cudaGetLastError(), "apply (SIMT)");
 }
 
+template <int CC>
+void launch_fp64(bse_handle* h, const double2* psi, double2* hpsi, int c0, int ncc, int nc) {
+  if (!hpsi) {
+    BSE_PROF(h, BSE_K_BAND_TO_GRID,
+             b2g_fp64<CC><<<dim3((unsigned)((h->nx + 31) / 32), (unsigned)h->nk), 128, 0, h->stream>>>(
+                 (const double2*)h->u, psi, (double2*)h->phi, h->nk, h->nx, h->nb, c0, ncc, nc));
+  } else {
+    BSE_PROF(h, BSE_K_GRID_TO_BAND,
+             g2b_fp64<CC><<<dim3((unsigned)((h->nb + 15) / 16), (unsigned)h->nk), 256, 0, h->stream>>>(
+                 (const double2*)h->u, (const double2*)h->phi, psi, hpsi, h->e_nk, h->chi, h->a_proj, h->sr_cp, h->nk,
+                 h->nx, h->nb, h->na, h->np, c0, ncc, nc));
+  }
+}
+// hpsi == nullptr: band->grid of psi; else grid->band into hpsi
+void contract_fp64(bse_handle* h, const double2* psi, double2* hpsi, int nc) {
+  for (int c0 = 0; c0 < nc;) {
+    const int n = nc - c0 < 8 ? nc - c0 : 8;
+    if (n == 1) launch_fp64<1>(h, psi, hpsi, c0, n, nc);
+    else if (n == 2) launch_fp64<2>(h, psi, hpsi, c0, n, nc);
+    else if (n <= 4) launch_fp64<4>(h, psi, hpsi, c0, n, nc);
+    else if (n <= 6) launch_fp64<6>(h, psi, hpsi, c0, n, nc);
+    else launch_fp64<8>(h, psi, hpsi, c0, n, nc);
+    c0 += n;
+  }
+}
+
+bse_status apply_fp64(bse_handle* h, const double2* psi, double2* hpsi, int n_vec) {
+  const int nc = n_vec * h->na;
+  if (bse_ozh_takes(h, nc)) {
+    bse_status s = bse_ozh_band_to_grid(h, psi, nc);
+    if (s == BSE_OK) s = bse_kconv_inplace(h, n_vec);
+    if (s == BSE_OK) s = bse_ozh_grid_to_band(h, psi, hpsi, nc);
+    return s;
+  }
+  contract_fp64(h, psi, nullptr, nc);
+  const bse_status s = bse_kconv_inplace(h, n_vec);
+  if (s != BSE_OK) return s;
+  if (h->np > 0) cudaStreamWaitEvent(h->stream, h->ev_join, 0);   // short-range c' ready
+  contract_fp64(h, psi, hpsi, nc);
+  return bse_cuda_check(h, cudaGetLastError(), "apply (FP64)");
+}
+
 template <typename T>
 void launch_sr_in(bse_handle* h, const double2* psi, int nc, int nkb, int nblk, int srt) {
   typedef typename Cx<T>::type C;
@@ -351,7 +491,7 @@ bse_status bse_apply_device(bse_handle* h, const double2* psi, double2* hpsi, in
       if (fuse) return BSE_ERR_UNSUPPORTED;
       s = bse_sr_terms(h, psi, n_vec);
       if (s != BSE_OK) return s;
-      return apply_simt<double>(h, psi, hpsi, n_vec);
+      return apply_fp64(h, psi, hpsi, n_vec);
     case BSE_PREC_FP32:
       if (fuse) return BSE_ERR_UNSUPPORTED;
       s = bse_sr_terms(h, psi, n_vec);

@@ -318,11 +318,11 @@ __global__ void __launch_bounds__(256) oz_split_rows(const double2* __restrict__
   const size_t digit = (size_t)nr * (kp / 2);
   for (int k = threadIdx.x; k < kp / 2; k += blockDim.x) {
     const double2 v = k < n ? entry(k) : make_double2(0.0, 0.0);
-    const unsigned long long fr = oz_fixed(v.x, e), fi = oz_fixed(v.y, e);
+    const oz_fix fr = oz_fixed(v.x, e), fi = oz_fixed(v.y, e);
 #pragma unroll
     for (int i = 0; i < OZ_S; ++i) out[i * digit + k] = oz_digit2(fr, fi, i);
     if (pair) {
-      const unsigned long long fm = oz_fixed(-v.y, e);
+      const oz_fix fm = oz_fixed(-v.y, e);
 #pragma unroll
       for (int i = 0; i < OZ_S; ++i) out[i * digit + kp / 2 + k] = oz_digit2(fm, fr, i);
     }
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(256) oz_split_bloch(const double2* __restrict_
       scale[(size_t)kl * nb + n] = scalbn(1.0, e);
       if (flag) atomicOr(bad, 1);
     }
-    unsigned long long f[8];
+    oz_fix f[8];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const double2 w = x + i < nx ? u[((size_t)k * nx + x + i) * nb + n] : make_double2(0.0, 0.0);

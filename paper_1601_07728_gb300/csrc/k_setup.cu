@@ -264,5 +264,6 @@ bse_status bse_setup_device(bse_handle* h, const bse_system_desc* d) {
   if (w64) cudaFree(w64);
   if (wbar) cudaFree(wbar);
   if (lr) cudaFree(lr);
+  if (s == BSE_OK && h->prec == BSE_PREC_FP64) bse_ozh_prepare(h);
   return s;
 }

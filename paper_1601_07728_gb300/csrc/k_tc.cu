@@ -1466,6 +1466,7 @@ extern "C" bse_status bse_autotune(bse_handle* h, int n_vec, int reps, int* spli
 }
 
 bse_status bse_tc_status(bse_handle* h) {
+  if (h->ozh) return bse_ozh_status(h);
   if (h->prec != BSE_PREC_SPLIT_BF16 || !h->tmap_host) return BSE_OK;
   TcState* ts = (TcState*)h->tmap_host;
   int e = 0;

@@ -39,31 +39,49 @@ __device__ __forceinline__ int oz_exponent(unsigned key, int* bad) {
   return e;
 }
 
-// round(x 2^(55-e)) biased so that each byte of the result is a digit + 128
-__device__ __forceinline__ unsigned long long oz_fixed(double x, int e) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int ex = (int)((b >> 52) & 0x7ff);
-  unsigned long long m = (b & 0xfffffffffffffull) | (ex ? 0x10000000000000ull : 0ull);
-  int sh = ex - 1020 - e;   // at most 2 where |x| < 2^e
-  if (sh > 2) sh = 2;       // only rows flagged out of range
-  if (sh >= 0) {
-    m <<= sh;
-  } else {
-    const int r = -sh > 62 ? 62 : -sh;
-    m = (m + (1ull << (r - 1))) >> r;
+// f = round(x 2^(55-e)) + 0x80808080808080: each byte of f is a digit + 128 (the
+// leading one with its carry above).  Integer arithmetic: at two FP64
+// operations per SM and clock the FP64 pipe would take longer than HBM.  An
+// entry far below the row's scale (every zero among them) shifts out to 0;
+// e >= -960, or e = 0 for a row that counts as zero.
+struct oz_fix {
+  uint32_t lo, hi;
+};
+__device__ __forceinline__ oz_fix oz_fixed(double x, int e) {
+  const uint32_t xh = (uint32_t)__double2hiint(x), xl = (uint32_t)__double2loint(x);
+  // |x| 2^(56-e) = (mantissa << 3) >> r with the leading bit of the mantissa at 52
+  int r = 1022 + e - (int)((xh >> 20) & 0x7ffu);
+  r = max(0, min(r, 63));   // below 0 only in rows flagged out of range
+  uint32_t h = __funnelshift_l(xl, (xh & 0xfffffu) | 0x100000u, 3), l = xl << 3;
+  if (r & 32) {
+    l = h;
+    h = 0;
   }
-  const long long q = (long long)b < 0 ? -(long long)m : (long long)m;
-  return (unsigned long long)q + 0x80808080808080ull;
+  l = __funnelshift_r(l, h, r);
+  h >>= r & 31;
+  // (v + 1 + 2 * 0x80808080808080) >> 1 rounds v / 2 to the nearest; with the
+  // complement ~v = -v - 1 of a negative entry the same sum rounds -v / 2
+  const uint32_t s = (uint32_t)((int)xh >> 31);
+  const unsigned long long t = (((unsigned long long)(h ^ s) << 32) | (l ^ s)) + 0x0101010101010101ull;
+  oz_fix f;
+  f.lo = __funnelshift_r((uint32_t)t, (uint32_t)(t >> 32), 1);
+  f.hi = (uint32_t)(t >> 32) >> 1;
+  return f;
 }
 
-// digit i (0 = leading) of two entries as packed FP16; f from oz_fixed
-__device__ __forceinline__ uint32_t oz_digit2(unsigned long long f0, unsigned long long f1, int i) {
-  const int sh = 8 * (OZ_S - 1 - i);
-  // the leading digit keeps the carry above its byte (128 at most)
-  const uint32_t mask = i == 0 ? 0x1ffu : 0xffu;
-  const uint32_t b0 = (uint32_t)(f0 >> sh) & mask, b1 = (uint32_t)(f1 >> sh) & mask;
-  const uint32_t w = b0 | (b1 << 16) | 0x64006400u;   // FP16 1024 + digit + 128, exact
-  const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&w), __floats2half2_rn(1152.f, 1152.f));
+// digit i (0 = leading) of two entries as packed FP16: the bytes b become
+// 0x6400 | b = 1024 + digit + 128, less 1152
+__device__ __forceinline__ uint32_t oz_digit2(oz_fix f0, oz_fix f1, int i) {
+  uint32_t w;
+  if (i == 0) {
+    w = (__byte_perm(f0.hi, f1.hi, 0x7632) & 0x01ff01ffu) | 0x64006400u;   // nine bits: 256 for the digit 128
+  } else {
+    const int b = OZ_S - 1 - i;   // byte of the 64-bit word
+    const uint32_t sel = (uint32_t)((b & 3) * 0x1111 + 0x4400);
+    w = (__byte_perm(b >= 4 ? f0.hi : f0.lo, b >= 4 ? f1.hi : f1.lo, sel) & 0x00ff00ffu) | 0x64006400u;
+  }
+  const uint32_t c = 0x64806480u;   // 1152 twice
+  const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&w), *reinterpret_cast<const __half2*>(&c));
   return *reinterpret_cast<const uint32_t*>(&d);
 }
 
