@@ -453,8 +453,9 @@ int bse_schedule(const bse_handle* h);
  * wait that gives up makes the kernel stop issuing work, wait for its own
  * copies and MMAs in flight (with a fixed 2 s bound), free its tensor memory
  * and return; the call reports BSE_ERR_TIMEOUT (its outputs are not valid)
- * and the handle stays usable.  Other precisions have no such waits.
- * Synchronises the handle's stream. */
+ * and the handle stays usable.  The same holds for the tensor-core kernels of
+ * the FP64 form; the FP32 form has no such waits.  Synchronises the handle's
+ * stream. */
 bse_status bse_set_wait_limit(bse_handle* h, double seconds);
 
 /* Measurement aid, no counterpart in the paper: when enabled, every kernel

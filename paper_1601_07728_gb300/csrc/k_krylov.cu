@@ -54,6 +54,15 @@ __device__ double2 block_sum2(double2 v) {
   return r;
 }
 
+// 1 / x by one thread of the block (an FP64 division in every thread costs more
+// than the element it is for)
+__device__ double block_inverse(double x) {
+  __shared__ double inv;
+  if (threadIdx.x == 0) inv = 1.0 / x;
+  __syncthreads();
+  return inv;
+}
+
 // partial[v][blk] = sum over the block's slice of conj(x) * y   (y == nullptr: |x|^2)
 // x, y of vector v start at v * xs, v * ys (xs = ys = N for packed batches).
 __global__ void __launch_bounds__(RB) dot_partial_s(const double2* __restrict__ x, long long xs,
@@ -123,7 +132,7 @@ __global__ void hay_scale(const double2* __restrict__ x, double2* __restrict__ y
                           const double* __restrict__ bco, int col, int stride, const int* __restrict__ active) {
   const int v = blockIdx.y;
   if (!active[v]) return;
-  const double inv = 1.0 / bco[(size_t)v * stride + col];
+  const double inv = block_inverse(bco[(size_t)v * stride + col]);
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
     double2 a = x[(size_t)v * N + i];
     y[(size_t)v * N + i] = make_double2(a.x * inv, a.y * inv);
@@ -287,14 +296,16 @@ bse_status apply_chunked(bse_handle* h, const double2* in, double2* out, int n_v
 // The 16 sums of a warp are reduced by exchanging halves: the same pairs as a
 // butterfly per sum, at 16 FP64 additions per lane instead of 80, which at two
 // FP64 operations per SM and clock were most of the kernel on short vectors,
-// and the groups of a long basis run beside one another.  Mean over j = 1..12:
-// 16 systems of 12,288 rows 86 -> 35 us, 32 systems of 196,608 rows 850 -> 746
-// (FP64 pipe: 6 operations per entry, 2 per SM and clock, 460 us).
-constexpr int GS_JB = 8;
-__global__ void __launch_bounds__(RB) gs_dot_multi(const double2* __restrict__ basis, long long bstride,
-                                                   long long jstride, const double2* __restrict__ w,
-                                                   long long wstride, long long N, int nj,
-                                                   double2* __restrict__ partial, const int* __restrict__ mask) {
+// and the groups of a long basis run beside one another.  Groups of four with
+// two rows in flight keep three blocks on an SM (groups of eight: two, 746 us).
+// Mean over j = 1..12: 16 systems of 12,288 rows 86 -> 32 us, 32 systems of
+// 196,608 rows 850 -> 560 (FP64 pipe: 6 operations per entry, 2 per SM and
+// clock, 400 us).
+constexpr int GS_JB = 4;
+__global__ void __launch_bounds__(RB, 3) gs_dot_multi(const double2* __restrict__ basis, long long bstride,
+                                                      long long jstride, const double2* __restrict__ w,
+                                                      long long wstride, long long N, int nj,
+                                                      double2* __restrict__ partial, const int* __restrict__ mask) {
   const int v = blockIdx.z, j0 = blockIdx.y * GS_JB;
   if (mask && !mask[v]) return;
   const double2* bv = basis + (size_t)v * bstride + (size_t)j0 * jstride;
@@ -303,34 +314,46 @@ __global__ void __launch_bounds__(RB) gs_dot_multi(const double2* __restrict__ b
   double acc[2 * GS_JB];
 #pragma unroll
   for (int q = 0; q < 2 * GS_JB; ++q) acc[q] = 0.0;
-  for (long long e = (long long)blockIdx.x * RB + threadIdx.x; e < N; e += (long long)gridDim.x * RB) {
-    const double2 b = wv[e];
-    double2 a[GS_JB];
+  const long long step = (long long)gridDim.x * RB;
+  for (long long e = (long long)blockIdx.x * RB + threadIdx.x; e < N; e += 2 * step) {
+    // two rows' loads in flight, their terms added in order
+    const bool two = e + step < N;
+    double2 b[2], a[2][GS_JB];
+    b[0] = wv[e];
+    if (two) b[1] = wv[e + step];
 #pragma unroll
     for (int q = 0; q < GS_JB; ++q)
-      if (q < njg) a[q] = bv[(size_t)q * jstride + e];
-#pragma unroll
-    for (int q = 0; q < GS_JB; ++q) {
       if (q < njg) {
-        acc[2 * q] += a[q].x * b.x + a[q].y * b.y;
-        acc[2 * q + 1] += a[q].x * b.y - a[q].y * b.x;
+        a[0][q] = bv[(size_t)q * jstride + e];
+        if (two) a[1][q] = bv[(size_t)q * jstride + e + step];
+      }
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      if (t && !two) break;
+#pragma unroll
+      for (int q = 0; q < GS_JB; ++q) {
+        if (q < njg) {
+          acc[2 * q] += a[t][q].x * b[t].x + a[t][q].y * b[t].y;
+          acc[2 * q + 1] += a[t][q].x * b[t].y - a[t][q].y * b[t].x;
+        }
       }
     }
   }
-  // lane L ends with sum L >> 1
+  // the pairs of a butterfly (16, 8, 4, 2, 1); lane L ends with sum L >> 2
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int h = GS_JB; h >= 1; h >>= 1) {
-    const bool up = (lane & (2 * h)) != 0;
+    const bool up = (lane & (4 * h)) != 0;
 #pragma unroll
     for (int i = 0; i < h; ++i) {
       const double mine = up ? acc[h + i] : acc[i], other = up ? acc[i] : acc[h + i];
-      acc[i] = mine + __shfl_xor_sync(0xffffffffu, other, 2 * h);
+      acc[i] = mine + __shfl_xor_sync(0xffffffffu, other, 4 * h);
     }
   }
+  acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
   acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
   __shared__ double sred[RB / 32][2 * GS_JB];
-  if ((lane & 1) == 0) sred[threadIdx.x >> 5][lane >> 1] = acc[0];
+  if ((lane & 3) == 0) sred[threadIdx.x >> 5][lane >> 2] = acc[0];
   __syncthreads();
   if ((int)threadIdx.x < 2 * njg) {
     double t = 0.0;
@@ -607,7 +630,7 @@ __global__ void gm_next(const double2* w, long long wstride, double2* V, long lo
                         const double* __restrict__ hnorm, const int* __restrict__ mask) {
   const int v = blockIdx.y;
   if (!mask[v] || !(hnorm[v] > 0)) return;
-  const double inv = 1.0 / hnorm[v];
+  const double inv = block_inverse(hnorm[v]);
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < N; e += (long long)gridDim.x * blockDim.x) {
     double2 a = w[(size_t)v * wstride + e];
     V[(size_t)v * vstride + e] = make_double2(a.x * inv, a.y * inv);
