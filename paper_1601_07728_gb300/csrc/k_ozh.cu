@@ -556,24 +556,15 @@ __global__ void __launch_bounds__(256) ozh_final(const double2* __restrict__ par
   }
 }
 
-typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                             const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                             CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
 // digits [nk * 7][H_J][kp] FP16: box of 32 K elements x 16 rows x 7 digits, 64-byte swizzle
 bool stacked_map(CUtensorMap* m, const __half* base, int kp, int nk) {
-  void* f = nullptr;
-  cudaDriverEntryPointQueryResult q;
-  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-      q != cudaDriverEntryPointSuccess) {
-    cudaGetLastError();
-    return false;
-  }
+  const EncodeTiledFn f = bse_encode_tiled_fn();
+  if (!f) return false;
   cuuint64_t dims[3] = {(cuuint64_t)kp, (cuuint64_t)H_J, (cuuint64_t)nk * OZ_S};
   cuuint64_t strides[2] = {(cuuint64_t)kp * 2, (cuuint64_t)H_J * kp * 2};
   cuuint32_t box[3] = {(cuuint32_t)H_KB, (cuuint32_t)H_J, (cuuint32_t)OZ_S};
   cuuint32_t es[3] = {1, 1, 1};
-  return ((EncodeFn)f)(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half*>(base), dims, strides, box, es,
+  return f(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half*>(base), dims, strides, box, es,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }

@@ -27,6 +27,19 @@
 
 #include <algorithm>
 
+EncodeTiledFn bse_encode_tiled_fn() {
+  static EncodeTiledFn fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      return (EncodeTiledFn)p;
+    cudaGetLastError();
+    return (EncodeTiledFn) nullptr;
+  }();
+  return fn;
+}
+
 namespace {
 
 constexpr int TC_M = 128;
@@ -40,7 +53,6 @@ constexpr int SMEM_BUDGET = 224 * 1024;
 // persistent split-bf16 GEMM
 // ---------------------------------------------------------------------------
 struct TcParams {
-  int mode;            // 0: band->grid (phi out), 1: grid->band (split-K partials out)
   int ntiles;          // work units = batch * mtiles * nsplit * ntn
   int mtiles, nsplit;
   int kb_per_split, kb_total;
@@ -56,6 +68,9 @@ struct TcParams {
   int* err;
   unsigned long long wait_ns;   // limit of each pipeline wait (the drain after an abort keeps WAIT_NS)
   uint32_t lbo, sbo;   // mode 2: MN-major descriptor offsets of the A operand (bytes)
+  int k_len;           // K elements (of band->grid: padded row length; of grid->band: Nx)
+  int m_tail;          // last M tile: rows its A boxes hold (0: the full boxes)
+  int mt_last;
 };
 
 struct Tile {
@@ -78,8 +93,20 @@ __device__ __forceinline__ Tile decode(const TcParams& p, int t) {
   return r;
 }
 
+// What padding costs: a K block or M tile that is mostly padding used to take
+// as long as a full one, because the products of a stage took about as long to
+// issue as its 36 KB to arrive.  The MMA loop is therefore one straight line of
+// twelve products whose descriptors differ by constants (a product of N = 16
+// takes 39 clocks issued so, over 100 with descriptors put together in the
+// loop), K steps beyond the last element are left out, and the last M tile has
+// A boxes of its own height.  512 k, 18^3 points, 140 bands (K blocks 88 %, M
+// tiles 73 % filled), one column: band->grid 597 -> 501 us (496 at the copy
+// rate), grid->band 707 -> 558 (521); 8^3 k, 16^3 points, 64 bands (no padding),
+// six columns: 185 -> 171 and 185 -> 174 us (174 and 177 at the copy rate).
+template <int MODE>   // 0: band->grid, 1: grid->band, 2: grid->band from the row-major U~
 __global__ void __launch_bounds__(TC_THREADS, 1)
     tc_gemm(const __grid_constant__ CUtensorMap ma_hi, const __grid_constant__ CUtensorMap ma_lo,
+            const __grid_constant__ CUtensorMap mt_hi, const __grid_constant__ CUtensorMap mt_lo,
             const __grid_constant__ CUtensorMap mb_hi, const __grid_constant__ CUtensorMap mb_lo, const TcParams p) {
   extern __shared__ unsigned char smraw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
@@ -131,30 +158,33 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&ma_lo) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&mb_hi) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"((unsigned long long)&mb_lo) : "memory");
-    int it = 0;
+    int it = 0, s = 0;
+    uint32_t ph = 1;
     bool ok = true;
     for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
       Tile tl = decode(p, t);
+      const bool tail = MODE != 2 && p.m_tail && tl.mt == p.mt_last;
+      const CUtensorMap* a_hi = tail ? &mt_hi : &ma_hi;
+      const CUtensorMap* a_lo = tail ? &mt_lo : &ma_lo;
+      const uint32_t bytes = 2 * (tail ? (uint32_t)p.m_tail * 128 : a_bytes) + 2 * b_bytes;
       for (int kb = 0; kb < tl.nkb; ++kb, ++it) {
-        const int s = it % S;
-        const uint32_t ph = (uint32_t)(it / S) & 1u;
-        if (!mbar_wait(empty(s), ph ^ 1u, abort_flag, p.wait_ns)) {
+        if (!mbar_wait(empty(s), ph, abort_flag, p.wait_ns)) {
           ok = false;
           break;
         }
         const uint32_t st = sbase + (uint32_t)s * stage_bytes;
-        mbar_expect_tx(full(s), stage_bytes);
-        if (p.mode == 0) {
+        mbar_expect_tx(full(s), bytes);
+        const int kt = tl.kb0 + kb;
+        if constexpr (MODE == 0) {
           // row-major operands [batch][rows][K]: K block = 64 consecutive elements of each row
-          const int kc = (tl.kb0 + kb) * TC_KB;
-          tma_load_3d(st, &ma_hi, full(s), kc, tl.mt * TC_M, tl.batch);
-          tma_load_3d(st + a_bytes, &ma_lo, full(s), kc, tl.mt * TC_M, tl.batch);
+          const int kc = kt * TC_KB;
+          tma_load_3d(st, a_hi, full(s), kc, tl.mt * TC_M, tl.batch);
+          tma_load_3d(st + a_bytes, a_lo, full(s), kc, tl.mt * TC_M, tl.batch);
           tma_load_3d(st + 2 * a_bytes, &mb_hi, full(s), kc, tl.nt * p.nn, tl.batch);
           tma_load_3d(st + 2 * a_bytes + b_bytes, &mb_lo, full(s), kc, tl.nt * p.nn, tl.batch);
-        } else if (p.mode == 2) {
+        } else if constexpr (MODE == 2) {
           // grid->band from the row-major U~ [k][x][q]: rows x = 64 kt .. 64 kt + 63
           // of q 0..63 and 64..127 of the M tile, an MN-major A operand
-          const int kt = tl.kb0 + kb;
           const int q0 = tl.mt * TC_M;
           tma_load_3d(st, &ma_hi, full(s), q0, kt * TC_KB, tl.batch);
           tma_load_3d(st + a_bytes / 2, &ma_hi, full(s), q0 + TC_KB, kt * TC_KB, tl.batch);
@@ -164,13 +194,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           tma_load_4d(st + 2 * a_bytes + b_bytes, &mb_lo, full(s), 0, tl.nt * p.nn, kt, tl.batch);
         } else {
           // K-tiled operands [batch][K/64][rows][64]: one contiguous block per K block
-          const int kt = tl.kb0 + kb;
-          tma_load_4d(st, &ma_hi, full(s), 0, tl.mt * TC_M, kt, tl.batch);
-          tma_load_4d(st + a_bytes, &ma_lo, full(s), 0, tl.mt * TC_M, kt, tl.batch);
+          tma_load_4d(st, a_hi, full(s), 0, tl.mt * TC_M, kt, tl.batch);
+          tma_load_4d(st + a_bytes, a_lo, full(s), 0, tl.mt * TC_M, kt, tl.batch);
           tma_load_4d(st + 2 * a_bytes, &mb_hi, full(s), 0, tl.nt * p.nn, kt, tl.batch);
           tma_load_4d(st + 2 * a_bytes + b_bytes, &mb_lo, full(s), 0, tl.nt * p.nn, kt, tl.batch);
         }
         *(volatile int*)issued = it + 1;
+        if (++s == S) s = 0, ph ^= 1u;
       }
     }
     if (!ok) {
@@ -179,8 +209,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
   } else if (warp == 1 && lane == 0) {
     // ---------------- MMA issuer ----------------
-    const uint32_t idesc = idesc_bf16(TC_M, p.nn) | (p.mode == 2 ? IDESC_A_MN : 0u);
-    int it = 0, local = 0;
+    const uint32_t idesc = idesc_bf16(TC_M, p.nn) | (MODE == 2 ? IDESC_A_MN : 0u);
+    int it = 0, local = 0, s = 0;
+    uint32_t ph = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x, ++local) {
       Tile tl = decode(p, t);
@@ -193,8 +224,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       tc_fence_after();
       const uint32_t d = tmem_base + (uint32_t)(acc * p.nn);
       for (int kb = 0; kb < tl.nkb; ++kb, ++it) {
-        const int s = it % S;
-        const uint32_t ph = (uint32_t)(it / S) & 1u;
         if (!mbar_wait(full(s), ph, abort_flag, p.wait_ns)) {
           ok = false;
           break;
@@ -202,21 +231,29 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         *(volatile int*)consumed = it + 1;
         tc_fence_after();
         const uint32_t st = sbase + (uint32_t)s * stage_bytes;
+        // K-major A: 16 K elements = 32 bytes along the row; MN-major A (mode 2):
+        // 16 rows of K = 2048 bytes
+        constexpr int ASTEP = MODE == 2 ? 2048 / 16 : 32 / 16;
+        const unsigned long long a_hi = MODE == 2 ? sdesc_mn_sw128(st, p.lbo, p.sbo) : sdesc_sw128(st);
+        const unsigned long long a_lo = a_hi + (TC_M * 128) / 16;
+        const unsigned long long b_hi = sdesc_sw128(st + 2 * a_bytes), b_lo = b_hi + b_bytes / 16;
+        const int left = p.k_len - (tl.kb0 + kb) * TC_KB;
+        if (left >= TC_KB) {
 #pragma unroll
-        for (int ks = 0; ks < TC_KB / 16; ++ks) {
-          // K-major A: 16 K elements = 32 bytes along the row; MN-major A (mode 2):
-          // 16 rows of K = 2048 bytes
-          const unsigned long long a_hi =
-              p.mode == 2 ? sdesc_mn_sw128(st + ks * 2048, p.lbo, p.sbo) : sdesc_sw128(st + ks * 32);
-          const unsigned long long a_lo = p.mode == 2 ? sdesc_mn_sw128(st + a_bytes + ks * 2048, p.lbo, p.sbo)
-                                                      : sdesc_sw128(st + a_bytes + ks * 32);
-          const unsigned long long b_hi = sdesc_sw128(st + 2 * a_bytes + ks * 32);
-          const unsigned long long b_lo = sdesc_sw128(st + 2 * a_bytes + b_bytes + ks * 32);
-          mma_bf16(d, a_hi, b_hi, idesc, (kb | ks) != 0);
-          mma_bf16(d, a_hi, b_lo, idesc, 1);
-          mma_bf16(d, a_lo, b_hi, idesc, 1);
+          for (int ks = 0; ks < TC_KB / 16; ++ks) {
+            mma_bf16(d, a_hi + ks * ASTEP, b_hi + ks * 2, idesc, (kb | ks) != 0);
+            mma_bf16(d, a_hi + ks * ASTEP, b_lo + ks * 2, idesc, 1);
+            mma_bf16(d, a_lo + ks * ASTEP, b_hi + ks * 2, idesc, 1);
+          }
+        } else {
+          for (int ks = 0; ks * 16 < left; ++ks) {
+            mma_bf16(d, a_hi + ks * ASTEP, b_hi + ks * 2, idesc, (kb | ks) != 0);
+            mma_bf16(d, a_hi + ks * ASTEP, b_lo + ks * 2, idesc, 1);
+            mma_bf16(d, a_lo + ks * ASTEP, b_hi + ks * 2, idesc, 1);
+          }
         }
         mma_commit(empty(s));
+        if (++s == S) s = 0, ph ^= 1u;
       }
       if (!ok) break;
       mma_commit(tfull(acc));
@@ -256,7 +293,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       for (int c16 = 0; c16 < p.nn / 16; ++c16) {
         float v[16];
         tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * p.nn + c16 * 16), v);
-        if (p.mode == 0) {
+        if constexpr (MODE == 0) {
           // phi[k][c][x], x = row
           if (row < p.nx) {
 #pragma unroll
@@ -692,7 +729,7 @@ __global__ void __launch_bounds__(256, 4) g2b_final_na(const float2* __restrict_
       }
       const double2 val = make_double2((double)rx + e_kn * ps.x, (double)ry + e_kn * ps.y);
       out[(size_t)c * nkb + kn] = val;
-      dre += ps.x * val.x + ps.y * val.y;   // Re <psi|H psi>: the only part the recursion uses
+      if (f.partial) dre += ps.x * val.x + ps.y * val.y;   // Re <psi|H psi>: the only part the recursion uses
     }
   }
   if (f.partial) fused_dot_tail(f, dre, 0.0);
@@ -756,23 +793,7 @@ __global__ void __launch_bounds__(256) g2b_final(const float2* __restrict__ part
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (EncodeTiledFn)p;
-    else
-      cudaGetLastError();
-  }
-  return fn;
-}
+EncodeTiledFn encode_fn() { return bse_encode_tiled_fn(); }
 
 // 3-D bf16 map {inner, rows, batch} with row stride `inner_stride` elements and
 // batch stride `batch_stride` elements; box {64, box_rows, 1}, 128-byte swizzle.
@@ -817,6 +838,8 @@ struct TcState {
   // a2: U~ row-major, box 64 x 128 rows (band->grid A); a2m: the same array,
   // box 64 x 64 rows (grid->band A read MN-major); a6: the K-tiled transposed copy
   CUtensorMap a2_hi, a2_lo, a2m_hi, a2m_lo, a6_hi, a6_lo;
+  // a2 and a6 with boxes of the height of their last M tile
+  CUtensorMap a2t_hi, a2t_lo, a6t_hi, a6t_lo;
 };
 
 inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
@@ -850,8 +873,10 @@ int pick_stages(int nn, int tuned) {
   return s;
 }
 
-bse_status launch_gemm(bse_handle* h, TcState* ts, int mode, const CUtensorMap& a_hi, const CUtensorMap& a_lo,
-                       const CUtensorMap& b_hi, const CUtensorMap& b_lo, TcParams p, int kind, cudaStream_t st) {
+template <int MODE>
+bse_status launch_gemm(bse_handle* h, TcState* ts, const CUtensorMap& a_hi, const CUtensorMap& a_lo,
+                       const CUtensorMap& t_hi, const CUtensorMap& t_lo, const CUtensorMap& b_hi,
+                       const CUtensorMap& b_lo, TcParams p, int kind, cudaStream_t st) {
   p.stages = pick_stages(p.nn, ts->stages);
   if (p.stages < 2) return bse_fail(h, BSE_ERR_UNSUPPORTED, "tensor-core tile does not fit shared memory");
   uint32_t cols = 32;
@@ -862,13 +887,15 @@ bse_status launch_gemm(bse_handle* h, TcState* ts, int mode, const CUtensorMap& 
   p.lbo = ts->lbo;
   p.sbo = ts->sbo;
   const size_t smem = 1024 + (size_t)p.stages * (2 * TC_M * 128 + 2 * p.nn * 128) + 256;
-  cudaFuncSetAttribute(tc_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(tc_gemm<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int grid = p.ntiles < ts->sms ? p.ntiles : ts->sms;
   if (grid < 1) return BSE_OK;
-  BSE_PROF(h, kind, tc_gemm<<<grid, TC_THREADS, smem, st>>>(a_hi, a_lo, b_hi, b_lo, p));
-  (void)mode;
+  BSE_PROF(h, kind, tc_gemm<MODE><<<grid, TC_THREADS, smem, st>>>(a_hi, a_lo, t_hi, t_lo, b_hi, b_lo, p));
   return bse_cuda_check(h, cudaGetLastError(), "tc_gemm launch");
 }
+
+// rows of the A boxes of a last M tile that holds `rows` in all (0: a full tile)
+inline int tail_rows(int rows) { return rows % TC_M == 0 ? 0 : (rows % TC_M + 7) / 8 * 8; }
 
 }  // namespace
 
@@ -914,6 +941,16 @@ bse_status bse_tc_prepare(bse_handle* h) {
             make_map(&ts->a2m_lo, h->u_lo, kp, h->nx, h->nk, kp, (uint64_t)h->nx * kp, TC_KB) &&
             make_map_tiled(&ts->a6_hi, h->ut_hi, 2 * h->nb, 2 * h->nb, x64, h->nk, TC_M) &&
             make_map_tiled(&ts->a6_lo, h->ut_lo, 2 * h->nb, 2 * h->nb, x64, h->nk, TC_M);
+  ts->a2t_hi = ts->a2_hi;
+  ts->a2t_lo = ts->a2_lo;
+  ts->a6t_hi = ts->a6_hi;
+  ts->a6t_lo = ts->a6_lo;
+  if (const int r = tail_rows(h->nx))
+    ok = ok && make_map(&ts->a2t_hi, h->u_hi, kp, h->nx, h->nk, kp, (uint64_t)h->nx * kp, r) &&
+         make_map(&ts->a2t_lo, h->u_lo, kp, h->nx, h->nk, kp, (uint64_t)h->nx * kp, r);
+  if (const int r = tail_rows(2 * h->nb))
+    ok = ok && make_map_tiled(&ts->a6t_hi, h->ut_hi, 2 * h->nb, 2 * h->nb, x64, h->nk, r) &&
+         make_map_tiled(&ts->a6t_lo, h->ut_lo, 2 * h->nb, 2 * h->nb, x64, h->nk, r);
   if (!ok) return bse_fail(h, BSE_ERR_CUDA, "tensor map encoding failed");
   return bse_cuda_check(h, cudaStreamSynchronize(h->stream), "tc prepare");
 }
@@ -958,7 +995,9 @@ bse_status b2g_range(bse_handle* h, int n_vec, int mt_b, int mt_e, cudaStream_t 
       !make_map(&b_lo, bl, ts->kp, rows, h->nk, ts->kp, (uint64_t)ts->nnmax * ts->kp, nn))
     return bse_fail(h, BSE_ERR_CUDA, "tensor map encoding failed");
   TcParams p{};
-  p.mode = 0;
+  p.k_len = ts->kp;
+  p.m_tail = tail_rows(h->nx);
+  p.mt_last = (h->nx + TC_M - 1) / TC_M - 1;
   p.mt0 = mt_b;
   p.mtiles = mt_e - mt_b;
   p.nsplit = 1;
@@ -972,7 +1011,7 @@ bse_status b2g_range(bse_handle* h, int n_vec, int mt_b, int mt_e, cudaStream_t 
   p.nx = h->nx;
   p.nb = h->nb;
   p.nc = nc;
-  return launch_gemm(h, ts, 0, ts->a2_hi, ts->a2_lo, b_hi, b_lo, p, BSE_K_BAND_TO_GRID, st);
+  return launch_gemm<0>(h, ts, ts->a2_hi, ts->a2_lo, ts->a2t_hi, ts->a2t_lo, b_hi, b_lo, p, BSE_K_BAND_TO_GRID, st);
 }
 
 // grid->band over the K blocks [kb_b, kb_e) (x = kb*64 ..), split into at
@@ -991,7 +1030,9 @@ bse_status g2b_range(bse_handle* h, int n_vec, int kb_b, int kb_e, int split_bas
       !make_map_tiled(&b_lo, h->bphi + nbf, rows, ts->nnmax, x64, h->nk, nn))
     return bse_fail(h, BSE_ERR_CUDA, "tensor map encoding failed");
   TcParams p{};
-  p.mode = h->sched == BSE_SCHED_TWO_PASS_ROWMAJOR ? 2 : 1;
+  p.k_len = h->nx;
+  p.m_tail = tail_rows(2 * h->nb);
+  p.mt_last = (2 * h->nb + TC_M - 1) / TC_M - 1;
   p.mtiles = (2 * h->nb + TC_M - 1) / TC_M;
   p.kb_base = kb_b;
   p.kb_total = kb_e - kb_b;
@@ -1009,8 +1050,9 @@ bse_status g2b_range(bse_handle* h, int n_vec, int kb_b, int kb_e, int split_bas
   p.nb = h->nb;
   p.nc = nc;
   *nsplit_out = p.nsplit;
-  if (p.mode == 2) return launch_gemm(h, ts, 2, ts->a2m_hi, ts->a2m_lo, b_hi, b_lo, p, BSE_K_GRID_TO_BAND, st);
-  return launch_gemm(h, ts, 1, ts->a6_hi, ts->a6_lo, b_hi, b_lo, p, BSE_K_GRID_TO_BAND, st);
+  if (h->sched == BSE_SCHED_TWO_PASS_ROWMAJOR)
+    return launch_gemm<2>(h, ts, ts->a2m_hi, ts->a2m_lo, ts->a2m_hi, ts->a2m_lo, b_hi, b_lo, p, BSE_K_GRID_TO_BAND, st);
+  return launch_gemm<1>(h, ts, ts->a6_hi, ts->a6_lo, ts->a6t_hi, ts->a6t_lo, b_hi, b_lo, p, BSE_K_GRID_TO_BAND, st);
 }
 
 }  // namespace
@@ -1037,24 +1079,34 @@ bse_status g2b_epilogue(bse_handle* h, const double2* psi, double2* hpsi, int n_
     int nsplit;
   } p{nsplit};
   if (wait_side) cudaStreamWaitEvent(h->stream, h->ev_join, 0);   // short-range c' ready
-  const int blocks = bse_tc_final_blocks(h);
+  int blocks = bse_tc_final_blocks(h);
   bse_dotfuse f = fuse ? *fuse : bse_dotfuse();
+  // H psi alone, from about eight warps per SM on: two core states per thread
+  // share their projectors and psi, one thread per pair (with <psi|H psi> the
+  // grid, and with it the order of the sums, stay those of the recursion).  32
+  // vectors of the L2,3 workload 307 -> 215 us; 3 vectors of the reduced one
+  // would take 11.2 us instead of 9.8
+  const bool pairs = h->na == 6 && !f.partial && (long long)h->nk * h->nb * 3 * n_vec >= 40000;
+  if (pairs) blocks = (int)std::min<size_t>(((size_t)h->nk * h->nb * 3 + 255) / 256, 65535);
   auto final_grid = [&](int) { return dim3((unsigned)blocks, (unsigned)n_vec); };
   const double2* srp = h->sr_cp;
   const float2* apf = h->a_proj_f;
-#define G2B_NA(NA_, FUSED_)                                                                                      \
+#define G2B_NA(NA_, G_, FUSED_)                                                                                  \
   BSE_PROF(h, BSE_K_PREP,                                                                                         \
-           (g2b_final_na<NA_, 1, FUSED_><<<final_grid(NA_), 256, 0, h->stream>>>(                                 \
+           (g2b_final_na<NA_, G_, FUSED_><<<final_grid(NA_), 256, 0, h->stream>>>(                                 \
                (const float2*)h->part, p.nsplit, const_cast<double2*>(psi), h->psi_f, hpsi, h->e_nk, h->chi, apf, \
                srp, h->nk, h->nb, h->np, nc, f)))
   if (h->na == 6 && f.fused_update) {
-    G2B_NA(6, true);
+    G2B_NA(6, 1, true);
   } else if (h->na == 6) {
-    G2B_NA(6, false);
+    if (pairs)
+      G2B_NA(6, 2, false);
+    else
+      G2B_NA(6, 1, false);
   } else if (h->na == 1 && f.fused_update) {
-    G2B_NA(1, true);
+    G2B_NA(1, 1, true);
   } else if (h->na == 1) {
-    G2B_NA(1, false);
+    G2B_NA(1, 1, false);
   } else {
     if (f.fused_update) return bse_fail(h, BSE_ERR_UNSUPPORTED, "fused Haydock update needs 1 or 6 core states");
     BSE_PROF(h, BSE_K_PREP,

@@ -7,6 +7,12 @@
 #include <cuda.h>
 #include <stdint.h>
 
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+// cuTensorMapEncodeTiled of the driver, nullptr where it has none (k_tc.cu)
+EncodeTiledFn bse_encode_tiled_fn();
+
 namespace {
 
 // ---------------------------------------------------------------------------
