@@ -850,11 +850,16 @@ size_t tc_word_bytes(const bse_handle* h) {
   return 256 + ((2 * nslab + 3) * sizeof(unsigned) + 255) / 256 * 256;
 }
 
-// MMA N of one tile for `rows` B rows (two per complex column): one tile up
-// to 256 rows (the tcgen05 maximum, two accumulators filling TMEM's 512
-// columns); wider operands in 256-row tiles (the last one partly out of the
-// tensor, zero-filled by TMA, its columns not stored)
-inline int tile_n(int rows) { return rows <= 256 ? rows : 256; }
+// MMA N of one tile for `rows` B rows (two per complex column): the fewest tiles
+// of at most 256 rows (the tcgen05 maximum, two accumulators filling TMEM's 512
+// columns), all of the same height -- 384 rows as 2 x 192 and not as 256 + 128 of
+// 256 (192 columns of the L2,3 workload: band->grid 1104 -> 859 us, grid->band
+// 742 -> 646); what the last one has past the tensor is zero-filled by TMA and
+// not stored
+inline int tile_n(int rows) {
+  const int nt = (rows + 255) / 256;
+  return round_up((rows + nt - 1) / nt, 16);
+}
 
 // most pipeline stages that fit shared memory for MMA width nn (at most 8)
 int fit_stages(int nn) {
