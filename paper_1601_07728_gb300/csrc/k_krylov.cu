@@ -208,6 +208,7 @@ __global__ void __launch_bounds__(RB) hay_b_finalize(const double2* partial, int
 // coef[v][j] = sum of the 64 partials (one warp per j; grid (ceil(nj/8), nv)),
 // only where mask[v] != 0 (mask may be null); optionally accumulated into hacc
 constexpr int GS_BLK = 64;   // blocks per vector of the multi-dot
+constexpr int GS_CH = 512;   // coefficients staged at a time
 __global__ void __launch_bounds__(256) gs_dot_finalize(const double2* __restrict__ partial, int nj, double2* coef,
                                                        long long coef_vs, long long coef_js, double2* hacc,
                                                        int hacc_stride, const int* __restrict__ mask) {
@@ -242,6 +243,57 @@ __global__ void gs_subtract(const double2* __restrict__ basis, long long bstride
     }
     w[(size_t)v * N + e] = acc;
   }
+}
+
+// The same for small problems, where the launches count: the block sums the
+// multi-dot's 64 partials itself (one warp per j; the first block records the
+// coefficients and adds them to hacc) and leaves its partial of |w|^2.  Grid and
+// order are those of dot_partial_s with one element per thread.
+__global__ void __launch_bounds__(RB) gs_subtract_small(const double2* __restrict__ basis, long long bstride,
+                                                        double2* __restrict__ w, long long N,
+                                                        const double2* __restrict__ partial, double2* coef,
+                                                        int coef_stride, double2* hacc, int hacc_stride, int nj,
+                                                        const int* __restrict__ mask, double2* __restrict__ npart) {
+  __shared__ double2 cs[GS_CH];
+  const int v = blockIdx.y;
+  if (mask && !mask[v]) return;
+  double2 nrm = make_double2(0, 0);
+  for (int j0 = 0; j0 < nj; j0 += GS_CH) {
+    const int n = nj - j0 < GS_CH ? nj - j0 : GS_CH;
+    __syncthreads();
+    for (int j = threadIdx.x >> 5; j < n; j += RB / 32) {
+      const int lane = threadIdx.x & 31;
+      const double2* p = partial + ((size_t)v * nj + j0 + j) * GS_BLK;
+      double2 s = cadd(p[lane], p[lane + 32]);
+      for (int off = 16; off > 0; off >>= 1) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+      }
+      if (lane == 0) {
+        cs[j] = s;
+        if (blockIdx.x == 0) {
+          coef[(size_t)v * coef_stride + j0 + j] = s;
+          if (hacc) hacc[(size_t)v * hacc_stride + j0 + j] = cadd(hacc[(size_t)v * hacc_stride + j0 + j], s);
+        }
+      }
+    }
+    __syncthreads();
+    const double2* bv = basis + (size_t)v * bstride + (size_t)j0 * N;
+    for (long long e = (long long)blockIdx.x * RB + threadIdx.x; e < N; e += (long long)gridDim.x * RB) {
+      double2 acc = w[(size_t)v * N + e];
+#pragma unroll 4
+      for (int j = 0; j < n; ++j) {
+        const double2 c = cs[j], b = bv[(size_t)j * N + e];
+        // the contraction is spelt out: the sums' bits depend on it
+        acc.x -= fma(c.x, b.x, -__dmul_rn(c.y, b.y));
+        acc.y -= fma(c.y, b.x, __dmul_rn(c.x, b.y));
+      }
+      w[(size_t)v * N + e] = acc;
+      if (j0 + n == nj) nrm.x += acc.x * acc.x + acc.y * acc.y;
+    }
+  }
+  const double2 s = block_sum2(nrm);
+  if (threadIdx.x == 0) npart[(size_t)v * gridDim.x + blockIdx.x] = s;
 }
 
 __global__ void copy_vecs(const double2* __restrict__ src, double2* __restrict__ dst, long long N,
@@ -291,6 +343,34 @@ bse_status apply_chunked(bse_handle* h, const double2* in, double2* out, int n_v
   return BSE_OK;
 }
 
+struct gs_second {   // second pass of cgs_dgks (mask2 null: none)
+  int* mask2;
+  const double2* npart;   // |w|^2 after the first pass, [nv][nblk]
+  int nblk;
+  const double2* coef;    // coefficients of the first pass
+  int coef_stride;
+};
+// DGKS test after one classical Gram-Schmidt pass: with s_after = |w|^2 and
+// s_proj = sum_j |h_j|^2 of the coefficients just removed, |w_before|^2 =
+// s_after + s_proj, and a second pass is needed where more than half of |w|^2
+// was removed (|w_after| < |w_before| / sqrt 2, i.e. s_after < s_proj; NaN also
+// takes it).
+__device__ bool needs_second_pass(const gs_second& a, int v, int nj) {
+  double2 acc = make_double2(0, 0);
+  for (int i = threadIdx.x; i < a.nblk; i += RB) acc.x += a.npart[(size_t)v * a.nblk + i].x;
+  for (int j = threadIdx.x; j < nj; j += RB) {
+    const double2 c = a.coef[(size_t)v * a.coef_stride + j];
+    acc.y += c.x * c.x + c.y * c.y;
+  }
+  const double2 s = block_sum2(acc);
+  return !(s.x >= s.y);
+}
+__global__ void __launch_bounds__(RB) gs_dgks_mask(gs_second a, int nj, const int* __restrict__ mask) {
+  const int v = blockIdx.x;
+  const bool on = (!mask || mask[v]) && needs_second_pass(a, v, nj);
+  if (threadIdx.x == 0) a.mask2[v] = on;
+}
+
 // Gram-Schmidt projections <basis_j|w> of GS_JB basis vectors per block (w is
 // read once per group of GS_JB).  partial[v][j][blk]; grid (GS_BLK, groups, nv).
 // The 16 sums of a warp are reduced by exchanging halves: the same pairs as a
@@ -305,9 +385,18 @@ constexpr int GS_JB = 4;
 __global__ void __launch_bounds__(RB, 3) gs_dot_multi(const double2* __restrict__ basis, long long bstride,
                                                       long long jstride, const double2* __restrict__ w,
                                                       long long wstride, long long N, int nj,
-                                                      double2* __restrict__ partial, const int* __restrict__ mask) {
+                                                      double2* __restrict__ partial, const int* __restrict__ mask,
+                                                      gs_second again) {
   const int v = blockIdx.z, j0 = blockIdx.y * GS_JB;
-  if (mask && !mask[v]) return;
+  if (mask && !mask[v]) {
+    if (again.mask2 && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) again.mask2[v] = 0;
+    return;
+  }
+  if (again.mask2) {   // every block decides for itself, the first records it
+    const bool on = needs_second_pass(again, v, nj);
+    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) again.mask2[v] = on;
+    if (!on) return;
+  }
   const double2* bv = basis + (size_t)v * bstride + (size_t)j0 * jstride;
   const double2* wv = w + (size_t)v * wstride;
   const int njg = nj - j0 < GS_JB ? nj - j0 : GS_JB;
@@ -368,7 +457,7 @@ void gs_project(bse_handle* h, const double2* basis, long long bstride, const do
                 double2* partial, double2* coef, int coef_stride, double2* hacc, int hacc_stride, const int* mask) {
   BSE_PROF(h, BSE_K_RECURSION,
            gs_dot_multi<<<dim3(GS_BLK, (nj + GS_JB - 1) / GS_JB, nv), RB, 0, h->stream>>>(
-               basis, bstride, h->N, w, h->N, h->N, nj, partial, mask));
+               basis, bstride, h->N, w, h->N, h->N, nj, partial, mask, gs_second{}));
   BSE_PROF(h, BSE_K_RECURSION,
            gs_dot_finalize<<<dim3((nj + 7) / 8, nv), 256, 0, h->stream>>>(partial, nj, coef, coef_stride, 1, hacc,
                                                                            hacc_stride, mask));
@@ -386,35 +475,33 @@ bse_status cgs2(bse_handle* h, const double2* basis, long long bstride, double2*
   return BSE_OK;
 }
 
-// DGKS test after one classical Gram-Schmidt pass: with s_after = |w|^2 (from
-// partial sums) and s_proj = sum_j |h_j|^2 of the coefficients just removed,
-// |w_before|^2 = s_after + s_proj, and a second pass is needed where more than
-// half of |w|^2 was removed (|w_after| < |w_before| / sqrt 2, i.e. s_after < s_proj).
-__global__ void __launch_bounds__(RB) gs_dgks_mask(const double2* __restrict__ npart, int nblk,
-                                                   const double2* __restrict__ coef, int coef_stride, int nj,
-                                                   const int* __restrict__ mask, int* __restrict__ mask2) {
-  const int v = blockIdx.x;
-  if (mask && !mask[v]) {
-    if (threadIdx.x == 0) mask2[v] = 0;
-    return;
-  }
-  double2 acc = make_double2(0, 0);
-  for (int i = threadIdx.x; i < nblk; i += RB) acc.x += npart[(size_t)v * nblk + i].x;
-  for (int j = threadIdx.x; j < nj; j += RB) {
-    const double2 c = coef[(size_t)v * coef_stride + j];
-    acc.y += c.x * c.x + c.y * c.y;
-  }
-  const double2 s = block_sum2(acc);
-  if (threadIdx.x == 0) mask2[v] = !(s.x >= s.y);   // NaN also takes the second pass
-}
-
 // Classical Gram-Schmidt with the DGKS criterion: one pass, and a second only
 // for the systems whose first pass cancelled more than half of |w|^2.  npart
-// receives the partials of the new |w|^2 (norm_blocks per system).
+// receives the partials of the new |w|^2 (norm_blocks per system).  Where the
+// norm's grid has a thread for every element the small kernels around the two
+// passes (coefficient sums, |w|^2, the criterion) are done inside them: four
+// launches instead of nine, 51.0 -> 47.7 ms for a resonant spectrum of 10 x 3
+// systems of 12,288 rows.  With more elements the repeated sums and the smaller
+// grid cost more than the launches: 43.6 -> 47.0 ms for 16 such systems at
+// once, 488 -> 505 ms for 32 systems of 196,608 rows.
 bse_status cgs_dgks(bse_handle* h, const double2* basis, long long bstride, double2* w, int nv, int nj,
                     double2* partial, double2* coef, int coef_stride, double2* hacc, int hacc_stride,
                     const int* mask, int* mask2, double2* npart) {
-  const int nbn = norm_blocks(h->N, nv);
+  const long long N = h->N;
+  const int nbn = norm_blocks(N, nv);
+  if ((long long)nbn * RB >= N) {
+    gs_second again{};
+    for (int pass = 0; pass < 2; ++pass) {
+      BSE_PROF(h, BSE_K_RECURSION,
+               gs_dot_multi<<<dim3(GS_BLK, (nj + GS_JB - 1) / GS_JB, nv), RB, 0, h->stream>>>(
+                   basis, bstride, N, w, N, N, nj, partial, mask, again));
+      BSE_PROF(h, BSE_K_RECURSION,
+               gs_subtract_small<<<dim3(nbn, nv), RB, 0, h->stream>>>(basis, bstride, w, N, partial, coef, coef_stride,
+                                                                      hacc, hacc_stride, nj, pass ? mask2 : mask, npart));
+      again = gs_second{mask2, npart, nbn, coef, coef_stride};
+    }
+    return BSE_OK;
+  }
   const int* mk = mask;
   for (int pass = 0; pass < 2; ++pass) {
     gs_project(h, basis, bstride, w, nv, nj, partial, coef, coef_stride, hacc, hacc_stride, mk);
@@ -423,7 +510,7 @@ bse_status cgs_dgks(bse_handle* h, const double2* basis, long long bstride, doub
     BSE_PROF(h, BSE_K_RECURSION, dot_partial_s<<<dim3(nbn, nv), RB, 0, h->stream>>>(w, h->N, nullptr, 0, h->N, npart));
     if (pass == 0) {
       BSE_PROF(h, BSE_K_RECURSION,
-               gs_dgks_mask<<<nv, RB, 0, h->stream>>>(npart, nbn, coef, coef_stride, nj, mask, mask2));
+               gs_dgks_mask<<<nv, RB, 0, h->stream>>>(gs_second{mask2, npart, nbn, coef, coef_stride}, nj, mask));
     }
     mk = mask2;
   }
@@ -575,35 +662,40 @@ __global__ void __launch_bounds__(32) gm_givens(const double2* npart, int nblk, 
     }
   }
   __syncwarp();
+  // the chain of rotations on every lane alike; square roots and divisions that do
+  // not depend on one another on lanes of their own (14.8 -> 13 us at j = 9)
+  const double hn = sqrt(s);
+  double2 h0 = col[0];
+  for (int i = 0; i < j; ++i) {
+    const double2 h1 = col[i + 1], si = ssn[i];
+    const double ci = scs[i];
+    // t1 = c h0 + s h1 ; t2 = -conj(s) h0 + c h1
+    const double2 t1 = make_double2(ci * h0.x + si.x * h1.x - si.y * h1.y, ci * h0.y + si.x * h1.y + si.y * h1.x);
+    const double2 t2 =
+        make_double2(-(si.x * h0.x + si.y * h0.y) + ci * h1.x, -(si.x * h0.y - si.y * h0.x) + ci * h1.y);
+    __syncwarp();
+    if (lane == 0) col[i] = t1;
+    h0 = t2;
+  }
+  const double2 aa = h0;
+  const double hy = hypot(lane == 0 ? aa.x : hn, lane == 0 ? aa.y : 0.0);
+  const double na_ = __shfl_sync(0xffffffffu, hy, 0), nb_ = __shfl_sync(0xffffffffu, hy, 1);
+  const double rr = hypot(na_, nb_);
+  const double q1 = (lane == 0 ? aa.x : lane == 1 ? aa.y : na_) / (lane == 2 ? rr : na_);
+  const double2 ph = make_double2(__shfl_sync(0xffffffffu, q1, 0), __shfl_sync(0xffffffffu, q1, 1));
+  const double q2 = (lane == 0 ? ph.x * hn : ph.y * hn) / rr;   // ph conj(|w|) / rr
+  double cj = __shfl_sync(0xffffffffu, q1, 2);
+  double2 sj = make_double2(__shfl_sync(0xffffffffu, q2, 0), __shfl_sync(0xffffffffu, q2, 1));
+  double2 hjj = make_double2(ph.x * rr, ph.y * rr);
+  if (na_ == 0.0) {
+    cj = 0.0;
+    sj = make_double2(1, 0);
+    hjj = make_double2(hn, 0);
+  }
+  __syncwarp();
   if (lane == 0) {
-    const double hn = sqrt(s);
     hnorm[v] = hn;
-    double2 h0 = col[0];
-    for (int i = 0; i < j; ++i) {
-      const double2 h1 = col[i + 1], si = ssn[i];
-      const double ci = scs[i];
-      // t1 = c h0 + s h1 ; t2 = -conj(s) h0 + c h1
-      const double2 t1 = make_double2(ci * h0.x + si.x * h1.x - si.y * h1.y, ci * h0.y + si.x * h1.y + si.y * h1.x);
-      const double2 t2 =
-          make_double2(-(si.x * h0.x + si.y * h0.y) + ci * h1.x, -(si.x * h0.y - si.y * h0.x) + ci * h1.y);
-      col[i] = t1;
-      h0 = t2;
-    }
-    const double2 aa = h0;
-    double2 sj;
-    double cj;
-    const double na_ = hypot(aa.x, aa.y);
-    const double rr = hypot(na_, hypot(hn, 0.0));
-    if (na_ == 0.0) {
-      cj = 0.0;
-      sj = make_double2(1, 0);
-      col[j] = make_double2(hn, 0);
-    } else {
-      const double2 ph = make_double2(aa.x / na_, aa.y / na_);
-      cj = na_ / rr;
-      sj = make_double2(ph.x * hn / rr, ph.y * hn / rr);   // ph conj(|w|)/rr
-      col[j] = make_double2(ph.x * rr, ph.y * rr);
-    }
+    col[j] = hjj;
     c[j] = cj;
     sv[j] = sj;
     HS(H, j + 1, j) = make_double2(0, 0);
@@ -725,7 +817,7 @@ void bse_multi_dot(bse_handle* h, const double2* basis, long long vstride, long 
                    long long wstride, int nv, int nj, double2* partial, double2* out, long long ovs, long long ojs) {
   BSE_PROF(h, BSE_K_PREP,
            gs_dot_multi<<<dim3(MD_BLK, (nj + GS_JB - 1) / GS_JB, nv), RB, 0, h->stream>>>(
-               basis, vstride, jstride, w, wstride, h->N, nj, partial, nullptr));
+               basis, vstride, jstride, w, wstride, h->N, nj, partial, nullptr, gs_second{}));
   BSE_PROF(h, BSE_K_PREP,
            multi_dot_finalize<<<dim3((nj + 7) / 8, nv), 256, 0, h->stream>>>(partial, nj, out, ovs, ojs));
 }
