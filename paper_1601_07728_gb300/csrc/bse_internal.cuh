@@ -235,16 +235,15 @@ struct bse_oz_operand {
   int batches = 1, rows = 0, kp = 0;
 };
 size_t bse_oz_digit_bytes(int batches, int rows, int kp);
-int bse_oz_tiles(int rows_a, int rows_b);   // output tiles of one batch
 int bse_oz_kp(int k);   // K padded to whole blocks
 // digits of complex rows x [rows][n], entries times d[batch][n] if given; pair = 1 writes two
 // real rows per complex row so that a product with pair = 0 rows is sum a conj(x)
 bse_status bse_oz_split_rows(const double2* x, int rows, int n, const double2* d, int batches, int pair,
                              const bse_oz_operand& o, int* bad, cudaStream_t st);
-// digits of e^{ik.x} u_nk(x) as rows n, K = (x; re, im), for the nkc k points from k0; u is the
-// whole [Nk][Nx][Nb] array, keys [nkc][nb] scratch
-bse_status bse_oz_split_bloch(const double2* u, const int* nk, const int* nx, const double* kshift, int nb, int k0,
-                              int nkc, const bse_oz_operand& o, unsigned* keys, int* bad, cudaStream_t st);
+// the projection of bse_local_projection_device on the tensor cores; *done = false where the
+// scratch cannot be had or u or f hold Inf/NaN or magnitudes outside 2^+-400
+bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb, const double* kshift,
+                          const double2* f, int np, double dv, double2* a, cudaStream_t st, bool* done);
 // out = alpha A_b B_b^T for every batch (an operand with one batch serves all);
 // element (b, row, col) at out + b sb + (row/2) sr2 + (row%2) sr1 + col sc
 bse_status bse_oz_gemm(const bse_oz_operand& a, const bse_oz_operand& b, int batches, double alpha, double* out,

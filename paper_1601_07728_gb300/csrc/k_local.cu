@@ -7,8 +7,6 @@
 // system, before bse_setup (whose short-range term takes A as input).
 #include "bse_internal.cuh"
 
-#include <algorithm>
-
 namespace {
 
 constexpr int LP = 16, LN = 16, LX = 32;   // projector, band and grid tile of one 256-thread block
@@ -66,77 +64,6 @@ __global__ void __launch_bounds__(256) local_proj_kernel(const double2* __restri
   if (p < np && n < nb) a[((size_t)p * nkt + k) * nb + n] = make_double2(ar * dv, ai * dv);
 }
 
-struct Scratch {
-  void* p = nullptr;
-  ~Scratch() {
-    if (p) cudaFree(p);
-  }
-};
-
-// The projection on the tensor cores (k_oz.cu), as many k points per pass as
-// the scratch holds.  *done = false where the scratch cannot be had or u or f
-// hold Inf/NaN or magnitudes outside 2^+-400.
-bse_status projection_tensor(const double2* u, const int* nk, const int* nx, int nb, const double* kshift,
-                             const double2* f, int np, double dv, double2* a, cudaStream_t st, bool* done) {
-  *done = false;
-  const int nkt = nk[0] * nk[1] * nk[2], nxt = nx[0] * nx[1] * nx[2];
-  const int kp = bse_oz_kp(2 * nxt);
-  const size_t per = bse_oz_digit_bytes(1, nb, kp), fixed = bse_oz_digit_bytes(1, 2 * np, kp);
-  const size_t budget = (size_t)1200 << 20;
-  int nkc = (int)(budget / per);
-  nkc = nkc < 1 ? 1 : (nkc > nkt ? nkt : nkc);
-  if (nkc > 32768) nkc = 32768;   // grid extents
-  // whole waves of the product kernel (one CTA per SM) where several passes are needed
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return BSE_ERR_CUDA;
-  const int tiles = bse_oz_tiles(2 * np, nb);
-  if (nkc < nkt && nkc * (long long)tiles > sms) nkc = std::max(1, (int)(nkc * (long long)tiles / sms * sms / tiles));
-  const size_t ud = bse_oz_digit_bytes(nkc, nb, kp);
-  const size_t scu = ((size_t)nkc * nb * sizeof(double) + 255) / 256 * 256;
-  const size_t scf = ((size_t)2 * np * sizeof(double) + 255) / 256 * 256;
-  const size_t key = ((size_t)nkc * nb * sizeof(unsigned) + 255) / 256 * 256;
-  Scratch sc;
-  if (cudaMalloc(&sc.p, ud + fixed + scu + scf + key + 256) != cudaSuccess) {
-    cudaGetLastError();
-    sc.p = nullptr;
-    return BSE_OK;
-  }
-  char* q = (char*)sc.p;
-  bse_oz_operand A, B;
-  B.digits = q, q += ud;
-  A.digits = q, q += fixed;
-  B.scale = (double*)q, q += scu;
-  A.scale = (double*)q, q += scf;
-  unsigned* keys = (unsigned*)q;
-  q += key;
-  int* word = (int*)q;   // {wait gave up, out of range}
-  A.rows = 2 * np, B.rows = nb;
-  A.kp = B.kp = kp;
-  cudaMemsetAsync(word, 0, 2 * sizeof(int), st);
-  // rows (Re f, Im f) and (-Im f, Re f): real and imaginary part of conj(f) times a column
-  bse_status s = bse_oz_split_rows(f, np, nxt, nullptr, 1, 1, A, word + 1, st);
-  for (int k = 0; k < nkt && s == BSE_OK; k += nkc) {
-    const int n = nkt - k < nkc ? nkt - k : nkc;
-    B.batches = n;
-    s = bse_oz_split_bloch(u, nk, nx, kshift, nb, k, n, B, keys, word + 1, st);
-    if (s == BSE_OK)
-      s = bse_oz_gemm(A, B, n, dv, (double*)(a + (size_t)k * nb), 2ll * nb, 2ll * nkt * nb, 1, 2, word, st);
-  }
-  int hw[2] = {0, 0};
-  if (s == BSE_OK && (cudaMemcpyAsync(hw, word, sizeof(hw), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-                      cudaStreamSynchronize(st) != cudaSuccess))
-    s = BSE_ERR_CUDA;
-  if (s != BSE_OK) {
-    cudaStreamSynchronize(st);   // before the scratch goes
-    return s;
-  }
-  if (hw[0]) return BSE_ERR_TIMEOUT;
-  *done = hw[1] == 0;
-  return BSE_OK;
-}
-
 }  // namespace
 
 bse_status bse_local_projection_device(const double2* u, const int* nk, const int* nx, int nb, const double* kshift,
@@ -147,7 +74,7 @@ bse_status bse_local_projection_device(const double2* u, const int* nk, const in
   const double nxd = (double)nx[0] * nx[1] * nx[2];
   if ((double)nkt * nxd * nb * np >= 4194304.0 && nxd <= 1048576.0) {
     bool done = false;
-    const bse_status s = projection_tensor(u, nk, nx, nb, kshift, f, np, dv, a, st, &done);
+    const bse_status s = bse_oz_project(u, nk, nx, nb, kshift, f, np, dv, a, st, &done);
     if (s != BSE_OK || done) return s;
   }
   const dim3 g((unsigned)nkt, (unsigned)((nb + LN - 1) / LN), (unsigned)((np + LP - 1) / LP));

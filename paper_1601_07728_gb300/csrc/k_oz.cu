@@ -9,10 +9,11 @@
 // Green's functions of 900 points, 4096 states and 16 frequencies 682 ms
 // (FP64 kernel) -> 14.0 ms (this one 12.9, writing the digits 0.97); the
 // projection of 8^3 k x 16^3 points x 64 bands onto 64 functions 102.6 ms ->
-// 4.4 ms (this one 2.0, digits 2.07, row scales 0.32).  The error against 64
-// bits fell from 1.9e-15 to 1.3e-15 and from 1.3e-15 to 0.9e-15.  What bounds
-// it now: operand tiles from L2 (35 bytes per SM and clock) beside the
-// products' 64 clocks each.
+// 5.4 ms with the Bloch functions' digits in memory -> 3.3 ms with the digits
+// made on the way into shared memory (oz_project 2.6, row scales 0.29).  The
+// error against 64 bits fell from 1.9e-15 to 1.3e-15 and from 1.4e-15 to
+// 1.2e-15.  What bounds oz_gemm now: operand tiles from L2 (35 bytes per SM and
+// clock) beside the products' 64 clocks each.
 #include "bse_internal.cuh"
 #include "oz_dev.cuh"
 #include "tc_ptx.cuh"
@@ -49,17 +50,57 @@ struct OzParams {
   int* err;
 };
 
-// Persistent warp-specialised kernel, one CTA per SM: warp 0 streams digit
-// tiles with TMA (the seven B tiles of a K block as one box, each A digit in
-// a slot of its own), warp 1 issues the digit products, warps 2-9 drain the
-// accumulators every 128 K elements into 64-bit integers.
+// Digit products of one K block against the B tiles at descriptor db, one A
+// digit after the other out of the ring (slot sl, phase ph); `first`: the
+// accumulators start over, each as soon as it is drained.
 // A product of N = 64 or less takes the tensor core as long as one of N = 128
 // (about 64 clocks measured at N = 32 and 64), so two neighbouring B digits
 // form one operand of 128 rows and the accumulators of s = 2P, 2P + 1 one of
 // 128 columns: digit A_i meets (B_0, B_1), (B_2, B_3), ... for even i and (0,
 // B_0), (B_1, B_2), ... for odd i, 19 products instead of 28 per 16 K elements
-// and all of one shape (s = 7 is computed along and not used).  M tiles are the fastest tile index: the CTAs running at one
-// time then share both operands' tiles in L2.
+// and all of one shape (s = 7 is computed along and not used).
+__device__ __forceinline__ bool issue_block(uint32_t tmem, uint32_t sa, unsigned long long db, bool first, int chunk,
+                                            int& sl, uint32_t& ph, uint32_t afull, uint32_t aempty, uint32_t tempty,
+                                            volatile int* abort_flag) {
+  // FP16 A and B (K-major), FP32 D
+  constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(2 * OZ_N >> 3) << 17) | ((uint32_t)(OZ_M >> 4) << 24);
+#pragma unroll
+  for (int i = 0; i < OZ_S; ++i) {
+    if (!mbar_wait(afull + 8 * sl, ph, abort_flag, OZ_WAIT_NS)) return false;
+    tc_fence_after();
+    const unsigned long long da = sdesc_sw128(sa + sl * OZ_A);
+    if (i == 0 && first) {
+#pragma unroll
+      for (int P = 0; P < 4; ++P) {
+        if (!mbar_wait(tempty + 8 * (2 * P), ((uint32_t)chunk & 1u) ^ 1u, abort_flag, OZ_WAIT_NS)) return false;
+        if (P < 3 && !mbar_wait(tempty + 8 * (2 * P + 1), ((uint32_t)chunk & 1u) ^ 1u, abort_flag, OZ_WAIT_NS))
+          return false;
+        tc_fence_after();
+#pragma unroll
+        for (int ks = 0; ks < OZ_KB / 16; ++ks)
+          mma_bf16(tmem + 2 * P * OZ_N, da + ks * 2, db + (2 * P * OZ_BD + ks * 32) / 16, idesc, ks > 0);
+      }
+    } else {
+      // consecutive products go to different accumulators
+#pragma unroll
+      for (int ks = 0; ks < OZ_KB / 16; ++ks)
+#pragma unroll
+        for (int P = i / 2; P < 4; ++P)
+          mma_bf16(tmem + 2 * P * OZ_N, da + ks * 2,
+                   db + (unsigned long long)(long long)(((2 * P - i) * OZ_BD + ks * 32) / 16), idesc, 1);
+    }
+    mma_commit(aempty + 8 * sl);
+    if (++sl == OZ_AS) sl = 0, ph ^= 1u;
+  }
+  return true;
+}
+
+// Persistent warp-specialised kernel, one CTA per SM: warp 0 streams digit
+// tiles with TMA (the seven B tiles of a K block as one box, each A digit in
+// a slot of its own), warp 1 issues the digit products, warps 2-9 drain the
+// accumulators every 128 K elements into 64-bit integers.  M tiles are the
+// fastest tile index: the CTAs running at one time then share both operands'
+// tiles in L2.
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     oz_gemm(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb, const OzParams p) {
   extern __shared__ unsigned char oz_raw[];
@@ -135,8 +176,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       *abort_flag = 1;
     }
   } else if (warp == 1 && lane == 0) {
-    // FP16 A and B (K-major), FP32 D
-    constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(2 * OZ_N >> 3) << 17) | ((uint32_t)(OZ_M >> 4) << 24);
     int ib = 0, chunk = 0, sl = 0;
     uint32_t ph = 0;
     bool ok = true;
@@ -147,37 +186,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         if (!(ok = mbar_wait(bfull(s), (uint32_t)(ib / OZ_BS) & 1u, abort_flag, OZ_WAIT_NS))) break;
         ++ib;
         const unsigned long long db = sdesc_sw128(sb + s * (OZ_B + OZ_BD));
-#pragma unroll
-        for (int i = 0; i < OZ_S; ++i) {
-          if (!(ok = mbar_wait(afull(sl), ph, abort_flag, OZ_WAIT_NS))) break;
-          tc_fence_after();
-          const unsigned long long da = sdesc_sw128(sa + sl * OZ_A);
-          if (i == 0 && first) {
-            // each accumulator starts over as soon as it is drained
-#pragma unroll
-            for (int P = 0; P < 4; ++P) {
-              ok = mbar_wait(tempty(2 * P), ((uint32_t)chunk & 1u) ^ 1u, abort_flag, OZ_WAIT_NS);
-              if (ok && P < 3) ok = mbar_wait(tempty(2 * P + 1), ((uint32_t)chunk & 1u) ^ 1u, abort_flag, OZ_WAIT_NS);
-              if (!ok) break;
-              tc_fence_after();
-#pragma unroll
-              for (int ks = 0; ks < OZ_KB / 16; ++ks)
-                mma_bf16(tmem + 2 * P * OZ_N, da + ks * 2, db + (2 * P * OZ_BD + ks * 32) / 16, idesc, ks > 0);
-            }
-            if (!ok) break;
-          } else {
-            // consecutive products go to different accumulators
-#pragma unroll
-            for (int ks = 0; ks < OZ_KB / 16; ++ks)
-#pragma unroll
-              for (int P = i / 2; P < 4; ++P)
-                mma_bf16(tmem + 2 * P * OZ_N, da + ks * 2,
-                         db + (unsigned long long)(long long)(((2 * P - i) * OZ_BD + ks * 32) / 16), idesc, 1);
-          }
-          mma_commit(aempty(sl));
-          if (++sl == OZ_AS) sl = 0, ph ^= 1u;
-        }
-        if (!ok) break;
+        if (!(ok = issue_block(tmem, sa, db, first, chunk, sl, ph, afull(0), aempty(0), tempty(0), abort_flag))) break;
         mma_commit(bempty(s));
         if (last) {
           mma_commit(tfull);
@@ -354,56 +363,375 @@ __global__ void __launch_bounds__(256) oz_col_keys(const double2* __restrict__ u
   }
 }
 
-// Digits of the rows (n) of e^{ik.x} u_nk(x), K = 2x interleaved (re, im):
-// u [k][x][n] is read coalesced along n and written transposed.  One block:
-// 32 grid points of one k, every band; a warp holds 4 bands x 8 groups of 4
-// points, so that both the 64-byte reads and the 128-byte digit rows fill
-// their sectors.  |e^{ik.x} u| components are at most sqrt 2 times those of u:
-// the row scale has one more bit.
-__global__ void __launch_bounds__(256) oz_split_bloch(const double2* __restrict__ u, oz_mesh ms, int k0, int nb, int kp,
-                                                      const unsigned* __restrict__ keys, __half* __restrict__ dig,
-                                                      double* __restrict__ scale, int* __restrict__ bad) {
-  __shared__ double2 ph[32];
-  const int nx = ms.nx[0] * ms.nx[1] * ms.nx[2];
-  const int kl = blockIdx.y, k = k0 + kl, x0 = blockIdx.x * 32;
-  if (threadIdx.x < 32) {
-    const int x = x0 + threadIdx.x;
-    double sn = 0.0, cs = 1.0;
-    if (x < nx) {
-      const int m2 = k % ms.nk[2], m1 = (k / ms.nk[2]) % ms.nk[1], m0 = k / (ms.nk[1] * ms.nk[2]);
-      const int j2 = x % ms.nx[2], j1 = (x / ms.nx[2]) % ms.nx[1], j0 = x / (ms.nx[1] * ms.nx[2]);
-      double fr = (m0 + ms.s[0]) * j0 / ((double)ms.nk[0] * ms.nx[0]) + (m1 + ms.s[1]) * j1 / ((double)ms.nk[1] * ms.nx[1]) +
-                  (m2 + ms.s[2]) * j2 / ((double)ms.nk[2] * ms.nx[2]);
+// a load that stays where it stands: the compiler otherwise sinks the next
+// block's loads behind the waits, to their use
+__device__ __forceinline__ double2 load_in_place(const double2* p) {
+  double2 v;
+  asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
+
+// e^{ik.x} per dimension: tab_d[m][j] = e^{2 pi i (m + s_d) j / (nk_d nx_d)}, the
+// three tables one after the other
+__global__ void __launch_bounds__(256) oz_tables(oz_mesh ms, double2* __restrict__ tab) {
+  long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+  double2* t = tab;
+  for (int d = 0; d < 3; ++d) {
+    const long long n = (long long)ms.nk[d] * ms.nx[d];
+    if (i < n) {
+      double fr = ((int)(i / ms.nx[d]) + ms.s[d]) * (double)(i % ms.nx[d]) / ((double)ms.nk[d] * ms.nx[d]), sn, cs;
       fr -= floor(fr);
       sincospi(2.0 * fr, &sn, &cs);
+      t[i] = make_double2(cs, sn);
+      return;
     }
-    ph[threadIdx.x] = make_double2(cs, sn);
+    i -= n;
+    t += n;
+  }
+}
+
+// phases [k][xp] of the nkc k points from k0, xp grid points (zero beyond nx)
+__global__ void __launch_bounds__(256) oz_phases(oz_mesh ms, const double2* __restrict__ tab, int k0, int xp,
+                                                 double2* __restrict__ phase) {
+  const int x = blockIdx.x * 256 + threadIdx.x, k = k0 + blockIdx.y;
+  if (x >= xp) return;
+  double2 r = make_double2(0.0, 0.0);
+  if (x < ms.nx[0] * ms.nx[1] * ms.nx[2]) {
+    const int m2 = k % ms.nk[2], m1 = (k / ms.nk[2]) % ms.nk[1], m0 = k / (ms.nk[1] * ms.nk[2]);
+    const int j2 = x % ms.nx[2], j1 = (x / ms.nx[2]) % ms.nx[1], j0 = x / (ms.nx[1] * ms.nx[2]);
+    const double2* t1 = tab + (size_t)ms.nk[0] * ms.nx[0];
+    const double2* t2 = t1 + (size_t)ms.nk[1] * ms.nx[1];
+    const double2 a = tab[(size_t)m0 * ms.nx[0] + j0], b = t1[(size_t)m1 * ms.nx[1] + j1],
+                  c = t2[(size_t)m2 * ms.nx[2] + j2];
+    const double2 ab = make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+    r = make_double2(ab.x * c.x - ab.y * c.y, ab.x * c.y + ab.y * c.x);
+  }
+  phase[(size_t)blockIdx.y * xp + x] = r;
+}
+
+// row scales 2^e of the rotated Bloch functions: |e^{ik.x} u| components are at
+// most sqrt 2 times those of u, one more bit
+__global__ void __launch_bounds__(256) oz_bloch_scales(const unsigned* __restrict__ keys, int n, int* __restrict__ expo,
+                                                       double* __restrict__ scale, int* __restrict__ bad) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  int flag = 0;
+  const int e = oz_exponent(keys[i], &flag) + 1;
+  expo[i] = e;
+  scale[i] = scalbn(1.0, e);
+  if (flag) atomicOr(bad, 1);
+}
+
+constexpr int OZ_W = 16;                               // worker warps of oz_project
+constexpr int OZ_PT = 64 + 32 * OZ_W;                  // its threads
+constexpr int OZ_PH = 4;                               // phase slots
+constexpr size_t OZ_PSMEM = OZ_SMEM + OZ_PH * OZ_KB / 2 * sizeof(double2);
+
+struct OzProject {
+  const double2* u;       // the pass's first k point: [k][x][n]
+  const double2* phase;   // [k][32 kb]
+  const int* expo;        // [k][nb]
+  const double* scale;    // [k][nb]
+  const double* scale_a;
+  int nx, nb, np2, nkt, k0;
+  int mt, nt, ntiles, kb, cpt;   // M tiles, N tiles, all tiles, K blocks and chunks of a tile
+  double alpha;
+  double* out;            // [np][nkt][nb] complex
+  longlong2* part;        // [CTA][2][128][64] sums of the tiles that CTAs share
+  int* err;
+};
+
+// first chunk of CTA c: all tiles' chunks in one line, cut into equal parts
+__host__ __device__ inline long long oz_start(long long c, long long chunks, int grid) { return c * chunks / grid; }
+
+__device__ __forceinline__ void oz_store(const OzProject& p, int t, int row, int col, long long hi, long long lo) {
+  const int m = t % p.mt, r = t / p.mt, n = r % p.nt, k = r / p.nt;
+  const int gr = m * OZ_M + row, gc = n * OZ_N + col;
+  if (gr < p.np2 && gc < p.nb)
+    p.out[2 * (((size_t)(gr >> 1) * p.nkt + p.k0 + k) * p.nb + gc) + (gr & 1)] =
+        ((double)hi * 0x1p-30 + (double)lo * 0x1p-62) * (p.alpha * p.scale_a[gr] * p.scale[(size_t)k * p.nb + gc]);
+}
+
+// Projections a = alpha F (e^{ik.x} u)^T: the product kernel above with the Bloch
+// functions turned into digits on the way into shared memory instead of
+// written to memory in 14 bytes per 8 and read back.  Warp 0 streams the
+// projectors' digits and the phases of a K block (32 grid points), warp 1
+// issues, warps 2-17 both convert (thread: band tid / 8, four grid points: 64-
+// byte reads, and 16-byte stores that fill all banks) and drain (32 rows x 16
+// columns each).  A chunk is drained after the first block of the next one is
+// converted, so that the tensor core has that block while they drain.  The
+// phases' products (4 FP64 operations per complex entry: 4096 clocks a block at
+// two per SM and clock) run beside the digit products' 4864 clocks.
+// The CTAs take equal shares of all tiles' chunks; sums of a tile that two or more share
+// go to `part`, exact as they are, and oz_join adds them.
+__global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ CUtensorMap ma, const OzProject p) {
+  extern __shared__ unsigned char oz_raw[];
+  unsigned char* sm = (unsigned char*)(((uintptr_t)oz_raw + 1023) & ~(uintptr_t)1023);
+  unsigned char* const bs = sm + OZ_AS * OZ_A + OZ_BD;   // first B slot
+  double2* phs = (double2*)(sm + OZ_AS * OZ_A + OZ_BAREA);
+  unsigned long long* bars = (unsigned long long*)(phs + OZ_PH * (OZ_KB / 2));
+  constexpr int NBAR = 2 * OZ_AS + 2 * OZ_BS + 2 * OZ_PH + 1 + OZ_S + 1;
+  uint32_t* tmem_slot = (uint32_t*)(bars + NBAR);
+  volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+  volatile int* a_issued = (volatile int*)(tmem_slot + 2);
+  volatile int* p_issued = (volatile int*)(tmem_slot + 3);
+  const uint32_t sa = smem_u32(sm), sb = sa + OZ_AS * OZ_A + OZ_BD, sp = smem_u32(phs), b0 = smem_u32(bars);
+  auto afull = [&](int s) { return b0 + 8 * s; };
+  auto aempty = [&](int s) { return b0 + 8 * (OZ_AS + s); };
+  auto bfull = [&](int s) { return b0 + 8 * (2 * OZ_AS + s); };
+  auto bempty = [&](int s) { return b0 + 8 * (2 * OZ_AS + OZ_BS + s); };
+  auto pfull = [&](int s) { return b0 + 8 * (2 * OZ_AS + 2 * OZ_BS + s); };
+  auto pempty = [&](int s) { return b0 + 8 * (2 * OZ_AS + 2 * OZ_BS + OZ_PH + s); };
+  const uint32_t tfull = b0 + 8 * (2 * OZ_AS + 2 * OZ_BS + 2 * OZ_PH), tempty = tfull + 8, fin = b0 + 8 * (NBAR - 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < OZ_AS; ++s) {
+      mbar_init(afull(s), 1);
+      mbar_init(aempty(s), 1);
+    }
+    for (int s = 0; s < OZ_BS; ++s) {
+      mbar_init(bfull(s), OZ_W);
+      mbar_init(bempty(s), 1);
+    }
+    for (int s = 0; s < OZ_PH; ++s) {
+      mbar_init(pfull(s), 1);
+      mbar_init(pempty(s), OZ_W);
+    }
+    mbar_init(tfull, 1);
+    for (int s = 0; s < OZ_S; ++s) mbar_init(tempty + 8 * s, OZ_W);
+    mbar_init(fin, 1);
+    *abort_flag = 0;
+    *a_issued = 0;
+    *p_issued = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int z = 0; z <= OZ_BS; ++z)   // the tiles of zeros
+    for (int i = threadIdx.x; i < OZ_BD / 16; i += blockDim.x)
+      reinterpret_cast<uint4*>(sm + OZ_AS * OZ_A + z * (OZ_B + OZ_BD))[i] = make_uint4(0, 0, 0, 0);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  if (warp == 1) {
+    tmem_alloc(smem_u32(tmem_slot), 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  // this CTA's blocks: from block bq of tile tq, `total` of them
+  const long long chunks = (long long)p.ntiles * p.cpt;
+  const long long q0 = oz_start(blockIdx.x, chunks, gridDim.x), q1 = oz_start(blockIdx.x + 1, chunks, gridDim.x);
+  const int tq = (int)(q0 / p.cpt), bq = 2 * (int)(q0 % p.cpt), te = (int)((q1 - 1) / p.cpt);
+  const int be = min(2 * (int)((q1 - 1) % p.cpt) + 2, p.kb);
+  const int total = (te - tq) * p.kb + be - bq;
+
+  if (warp == 0 && lane == 0) {
+    int ia = 0, ip = 0, t = tq, b = bq, tp = tq, bp = bq;
+    bool ok = true;
+    auto phases = [&]() {
+      const int s = ip % OZ_PH;
+      if (!mbar_wait(pempty(s), ((uint32_t)(ip / OZ_PH) & 1u) ^ 1u, abort_flag, OZ_WAIT_NS)) return false;
+      mbar_expect_tx(pfull(s), OZ_KB / 2 * sizeof(double2));
+      bulk_load(sp + s * (OZ_KB / 2) * (int)sizeof(double2),
+                p.phase + ((size_t)(tp / p.mt / p.nt) * p.kb + bp) * (OZ_KB / 2), OZ_KB / 2 * sizeof(double2), pfull(s));
+      *p_issued = ++ip;
+      if (++bp == p.kb) bp = 0, ++tp;
+      return true;
+    };
+    for (int i = 0; i < total && ok; ++i) {
+      while (ok && ip < total && ip < i + OZ_PH - 1) ok = phases();
+      const int m = t % p.mt;
+      for (int j = 0; j < OZ_S && ok; ++j) {
+        const int q = ia % OZ_AS;
+        if (!(ok = mbar_wait(aempty(q), ((uint32_t)(ia / OZ_AS) & 1u) ^ 1u, abort_flag, OZ_WAIT_NS))) break;
+        mbar_expect_tx(afull(q), OZ_A);
+        tma_load_3d(sa + q * OZ_A, &ma, afull(q), b * OZ_KB, m * OZ_M, j);
+        *a_issued = ++ia;
+      }
+      if (++b == p.kb) b = 0, ++t;
+    }
+    if (!ok) {
+      atomicExch(p.err, 1);
+      *abort_flag = 1;
+    }
+  } else if (warp == 1 && lane == 0) {
+    int chunk = 0, sl = 0, b = bq;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int i = 0; i < total; ++i) {
+      const int s = i % OZ_BS;
+      if (!(ok = mbar_wait(bfull(s), (uint32_t)(i / OZ_BS) & 1u, abort_flag, OZ_WAIT_NS))) break;
+      const unsigned long long db = sdesc_sw128(sb + s * (OZ_B + OZ_BD));
+      if (!(ok = issue_block(tmem, sa, db, (b & 1) == 0, chunk, sl, ph, afull(0), aempty(0), tempty, abort_flag))) break;
+      mma_commit(bempty(s));
+      if ((b & 1) == 1 || b + 1 == p.kb) {
+        mma_commit(tfull);
+        ++chunk;
+      }
+      if (++b == p.kb) b = 0;
+    }
+    if (!ok) {
+      atomicExch(p.err, 1);
+      *abort_flag = 1;
+    }
+    mma_commit(fin);   // issued products retire before tensor memory is freed
+    const unsigned long long t0 = gtime();
+    while (!mbar_try(fin, 0) && gtime() - t0 < OZ_WAIT_NS) {
+    }
+  } else if (warp >= 2) {
+    const int tid = threadIdx.x - 64, nl = tid >> 3, xg = tid & 7;
+    const int row = (warp & 3) * 32 + lane, col0 = ((warp - 2) >> 2) * 16;
+    const uint32_t ta = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col0;
+    const uint32_t dst = smem_u32(bs) + nl * 128 + ((xg ^ (nl & 7)) << 4);
+    long long hi[16], lo[16];   // units 2^-30 (s < 3) and 2^-62
+#pragma unroll
+    for (int c = 0; c < 16; ++c) hi[c] = lo[c] = 0;
+    int chunk = 0;
+    // the accumulators of the oldest chunk not yet drained, which ends with block b of tile t
+    auto drain = [&](int t, int b, bool last) {
+      if (!__all_sync(0xffffffffu, mbar_wait(tfull, (uint32_t)chunk & 1u, abort_flag, OZ_WAIT_NS))) return false;
+      ++chunk;
+      tc_fence_after();
+#pragma unroll
+      for (int s = 0; s < OZ_S; ++s) {
+        float v[16];
+        tmem_ld16(ta + s * OZ_N, v);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty + 8 * s);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          const int d = __float2int_rn(v[c]);
+          if (s < 3)
+            hi[c] += (long long)d * (1 << (8 * (2 - s)));
+          else
+            lo[c] += (long long)d * (1 << (8 * (6 - s)));
+        }
+      }
+      if (b + 1 != p.kb && !last) return true;
+      if (b + 1 == p.kb && (t > tq || bq == 0)) {
+#pragma unroll
+        for (int c = 0; c < 16; ++c) oz_store(p, t, row, col0 + c, hi[c], lo[c]);
+      } else {
+        longlong2* o = p.part + ((size_t)(2 * blockIdx.x + (t > tq ? 1 : 0)) * OZ_M + row) * OZ_N + col0;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) o[c] = make_longlong2(hi[c], lo[c]);
+      }
+#pragma unroll
+      for (int c = 0; c < 16; ++c) hi[c] = lo[c] = 0;
+      return true;
+    };
+    double2 w[4];
+    const double2* base = nullptr;   // this thread's first entry of the tile, nullptr: a column beyond the last
+    int e = 0, en = 0;
+    auto tile = [&](int t) {
+      const int r = t / p.mt, n = (r % p.nt) * OZ_N + nl, k = r / p.nt;
+      const bool in = t <= te && n < p.nb;
+      base = in ? p.u + ((size_t)k * p.nx + 4 * xg) * p.nb + n : nullptr;
+      en = in ? p.expo[(size_t)k * p.nb + n] : 0;
+    };
+    auto load = [&](int b) {
+      const int left = base ? p.nx - b * (OZ_KB / 2) - 4 * xg : 0;
+      const double2* a = base + (size_t)b * (OZ_KB / 2) * p.nb;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        w[i] = make_double2(0.0, 0.0);
+        if (i < left) w[i] = load_in_place(a + (size_t)i * p.nb);
+      }
+      // lines of a block four ahead into L2: the loads then cover an L2 hit, not HBM's latency
+      if ((nl & 7) == 0 && b + 4 < p.kb) {
+        a += (size_t)4 * (OZ_KB / 2) * p.nb;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i < left - 4 * (OZ_KB / 2)) asm volatile("prefetch.global.L2 [%0];" ::"l"(a + (size_t)i * p.nb));
+      }
+    };
+    tile(tq);
+    load(bq);
+    int t = tq, b = bq, t1 = tq, b1 = bq;
+    bool ok = true;
+    for (int i = 0; i < total; ++i) {
+      if (b == 0 || i == 0) e = en;
+      const int s = i % OZ_BS, q = i % OZ_PH;
+      ok = __all_sync(0xffffffffu, mbar_wait(pfull(q), (uint32_t)(i / OZ_PH) & 1u, abort_flag, OZ_WAIT_NS) &&
+                                       mbar_wait(bempty(s), ((uint32_t)(i / OZ_BS) & 1u) ^ 1u, abort_flag, OZ_WAIT_NS));
+      if (!ok) break;
+      oz_fix f[8];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const double2 c = phs[q * (OZ_KB / 2) + 4 * xg + j];
+        f[2 * j] = oz_fixed(w[j].x * c.x - w[j].y * c.y, e);
+        f[2 * j + 1] = oz_fixed(w[j].x * c.y + w[j].y * c.x, e);
+      }
+#pragma unroll
+      for (int j = 0; j < OZ_S; ++j)
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + s * (OZ_B + OZ_BD) + j * OZ_BD),
+                     "r"(oz_digit2(f[0], f[1], j)), "r"(oz_digit2(f[2], f[3], j)), "r"(oz_digit2(f[4], f[5], j)),
+                     "r"(oz_digit2(f[6], f[7], j))
+                     : "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(bfull(s));
+        mbar_arrive(pempty(q));
+      }
+      const int tc = t, bc = b;
+      if (++b == p.kb) b = 0, tile(++t);
+      if (i + 1 < total) load(b);
+      if (i > 0 && (bc & 1) == 0 && !(ok = drain(t1, b1, false))) break;
+      t1 = tc, b1 = bc;
+    }
+    if (ok) ok = drain(t1, b1, true);
+    if (!ok && lane == 0) {
+      atomicExch(p.err, 1);
+      *abort_flag = 1;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag) {
+    // copies in flight land before the CTA leaves (the last use of each slot)
+    const int na = *a_issued, np = *p_issued;
+    for (int k = na > OZ_AS ? na - OZ_AS : 0; k < na; ++k) {
+      const unsigned long long t0 = gtime();
+      while (!mbar_try(afull(k % OZ_AS), (uint32_t)(k / OZ_AS) & 1u) && gtime() - t0 < OZ_WAIT_NS) {
+      }
+    }
+    for (int k = np > OZ_PH ? np - OZ_PH : 0; k < np; ++k) {
+      const unsigned long long t0 = gtime();
+      while (!mbar_try(pfull(k % OZ_PH), (uint32_t)(k / OZ_PH) & 1u) && gtime() - t0 < OZ_WAIT_NS) {
+      }
+    }
   }
   __syncthreads();
-  const int xg = threadIdx.x & 7, x = x0 + 4 * xg;
-  double2 c[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) c[i] = ph[4 * xg + i];
-  for (int n = threadIdx.x >> 3; n < nb; n += 32) {
-    int flag = 0;
-    const int e = oz_exponent(keys[(size_t)kl * nb + n], &flag) + 1;
-    if (xg == 0 && blockIdx.x == 0) {
-      scale[(size_t)kl * nb + n] = scalbn(1.0, e);
-      if (flag) atomicOr(bad, 1);
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+}
+
+// tiles shared by several CTAs of oz_project (grid of them): the sum of their
+// partial sums, one block per tile and 16 rows
+__global__ void __launch_bounds__(256) oz_join(const OzProject p, int grid) {
+  const int t = blockIdx.x;
+  const long long chunks = (long long)p.ntiles * p.cpt, qa = (long long)t * p.cpt, qb = qa + p.cpt - 1;
+  auto owner = [&](long long q) {
+    long long c = q * grid / chunks;
+    while (oz_start(c + 1, chunks, grid) <= q) ++c;
+    return (int)c;
+  };
+  const int ca = owner(qa), cb = owner(qb);
+  if (ca == cb) return;
+  for (int i = threadIdx.x; i < 16 * OZ_N; i += 256) {
+    const int row = blockIdx.y * 16 + i / OZ_N, col = i % OZ_N;
+    long long hi = 0, lo = 0;
+    for (int c = ca; c <= cb; ++c) {
+      const int slot = 2 * c + (oz_start(c, chunks, grid) / p.cpt < t ? 1 : 0);
+      const longlong2 v = p.part[((size_t)slot * OZ_M + row) * OZ_N + col];
+      hi += v.x;
+      lo += v.y;
     }
-    oz_fix f[8];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const double2 w = x + i < nx ? u[((size_t)k * nx + x + i) * nb + n] : make_double2(0.0, 0.0);
-      f[2 * i] = oz_fixed(w.x * c[i].x - w.y * c[i].y, e);
-      f[2 * i + 1] = oz_fixed(w.x * c[i].y + w.y * c[i].x, e);
-    }
-    __half* o = dig + ((size_t)kl * OZ_S * nb + n) * kp + 2 * x;
-#pragma unroll
-    for (int i = 0; i < OZ_S; ++i)
-      *reinterpret_cast<uint4*>(o + (size_t)i * nb * kp) =
-          make_uint4(oz_digit2(f[0], f[1], i), oz_digit2(f[2], f[3], i), oz_digit2(f[4], f[5], i),
-                     oz_digit2(f[6], f[7], i));
+    oz_store(p, t, row, col, hi, lo);
   }
 }
 
@@ -425,7 +753,6 @@ bool digit_map(CUtensorMap* m, const __half* base, int kp, int rows, int z, int 
 size_t bse_oz_digit_bytes(int batches, int rows, int kp) {
   return (((size_t)batches * OZ_S * rows * kp * sizeof(__half)) + 255) / 256 * 256;
 }
-int bse_oz_tiles(int rows_a, int rows_b) { return (rows_a + OZ_M - 1) / OZ_M * ((rows_b + OZ_N - 1) / OZ_N); }
 int bse_oz_kp(int k) { return (k + OZ_KB - 1) / OZ_KB * OZ_KB; }
 
 bse_status bse_oz_split_rows(const double2* x, int rows, int n, const double2* d, int batches, int pair,
@@ -435,22 +762,111 @@ bse_status bse_oz_split_rows(const double2* x, int rows, int n, const double2* d
   return cudaGetLastError() == cudaSuccess ? BSE_OK : BSE_ERR_CUDA;
 }
 
-bse_status bse_oz_split_bloch(const double2* u, const int* nk, const int* nx, const double* kshift, int nb, int k0,
-                              int nkc, const bse_oz_operand& o, unsigned* keys, int* bad, cudaStream_t st) {
+// The scratch holds the projectors' digits, the phases of as many k points per
+// pass as fit 256 MB, and the shared tiles' sums: 87 MB for 8^3 k x 16^3 points
+// (a gigabyte of Bloch digits took 1.0 ms to allocate and free).
+bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb, const double* kshift,
+                          const double2* f, int np, double dv, double2* a, cudaStream_t st, bool* done) {
+  *done = false;
   oz_mesh ms;
   for (int i = 0; i < 3; ++i) {
     ms.nk[i] = nk[i];
     ms.nx[i] = nx[i];
     ms.s[i] = kshift ? kshift[i] : 0.0;
   }
-  const int nxt = nx[0] * nx[1] * nx[2];
-  const int per = nxt > 8192 ? 1024 : 512;
-  cudaMemsetAsync(keys, 0, (size_t)nkc * nb * sizeof(unsigned), st);
-  oz_col_keys<<<dim3((unsigned)((nxt + per - 1) / per), (unsigned)((nb + 31) / 32), (unsigned)nkc), 256, 0, st>>>(
-      u + (size_t)k0 * nxt * nb, nxt, nb, per, keys);
-  oz_split_bloch<<<dim3((unsigned)(o.kp / OZ_KB), (unsigned)nkc), 256, 0, st>>>(u, ms, k0, nb, o.kp, keys,
-                                                                                (__half*)o.digits, o.scale, bad);
-  return cudaGetLastError() == cudaSuccess ? BSE_OK : BSE_ERR_CUDA;
+  const int nkt = nk[0] * nk[1] * nk[2], nxt = nx[0] * nx[1] * nx[2], kp = bse_oz_kp(2 * nxt);
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaFuncSetAttribute(oz_project, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_PSMEM) != cudaSuccess) {
+    cudaGetLastError();
+    return BSE_ERR_CUDA;
+  }
+  const size_t per = (size_t)kp / 2 * sizeof(double2);
+  const int nkc = (int)std::min<size_t>({(size_t)nkt, std::max<size_t>(((size_t)256 << 20) / per, 1), (size_t)32768});
+  auto pad = [](size_t n) { return (n + 255) / 256 * 256; };
+  long long ntab = 0;
+  for (int i = 0; i < 3; ++i) ntab += (long long)nk[i] * nx[i];
+  const size_t sd = bse_oz_digit_bytes(1, 2 * np, kp), sf = pad((size_t)2 * np * sizeof(double)), sph = pad(nkc * per);
+  const size_t stab = pad((size_t)ntab * sizeof(double2)), skey = pad((size_t)nkc * nb * sizeof(unsigned));
+  const size_t ssc = pad((size_t)nkc * nb * sizeof(double)), spart = (size_t)2 * sms * OZ_M * OZ_N * sizeof(longlong2);
+  struct Scratch {
+    void* p = nullptr;
+    ~Scratch() {
+      if (p) cudaFree(p);
+    }
+  } sc;
+  if (cudaMalloc(&sc.p, sd + sf + sph + stab + 2 * skey + ssc + spart + 256) != cudaSuccess) {
+    cudaGetLastError();
+    sc.p = nullptr;
+    return BSE_OK;
+  }
+  char* q = (char*)sc.p;
+  bse_oz_operand A;
+  A.digits = q, q += sd;
+  A.scale = (double*)q, q += sf;
+  A.rows = 2 * np, A.kp = kp;
+  OzProject p{};
+  double2* phase = (double2*)q;
+  q += sph;
+  double2* tab = (double2*)q;
+  q += stab;
+  unsigned* keys = (unsigned*)q;
+  q += skey;
+  int* expo = (int*)q;
+  q += skey;
+  double* scale = (double*)q;
+  q += ssc;
+  p.part = (longlong2*)q, q += spart;
+  int* word = (int*)q;   // {wait gave up, out of range}
+  p.phase = phase;
+  p.expo = expo;
+  p.scale = scale;
+  p.scale_a = A.scale;
+  p.nx = nxt;
+  p.nb = nb;
+  p.np2 = 2 * np;
+  p.nkt = nkt;
+  p.mt = (2 * np + OZ_M - 1) / OZ_M;
+  p.nt = (nb + OZ_N - 1) / OZ_N;
+  p.kb = kp / OZ_KB;
+  p.cpt = (p.kb + 1) / 2;
+  p.alpha = dv;
+  p.out = (double*)a;
+  p.err = word;
+  CUtensorMap ma;
+  if (!digit_map(&ma, (const __half*)A.digits, kp, A.rows, OZ_S, OZ_M, 1)) return BSE_ERR_CUDA;
+  cudaMemsetAsync(word, 0, 2 * sizeof(int), st);
+  // rows (Re f, Im f) and (-Im f, Re f): real and imaginary part of conj(f) times a column
+  bse_status s = bse_oz_split_rows(f, np, nxt, nullptr, 1, 1, A, word + 1, st);
+  oz_tables<<<(unsigned)((ntab + 255) / 256), 256, 0, st>>>(ms, tab);
+  const int xrows = nxt > 8192 ? 1024 : 512;   // grid points per block of the key kernel
+  for (int k = 0; k < nkt && s == BSE_OK; k += nkc) {
+    const int n = std::min(nkc, nkt - k);
+    p.u = u + (size_t)k * nxt * nb;
+    p.k0 = k;
+    p.ntiles = p.mt * p.nt * n;
+    cudaMemsetAsync(keys, 0, (size_t)n * nb * sizeof(unsigned), st);
+    oz_col_keys<<<dim3((unsigned)((nxt + xrows - 1) / xrows), (unsigned)((nb + 31) / 32), (unsigned)n), 256, 0, st>>>(
+        p.u, nxt, nb, xrows, keys);
+    oz_bloch_scales<<<(unsigned)(((long long)n * nb + 255) / 256), 256, 0, st>>>(keys, n * nb, expo, scale, word + 1);
+    oz_phases<<<dim3((unsigned)((kp / 2 + 255) / 256), (unsigned)n), 256, 0, st>>>(ms, tab, k, kp / 2, phase);
+    const int grid = (int)std::min<long long>(sms, (long long)p.ntiles * p.cpt);
+    oz_project<<<grid, OZ_PT, OZ_PSMEM, st>>>(ma, p);
+    oz_join<<<dim3((unsigned)p.ntiles, OZ_M / 16), 256, 0, st>>>(p, grid);
+    if (cudaGetLastError() != cudaSuccess) s = BSE_ERR_CUDA;
+  }
+  int hw[2] = {0, 0};
+  if (s == BSE_OK && (cudaMemcpyAsync(hw, word, sizeof(hw), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+                      cudaStreamSynchronize(st) != cudaSuccess))
+    s = BSE_ERR_CUDA;
+  if (s != BSE_OK) {
+    cudaStreamSynchronize(st);   // before the scratch goes
+    return s;
+  }
+  if (hw[0]) return BSE_ERR_TIMEOUT;
+  *done = hw[1] == 0;
+  return BSE_OK;
 }
 
 bse_status bse_oz_gemm(const bse_oz_operand& a, const bse_oz_operand& b, int batches, double alpha, double* out,

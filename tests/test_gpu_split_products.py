@@ -121,3 +121,15 @@ def test_projection_with_nan_takes_the_fp64_kernel():
     assert not np.any(np.isfinite(a[:, 3, 7]))
     a[:, 3, 7] = ref[:, 3, 7]
     assert np.abs(a - ref).max() <= 1e-12 * np.abs(ref).max()
+
+
+def test_projection_in_several_passes():
+    """More k points than one pass's phases hold; an odd number of blocks a tile."""
+    nk, nx = (10, 8, 8), (32, 31, 29)
+    rng = np.random.default_rng(12)
+    u = rng.standard_normal((640, 32 * 31 * 29, 1)) + 1j * rng.standard_normal((640, 32 * 31 * 29, 1))
+    f = S.complex_normal(rng, (1, 32 * 31 * 29))
+    a = bse.local_projection(u, nk, nx, f, 0.11, (0.5, 0.0, 0.25))
+    ref = O.local_projection(u, nk, nx, f, 0.11, (0.5, 0.0, 0.25))
+    um = np.maximum(np.abs(u.real), np.abs(u.imag)).max(axis=1)
+    assert np.all(np.abs(a - ref) <= 4 * 2 * np.prod(nx) * 2.0 ** -51 * 0.11 * _row_max(f)[:, None, None] * um[None])
