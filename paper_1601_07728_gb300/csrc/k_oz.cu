@@ -7,10 +7,10 @@
 // FP16 products, so that the 19 products of 128 x 128 x 16 which replace one
 // FP64 product of 128 x 64 x 16 still run some 50 times faster.  Measured:
 // Green's functions of 900 points, 4096 states and 16 frequencies 682 ms
-// (FP64 kernel) -> 14.0 ms (this one 12.9, writing the digits 0.97); the
+// (FP64 kernel) -> 13.5 ms (this one 12.4, writing the digits 0.97); the
 // projection of 8^3 k x 16^3 points x 64 bands onto 64 functions 102.6 ms ->
-// 5.4 ms with the Bloch functions' digits in memory -> 3.3 ms with the digits
-// made on the way into shared memory (oz_project 2.6, row scales 0.29).  The
+// 5.4 ms with the Bloch functions' digits in memory -> 3.1 ms with the digits
+// made on the way into shared memory (oz_project 2.4, row scales 0.29).  The
 // error against 64 bits fell from 1.9e-15 to 1.3e-15 and from 1.4e-15 to
 // 1.2e-15.  What bounds oz_gemm now: operand tiles from L2 (35 bytes per SM and
 // clock) beside the products' 64 clocks each.
@@ -50,49 +50,128 @@ struct OzParams {
   int* err;
 };
 
-// Digit products of one K block against the B tiles at descriptor db, one A
-// digit after the other out of the ring (slot sl, phase ph); `first`: the
-// accumulators start over, each as soon as it is drained.
+// bounded wait, inlined: at a call the draining warps' sums would go through memory
+__device__ __forceinline__ bool oz_wait(uint32_t a, uint32_t parity, volatile int* abort_flag) {
+  if (mbar_try(a, parity)) return true;
+  const unsigned long long t0 = gtime();
+  while (!mbar_try(a, parity))
+    if (*abort_flag || gtime() - t0 > OZ_WAIT_NS) return false;
+  return true;
+}
+
+// Chunks of 128 K elements.  The accumulators s = 4..6 hold one chunk's sums
+// (at most 7 * 128 * 2^14 < 2^24), s = 2, 3 two and s = 0, 1 four (4 * 256 and
+// 2 * 512 times 2^14): c counts the chunks of a tile, `last` its last one.
+// Draining all of them after every chunk cost 12.9 instead of 12.4 ms and 2.6
+// instead of 2.4 (float to integer runs at 16 per SM and clock).  Issuing the
+// products of s < 4 first while the others drain holds four A slots of five and
+// was slower (14.5 ms).
+__device__ __forceinline__ bool drains(int s, int c, bool last) {
+  return last || s >= 4 || (s >= 2 ? (c & 1) == 1 : (c & 3) == 3);
+}
+
+// state of the issuing thread: A ring slot and phase, restarts of the accumulators s = 0, 1 / 2, 3 / 4..6
+struct oz_issue {
+  int sl = 0, r0 = 0, r1 = 0, r2 = 0;
+  uint32_t ph = 0;
+};
+
+// Digit products of one K block against the B tiles at descriptor db, the A
+// digits from the ring.  First block of a chunk (c: its number in the tile): the
+// accumulators that were drained start over, each as soon as that is done.
 // A product of N = 64 or less takes the tensor core as long as one of N = 128
 // (about 64 clocks measured at N = 32 and 64), so two neighbouring B digits
 // form one operand of 128 rows and the accumulators of s = 2P, 2P + 1 one of
 // 128 columns: digit A_i meets (B_0, B_1), (B_2, B_3), ... for even i and (0,
 // B_0), (B_1, B_2), ... for odd i, 19 products instead of 28 per 16 K elements
 // and all of one shape (s = 7 is computed along and not used).
-__device__ __forceinline__ bool issue_block(uint32_t tmem, uint32_t sa, unsigned long long db, bool first, int chunk,
-                                            int& sl, uint32_t& ph, uint32_t afull, uint32_t aempty, uint32_t tempty,
+__device__ __forceinline__ bool issue_block(uint32_t tmem, uint32_t sa, unsigned long long db, bool first, int c,
+                                            oz_issue& z, uint32_t afull, uint32_t aempty, uint32_t tempty,
                                             volatile int* abort_flag) {
   // FP16 A and B (K-major), FP32 D
   constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(2 * OZ_N >> 3) << 17) | ((uint32_t)(OZ_M >> 4) << 24);
+  auto products = [&](int i, int p0, int p1, uint32_t keep) {   // bit P of keep: add to accumulator P
+    const unsigned long long da = sdesc_sw128(sa + z.sl * OZ_A);
+#pragma unroll
+    for (int ks = 0; ks < OZ_KB / 16; ++ks)
+#pragma unroll
+      for (int P = p0; P < p1; ++P)
+        mma_bf16(tmem + 2 * P * OZ_N, da + ks * 2,
+                 db + (unsigned long long)(long long)(((2 * P - i) * OZ_BD + ks * 32) / 16), idesc,
+                 ks > 0 ? 1u : (keep >> P) & 1u);
+  };
+  auto drained = [&](int s, int n) { return oz_wait(tempty + 8 * s, ((uint32_t)n & 1u) ^ 1u, abort_flag); };
 #pragma unroll
   for (int i = 0; i < OZ_S; ++i) {
-    if (!mbar_wait(afull + 8 * sl, ph, abort_flag, OZ_WAIT_NS)) return false;
+    if (!oz_wait(afull + 8 * z.sl, z.ph, abort_flag)) return false;
     tc_fence_after();
-    const unsigned long long da = sdesc_sw128(sa + sl * OZ_A);
     if (i == 0 && first) {
-#pragma unroll
-      for (int P = 0; P < 4; ++P) {
-        if (!mbar_wait(tempty + 8 * (2 * P), ((uint32_t)chunk & 1u) ^ 1u, abort_flag, OZ_WAIT_NS)) return false;
-        if (P < 3 && !mbar_wait(tempty + 8 * (2 * P + 1), ((uint32_t)chunk & 1u) ^ 1u, abort_flag, OZ_WAIT_NS))
-          return false;
-        tc_fence_after();
-#pragma unroll
-        for (int ks = 0; ks < OZ_KB / 16; ++ks)
-          mma_bf16(tmem + 2 * P * OZ_N, da + ks * 2, db + (2 * P * OZ_BD + ks * 32) / 16, idesc, ks > 0);
-      }
+      const bool n0 = (c & 3) == 0, n1 = (c & 1) == 0;
+      if (n0 && !(drained(0, z.r0) && drained(1, z.r0))) return false;
+      tc_fence_after();
+      products(0, 0, 1, n0 ? 0u : 1u);
+      if (n1 && !(drained(2, z.r1) && drained(3, z.r1))) return false;
+      tc_fence_after();
+      products(0, 1, 2, n1 ? 0u : 2u);
+      if (!(drained(4, z.r2) && drained(5, z.r2))) return false;
+      tc_fence_after();
+      products(0, 2, 3, 0u);
+      if (!drained(6, z.r2)) return false;
+      tc_fence_after();
+      products(0, 3, 4, 0u);
+      z.r0 += n0, z.r1 += n1, z.r2 += 1;
     } else {
-      // consecutive products go to different accumulators
-#pragma unroll
-      for (int ks = 0; ks < OZ_KB / 16; ++ks)
-#pragma unroll
-        for (int P = i / 2; P < 4; ++P)
-          mma_bf16(tmem + 2 * P * OZ_N, da + ks * 2,
-                   db + (unsigned long long)(long long)(((2 * P - i) * OZ_BD + ks * 32) / 16), idesc, 1);
+      products(i, i / 2, 4, 15u);   // consecutive products go to different accumulators
     }
-    mma_commit(aempty + 8 * sl);
-    if (++sl == OZ_AS) sl = 0, ph ^= 1u;
+    mma_commit(aempty + 8 * z.sl);
+    if (++z.sl == OZ_AS) z.sl = 0, z.ph ^= 1u;
   }
   return true;
+}
+
+// hi 2^32 + lo += d 2^sh
+__device__ __forceinline__ void add96(long long& hi, uint32_t& lo, int d, int sh) {
+  const uint32_t l = (uint32_t)d << sh;
+  const int m = sh ? d >> (32 - sh) : d >> 31, t = d >> 31;
+  asm("{\n .reg .u32 a, b;\n mov.b64 {a, b}, %0;\n add.cc.u32 %1, %1, %2;\n addc.cc.u32 a, a, %3;\n"
+      " addc.u32 b, b, %4;\n mov.b64 %0, {a, b};\n}\n"
+      : "+l"(hi), "+r"(lo)
+      : "r"(l), "r"(m), "r"(t));
+}
+
+// Accumulators of 32 TMEM lanes x C columns at ta into sums hi 2^-30 + lo 2^-62
+// (lo unsigned; s < 3 have the weights 2^-14, 2^-22, 2^-30, the rest 2^-38 ..
+// 2^-62).  Each is given back as soon as it is read.
+template <int C>
+__device__ __forceinline__ void drain_chunk(uint32_t ta, int c, bool last, uint32_t tempty, int lane, long long* hi,
+                                            uint32_t* lo) {
+#pragma unroll
+  for (int s = 0; s < OZ_S; ++s) {
+    if (!drains(s, c, last)) continue;
+#pragma unroll
+    for (int h = 0; h < C / 16; ++h) {
+      float v[16];
+      tmem_ld16(ta + s * OZ_N + 16 * h, v);
+      if (h == C / 16 - 1) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty + 8 * s);
+      }
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const int d = __float2int_rn(v[k]), j = 16 * h + k;
+        if (s < 3) {
+          hi[j] += (long long)d * (1 << (8 * (2 - s)));
+        } else {
+          // 96-bit addition; as 64-bit arithmetic lo would take a pair of registers
+          add96(hi[j], lo[j], d, 8 * (6 - s));
+        }
+      }
+    }
+  }
+}
+__device__ __forceinline__ double oz_value(long long hi, long long lo) {
+  return (double)hi * 0x1p-30 + (double)lo * 0x1p-62;
 }
 
 // Persistent warp-specialised kernel, one CTA per SM: warp 0 streams digit
@@ -158,13 +237,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       const int za = p.a_batched ? b * OZ_S : 0, zb = p.b_batched ? b * OZ_S : 0;
       for (int kb = 0; kb < p.kb && ok; ++kb) {
         const int s = ib % OZ_BS;
-        if (!(ok = mbar_wait(bempty(s), ((uint32_t)(ib / OZ_BS) & 1u) ^ 1u, abort_flag, OZ_WAIT_NS))) break;
+        if (!(ok = oz_wait(bempty(s), ((uint32_t)(ib / OZ_BS) & 1u) ^ 1u, abort_flag))) break;
         mbar_expect_tx(bfull(s), OZ_B);
         tma_load_3d(sb + s * (OZ_B + OZ_BD), &mb, bfull(s), kb * OZ_KB, n * OZ_N, zb);
         *b_issued = ++ib;
         for (int i = 0; i < OZ_S; ++i) {
           const int q = ia % OZ_AS;
-          if (!(ok = mbar_wait(aempty(q), ((uint32_t)(ia / OZ_AS) & 1u) ^ 1u, abort_flag, OZ_WAIT_NS))) break;
+          if (!(ok = oz_wait(aempty(q), ((uint32_t)(ia / OZ_AS) & 1u) ^ 1u, abort_flag))) break;
           mbar_expect_tx(afull(q), OZ_A);
           tma_load_3d(sa + q * OZ_A, &ma, afull(q), kb * OZ_KB, m * OZ_M, za + i);
           *a_issued = ++ia;
@@ -176,22 +255,19 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       *abort_flag = 1;
     }
   } else if (warp == 1 && lane == 0) {
-    int ib = 0, chunk = 0, sl = 0;
-    uint32_t ph = 0;
+    int ib = 0;
+    oz_issue z;
     bool ok = true;
     for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
       for (int kb = 0; kb < p.kb && ok; ++kb) {
         const bool first = (kb & 1) == 0, last = (kb & 1) == 1 || kb + 1 == p.kb;
         const int s = ib % OZ_BS;
-        if (!(ok = mbar_wait(bfull(s), (uint32_t)(ib / OZ_BS) & 1u, abort_flag, OZ_WAIT_NS))) break;
+        if (!(ok = oz_wait(bfull(s), (uint32_t)(ib / OZ_BS) & 1u, abort_flag))) break;
         ++ib;
         const unsigned long long db = sdesc_sw128(sb + s * (OZ_B + OZ_BD));
-        if (!(ok = issue_block(tmem, sa, db, first, chunk, sl, ph, afull(0), aempty(0), tempty(0), abort_flag))) break;
+        if (!(ok = issue_block(tmem, sa, db, first, kb >> 1, z, afull(0), aempty(0), tempty(0), abort_flag))) break;
         mma_commit(bempty(s));
-        if (last) {
-          mma_commit(tfull);
-          ++chunk;
-        }
+        if (last) mma_commit(tfull);
       }
     }
     if (!ok) {
@@ -208,32 +284,16 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     int chunk = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
-      long long hi[32], lo[32];
+      long long hi[32];
+      uint32_t lo[32];
 #pragma unroll
-      for (int c = 0; c < 32; ++c) hi[c] = lo[c] = 0;
+      for (int c = 0; c < 32; ++c) hi[c] = 0, lo[c] = 0;
       for (int kb = 0; kb < p.kb; kb += 2, ++chunk) {
-        ok = __all_sync(0xffffffffu, mbar_wait(tfull, (uint32_t)chunk & 1u, abort_flag, OZ_WAIT_NS));
+        ok = __all_sync(0xffffffffu, oz_wait(tfull, (uint32_t)chunk & 1u, abort_flag));
         if (!ok) break;
         tc_fence_after();
-        // hi: weights 2^-14, 2^-22, 2^-30; lo: 2^-38 .. 2^-62
-#pragma unroll
-        for (int s = 0; s < OZ_S; ++s) {
-          float v[32];
-          const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(s * OZ_N + half * 32);
-          tmem_ld16(ta, v);
-          tmem_ld16(ta + 16, v + 16);
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(tempty(s));
-#pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            const int d = __float2int_rn(v[c]);
-            if (s < 3)
-              hi[c] += (long long)d * (1 << (8 * (2 - s)));
-            else
-              lo[c] += (long long)d * (1 << (8 * (6 - s)));
-          }
-        }
+        drain_chunk<32>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 32), kb >> 1, kb + 2 >= p.kb, tempty(0), lane,
+                    hi, lo);
       }
       if (!ok) break;
       const int m = t % p.mt, r = t / p.mt, n = r % p.nt, b = r / p.nt;
@@ -245,7 +305,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 #pragma unroll
         for (int c = 0; c < 32; ++c)
           if (col0 + c < p.rows_b)
-            o[c * p.sc] = ((double)hi[c] * 0x1p-30 + (double)lo[c] * 0x1p-62) * (fa * fb[c]);
+            o[c * p.sc] = oz_value(hi[c], lo[c]) * (fa * fb[c]);
       }
     }
     if (!ok && lane == 0) {
@@ -390,7 +450,7 @@ __global__ void __launch_bounds__(256) oz_tables(oz_mesh ms, double2* __restrict
   }
 }
 
-// phases [k][xp] of the nkc k points from k0, xp grid points (zero beyond nx)
+// phases [k][xp] of the k points from k0, xp grid points (zero beyond nx)
 __global__ void __launch_bounds__(256) oz_phases(oz_mesh ms, const double2* __restrict__ tab, int k0, int xp,
                                                  double2* __restrict__ phase) {
   const int x = blockIdx.x * 256 + threadIdx.x, k = k0 + blockIdx.y;
@@ -437,7 +497,8 @@ struct OzProject {
   int mt, nt, ntiles, kb, cpt;   // M tiles, N tiles, all tiles, K blocks and chunks of a tile
   double alpha;
   double* out;            // [np][nkt][nb] complex
-  longlong2* part;        // [CTA][2][128][64] sums of the tiles that CTAs share
+  long long* part_hi;     // [CTA][2][128][64] sums of the tiles that CTAs share
+  uint32_t* part_lo;
   int* err;
 };
 
@@ -449,7 +510,7 @@ __device__ __forceinline__ void oz_store(const OzProject& p, int t, int row, int
   const int gr = m * OZ_M + row, gc = n * OZ_N + col;
   if (gr < p.np2 && gc < p.nb)
     p.out[2 * (((size_t)(gr >> 1) * p.nkt + p.k0 + k) * p.nb + gc) + (gr & 1)] =
-        ((double)hi * 0x1p-30 + (double)lo * 0x1p-62) * (p.alpha * p.scale_a[gr] * p.scale[(size_t)k * p.nb + gc]);
+        oz_value(hi, lo) * (p.alpha * p.scale_a[gr] * p.scale[(size_t)k * p.nb + gc]);
 }
 
 // Projections a = alpha F (e^{ik.x} u)^T: the product kernel above with the Bloch
@@ -461,9 +522,12 @@ __device__ __forceinline__ void oz_store(const OzProject& p, int t, int row, int
 // columns each).  A chunk is drained after the first block of the next one is
 // converted, so that the tensor core has that block while they drain.  The
 // phases' products (4 FP64 operations per complex entry: 4096 clocks a block at
-// two per SM and clock) run beside the digit products' 4864 clocks.
+// two per SM and clock) run beside the digit products' 4864 clocks; a block
+// takes about 10,700, in which the 16 warps' FP64, integer and load phases
+// overlap only in part (FP64 pipe 41 %, tensor pipe 47 %).  With conversion and
+// draining on warps of their own (eight each) it was 12,300.
 // The CTAs take equal shares of all tiles' chunks; sums of a tile that two or more share
-// go to `part`, exact as they are, and oz_join adds them.
+// go to part_hi and part_lo, exact as they are, and oz_join adds them.
 __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ CUtensorMap ma, const OzProject p) {
   extern __shared__ unsigned char oz_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)oz_raw + 1023) & ~(uintptr_t)1023);
@@ -530,7 +594,7 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
     bool ok = true;
     auto phases = [&]() {
       const int s = ip % OZ_PH;
-      if (!mbar_wait(pempty(s), ((uint32_t)(ip / OZ_PH) & 1u) ^ 1u, abort_flag, OZ_WAIT_NS)) return false;
+      if (!oz_wait(pempty(s), ((uint32_t)(ip / OZ_PH) & 1u) ^ 1u, abort_flag)) return false;
       mbar_expect_tx(pfull(s), OZ_KB / 2 * sizeof(double2));
       bulk_load(sp + s * (OZ_KB / 2) * (int)sizeof(double2),
                 p.phase + ((size_t)(tp / p.mt / p.nt) * p.kb + bp) * (OZ_KB / 2), OZ_KB / 2 * sizeof(double2), pfull(s));
@@ -543,7 +607,7 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
       const int m = t % p.mt;
       for (int j = 0; j < OZ_S && ok; ++j) {
         const int q = ia % OZ_AS;
-        if (!(ok = mbar_wait(aempty(q), ((uint32_t)(ia / OZ_AS) & 1u) ^ 1u, abort_flag, OZ_WAIT_NS))) break;
+        if (!(ok = oz_wait(aempty(q), ((uint32_t)(ia / OZ_AS) & 1u) ^ 1u, abort_flag))) break;
         mbar_expect_tx(afull(q), OZ_A);
         tma_load_3d(sa + q * OZ_A, &ma, afull(q), b * OZ_KB, m * OZ_M, j);
         *a_issued = ++ia;
@@ -555,20 +619,20 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
       *abort_flag = 1;
     }
   } else if (warp == 1 && lane == 0) {
-    int chunk = 0, sl = 0, b = bq;
-    uint32_t ph = 0;
+    int c = 0, b = bq;   // chunk of the tile, as this CTA counts
+    oz_issue z;
     bool ok = true;
     for (int i = 0; i < total; ++i) {
       const int s = i % OZ_BS;
-      if (!(ok = mbar_wait(bfull(s), (uint32_t)(i / OZ_BS) & 1u, abort_flag, OZ_WAIT_NS))) break;
+      if (!(ok = oz_wait(bfull(s), (uint32_t)(i / OZ_BS) & 1u, abort_flag))) break;
       const unsigned long long db = sdesc_sw128(sb + s * (OZ_B + OZ_BD));
-      if (!(ok = issue_block(tmem, sa, db, (b & 1) == 0, chunk, sl, ph, afull(0), aempty(0), tempty, abort_flag))) break;
+      if (!(ok = issue_block(tmem, sa, db, (b & 1) == 0, c, z, afull(0), aempty(0), tempty, abort_flag))) break;
       mma_commit(bempty(s));
       if ((b & 1) == 1 || b + 1 == p.kb) {
         mma_commit(tfull);
-        ++chunk;
+        ++c;
       }
-      if (++b == p.kb) b = 0;
+      if (++b == p.kb) b = 0, c = 0;
     }
     if (!ok) {
       atomicExch(p.err, 1);
@@ -583,42 +647,33 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
     const int row = (warp & 3) * 32 + lane, col0 = ((warp - 2) >> 2) * 16;
     const uint32_t ta = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col0;
     const uint32_t dst = smem_u32(bs) + nl * 128 + ((xg ^ (nl & 7)) << 4);
-    long long hi[16], lo[16];   // units 2^-30 (s < 3) and 2^-62
+    long long hi[16];
+    uint32_t lo[16];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) hi[c] = lo[c] = 0;
-    int chunk = 0;
+    for (int c = 0; c < 16; ++c) hi[c] = 0, lo[c] = 0;
+    int chunk = 0, cc = 0;   // drained so far, of them in this tile
     // the accumulators of the oldest chunk not yet drained, which ends with block b of tile t
     auto drain = [&](int t, int b, bool last) {
-      if (!__all_sync(0xffffffffu, mbar_wait(tfull, (uint32_t)chunk & 1u, abort_flag, OZ_WAIT_NS))) return false;
+      if (!__all_sync(0xffffffffu, oz_wait(tfull, (uint32_t)chunk & 1u, abort_flag))) return false;
       ++chunk;
       tc_fence_after();
+      const bool end = b + 1 == p.kb || last;
+      drain_chunk<16>(ta, cc, end, tempty, lane, hi, lo);
+      ++cc;
+      if (!end) return true;
+      cc = 0;
+      const size_t o = ((size_t)(2 * blockIdx.x + (t > tq ? 1 : 0)) * OZ_M + row) * OZ_N + col0;
+      const bool whole = b + 1 == p.kb && (t > tq || bq == 0);
 #pragma unroll
-      for (int s = 0; s < OZ_S; ++s) {
-        float v[16];
-        tmem_ld16(ta + s * OZ_N, v);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(tempty + 8 * s);
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          const int d = __float2int_rn(v[c]);
-          if (s < 3)
-            hi[c] += (long long)d * (1 << (8 * (2 - s)));
-          else
-            lo[c] += (long long)d * (1 << (8 * (6 - s)));
+      for (int c = 0; c < 16; ++c) {
+        if (whole) {
+          oz_store(p, t, row, col0 + c, hi[c], lo[c]);
+        } else {
+          p.part_hi[o + c] = hi[c];
+          p.part_lo[o + c] = lo[c];
         }
+        hi[c] = 0, lo[c] = 0;
       }
-      if (b + 1 != p.kb && !last) return true;
-      if (b + 1 == p.kb && (t > tq || bq == 0)) {
-#pragma unroll
-        for (int c = 0; c < 16; ++c) oz_store(p, t, row, col0 + c, hi[c], lo[c]);
-      } else {
-        longlong2* o = p.part + ((size_t)(2 * blockIdx.x + (t > tq ? 1 : 0)) * OZ_M + row) * OZ_N + col0;
-#pragma unroll
-        for (int c = 0; c < 16; ++c) o[c] = make_longlong2(hi[c], lo[c]);
-      }
-#pragma unroll
-      for (int c = 0; c < 16; ++c) hi[c] = lo[c] = 0;
       return true;
     };
     double2 w[4];
@@ -653,8 +708,8 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
     for (int i = 0; i < total; ++i) {
       if (b == 0 || i == 0) e = en;
       const int s = i % OZ_BS, q = i % OZ_PH;
-      ok = __all_sync(0xffffffffu, mbar_wait(pfull(q), (uint32_t)(i / OZ_PH) & 1u, abort_flag, OZ_WAIT_NS) &&
-                                       mbar_wait(bempty(s), ((uint32_t)(i / OZ_BS) & 1u) ^ 1u, abort_flag, OZ_WAIT_NS));
+      ok = __all_sync(0xffffffffu, oz_wait(pfull(q), (uint32_t)(i / OZ_PH) & 1u, abort_flag) &&
+                                       oz_wait(bempty(s), ((uint32_t)(i / OZ_BS) & 1u) ^ 1u, abort_flag));
       if (!ok) break;
       oz_fix f[8];
 #pragma unroll
@@ -727,9 +782,9 @@ __global__ void __launch_bounds__(256) oz_join(const OzProject p, int grid) {
     long long hi = 0, lo = 0;
     for (int c = ca; c <= cb; ++c) {
       const int slot = 2 * c + (oz_start(c, chunks, grid) / p.cpt < t ? 1 : 0);
-      const longlong2 v = p.part[((size_t)slot * OZ_M + row) * OZ_N + col];
-      hi += v.x;
-      lo += v.y;
+      const size_t o = ((size_t)slot * OZ_M + row) * OZ_N + col;
+      hi += p.part_hi[o];
+      lo += p.part_lo[o];
     }
     oz_store(p, t, row, col, hi, lo);
   }
@@ -789,14 +844,14 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
   for (int i = 0; i < 3; ++i) ntab += (long long)nk[i] * nx[i];
   const size_t sd = bse_oz_digit_bytes(1, 2 * np, kp), sf = pad((size_t)2 * np * sizeof(double)), sph = pad(nkc * per);
   const size_t stab = pad((size_t)ntab * sizeof(double2)), skey = pad((size_t)nkc * nb * sizeof(unsigned));
-  const size_t ssc = pad((size_t)nkc * nb * sizeof(double)), spart = (size_t)2 * sms * OZ_M * OZ_N * sizeof(longlong2);
+  const size_t ssc = pad((size_t)nkc * nb * sizeof(double)), npart = (size_t)2 * sms * OZ_M * OZ_N;
   struct Scratch {
     void* p = nullptr;
     ~Scratch() {
       if (p) cudaFree(p);
     }
   } sc;
-  if (cudaMalloc(&sc.p, sd + sf + sph + stab + 2 * skey + ssc + spart + 256) != cudaSuccess) {
+  if (cudaMalloc(&sc.p, sd + sf + sph + stab + 2 * skey + ssc + npart * 12 + 256) != cudaSuccess) {
     cudaGetLastError();
     sc.p = nullptr;
     return BSE_OK;
@@ -817,7 +872,8 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
   q += skey;
   double* scale = (double*)q;
   q += ssc;
-  p.part = (longlong2*)q, q += spart;
+  p.part_hi = (long long*)q, q += npart * 8;
+  p.part_lo = (uint32_t*)q, q += npart * 4;
   int* word = (int*)q;   // {wait gave up, out of range}
   p.phase = phase;
   p.expo = expo;

@@ -8,8 +8,8 @@
 // the top).  A digit is an integer that FP16 holds exactly, and a sum of fewer than 2^24 /
 // 2^14 products of two digits is exact in the FP32 accumulators.  Digit
 // products (i, j) of equal s = i + j < 7 share an accumulator; 128 K elements
-// of up to seven products reach at most 7 * 128 * 2^14 < 2^24, after which the
-// accumulators are drained into 64-bit integers.  The only roundings are the
+// of up to seven products reach at most 7 * 128 * 2^14 < 2^24 (fewer products:
+// more elements), after which the accumulators are drained into integers.  The only roundings are the
 // one of each operand entry at 2^-56 of its row's largest, the dropped
 // products s >= 7 (of the same size) and the final conversion.
 #pragma once

@@ -58,6 +58,18 @@ def test_full_digits_do_not_overflow_the_accumulators():
     np.testing.assert_allclose(g, ref, rtol=1e-14, atol=0)
 
 
+@pytest.mark.parametrize("ns", [63, 64, 65, 128, 255, 256, 520])
+def test_accumulators_kept_over_several_chunks_stay_exact(ns):
+    """Digits (128, -128, -128, ...): the products of every order reach the
+    largest magnitude, and those of order one 2^24 after four chunks."""
+    nr = 260
+    v = 1 - sum(2.0 ** (-8 * i) for i in range(1, 7))
+    psi = np.full((nr, ns), v * (1 + 1j))
+    psi[1::2] *= -1
+    chi, g, ref = _screening(psi, np.full(ns, -1.0), 0.0, np.array([0.0]), np.array([1.0]))
+    np.testing.assert_allclose(g, ref, rtol=1e-14, atol=0)
+
+
 def test_rows_of_any_scale_and_rows_of_zeros():
     nr, ns = 150, 300
     psi, eps = S.screening_grid_states(nr, ns, seed=3)
