@@ -293,12 +293,15 @@ bse_status bse_jacobi_diag(bse_handle* h, double* diag);
  * u [Nk][Nx][Nb] (periodic parts, as for bse_setup), f [n_proj][Nx] the local
  * functions sampled on the cell's grid (zero outside their radius), k and x
  * indexed as in bse_setup, kshift [3] or NULL, dv the volume per grid point;
- * a [n_proj][Nk][Nb].  All complex128, host or device; FP64 arithmetic.
- * Work runs on `stream` (NULL: legacy default) and the call returns when a is
- * written.  Allocates staging copies of host arrays.  Returns
+ * a [n_proj][Nk][Nb].  All complex128, host or device; FP64 accuracy (large
+ * problems as exactly split tensor-core products, with scratch allocated for
+ * the call; without it, or for Inf/NaN and magnitudes outside 2^+-400, on the
+ * FP64 pipe).  Work runs on `stream` (NULL: legacy default) and the call returns
+ * when a is written.  Allocates staging copies of host arrays.  Returns
  * BSE_ERR_INVALID_ARG (before any device work) for a NULL u, nk, nx, f or a,
  * n_bands < 1, n_proj outside 1..4096, nk[d] outside 1..16, nx[d] < 1 or
- * n_bands > Nx; BSE_ERR_OOM or BSE_ERR_CUDA from staging or the launch. */
+ * n_bands > Nx; BSE_ERR_OOM or BSE_ERR_CUDA from staging or the launch;
+ * BSE_ERR_TIMEOUT where a bounded wait of the tensor-core kernel gave up. */
 bse_status bse_local_projection(const bse_c128* u, const int* nk, const int* nx, int n_bands, const double* kshift,
                                 const bse_c128* f, int n_proj, double dv, bse_c128* a, void* stream);
 
@@ -312,9 +315,12 @@ bse_status bse_local_projection(const bse_c128* u, const int* nk, const int* nx,
  * [n_states] eV, chi0 [n_r][n_r]; green [n_t][n_r][n_r] receives the G_j or
  * may be NULL.  Complex128 / FP64, host or device; work on `stream` (NULL:
  * legacy default), returns when the outputs are written.  Allocates staging
- * and the G_j scratch.  Returns BSE_ERR_INVALID_ARG (before any device work)
- * for a NULL psi, eps, t, w or chi0, n_r, n_states or n_t < 1, n_r > 65535 or
- * n_t > 65535; BSE_ERR_OOM or BSE_ERR_CUDA from staging or the launches.  A
+ * and the G_j scratch, and for large problems that of exactly split tensor-core
+ * products (without it, or for Inf/NaN and magnitudes outside 2^+-400: the FP64
+ * pipe).  Returns BSE_ERR_INVALID_ARG (before any device work) for a NULL psi,
+ * eps, t, w or chi0, n_r, n_states or n_t < 1, n_r > 65535 or n_t > 65535;
+ * BSE_ERR_OOM or BSE_ERR_CUDA from staging or the launches; BSE_ERR_TIMEOUT
+ * where a bounded wait of the tensor-core kernel gave up.  A
  * node t_j = 0 with some eps[K] == mu sits on the integrand's pole and gives
  * non-finite values: the caller's nodes must avoid it (mu between two levels,
  * or t_j > 0). */

@@ -18,7 +18,7 @@
 //
 // L2,3 workload (8^3 k, 16^3 grid, 64 bands, 6 columns), FP64 kernels before:
 // band->grid 6.89 -> 0.92 ms, grid->band 8.53 -> 0.89 ms (+ 0.11 for phi's
-// digits, 0.07 for the last sum), H psi 15.0 -> 3.2 ms.  Against quadruple
+// digits, 0.07 for the last sum), H psi 15.0 -> 2.85 ms.  Against quadruple
 // precision the error of H psi falls from 6.3e-17..7.5e-17 to 4.8e-17..5.2e-17.
 // What bounds it: the integer instructions that split U (HBM would take 0.32 ms).
 #include "bse_internal.cuh"
