@@ -7,6 +7,9 @@
 // system, before bse_setup (whose short-range term takes A as input).
 #include "bse_internal.cuh"
 
+#include <algorithm>
+#include <cmath>
+
 namespace {
 
 constexpr int LP = 16, LN = 16, LX = 32;   // projector, band and grid tile of one 256-thread block
@@ -69,10 +72,18 @@ __global__ void __launch_bounds__(256) local_proj_kernel(const double2* __restri
 bse_status bse_local_projection_device(const double2* u, const int* nk, const int* nx, int nb, const double* kshift,
                                        const double2* f, int np, double dv, double2* a, cudaStream_t st) {
   const int nkt = nk[0] * nk[1] * nk[2];
-  // from 2^22 complex products on (FP64 kernel: about 0.1 ms) the tensor-core
-  // form; K is bounded by its 64-bit partial sums
+  // Tensor-core form or FP64 kernel, from their times (us) as measured over 1 to
+  // 512 k, 512 to 13,824 points, 16 to 64 bands and 1 to 64 functions.  FP64: a
+  // block walks the grid, 152 of them at a time.  Tensor cores: scratch and
+  // launches, and 5.6 per K block of 32 points and SM.  (4^3 k, 8^3 points, 32
+  // bands, 9 functions: 344 us against 355; 2^3 k, 9^3, 27, 27: 475 against 325.)
+  // K is bounded by the 64-bit partial sums.
   const double nxd = (double)nx[0] * nx[1] * nx[2];
-  if ((double)nkt * nxd * nb * np >= 4194304.0 && nxd <= 1048576.0) {
+  const double blocks = (double)nkt * ((nb + LN - 1) / LN) * ((np + LP - 1) / LP);
+  const double tiles = (double)nkt * ((nb + 63) / 64) * ((2 * np + 127) / 128);
+  const double fp64 = 50.0 + 0.585 * nxd * std::max(1.0, blocks / 152);
+  const double tensor = 320.0 + 5.6 * tiles * std::ceil(nxd / 32) / 152;
+  if (tensor < fp64 && nxd <= 1048576.0) {
     bool done = false;
     const bse_status s = bse_oz_project(u, nk, nx, nb, kshift, f, np, dv, a, st, &done);
     if (s != BSE_OK || done) return s;
