@@ -103,6 +103,10 @@ __device__ __forceinline__ Tile decode(const TcParams& p, int t) {
 // tiles 73 % filled), one column: band->grid 597 -> 501 us (496 at the copy
 // rate), grid->band 707 -> 558 (521); 8^3 k, 16^3 points, 64 bands (no padding),
 // six columns: 185 -> 171 and 185 -> 174 us (174 and 177 at the copy rate).
+// From N = 48 on the products are issued in a rolled loop: the longer ones hide
+// it, and the steadier release of the stages streams better (20 steps with 18
+// columns 14.43 -> 14.28 ms, the 48^3 supercell with 18 columns 2.47 -> 2.41; at
+// N = 16 and 32 the straight line wins, 9.69 -> 9.25 and 11.75 -> 11.55 ms).
 template <int MODE>   // 0: band->grid, 1: grid->band, 2: grid->band from the row-major U~
 __global__ void __launch_bounds__(TC_THREADS, 1)
     tc_gemm(const __grid_constant__ CUtensorMap ma_hi, const __grid_constant__ CUtensorMap ma_lo,
@@ -238,7 +242,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const unsigned long long a_lo = a_hi + (TC_M * 128) / 16;
         const unsigned long long b_hi = sdesc_sw128(st + 2 * a_bytes), b_lo = b_hi + b_bytes / 16;
         const int left = p.k_len - (tl.kb0 + kb) * TC_KB;
-        if (left >= TC_KB) {
+        if (left >= TC_KB && p.nn < 48) {
 #pragma unroll
           for (int ks = 0; ks < TC_KB / 16; ++ks) {
             mma_bf16(d, a_hi + ks * ASTEP, b_hi + ks * 2, idesc, (kb | ks) != 0);
@@ -246,7 +250,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             mma_bf16(d, a_lo + ks * ASTEP, b_hi + ks * 2, idesc, 1);
           }
         } else {
-          for (int ks = 0; ks * 16 < left; ++ks) {
+#pragma unroll 1
+          for (int ks = 0; ks < TC_KB / 16 && ks * 16 < left; ++ks) {
             mma_bf16(d, a_hi + ks * ASTEP, b_hi + ks * 2, idesc, (kb | ks) != 0);
             mma_bf16(d, a_hi + ks * ASTEP, b_lo + ks * 2, idesc, 1);
             mma_bf16(d, a_lo + ks * ASTEP, b_hi + ks * 2, idesc, 1);
