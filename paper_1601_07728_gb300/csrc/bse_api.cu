@@ -133,6 +133,13 @@ void free_handle(bse_handle* h) {
   delete h;
 }
 
+// status of a call that ends with s: BSE_ERR_TIMEOUT where a bounded wait gave
+// up under it (its outputs, and s with them, are then not to be used), else s
+bse_status with_waits(bse_handle* h, bse_status s) {
+  const bse_status t = bse_tc_status(h);
+  return t != BSE_OK ? t : s;
+}
+
 #define TRY(x)                   \
   do {                           \
     bse_status _s = (x);         \
@@ -291,13 +298,12 @@ bse_status bse_haydock(bse_handle* h, const bse_c128* b, int n_vec, int n_steps,
   TRY(stage_in(h, ss, steps_done, (size_t)n_vec * sizeof(int), false, "steps_done"));
   bse_status s = bse_haydock_device(h, (const double2*)sb.dev, n_vec, n_steps, reorth, (double*)sa.dev,
                                     (double*)sbb.dev, (int*)ss.dev);
-  if (s != BSE_OK && s != BSE_ERR_BREAKDOWN && s != BSE_ERR_NAN) return s;
+  if (s != BSE_OK && s != BSE_ERR_BREAKDOWN && s != BSE_ERR_NAN) return with_waits(h, s);
   TRY(stage_out(h, sa, a, (size_t)n_vec * n_steps * sizeof(double), "a copy-out"));
   TRY(stage_out(h, sbb, bcoef, (size_t)n_vec * (n_steps + 1) * sizeof(double), "b copy-out"));
   TRY(stage_out(h, ss, steps_done, (size_t)n_vec * sizeof(int), "steps copy-out"));
   TRY(bse_cuda_check(h, cudaStreamSynchronize(h->stream), "haydock sync"));
-  TRY(bse_tc_status(h));
-  return s;
+  return with_waits(h, s);
 }
 
 bse_status bse_haydock_batch(bse_handle* const* hs, const bse_c128* const* b, int n_sites, int n_vec, int n_steps,
@@ -332,6 +338,9 @@ bse_status bse_haydock_batch(bse_handle* const* hs, const bse_c128* const* b, in
     TRY(stage_out(h, sbb[s], bcoef[s], (size_t)n_vec * (n_steps + 1) * sizeof(double), "b copy-out"));
     TRY(stage_out(h, ss[s], steps_done[s], (size_t)n_vec * sizeof(int), "steps copy-out"));
     TRY(bse_cuda_check(h, cudaStreamSynchronize(h->stream), "batch sync"));
+    const bse_status w = with_waits(h, st[s]);
+    if (w != st[s]) worst = w;
+    site_status[s] = w;
   }
   return worst;
 }
@@ -420,13 +429,12 @@ bse_status bse_gmres(bse_handle* h, const bse_c128* b, const bse_c128* z, int n_
   TRY(stage_in(h, sr, rel_resid, (size_t)n_z * sizeof(double), false, "rel_resid"));
   bse_status s = bse_gmres_device(h, (const double2*)sb.dev, (const double2*)sz.dev, n_z, rtol, restart,
                                   max_iter, precond, (double2*)sx.dev, (int*)si.dev, (double*)sr.dev);
-  if (s != BSE_OK && s != BSE_ERR_NOT_CONVERGED) return s;
+  if (s != BSE_OK && s != BSE_ERR_NOT_CONVERGED) return with_waits(h, s);
   TRY(stage_out(h, sx, x, (size_t)n_z * h->N * sizeof(double2), "x copy-out"));
   TRY(stage_out(h, si, iters, (size_t)n_z * sizeof(int), "iters copy-out"));
   TRY(stage_out(h, sr, rel_resid, (size_t)n_z * sizeof(double), "rel copy-out"));
   TRY(bse_cuda_check(h, cudaStreamSynchronize(h->stream), "gmres sync"));
-  TRY(bse_tc_status(h));
-  return s;
+  return with_waits(h, s);
 }
 
 bse_status bse_gmres_set_mlp(bse_handle* h, bse_mlp* m) {

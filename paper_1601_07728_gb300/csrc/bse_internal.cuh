@@ -267,7 +267,7 @@ bool bse_ozh_takes(const bse_handle* h, int nc);   // nc columns are worth its l
 void bse_ozh_free(bse_handle* h);
 bse_status bse_ozh_band_to_grid(bse_handle* h, const double2* psi, int nc);
 bse_status bse_ozh_grid_to_band(bse_handle* h, const double2* psi, double2* hpsi, int nc);
-bse_status bse_ozh_status(bse_handle* h);
+int* bse_ozh_word(const bse_handle* h);   // device error word of its kernels
 
 // tensor-core band<->grid path (k_tc.cu)
 bse_status bse_tc_prepare(bse_handle* h);
@@ -296,7 +296,7 @@ bse_status bse_tc_apply_onepass(bse_handle* h, const double2* psi, double2* hpsi
                                 const bse_dotfuse* fuse, bool wait_side);
 // true if the k-transform can run on part of the grid (x-slabs)
 bool bse_kconv_takes_slabs(const bse_handle* h);
-bse_status bse_tc_status(bse_handle* h);   // device error word of the tensor-core pipeline
+bse_status bse_tc_status(bse_handle* h);   // BSE_ERR_TIMEOUT if a tensor-core pipeline wait of the handle gave up (once)
 void bse_tc_free(bse_handle* h);
 
 // Krylov drivers (k_krylov.cu)

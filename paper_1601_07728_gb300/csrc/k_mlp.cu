@@ -1131,6 +1131,9 @@ bse_status bse_mlp_loss_grad(bse_handle* h, bse_mlp* m, double omega, double gam
     s = bse_cuda_check(h, cudaMemcpyAsync(grad, m->g, (size_t)NPARAM * sizeof(float), cudaMemcpyDefault, h->stream),
                        "grad copy");
   if (s == BSE_OK) s = bse_cuda_check(h, cudaStreamSynchronize(h->stream), "grad sync");
+  // the products with H may have given up a bounded wait: the gradient is then no result
+  const bse_status t = bse_tc_status(h);
+  if (t != BSE_OK) s = t;
   cudaMemsetAsync(m->g, 0, (size_t)NPARAM * sizeof(float), h->stream);
   cudaFree(p);
   cudaFree(u);
@@ -1243,6 +1246,8 @@ extern "C" bse_status bse_mlp_train(bse_handle* const* hs, const bse_c128* const
       }
     }
     if (st == BSE_OK) st = bse_cuda_check(h, cudaStreamSynchronize(h->stream), "harvest sync");
+    const bse_status t = bse_tc_status(h);   // a bounded wait that gave up, whatever became of it since
+    if (t != BSE_OK) st = t;
     cudaFree(bd);
     cudaFree(zd);
     cudaFree(x);
@@ -1277,6 +1282,9 @@ extern "C" bse_status bse_mlp_train(bse_handle* const* hs, const bse_c128* const
       // probes with |r| <= 1e-5 |b| belong to an already converged solve and are skipped
       st = loss_grad(h, m, zh[zi].x, zh[zi].y, T, R[samples[k].sys] + (size_t)zi * T * N, p, u, v, &l,
                      1e-10 * b2[samples[k].sys], krylov_steps);
+      const bse_status t = bse_tc_status(h);   // before the weights take a step
+      if (t != BSE_OK) st = t;
+      if (st != BSE_OK) break;
       tot += l;
       if (++inb == batch || k + 1 == samples.size()) {
         m->t += 1;

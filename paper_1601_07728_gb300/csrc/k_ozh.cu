@@ -734,13 +734,5 @@ bse_status bse_ozh_grid_to_band(bse_handle* h, const double2* psi, double2* hpsi
   return bse_cuda_check(h, e == cudaSuccess ? cudaGetLastError() : e, "grid->band (split FP64)");
 }
 
-// reports (once) a wait that gave up in one of the kernels
-bse_status bse_ozh_status(bse_handle* h) {
-  OzhState* z = (OzhState*)h->ozh;
-  int e = 0;
-  if (cudaMemcpy(&e, z->err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return bse_cuda_check(h, cudaGetLastError(), "contraction status");
-  if (!e) return BSE_OK;
-  if (cudaMemset(z->err, 0, sizeof(int)) != cudaSuccess) return bse_cuda_check(h, cudaGetLastError(), "contraction status reset");
-  return bse_fail(h, BSE_ERR_TIMEOUT, "tensor-core pipeline wait timed out");
-}
+// the device word that a wait which gave up sets
+int* bse_ozh_word(const bse_handle* h) { return ((OzhState*)h->ozh)->err; }

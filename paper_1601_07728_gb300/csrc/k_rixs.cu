@@ -145,7 +145,12 @@ extern "C" bse_status bse_rixs(bse_handle* core, bse_handle* val, const bse_c128
   if (pk != BSE_PRECOND_NONE && pk != BSE_PRECOND_JACOBI && pk != BSE_PRECOND_MLP)
     return bse_fail(core, BSE_ERR_INVALID_ARG, "rixs: unknown preconditioner");
   const bse_status sg = bse_gmres_device(core, bd, zd, n_z, rtol, restart, max_iter, pk, (double2*)sx.p, id, rd);
-  if (sg != BSE_OK && sg != BSE_ERR_NOT_CONVERGED) return sg;
+  // the outcome `r`, or BSE_ERR_TIMEOUT where a bounded wait of either handle gave up before it
+  auto with_waits = [&](bse_status r) {
+    const bse_status tc = bse_tc_status(core), tv = bse_tc_status(val);
+    return tc != BSE_OK ? tc : tv != BSE_OK ? bse_fail(core, tv, val->err) : r;
+  };
+  if (sg != BSE_OK && sg != BSE_ERR_NOT_CONVERGED) return with_waits(sg);
   // 2. emission on the final state's stream, after the absorption
   cudaEvent_t ev = nullptr;
   if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
@@ -160,7 +165,8 @@ extern "C" bse_status bse_rixs(bse_handle* core, bse_handle* val, const bse_c128
   if (s != BSE_OK) return bse_fail(core, s, "rixs: emission launch failed");
   // 3. final-state recursion, every incoming energy as one start vector
   const bse_status sh = bse_haydock_device(val, (const double2*)sy.p, n_z, n_steps, 0, ad, bcd, sdd);
-  if (sh != BSE_OK && sh != BSE_ERR_BREAKDOWN) return bse_fail(core, sh, "rixs: final-state Haydock: " + val->err);
+  if (sh != BSE_OK && sh != BSE_ERR_BREAKDOWN)
+    return with_waits(bse_fail(core, sh, "rixs: final-state Haydock: " + val->err));
   if (!d_a) cudaMemcpyAsync(a, ad, nz * n_steps * sizeof(double), cudaMemcpyDeviceToHost, val->stream);
   if (!d_bc) cudaMemcpyAsync(bcoef, bcd, nz * (n_steps + 1) * sizeof(double), cudaMemcpyDeviceToHost, val->stream);
   if (!d_s) cudaMemcpyAsync(steps_done, sdd, nz * sizeof(int), cudaMemcpyDeviceToHost, val->stream);
@@ -168,9 +174,5 @@ extern "C" bse_status bse_rixs(bse_handle* core, bse_handle* val, const bse_c128
   if (!d_r) cudaMemcpyAsync(rel_resid, rd, nz * sizeof(double), cudaMemcpyDeviceToHost, st);
   if (cudaStreamSynchronize(val->stream) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
     return bse_cuda_check(core, cudaGetLastError(), "rixs sync");
-  s = bse_tc_status(core);
-  if (s == BSE_OK) s = bse_tc_status(val);
-  if (s != BSE_OK) return s;
-  if (sg == BSE_ERR_NOT_CONVERGED) return sg;
-  return sh;
+  return with_waits(sg == BSE_ERR_NOT_CONVERGED ? sg : sh);
 }

@@ -1528,16 +1528,20 @@ extern "C" bse_status bse_autotune(bse_handle* h, int n_vec, int reps, int* spli
 }
 
 bse_status bse_tc_status(bse_handle* h) {
-  if (h->ozh) return bse_ozh_status(h);
-  if (h->prec != BSE_PREC_SPLIT_BF16 || !h->tmap_host) return BSE_OK;
-  TcState* ts = (TcState*)h->tmap_host;
+  int* word = nullptr;
+  if (h->ozh)
+    word = bse_ozh_word(h);
+  else if (h->prec == BSE_PREC_SPLIT_BF16 && h->tmap_host)
+    word = ((TcState*)h->tmap_host)->err;
+  if (!word) return BSE_OK;
+  // on the handle's stream: other streams' work is not waited for
   int e = 0;
-  if (cudaMemcpy(&e, ts->err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return bse_cuda_check(h, cudaGetLastError(), "tc status");
-  if (e) {
-    // reported once: clear the word so that later calls on the handle start clean
-    if (cudaMemset(ts->err, 0, sizeof(int)) != cudaSuccess) return bse_cuda_check(h, cudaGetLastError(), "tc status reset");
-    return bse_fail(h, BSE_ERR_TIMEOUT, "tensor-core pipeline wait timed out");
-  }
-  return BSE_OK;
+  bse_status s = bse_cuda_check(h, cudaMemcpyAsync(&e, word, sizeof(int), cudaMemcpyDeviceToHost, h->stream), "tc status");
+  if (s == BSE_OK) s = bse_cuda_check(h, cudaStreamSynchronize(h->stream), "tc status");
+  if (s != BSE_OK || !e) return s;
+  // reported once: clear the word so that later calls on the handle start clean
+  s = bse_cuda_check(h, cudaMemsetAsync(word, 0, sizeof(int), h->stream), "tc status reset");
+  if (s == BSE_OK) s = bse_cuda_check(h, cudaStreamSynchronize(h->stream), "tc status reset");
+  if (s != BSE_OK) return s;
+  return bse_fail(h, BSE_ERR_TIMEOUT, "tensor-core pipeline wait timed out");
 }

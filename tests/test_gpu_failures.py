@@ -89,3 +89,40 @@ def test_device_memory_cap_gives_oom_without_leak(monkeypatch):
     out = g.apply_h(psi)
     g.close()
     assert rel(out[0], ref[0]) < 1e-5
+
+
+def _raises_timeout(f, *args, **kw):
+    with pytest.raises(bse.BSEError) as e:
+        f(*args, **kw)
+    assert e.value.status == bse.BSE_ERR_TIMEOUT
+
+
+@pytest.mark.parametrize("precision", ["fp64", "split_bf16"])
+def test_every_call_over_h_reports_a_wait_that_gave_up(l23, precision):
+    """The tensor-core kernels of the FP64 form and of the split-bf16 form, on a
+    size where a tile takes longer than the limit of 2 microseconds: each entry
+    point that applies H says BSE_ERR_TIMEOUT, and the call after it, with the
+    normal limit, has nothing left to report."""
+    torch = pytest.importorskip("torch")
+    s, psi, ref = l23
+    stream = torch.cuda.Stream()
+    sysg = bse.System(s, precision=precision, max_vec=4, stream=stream.cuda_stream)
+    net = bse.MLP(S.mlp_init(3))
+    r = torch.from_numpy(psi).cuda()
+    torch.cuda.synchronize()
+    z = np.array([2.0 + 0.5j])
+    calls = [lambda: sysg.apply_h(psi), lambda: sysg.haydock(psi[0], 4), lambda: bse.haydock_batch([sysg], [psi], 4),
+             lambda: sysg.gmres(psi[0], z, rtol=1e-3, restart=4, max_iter=4),
+             lambda: net.loss_grad(sysg, 2.0, 0.5, r, steps=0), lambda: net.loss_grad(sysg, 2.0, 0.5, r, steps=2),
+             lambda: net.train([sysg], [psi[0]], z, epochs=1, batch=1, lr=1e-3, steps=1)]
+    tol = 1e-13 if precision == "fp64" else 1e-5
+    weights = net.params()
+    for f in calls:
+        sysg.set_wait_limit(2e-6)
+        _raises_timeout(f)
+        sysg.set_wait_limit(2.0)
+        assert rel(sysg.apply_h(psi)[0], ref[0]) < tol
+    assert np.array_equal(net.params(), weights)   # no step on a gradient that is none
+    outs, sts = bse.haydock_batch([sysg], [psi], 4)
+    assert list(sts) == [bse.BSE_OK] and outs[0][2][0] == 4
+    sysg.close()
