@@ -67,7 +67,11 @@ typedef enum {
  * and short-range terms are FP64 in every mode. */
 typedef enum {
   BSE_PREC_FP64 = 0,        /* u complex128, sums to FP64 accuracy: FP64 FMAs, or exactly
-                               split FP16 tensor-core products where they are faster  */
+                               split FP16 tensor-core products where they are faster.
+                               Those hold an entry to 2^-56 of its row's (u: of a grid
+                               point over bands, of a band over the grid) or column's
+                               largest; sums a b whose error that could lift above
+                               about 2^-53 sum |a| |b| are formed by FP64 FMAs           */
   BSE_PREC_FP32 = 1,        /* u complex64, FP32 FMA, FP32 k-transforms               */
   BSE_PREC_SPLIT_BF16 = 2   /* u split into bf16 hi+lo, tcgen05 tensor-core MMAs with
                                3 products (hi*hi + hi*lo + lo*hi), FP32 accumulation */

@@ -16,11 +16,15 @@
 // 118 clocks each instead of 48, and N = 128 takes 64 where N = 16 takes 39).
 // An accumulator holds 128 K elements exactly and is then drained.
 //
-// L2,3 workload (8^3 k, 16^3 grid, 64 bands, 6 columns), FP64 kernels before:
-// band->grid 6.89 -> 0.92 ms, grid->band 8.53 -> 0.89 ms (+ 0.11 for phi's
-// digits, 0.07 for the last sum), H psi 15.0 -> 2.85 ms.  Against quadruple
-// precision the error of H psi falls from 6.3e-17..7.5e-17 to 4.8e-17..5.2e-17.
-// What bounds it: the integer instructions that split U (HBM would take 0.32 ms).
+// The digits hold an entry to 2^-56 of its row's largest, so every sum comes with
+// that of its magnitudes, and those for which this is not FP64 accuracy are
+// formed on the FP64 pipe (oz_accept; columns with Inf or NaN and columns below
+// 2^-960 wholly): band->grid's in the kernel, grid->band's in ozh_final.
+//
+// L2,3 workload (8^3 k, 16^3 grid, 64 bands, 6 columns): H psi 15.0 ms with the
+// FP64 kernels -> 2.88; of it band->grid 0.97, grid->band with the last sum 0.98,
+// digits of psi and phi 0.13, k-transform 1.08 (with the magnitude sums left out
+// 0.98, 0.96 and 0.13; 2.85 in all).
 #include "bse_internal.cuh"
 #include "oz_dev.cuh"
 #include "tc_ptx.cuh"
@@ -42,10 +46,10 @@ constexpr int H_BSTRIDE = H_B + (OZ_S - 1) * H_BD;   // a stage's B and the zero
 constexpr int H_N = 8 * H_J;                         // accumulator columns, s = 0..7
 constexpr int H_BAREA = H_STAGES * H_BSTRIDE + H_BD; // ... zeros after the last stage
 constexpr int H_CONV = 16;                           // conversion warps
-constexpr int H_THREADS = 32 * (2 + 4 + H_CONV);
+constexpr int H_MAG = 2;                             // warps of the magnitude sums
+constexpr int H_THREADS = 32 * (2 + 4 + H_CONV + H_MAG);
 constexpr size_t H_SMEM = 1024 + (size_t)H_STAGES * OZ_S * H_A + H_BAREA + 256;
 constexpr int H_CHUNK = 128 / H_KB;                  // K blocks until an accumulator is drained
-constexpr int E_NAN = 1 << 20;                       // exponent of a row that holds Inf or NaN
 constexpr unsigned long long H_DRAIN_NS = 2000000000ull;
 
 // K-major operand in rows of 64 bytes (64-byte swizzle, 8-row groups 512 bytes apart)
@@ -77,11 +81,84 @@ __device__ __forceinline__ double h_value(long long hi, long long lo, int e) {
   return __hiloint2double(h + (e << 20), __double2loint(v));
 }
 
+// a warp's 8 x 8 matrices of FP16 at the lanes' row addresses, as magnitudes
+__device__ __forceinline__ void ldmatrix4_abs(uint32_t a, uint32_t* r) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) r[i] &= 0x7fff7fffu;
+}
+__device__ __forceinline__ void mma_16x8x16(float* c, const uint32_t* a, const uint32_t* b) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+// FP64 sums over i < n of u_i p_c,i for the H_C columns p_c = p + c cs (those
+// from nc on repeat the first), by one warp: lane L returns part (L >> 1) & 1 of column L >> 2
+__device__ __noinline__ double warp_columns(const double2* __restrict__ u, const double2* __restrict__ p, size_t cs, int nc,
+                                            int n) {
+  double v[2 * H_C];
+#pragma unroll
+  for (int j = 0; j < 2 * H_C; ++j) v[j] = 0.0;
+  const int lane = threadIdx.x & 31;
+  for (int i = lane; i < n; i += 32) {
+    const double2 a = u[i];
+#pragma unroll
+    for (int c = 0; c < H_C; ++c) {
+      const double2 b = p[(c < nc ? c : 0) * cs + i];
+      v[2 * c] = fma(a.x, b.x, fma(-a.y, b.y, v[2 * c]));
+      v[2 * c + 1] = fma(a.x, b.y, fma(a.y, b.x, v[2 * c + 1]));
+    }
+  }
+  // sums by exchanged halves: lane L ends with number L >> 1
+#pragma unroll
+  for (int h = H_C; h >= 1; h >>= 1) {
+    const bool up = (lane & (2 * h)) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double mine = up ? v[h + i] : v[i], other = up ? v[i] : v[h + i];
+      v[i] = mine + __shfl_xor_sync(0xffffffffu, other, 2 * h);
+    }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+// FP64 sum of conj(u_i) p_i over i < n, entries of u `us` apart, by one warp; every lane returns it
+__device__ double2 warp_dot(const double2* __restrict__ u, long long us, const double2* __restrict__ p, int n) {
+  double x = 0.0, y = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x & 31; i < n; i += 32) {
+    const double2 a = u[i * us], b = p[i];
+    x = fma(a.x, b.x, fma(a.y, b.y, x));
+    y = fma(a.x, b.y, fma(-a.y, b.x, y));
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    x += __shfl_xor_sync(0xffffffffu, x, off);
+    y += __shfl_xor_sync(0xffffffffu, y, off);
+  }
+  return make_double2(x, y);
+}
+
+// A column of psi or phi: its norm in units of its scale and sqrt(2 n) of its n
+// entries other than 0; norm < 0: not to be summed from digits (Inf, NaN, or too small for them)
+struct __align__(8) HColumn {
+  float norm, root;
+};
+// norm_a: norm of the row of U; m: sum of magnitudes
+__device__ __forceinline__ bool column_accepts(HColumn c, float norm_a, float m) {
+  return c.norm >= 0.f && (c.norm == 0.f || norm_a == 0.f || oz_accept(m, fminf(norm_a, c.root), c.norm));
+}
+
 struct HParams {
   const double2* u;       // [nk][nx][nb]
   const short* ea;        // exponent per A row: [nk][nx] (mode 0) or [nk][nb] (mode 1)
+  const float* na;        // mode 0: norm per grid row in units of its scale
   const int* eb;          // exponent per column: [nk][H_C]
+  const HColumn* cb;      // mode 0: columns [nk][H_C]
+  const double2* psi;     // mode 0: this pass's columns of psi [c][nk][nb]
   double2* out;           // mode 0: phi; mode 1: partial sums [split][nk][H_C][nb]
+  float* sums;            // mode 1: sums of magnitudes, as out
   int nk, nx, nb, mt, nsplit, ntiles, kb, kb_per_split;
   int nc, c0, ncc;        // mode 0: columns of phi, first column, columns of this pass
   int* err;
@@ -89,14 +166,15 @@ struct HParams {
 };
 
 // Persistent, one CTA per SM: warp 0 brings B with TMA, warp 1 issues the
-// products, warps 2-5 drain tensor memory, warps 6-13 read U (the next stage's
-// loads are in flight while one is split) and write its digits.
+// products, warps 2-5 drain tensor memory, warps 6-21 read U (the next stage's
+// loads are in flight while one is split) and write its digits, warps 22 and 23
+// sum the magnitudes and say which results they accept (oz_accept).
 template <int MODE>
 __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constant__ CUtensorMap mb, const HParams p) {
   extern __shared__ unsigned char ozh_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)ozh_raw + 1023) & ~(uintptr_t)1023);
   unsigned long long* bars = (unsigned long long*)(sm + H_STAGES * OZ_S * H_A + H_BAREA);
-  uint32_t* tmem_slot = (uint32_t*)(bars + 3 * H_STAGES + 5);
+  uint32_t* tmem_slot = (uint32_t*)(bars + 3 * H_STAGES + 9);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   volatile int* issued = (volatile int*)(tmem_slot + 2);
   const uint32_t sbase = smem_u32(sm);
@@ -107,17 +185,19 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
   auto tfull = [&](int a) { return smem_u32(&bars[3 * H_STAGES + a]); };
   auto tempty = [&](int a) { return smem_u32(&bars[3 * H_STAGES + 2 + a]); };
   const uint32_t fin = smem_u32(&bars[3 * H_STAGES + 4]);
+  auto stored = [&](int a) { return smem_u32(&bars[3 * H_STAGES + 5 + a]); };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < H_STAGES; ++s) {
       mbar_init(afull(s), H_CONV);
       mbar_init(bfull(s), 1);
-      mbar_init(empty(s), 1);
+      mbar_init(empty(s), 1 + H_MAG);   // read by the products and the magnitude sums
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(tfull(a), 1);
       mbar_init(tempty(a), 4);
     }
+    for (int a = 0; a < 4; ++a) mbar_init(stored(a), 4);
     mbar_init(fin, 1);
     *abort_flag = 0;
     *issued = 0;
@@ -210,9 +290,9 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
   } else if (warp < 6) {
     const int q = warp & 3, row = q * 32 + lane;
     const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16);
-    int chunk = 0;
+    int chunk = 0, tiles = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
+    for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x, ++tiles) {
       int k, m, sp, b0, b1;
       tile(t, k, m, sp, b0, b1);
       long long hi[H_J], lo[H_J];   // units 2^-38 (s <= 3) and 2^-70 (s = 4..7)
@@ -249,14 +329,13 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
 #pragma unroll
           for (int c = 0; c < H_C; ++c)
             if (c < p.ncc) {
-              const int e = eb[c];
-              double2 o = make_double2(nan(""), nan(""));
-              if (e != E_NAN)
-                o = make_double2(h_value(hi[2 * c], lo[2 * c], ea + e - 70),
-                                 h_value(hi[2 * c + 1], lo[2 * c + 1], ea + e - 70));
-              p.out[((size_t)k * p.nc + p.c0 + c) * p.nx + x] = o;
+              const int e = eb[c] + ea - 70;
+              p.out[((size_t)k * p.nc + p.c0 + c) * p.nx + x] =
+                  make_double2(h_value(hi[2 * c], lo[2 * c], e), h_value(hi[2 * c + 1], lo[2 * c + 1], e));
             }
         }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(stored(tiles & 3));
       } else {
         double v[H_J];
         const int n = (m * H_M + row) >> 1;
@@ -264,16 +343,112 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
 #pragma unroll
         for (int j = 0; j < H_J; ++j) {
           if ((j >> 1) >= p.ncc) continue;
-          const int e = eb[j >> 1];
-          v[j] = e == E_NAN ? nan("") : h_value(hi[j], lo[j], ea + e - 70);
+          v[j] = h_value(hi[j], lo[j], ea + eb[j >> 1] - 70);
         }
         // psi'_{c,n} = (D[2n][2c] + D[2n+1][2c+1]) + i (D[2n][2c+1] - D[2n+1][2c])
-        double2* o = p.out + ((size_t)sp * p.nk + k) * H_C * p.nb + n;
+        const size_t o = ((size_t)sp * p.nk + k) * H_C * p.nb + n;
 #pragma unroll
         for (int c = 0; c < H_C; ++c) {
           if (c >= p.ncc) continue;
           const double w0 = __shfl_xor_sync(0xffffffffu, v[2 * c], 1), w1 = __shfl_xor_sync(0xffffffffu, v[2 * c + 1], 1);
-          if ((lane & 1) == 0 && n < p.nb) o[(size_t)c * p.nb] = make_double2(v[2 * c] + w1, v[2 * c + 1] - w0);
+          if ((lane & 1) == 0 && n < p.nb) p.out[o + (size_t)c * p.nb] = make_double2(v[2 * c] + w1, v[2 * c + 1] - w0);
+        }
+      }
+    }
+    if (!ok && lane == 0) {
+      atomicExch(p.err, 1);
+      *abort_flag = 1;
+    }
+  } else if (warp >= 6 + H_CONV) {
+    // ---------------- sums of magnitudes ----------------
+    // 64 rows x 16 columns each with a product of the older tensor-core form on
+    // the leading digits' tiles, beside the stage's seven products of 128 x 128.
+    // Done by the draining warps it held the stages up (band->grid 1.4 instead
+    // of 0.98 ms); their comparison with the norms there alone cost 0.23 ms.
+    const int w = warp - (6 + H_CONV), br = (lane & 7) + ((lane >> 4) << 3);
+    const int row0 = w * 64 + (lane >> 2);   // first of this lane's rows, 8 apart; its columns lane & 3 and 4 on
+    int it = 0, tiles = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x, ++tiles) {
+      int k, m, sp, b0, b1;
+      tile(t, k, m, sp, b0, b1);
+      float c[4][2][4], na[8];
+      HColumn cb[2];
+      if constexpr (MODE == 0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int x = m * H_M + row0 + 8 * i;
+          na[i] = x < p.nx ? p.na[(size_t)k * p.nx + x] : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int col = (lane & 3) + 4 * i;
+          cb[i] = col < p.ncc ? p.cb[(size_t)k * H_C + col] : HColumn{0.f, 0.f};
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 32; ++i) c[i >> 3][(i >> 2) & 1][i & 3] = 0.f;
+      for (int b = b0; b < b1; ++b, ++it) {
+        const int s = it % H_STAGES;
+        const uint32_t ph = (uint32_t)(it / H_STAGES) & 1u;
+        ok = __all_sync(0xffffffffu, mbar_wait(bfull(s), ph, abort_flag, p.wait_ns) &&
+                                         mbar_wait(afull(s), ph, abort_flag, p.wait_ns));
+        if (!ok) break;
+        const uint32_t at = sbase + s * (OZ_S * H_A), bt = bbase + s * H_BSTRIDE;
+#pragma unroll
+        for (int ks = 0; ks < H_KB / 16; ++ks) {
+          uint32_t bq[4];
+          ldmatrix4_abs(bt + br * 64 + (((2 * ks + ((lane >> 3) & 1)) ^ ((br >> 1) & 3)) << 4), bq);
+#pragma unroll
+          for (int mt = 0; mt < 4; ++mt) {
+            const int ar = w * 64 + mt * 16 + (lane & 15);
+            uint32_t aq[4];
+            ldmatrix4_abs(at + ar * 64 + (((2 * ks + (lane >> 4)) ^ ((ar >> 1) & 3)) << 4), aq);
+            mma_16x8x16(c[mt][0], aq, bq);
+            mma_16x8x16(c[mt][1], aq, bq + 2);
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty(s));
+      }
+      if (!ok) break;
+      // both parts of a complex column together, in units of the two scales
+      auto sum = [&](int i, int nt) { return (c[i >> 1][nt][2 * (i & 1)] + c[i >> 1][nt][2 * (i & 1) + 1]) * 0x1p-14f; };
+      if constexpr (MODE == 0) {
+        // bit i * 2 + nt: row row0 + 8 i, column (lane & 3) + 4 nt
+        unsigned refused = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt)
+            if (!column_accepts(cb[nt], na[i], sum(i, nt)) && m * H_M + row0 + 8 * i < p.nx) refused |= 1u << (2 * i + nt);
+        if (!__any_sync(0xffffffffu, refused)) continue;
+        // Those of FP64, over what the draining warps store.  They may be three
+        // tiles ahead (of one stage each), hence four barriers.
+        ok = __all_sync(0xffffffffu, mbar_wait(stored(tiles & 3), (uint32_t)(tiles >> 2) & 1u, abort_flag, p.wait_ns));
+        if (!ok) break;
+        for (int i = 0; i < 64; ++i) {
+          const unsigned f = __shfl_sync(0xffffffffu, refused, 4 * (i & 7) + ((lane >> 2) & 3)) >> (2 * (i >> 3) + (lane >> 4));
+          if (!__any_sync(0xffffffffu, f & 1u)) continue;
+          const int x = m * H_M + w * 64 + i, col = lane >> 2;
+          const double v = warp_columns(p.u + ((size_t)k * p.nx + x) * p.nb, p.psi + (size_t)k * p.nb, (size_t)p.nk * p.nb,
+                                        p.ncc, p.nb);
+          if ((lane & 1) == 0 && (f & 1u))
+            reinterpret_cast<double*>(p.out + ((size_t)k * p.nc + p.c0 + col) * p.nx + x)[(lane >> 1) & 1] = v;
+        }
+      } else {
+        // rows 2n and 2n + 1 (lanes 4 apart) are the parts of band n
+        const size_t o = ((size_t)sp * p.nk + k) * H_C * p.nb;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int n = (m * H_M + row0 + 8 * i) >> 1;
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) {
+            const int col = (lane & 3) + 4 * nt;
+            float v = sum(i, nt);
+            v += __shfl_xor_sync(0xffffffffu, v, 4);
+            if ((lane & 4) == 0 && n < p.nb && col < p.ncc) p.sums[o + (size_t)col * p.nb + n] = v;
+          }
         }
       }
     }
@@ -417,9 +592,20 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
   }
 }
 
-// exponent of every grid row (k, x) over its bands: one warp per row
+// |v|^2 in units of 2^2e
+__device__ __forceinline__ float unit_square(double2 v, int e) {
+  const float x = oz_unit(v.x, e), y = oz_unit(v.y, e);
+  return x * x + y * y;
+}
+__device__ __forceinline__ float warp_sum(float v) {
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
+// exponent and norm (in units of 2^exponent) of every grid row (k, x) over its bands: one warp per row
 __global__ void __launch_bounds__(256) ozh_row_exponents(const double2* __restrict__ u, long long rows, int nb,
-                                                         short* __restrict__ e, int* __restrict__ bad) {
+                                                         short* __restrict__ e, float* __restrict__ norm,
+                                                         int* __restrict__ bad) {
   const int lane = threadIdx.x & 31;
   for (long long r = blockIdx.x * 8ll + (threadIdx.x >> 5); r < rows; r += gridDim.x * 8ll) {
     unsigned key = 0;
@@ -428,18 +614,25 @@ __global__ void __launch_bounds__(256) ozh_row_exponents(const double2* __restri
       key = max(key, max(oz_key(v.x), oz_key(v.y)));
     }
     key = __reduce_max_sync(0xffffffffu, key);
+    int flag = 0;
+    const int er = oz_exponent(key, &flag);
+    float s = 0.f;
+    for (int n = lane; n < nb; n += 32) s += unit_square(u[(size_t)r * nb + n], er);
+    s = warp_sum(s);
     if (lane == 0) {
-      int flag = 0;
-      e[r] = (short)oz_exponent(key, &flag);
+      e[r] = (short)er;
+      norm[r] = sqrtf(s);
       if (flag) atomicOr(bad, 1);
     }
   }
 }
 
-// exponent of every band (k, n) over the grid: blocks of 32 bands x 8 points
+// exponent and norm of every band (k, n) over the grid: blocks of 32 bands x 8 points
 __global__ void __launch_bounds__(256) ozh_band_exponents(const double2* __restrict__ u, int nx, int nb,
-                                                          short* __restrict__ e, int* __restrict__ bad) {
+                                                          short* __restrict__ e, float* __restrict__ norm,
+                                                          int* __restrict__ bad) {
   __shared__ unsigned sk[8][32];
+  __shared__ float ss[8][32];
   const int n = blockIdx.x * 32 + (threadIdx.x & 31), g = threadIdx.x >> 5, k = blockIdx.y;
   unsigned key = 0;
   if (n < nb)
@@ -449,19 +642,30 @@ __global__ void __launch_bounds__(256) ozh_band_exponents(const double2* __restr
     }
   sk[g][threadIdx.x & 31] = key;
   __syncthreads();
+  for (int i = 0; i < 8; ++i) key = max(key, sk[i][threadIdx.x & 31]);
+  int flag = 0;
+  const int en = oz_exponent(key, &flag);
+  float s = 0.f;
+  if (n < nb)
+    for (int x = g; x < nx; x += 8) s += unit_square(u[((size_t)k * nx + x) * nb + n], en);
+  ss[g][threadIdx.x & 31] = s;
+  __syncthreads();
   if (g == 0 && n < nb) {
-    for (int i = 1; i < 8; ++i) key = max(key, sk[i][threadIdx.x]);
-    int flag = 0;
-    e[(size_t)k * nb + n] = (short)oz_exponent(key, &flag);
+    for (int i = 1; i < 8; ++i) s += ss[i][threadIdx.x];
+    e[(size_t)k * nb + n] = (short)en;
+    norm[(size_t)k * nb + n] = sqrtf(s);
     if (flag) atomicOr(bad, 1);
   }
 }
 
-// exponent of a column from the key of its largest entry: any finite scale is
-// accepted, columns below 2^-960 count as zero
-__device__ __forceinline__ int column_exponent(unsigned key) {
-  const int e = (int)(key >> 20) - 1022;
-  return key >= 0x7ff00000u ? E_NAN : e < -960 ? 0 : e;
+// Exponent of a column from the key of its largest entry.  Digits cannot stand
+// for columns with Inf or NaN, or whose largest entry is below 2^-960 (with 2^-e
+// and its products out of range): exponent 0, the sums from the FP64 pipe.
+__device__ __forceinline__ bool column_exponent(unsigned key, int* e) {
+  *e = key ? (int)(key >> 20) - 1022 : 0;
+  if (key < 0x7ff00000u && *e >= -960) return true;
+  *e = 0;
+  return false;
 }
 __device__ unsigned block_key(unsigned v) {
   __shared__ unsigned wm[8];
@@ -472,20 +676,46 @@ __device__ unsigned block_key(unsigned v) {
   for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, wm[w]);
   return m;
 }
+// thread 0 records the column of exponent e from every thread's sum of squares and count of entries
+__device__ void record_column(bool fits, int e, float sq, int count, int* eb, HColumn* cb) {
+  __shared__ float ws[8];
+  __shared__ int wc[8];
+  sq = warp_sum(sq);
+  count = __reduce_add_sync(0xffffffffu, count);
+  if ((threadIdx.x & 31) == 0) {
+    ws[threadIdx.x >> 5] = sq;
+    wc[threadIdx.x >> 5] = count;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
+    sq += ws[w];
+    count += wc[w];
+  }
+  *eb = e;
+  cb->norm = fits ? sqrtf(sq) : -1.f;
+  cb->root = sqrtf(2.f * (float)count);
+}
+__device__ __forceinline__ bool nonzero(double2 v) { return v.x != 0.0 || v.y != 0.0; }
 
 // Digits of psi for band->grid, one block per (k, column): rows 2c = (psi_r,
 // -psi_i) and 2c + 1 = (psi_i, psi_r) along (n; re, im).  dig [k][7][H_J][kp]
 __global__ void __launch_bounds__(64) ozh_psi_digits(const double2* __restrict__ psi, int nk, int nb, int kp,
-                                                     __half* __restrict__ dig, int* __restrict__ eb) {
+                                                     __half* __restrict__ dig, int* __restrict__ eb,
+                                                     HColumn* __restrict__ cb) {
   const int k = blockIdx.x, c = blockIdx.y;
   const double2* p = psi + ((size_t)c * nk + k) * nb;
   unsigned key = 0;
   for (int n = threadIdx.x; n < nb; n += blockDim.x) key = max(key, max(oz_key(p[n].x), oz_key(p[n].y)));
-  const int e = column_exponent(block_key(key));
-  if (threadIdx.x == 0) eb[k * H_C + c] = e;
+  int e;
+  const bool fits = column_exponent(block_key(key), &e);
+  float sq = 0.f;
+  int count = 0;
   uint32_t* o = reinterpret_cast<uint32_t*>(dig) + ((size_t)k * OZ_S * H_J + 2 * c) * (kp / 2);
   for (int n = threadIdx.x; n < nb; n += blockDim.x) {
     const double2 v = p[n];
+    sq += unit_square(v, e);
+    count += nonzero(v);
     const oz_fix fr = oz_fixed(v.x, e), fi = oz_fixed(v.y, e), fm = oz_fixed(-v.y, e);
 #pragma unroll
     for (int i = 0; i < OZ_S; ++i) {
@@ -493,12 +723,14 @@ __global__ void __launch_bounds__(64) ozh_psi_digits(const double2* __restrict__
       o[(size_t)i * H_J * (kp / 2) + kp / 2 + n] = oz_digit2(fi, fr, i);
     }
   }
+  record_column(fits, e, sq, count, eb + k * H_C + c, cb + k * H_C + c);
 }
 
 // Digits of phi[k][c][x] for grid->band, one block per (k, column): row 2c its
 // real, 2c + 1 its imaginary part along x.  dig [k][7][H_J][kp]
 __global__ void __launch_bounds__(256) ozh_phi_digits(const double2* __restrict__ phi, int nx, int nc, int c0, int kp,
-                                                      __half* __restrict__ dig, int* __restrict__ eb) {
+                                                      __half* __restrict__ dig, int* __restrict__ eb,
+                                                      HColumn* __restrict__ cb) {
   const int k = blockIdx.x, c = blockIdx.y;
   const double2* p = phi + ((size_t)k * nc + c0 + c) * nx;
   unsigned key = 0;
@@ -507,11 +739,15 @@ __global__ void __launch_bounds__(256) ozh_phi_digits(const double2* __restrict_
     const double2 v = p[x];
     key = max(key, max(oz_key(v.x), oz_key(v.y)));
   }
-  const int e = column_exponent(block_key(key));
-  if (threadIdx.x == 0) eb[k * H_C + c] = e;
+  int e;
+  const bool fits = column_exponent(block_key(key), &e);
+  float sq = 0.f;
+  int count = 0;
   uint32_t* o = reinterpret_cast<uint32_t*>(dig) + ((size_t)k * OZ_S * H_J + 2 * c) * (kp / 2);
   for (int x = 2 * threadIdx.x; x < nx; x += 2 * blockDim.x) {
     const double2 v0 = p[x], v1 = x + 1 < nx ? p[x + 1] : make_double2(0.0, 0.0);
+    sq += unit_square(v0, e) + unit_square(v1, e);
+    count += nonzero(v0) + nonzero(v1);
     const oz_fix r0 = oz_fixed(v0.x, e), r1 = oz_fixed(v1.x, e), i0 = oz_fixed(v0.y, e), i1 = oz_fixed(v1.y, e);
 #pragma unroll
     for (int i = 0; i < OZ_S; ++i) {
@@ -519,40 +755,62 @@ __global__ void __launch_bounds__(256) ozh_phi_digits(const double2* __restrict_
       o[(size_t)i * H_J * (kp / 2) + kp / 2 + x / 2] = oz_digit2(i0, i1, i);
     }
   }
+  record_column(fits, e, sq, count, eb + k * H_C + c, cb + k * H_C + c);
 }
 
-// out[c][k][n] = sum_split part + E psi - sum_b chi psi_b + short-range out, FP64
-__global__ void __launch_bounds__(256) ozh_final(const double2* __restrict__ part, int nsplit,
-                                                 const double2* __restrict__ psi, double2* __restrict__ out,
-                                                 const double* __restrict__ e_nk, const double2* __restrict__ chi,
-                                                 const double2* __restrict__ a_proj, const double2* __restrict__ srcp,
-                                                 int nk, int nb, int na, int np, int c0, int ncc) {
-  const size_t nkb = (size_t)nk * nb;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nkb * ncc; i += (size_t)gridDim.x * blockDim.x) {
-    const int cc = (int)(i / nkb), c = c0 + cc, v = c / na, a = c % na;
+// out[c][k][n] = sum_split part + E psi - sum_b chi psi_b + short-range out, FP64.
+// Sums over the grid that the digits may not stand for are formed here again,
+// one warp each.
+struct HFinal {
+  const double2 *part, *psi;
+  double2* out;
+  const double* e_nk;
+  const double2 *chi, *a_proj, *srcp, *u, *phi;
+  const float *sums, *norm;   // sums of magnitudes (as part), norms of the bands [nk][nb]
+  const HColumn* cb;          // columns of phi [nk][H_C]
+  int nsplit, nk, nx, nb, na, np, c0, ncc, nc;
+};
+__global__ void __launch_bounds__(256) ozh_final(const HFinal p) {
+  const size_t nkb = (size_t)p.nk * p.nb, total = nkb * p.ncc;
+  const int lane = threadIdx.x & 31;
+  for (size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x - lane; i0 < total; i0 += (size_t)gridDim.x * blockDim.x) {
+    const bool in = i0 + lane < total;
+    const size_t i = in ? i0 + lane : total - 1;
+    const int cc = (int)(i / nkb), c = p.c0 + cc, v = c / p.na, a = c % p.na;
     const size_t kn = i % nkb;
-    const int k = (int)(kn / nb), n = (int)(kn % nb);
+    const int k = (int)(kn / p.nb), n = (int)(kn % p.nb);
     double2 lr = make_double2(0.0, 0.0), rest = make_double2(0.0, 0.0);
-    for (int s = 0; s < nsplit; ++s) {
-      const double2 t = part[(((size_t)s * nk + k) * H_C + cc) * nb + n];
+    float m = 0.f;
+    for (int s = 0; s < p.nsplit; ++s) {
+      const size_t o = (((size_t)s * p.nk + k) * H_C + cc) * p.nb + n;
+      const double2 t = p.part[o];
       lr.x += t.x;
       lr.y += t.y;
+      m += p.sums[o];
     }
-    for (int b = 0; b < na; ++b) {
-      const double2 ch = chi[a * na + b], pb = psi[(size_t)(v * na + b) * nkb + kn];
+    const bool good = column_accepts(p.cb[(size_t)k * H_C + cc], p.norm[kn], m);
+    for (unsigned w = __ballot_sync(0xffffffffu, in && !good); w; w &= w - 1) {
+      const int r = __ffs(w) - 1;
+      const int kr = __shfl_sync(0xffffffffu, k, r), nr = __shfl_sync(0xffffffffu, n, r), cr = __shfl_sync(0xffffffffu, c, r);
+      const double2 t = warp_dot(p.u + (size_t)kr * p.nx * p.nb + nr, p.nb, p.phi + ((size_t)kr * p.nc + cr) * p.nx, p.nx);
+      if (lane == r) lr = t;
+    }
+    if (!in) continue;
+    for (int b = 0; b < p.na; ++b) {
+      const double2 ch = p.chi[a * p.na + b], pb = p.psi[(size_t)(v * p.na + b) * nkb + kn];
       rest.x = fma(-ch.x, pb.x, fma(ch.y, pb.y, rest.x));
       rest.y = fma(-ch.x, pb.y, fma(-ch.y, pb.x, rest.y));
     }
-    const double2* cp = srcp + (size_t)v * na * np + (size_t)a * np;
+    const double2* cp = p.srcp + (size_t)v * p.na * p.np + (size_t)a * p.np;
 #pragma unroll 4
-    for (int p = 0; p < np; ++p) {
-      const double2 ap = a_proj[(size_t)p * nkb + kn], q = cp[p];
+    for (int j = 0; j < p.np; ++j) {
+      const double2 ap = p.a_proj[(size_t)j * nkb + kn], q = cp[j];
       rest.x = fma(ap.x, q.x, fma(ap.y, q.y, rest.x));
       rest.y = fma(ap.x, q.y, fma(-ap.y, q.x, rest.y));
     }
-    const double2 ps = psi[(size_t)c * nkb + kn];
-    const double e = e_nk[kn];
-    out[(size_t)c * nkb + kn] = make_double2(lr.x + rest.x + e * ps.x, lr.y + rest.y + e * ps.y);
+    const double2 ps = p.psi[(size_t)c * nkb + kn];
+    const double e = p.e_nk[kn];
+    p.out[(size_t)c * nkb + kn] = make_double2(lr.x + rest.x + e * ps.x, lr.y + rest.y + e * ps.y);
   }
 }
 
@@ -573,14 +831,18 @@ struct OzhState {
   short *ex = nullptr, *en = nullptr;           // exponents of U per grid row and per band
   int *epsi = nullptr, *ephi = nullptr;         // exponents of the columns, [nk][H_C]
   __half *dpsi = nullptr, *dphi = nullptr;      // digits, [nk][7][H_J][kp]
+  float *nx = nullptr, *nn = nullptr;           // norms of U's rows and bands in units of their scales
+  HColumn *cpsi = nullptr, *cphi = nullptr;     // the columns, [nk][H_C]
   double2* part = nullptr;                      // [nsplit][nk][H_C][nb]
+  float* sums = nullptr;                        // their sums of magnitudes
   int* err = nullptr;
   CUtensorMap mpsi, mphi;
   int kp = 0, kpx = 0, nsplit = 1, sms = 0;
 };
 
 void free_state(OzhState* z) {
-  void* ptrs[] = {z->ex, z->en, z->epsi, z->ephi, z->dpsi, z->dphi, z->part, z->err};
+  void* ptrs[] = {z->ex,   z->en,   z->epsi, z->ephi, z->dpsi, z->dphi, z->nx,
+                  z->nn, z->cpsi, z->cphi, z->part, z->sums, z->err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete z;
@@ -637,7 +899,12 @@ void bse_ozh_prepare(bse_handle* h) {
               {(void**)&z->ephi, nk * H_C * sizeof(int)},
               {(void**)&z->dpsi, bpsi},
               {(void**)&z->dphi, bphi},
+              {(void**)&z->nx, nk * h->nx * sizeof(float)},
+              {(void**)&z->nn, nk * h->nb * sizeof(float)},
+              {(void**)&z->cpsi, nk * H_C * sizeof(HColumn)},
+              {(void**)&z->cphi, nk * H_C * sizeof(HColumn)},
               {(void**)&z->part, (size_t)z->nsplit * nk * H_C * h->nb * sizeof(double2)},
+              {(void**)&z->sums, (size_t)z->nsplit * nk * H_C * h->nb * sizeof(float)},
               {(void**)&z->err, 256}};
   bool ok = z->sms > 0;
   for (auto& w : want) ok = ok && bse_handle_malloc(h, w.p, w.bytes, "tensor-core form of the FP64 contractions") == BSE_OK;
@@ -648,9 +915,9 @@ void bse_ozh_prepare(bse_handle* h) {
     cudaMemsetAsync(z->err, 0, 256, h->stream);
     const long long rows = (long long)h->nk * h->nx;
     ozh_row_exponents<<<(unsigned)std::min<long long>((rows + 7) / 8, 16 * z->sms), 256, 0, h->stream>>>(
-        (const double2*)h->u, rows, h->nb, z->ex, z->err + 1);
+        (const double2*)h->u, rows, h->nb, z->ex, z->nx, z->err + 1);
     ozh_band_exponents<<<dim3((unsigned)((h->nb + 31) / 32), (unsigned)h->nk), 256, 0, h->stream>>>(
-        (const double2*)h->u, h->nx, h->nb, z->en, z->err + 1);
+        (const double2*)h->u, h->nx, h->nb, z->en, z->nn, z->err + 1);
     ok = cudaMemcpyAsync(&bad, z->err + 1, sizeof(int), cudaMemcpyDeviceToHost, h->stream) == cudaSuccess &&
          cudaStreamSynchronize(h->stream) == cudaSuccess && stacked_map(&z->mpsi, z->dpsi, z->kp, h->nk) &&
          stacked_map(&z->mphi, z->dphi, z->kpx, h->nk);
@@ -679,7 +946,9 @@ bse_status bse_ozh_band_to_grid(bse_handle* h, const double2* psi, int nc) {
   HParams p{};
   p.u = (const double2*)h->u;
   p.ea = z->ex;
+  p.na = z->nx;
   p.eb = z->epsi;
+  p.cb = z->cpsi;
   p.out = (double2*)h->phi;
   p.nk = h->nk, p.nx = h->nx, p.nb = h->nb;
   p.mt = (h->nx + H_M - 1) / H_M;
@@ -693,9 +962,10 @@ bse_status bse_ozh_band_to_grid(bse_handle* h, const double2* psi, int nc) {
   for (int c0 = 0; c0 < nc && e == cudaSuccess; c0 += H_C) {
     p.c0 = c0;
     p.ncc = std::min(H_C, nc - c0);
+    p.psi = psi + (size_t)c0 * h->nk * h->nb;
     BSE_PROF(h, BSE_K_PREP,
              ozh_psi_digits<<<dim3((unsigned)h->nk, (unsigned)p.ncc), 64, 0, h->stream>>>(
-                 psi + (size_t)c0 * h->nk * h->nb, h->nk, h->nb, z->kp, z->dpsi, z->epsi));
+                 p.psi, h->nk, h->nb, z->kp, z->dpsi, z->epsi, z->cpsi));
     BSE_PROF(h, BSE_K_BAND_TO_GRID, e = launch<0>(z->mpsi, p, z->sms, h->stream));
   }
   return bse_cuda_check(h, e, "band->grid (split FP64)");
@@ -709,6 +979,7 @@ bse_status bse_ozh_grid_to_band(bse_handle* h, const double2* psi, double2* hpsi
   p.ea = z->en;
   p.eb = z->ephi;
   p.out = z->part;
+  p.sums = z->sums;
   p.nk = h->nk, p.nx = h->nx, p.nb = h->nb;
   p.mt = (2 * h->nb + H_M - 1) / H_M;
   p.kb = z->kpx / H_KB;
@@ -717,19 +988,21 @@ bse_status bse_ozh_grid_to_band(bse_handle* h, const double2* psi, double2* hpsi
   p.ntiles = h->nk * p.mt * p.nsplit;
   p.err = z->err;
   p.wait_ns = h->tc_wait_ns;
+  HFinal f = {z->part, psi, hpsi, h->e_nk, h->chi, h->a_proj, h->sr_cp, (const double2*)h->u, (const double2*)h->phi,
+                      z->sums, z->nn, z->cphi, p.nsplit, h->nk, h->nx, h->nb, h->na, h->np, 0, 0, nc};
   cudaError_t e = cudaSuccess;
   const size_t nkb = (size_t)h->nk * h->nb;
   for (int c0 = 0; c0 < nc && e == cudaSuccess; c0 += H_C) {
     p.ncc = std::min(H_C, nc - c0);
     BSE_PROF(h, BSE_K_PREP,
              ozh_phi_digits<<<dim3((unsigned)h->nk, (unsigned)p.ncc), 256, 0, h->stream>>>(
-                 (const double2*)h->phi, h->nx, nc, c0, z->kpx, z->dphi, z->ephi));
+                 (const double2*)h->phi, h->nx, nc, c0, z->kpx, z->dphi, z->ephi, z->cphi));
     BSE_PROF(h, BSE_K_GRID_TO_BAND, e = launch<1>(z->mphi, p, z->sms, h->stream));
     if (h->np > 0 && c0 == 0) cudaStreamWaitEvent(h->stream, h->ev_join, 0);   // short-range c' ready
+    f.c0 = c0;
+    f.ncc = p.ncc;
     BSE_PROF(h, BSE_K_GRID_TO_BAND,
-             ozh_final<<<(unsigned)std::min<size_t>((nkb * p.ncc + 255) / 256, (size_t)32 * z->sms), 256, 0, h->stream>>>(
-                 z->part, p.nsplit, psi, hpsi, h->e_nk, h->chi, h->a_proj, h->sr_cp, h->nk, h->nb, h->na, h->np, c0,
-                 p.ncc));
+             ozh_final<<<(unsigned)std::min<size_t>((nkb * p.ncc + 255) / 256, (size_t)32 * z->sms), 256, 0, h->stream>>>(f));
   }
   return bse_cuda_check(h, e == cudaSuccess ? cudaGetLastError() : e, "grid->band (split FP64)");
 }

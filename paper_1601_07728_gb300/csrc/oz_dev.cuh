@@ -69,6 +69,28 @@ __device__ __forceinline__ oz_fix oz_fixed(double x, int e) {
   return f;
 }
 
+// |x| 2^-e as FP32, rounded down (0 below 2^-126): integer arithmetic as above
+__device__ __forceinline__ float oz_unit(double x, int e) {
+  const uint32_t xh = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+  const int f = (int)(xh >> 20) - e - (1023 - 127);
+  return f <= 0 ? 0.f : __uint_as_float(((uint32_t)min(f, 254) << 23) | ((xh & 0xfffffu) << 3));
+}
+
+// Which sums the digits may stand for.  With every entry held to 2^-56 of its
+// row's scale, the error of a sum over k is about 0.58 * 2^-56 (|a|^2 + |b|^2)^1/2
+// in units of the two scales (|.| the norms of the two rows there), whatever the
+// sum itself is: where one row is large the other may be small throughout, and
+// FP64 products keep the digits that are lost here.  So the magnitudes' sum
+// S = sum |a_k| |b_k| is taken along from the leading digits (entries below
+// 2^-8 of their row's scale count as zero, so that S is rather too small), and
+// a sum is accepted where the error is below 2^-53 S, one rounding of it:
+// S >= 0.0725 (|a|^2 + |b|^2)^1/2.  The rest is summed on the FP64 pipe.  Rows
+// of n normal random entries reach about 0.6 n / (r_a r_b) against a limit of
+// 0.1 sqrt(n) (1 / r_a + 1 / r_b), r = 3..8 their scale over their deviation.
+__device__ __forceinline__ bool oz_accept(float s, float norm_a, float norm_b) {
+  return s >= 0.1f * (norm_a + norm_b);
+}
+
 // digit i (0 = leading) of two entries as packed FP16: the bytes b become
 // 0x6400 | b = 1024 + digit + 128, less 1152
 __device__ __forceinline__ uint32_t oz_digit2(oz_fix f0, oz_fix f1, int i) {

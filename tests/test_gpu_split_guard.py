@@ -1,0 +1,99 @@
+"""Sums over rows of wide range: where one operand's entries are large the
+other's are small, so that what the sum consists of lies far below the rows'
+largest entries.  The tensor-core forms hold every entry to 2^-56 of its row's
+largest only; their results have to keep FP64's accuracy all the same.
+
+Bound: a sum of n complex products in FP64, in any order, is off by at most
+2 (n + 2) 2^-53 sum |a| |b|; chained sums add their factors.
+"""
+import numpy as np
+import pytest
+
+from oracle import bse_oracle as O
+from paper_1601_07728_gb300 import bse, synth as S
+
+pytestmark = pytest.mark.gpu
+U64 = 2.0 ** -53
+
+
+def graded_system(nk, nx, nb, na, npj, decades, ks=(0.0, 0.0, 0.0), seed=1):
+    """Two groups of bands, each `decades` smaller on the other's half of the grid."""
+    s = S.make_system_from(dict(id=971, n_alpha=na, nk=nk, n_bands=nb, nx=nx, cell=7.4, eps=5.0, n_proj=npj,
+                                so_split=5.7, m_scale=0.5, kshift=ks), seed)
+    s.chi = np.zeros_like(s.chi)   # no coupling that would lift the small entries
+    if npj:
+        s.a_proj = s.a_proj * 0.0
+    half = np.arange(s.n_x) < s.n_x // 2
+    group = np.arange(nb) % 2 == 0
+    s.u = s.u * np.where(half[:, None] == group[None, :], 1.0, 10.0 ** -decades)
+    return s, group
+
+
+def apply_bound(s, psi):
+    """(2 (n_b + 2) + 2 (n_x + 2) + 2 (n_k + 8)) 2^-53 |U|^H |W| |U| |psi|, the k sums from |phi| and |W|."""
+    a = np.abs(s.u)
+    p = np.abs(psi.reshape(s.n_alpha, s.n_k, s.n_bands))
+    phi = np.einsum("kxn,akn->akx", a, p)
+    conv = np.abs(s.w_rx).sum(0)[None, :] * phi.sum(1) / s.n_k
+    out = np.einsum("kxn,ax->akn", a, conv) + np.abs(s.e_nk)[None] * p
+    return (2 * (s.n_bands + s.n_x + s.n_k) + 40) * U64 * out.reshape(-1)
+
+
+# one block of bands and several, the grid split over blocks and not, 1 to 12
+# columns (two passes of eight), bands beyond one accumulator of 128 reals
+@pytest.mark.parametrize("decades", [4, 12, 20])
+@pytest.mark.parametrize("case", [((2, 1, 1), (16, 9, 11), 24, 6, 1), ((1, 1, 1), (16, 16, 16), 40, 1, 1),
+                                  ((2, 2, 1), (13, 10, 10), 150, 6, 2)])
+def test_graded_bands_keep_fp64_accuracy(case, decades):
+    nk, nx, nb, na, nv = case
+    s, group = graded_system(nk, nx, nb, na, 0, decades)
+    rng = np.random.default_rng(decades)
+    psi = S.complex_normal(rng, (nv, na, s.n_k, nb)) * group * 10.0 ** -(np.arange(nb) % 6.0)
+    psi = psi.reshape(nv, -1)
+    out = bse.System(s, precision="fp64", max_vec=nv).apply_h(psi)
+    for v in range(nv):
+        assert np.all(np.abs(out[v] - O.apply_h(s, psi[v])) <= 2 * apply_bound(s, psi[v]))
+
+
+def test_sparse_real_and_empty_columns():
+    """Columns of one entry, of real entries (with real Bloch functions: no
+    imaginary part at all) and of zeros, beside full ones."""
+    s, _ = graded_system((1, 1, 1), (16, 16, 16), 32, 6, 0, 0)
+    s.u = s.u.real.astype(complex)
+    rng = np.random.default_rng(5)
+    psi = S.complex_normal(rng, (6, 1, 32))
+    psi[0] = 0
+    psi[1] = 0
+    psi[1, 0, 7] = 1e-5
+    psi[2] = psi[2].real
+    psi = psi.reshape(1, -1)
+    h = bse.System(s, precision="fp64")
+    out = h.apply_h(psi)[0]
+    assert np.all(np.abs(out - O.apply_h(s, psi[0])) <= 2 * apply_bound(s, psi[0]))
+    assert np.all(out[:32] == 0) and np.all(out[64:96].imag == 0)
+    h.profile()
+    h.apply_h(psi)
+    assert h.profile_read()["prep"][0] == 2   # digits of psi and phi: the split kernels
+
+
+@pytest.mark.parametrize("power", [-1000, -965, 1000])
+def test_columns_of_extreme_scale_keep_fp64_accuracy(power):
+    s, _ = graded_system((2, 1, 1), (16, 9, 11), 24, 6, 0, 3)
+    psi = S.make_start_vectors(s, 1)
+    scale = 2.0 ** power
+    out = bse.System(s, precision="fp64").apply_h(psi * scale)[0]
+    ref = O.apply_h(s, psi[0])
+    # 2^-1074: what subnormal products and sums lose at the smallest scale
+    assert np.all(np.abs(out / scale - ref) <= 2 * apply_bound(s, psi[0]) + 1e5 * 2.0 ** (-1074 - power))
+
+
+def test_non_finite_entries_reach_what_they_reached_in_fp64():
+    s, _ = graded_system((1, 1, 1), (16, 16, 16), 32, 6, 0, 0)
+    psi = S.make_start_vectors(s, 1)
+    h = bse.System(s, precision="fp64")
+    ref = h.apply_h(psi)[0].reshape(6, 32)
+    psi[0, 32 + 3] = np.inf   # core state 1, band 3
+    out = h.apply_h(psi)[0].reshape(6, 32)
+    assert not np.any(np.isfinite(out[1]))
+    others = np.ix_([0, 2, 3, 4, 5], [n for n in range(32) if n != 3])   # 0 * inf of the spin-orbit term in band 3
+    assert np.array_equal(out[others], ref[others])
