@@ -299,13 +299,14 @@ bse_status bse_jacobi_diag(bse_handle* h, double* diag);
  * indexed as in bse_setup, kshift [3] or NULL, dv the volume per grid point;
  * a [n_proj][Nk][Nb].  All complex128, host or device; FP64 accuracy (large
  * problems as exactly split tensor-core products, with scratch allocated for
- * the call; without it, or for Inf/NaN and magnitudes outside 2^+-400, on the
- * FP64 pipe).  Work runs on `stream` (NULL: legacy default) and the call returns
+ * the call; without it, for Inf/NaN and magnitudes outside 2^+-400, or where a
+ * bounded wait of that kernel gives up, on the FP64 pipe).  Work runs on `stream` (NULL: legacy default) and the call returns
  * when a is written.  Allocates staging copies of host arrays.  Returns
  * BSE_ERR_INVALID_ARG (before any device work) for a NULL u, nk, nx, f or a,
  * n_bands < 1, n_proj outside 1..4096, nk[d] outside 1..16, nx[d] < 1 or
- * n_bands > Nx; BSE_ERR_OOM or BSE_ERR_CUDA from staging or the launch;
- * BSE_ERR_TIMEOUT where a bounded wait of the tensor-core kernel gave up. */
+ * n_bands > Nx; BSE_ERR_OOM or BSE_ERR_CUDA from staging or the launch.
+ * Failure-detection aid: BSE_SPLIT_WAIT_NS in the environment (decimal, 1000
+ * to 2000000000, the default) limits each of those waits. */
 bse_status bse_local_projection(const bse_c128* u, const int* nk, const int* nx, int n_bands, const double* kshift,
                                 const bse_c128* f, int n_proj, double dv, bse_c128* a, void* stream);
 
@@ -320,11 +321,10 @@ bse_status bse_local_projection(const bse_c128* u, const int* nk, const int* nx,
  * may be NULL.  Complex128 / FP64, host or device; work on `stream` (NULL:
  * legacy default), returns when the outputs are written.  Allocates staging
  * and the G_j scratch, and for large problems that of exactly split tensor-core
- * products (without it, or for Inf/NaN and magnitudes outside 2^+-400: the FP64
- * pipe).  Returns BSE_ERR_INVALID_ARG (before any device work) for a NULL psi,
+ * products (without it, for Inf/NaN and magnitudes outside 2^+-400, or where a
+ * bounded wait of that kernel gives up, BSE_SPLIT_WAIT_NS as above: the FP64 pipe).  Returns BSE_ERR_INVALID_ARG (before any device work) for a NULL psi,
  * eps, t, w or chi0, n_r, n_states or n_t < 1, n_r > 65535 or n_t > 65535;
- * BSE_ERR_OOM or BSE_ERR_CUDA from staging or the launches; BSE_ERR_TIMEOUT
- * where a bounded wait of the tensor-core kernel gave up.  A
+ * BSE_ERR_OOM or BSE_ERR_CUDA from staging or the launches.  A
  * node t_j = 0 with some eps[K] == mu sits on the integrand's pole and gives
  * non-finite values: the caller's nodes must avoid it (mu between two levels,
  * or t_j > 0). */

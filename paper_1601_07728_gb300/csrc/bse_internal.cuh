@@ -240,12 +240,14 @@ int bse_oz_kp(int k);   // K padded to whole blocks
 // real rows per complex row so that a product with pair = 0 rows is sum a conj(x)
 bse_status bse_oz_split_rows(const double2* x, int rows, int n, const double2* d, int batches, int pair,
                              const bse_oz_operand& o, int* bad, cudaStream_t st);
-// the projection of bse_local_projection_device on the tensor cores; *done = false where the
-// scratch cannot be had or u or f hold Inf/NaN or magnitudes outside 2^+-400
+// the projection of bse_local_projection_device on the tensor cores; *done = false (a not to be
+// used) where the scratch or the kernel's set-up cannot be had, u or f hold Inf/NaN or magnitudes
+// outside 2^+-400, or a bounded wait gave up
 bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb, const double* kshift,
                           const double2* f, int np, double dv, double2* a, cudaStream_t st, bool* done);
 // out = alpha A_b B_b^T for every batch (an operand with one batch serves all);
-// element (b, row, col) at out + b sb + (row/2) sr2 + (row%2) sr1 + col sc
+// element (b, row, col) at out + b sb + (row/2) sr2 + (row%2) sr1 + col sc; *err is set where a
+// bounded wait gave up; BSE_ERR_UNSUPPORTED (nothing launched) where the set-up fails
 bse_status bse_oz_gemm(const bse_oz_operand& a, const bse_oz_operand& b, int batches, double alpha, double* out,
                        long long sb, long long sr2, long long sr1, long long sc, int* err, cudaStream_t st);
 // screening: G_j = psi diag(1/(mu + i t_j - eps)) psi^H for all j, chi0 from them (k_screen.cu)

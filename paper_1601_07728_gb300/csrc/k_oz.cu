@@ -18,6 +18,8 @@
 #include "oz_dev.cuh"
 #include "tc_ptx.cuh"
 
+#include <stdlib.h>
+
 #include <algorithm>
 
 namespace {
@@ -31,7 +33,16 @@ constexpr int OZ_THREADS = 320;
 // B slots lie between tiles of zeros: 0 B_0..B_6 0 B_0..B_6 0
 constexpr int OZ_BAREA = OZ_BS * (OZ_B + OZ_BD) + OZ_BD;
 constexpr size_t OZ_SMEM = 1024 + (size_t)OZ_AS * OZ_A + OZ_BAREA + 512;
-constexpr unsigned long long OZ_WAIT_NS = 2000000000ull;
+constexpr unsigned long long OZ_WAIT_NS = 2000000000ull;   // limit of a wait, and of the drain after an abort
+
+// limit of the pipeline waits of one call: OZ_WAIT_NS, or BSE_SPLIT_WAIT_NS of the environment (see bse.h)
+unsigned long long wait_limit() {
+  const char* v = getenv("BSE_SPLIT_WAIT_NS");
+  if (!v) return OZ_WAIT_NS;
+  char* end = nullptr;
+  const unsigned long long n = strtoull(v, &end, 10);
+  return end == v || *end != '\0' || n < 1000 || n > OZ_WAIT_NS ? OZ_WAIT_NS : n;
+}
 
 struct oz_mesh {
   int nk[3], nx[3];
@@ -48,14 +59,15 @@ struct OzParams {
   double* out;                  // element (b, row, col) at b sb + (row>>1) sr2 + (row&1) sr1 + col sc
   long long sb, sr2, sr1, sc;
   int* err;
+  unsigned long long wait_ns;
 };
 
 // bounded wait, inlined: at a call the draining warps' sums would go through memory
-__device__ __forceinline__ bool oz_wait(uint32_t a, uint32_t parity, volatile int* abort_flag) {
+__device__ __forceinline__ bool oz_wait(uint32_t a, uint32_t parity, volatile int* abort_flag, unsigned long long limit_ns) {
   if (mbar_try(a, parity)) return true;
   const unsigned long long t0 = gtime();
   while (!mbar_try(a, parity))
-    if (*abort_flag || gtime() - t0 > OZ_WAIT_NS) return false;
+    if (*abort_flag || gtime() - t0 > limit_ns) return false;
   return true;
 }
 
@@ -87,7 +99,7 @@ struct oz_issue {
 // and all of one shape (s = 7 is computed along and not used).
 __device__ __forceinline__ bool issue_block(uint32_t tmem, uint32_t sa, unsigned long long db, bool first, int c,
                                             oz_issue& z, uint32_t afull, uint32_t aempty, uint32_t tempty,
-                                            volatile int* abort_flag) {
+                                            volatile int* abort_flag, unsigned long long limit_ns) {
   // FP16 A and B (K-major), FP32 D
   constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(2 * OZ_N >> 3) << 17) | ((uint32_t)(OZ_M >> 4) << 24);
   auto products = [&](int i, int p0, int p1, uint32_t keep) {   // bit P of keep: add to accumulator P
@@ -100,10 +112,10 @@ __device__ __forceinline__ bool issue_block(uint32_t tmem, uint32_t sa, unsigned
                  db + (unsigned long long)(long long)(((2 * P - i) * OZ_BD + ks * 32) / 16), idesc,
                  ks > 0 ? 1u : (keep >> P) & 1u);
   };
-  auto drained = [&](int s, int n) { return oz_wait(tempty + 8 * s, ((uint32_t)n & 1u) ^ 1u, abort_flag); };
+  auto drained = [&](int s, int n) { return oz_wait(tempty + 8 * s, ((uint32_t)n & 1u) ^ 1u, abort_flag, limit_ns); };
 #pragma unroll
   for (int i = 0; i < OZ_S; ++i) {
-    if (!oz_wait(afull + 8 * z.sl, z.ph, abort_flag)) return false;
+    if (!oz_wait(afull + 8 * z.sl, z.ph, abort_flag, limit_ns)) return false;
     tc_fence_after();
     if (i == 0 && first) {
       const bool n0 = (c & 3) == 0, n1 = (c & 1) == 0;
@@ -237,13 +249,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       const int za = p.a_batched ? b * OZ_S : 0, zb = p.b_batched ? b * OZ_S : 0;
       for (int kb = 0; kb < p.kb && ok; ++kb) {
         const int s = ib % OZ_BS;
-        if (!(ok = oz_wait(bempty(s), ((uint32_t)(ib / OZ_BS) & 1u) ^ 1u, abort_flag))) break;
+        if (!(ok = oz_wait(bempty(s), ((uint32_t)(ib / OZ_BS) & 1u) ^ 1u, abort_flag, p.wait_ns))) break;
         mbar_expect_tx(bfull(s), OZ_B);
         tma_load_3d(sb + s * (OZ_B + OZ_BD), &mb, bfull(s), kb * OZ_KB, n * OZ_N, zb);
         *b_issued = ++ib;
         for (int i = 0; i < OZ_S; ++i) {
           const int q = ia % OZ_AS;
-          if (!(ok = oz_wait(aempty(q), ((uint32_t)(ia / OZ_AS) & 1u) ^ 1u, abort_flag))) break;
+          if (!(ok = oz_wait(aempty(q), ((uint32_t)(ia / OZ_AS) & 1u) ^ 1u, abort_flag, p.wait_ns))) break;
           mbar_expect_tx(afull(q), OZ_A);
           tma_load_3d(sa + q * OZ_A, &ma, afull(q), kb * OZ_KB, m * OZ_M, za + i);
           *a_issued = ++ia;
@@ -262,10 +274,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       for (int kb = 0; kb < p.kb && ok; ++kb) {
         const bool first = (kb & 1) == 0, last = (kb & 1) == 1 || kb + 1 == p.kb;
         const int s = ib % OZ_BS;
-        if (!(ok = oz_wait(bfull(s), (uint32_t)(ib / OZ_BS) & 1u, abort_flag))) break;
+        if (!(ok = oz_wait(bfull(s), (uint32_t)(ib / OZ_BS) & 1u, abort_flag, p.wait_ns))) break;
         ++ib;
         const unsigned long long db = sdesc_sw128(sb + s * (OZ_B + OZ_BD));
-        if (!(ok = issue_block(tmem, sa, db, first, kb >> 1, z, afull(0), aempty(0), tempty(0), abort_flag))) break;
+        if (!(ok = issue_block(tmem, sa, db, first, kb >> 1, z, afull(0), aempty(0), tempty(0), abort_flag, p.wait_ns))) break;
         mma_commit(bempty(s));
         if (last) mma_commit(tfull);
       }
@@ -289,7 +301,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 #pragma unroll
       for (int c = 0; c < 32; ++c) hi[c] = 0, lo[c] = 0;
       for (int kb = 0; kb < p.kb; kb += 2, ++chunk) {
-        ok = __all_sync(0xffffffffu, oz_wait(tfull, (uint32_t)chunk & 1u, abort_flag));
+        ok = __all_sync(0xffffffffu, oz_wait(tfull, (uint32_t)chunk & 1u, abort_flag, p.wait_ns));
         if (!ok) break;
         tc_fence_after();
         drain_chunk<32>(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 32), kb >> 1, kb + 2 >= p.kb, tempty(0), lane,
@@ -500,6 +512,7 @@ struct OzProject {
   long long* part_hi;     // [CTA][2][128][64] sums of the tiles that CTAs share
   uint32_t* part_lo;
   int* err;
+  unsigned long long wait_ns;
 };
 
 // first chunk of CTA c: all tiles' chunks in one line, cut into equal parts
@@ -594,7 +607,7 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
     bool ok = true;
     auto phases = [&]() {
       const int s = ip % OZ_PH;
-      if (!oz_wait(pempty(s), ((uint32_t)(ip / OZ_PH) & 1u) ^ 1u, abort_flag)) return false;
+      if (!oz_wait(pempty(s), ((uint32_t)(ip / OZ_PH) & 1u) ^ 1u, abort_flag, p.wait_ns)) return false;
       mbar_expect_tx(pfull(s), OZ_KB / 2 * sizeof(double2));
       bulk_load(sp + s * (OZ_KB / 2) * (int)sizeof(double2),
                 p.phase + ((size_t)(tp / p.mt / p.nt) * p.kb + bp) * (OZ_KB / 2), OZ_KB / 2 * sizeof(double2), pfull(s));
@@ -607,7 +620,7 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
       const int m = t % p.mt;
       for (int j = 0; j < OZ_S && ok; ++j) {
         const int q = ia % OZ_AS;
-        if (!(ok = oz_wait(aempty(q), ((uint32_t)(ia / OZ_AS) & 1u) ^ 1u, abort_flag))) break;
+        if (!(ok = oz_wait(aempty(q), ((uint32_t)(ia / OZ_AS) & 1u) ^ 1u, abort_flag, p.wait_ns))) break;
         mbar_expect_tx(afull(q), OZ_A);
         tma_load_3d(sa + q * OZ_A, &ma, afull(q), b * OZ_KB, m * OZ_M, j);
         *a_issued = ++ia;
@@ -624,9 +637,9 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
     bool ok = true;
     for (int i = 0; i < total; ++i) {
       const int s = i % OZ_BS;
-      if (!(ok = oz_wait(bfull(s), (uint32_t)(i / OZ_BS) & 1u, abort_flag))) break;
+      if (!(ok = oz_wait(bfull(s), (uint32_t)(i / OZ_BS) & 1u, abort_flag, p.wait_ns))) break;
       const unsigned long long db = sdesc_sw128(sb + s * (OZ_B + OZ_BD));
-      if (!(ok = issue_block(tmem, sa, db, (b & 1) == 0, c, z, afull(0), aempty(0), tempty, abort_flag))) break;
+      if (!(ok = issue_block(tmem, sa, db, (b & 1) == 0, c, z, afull(0), aempty(0), tempty, abort_flag, p.wait_ns))) break;
       mma_commit(bempty(s));
       if ((b & 1) == 1 || b + 1 == p.kb) {
         mma_commit(tfull);
@@ -654,7 +667,7 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
     int chunk = 0, cc = 0;   // drained so far, of them in this tile
     // the accumulators of the oldest chunk not yet drained, which ends with block b of tile t
     auto drain = [&](int t, int b, bool last) {
-      if (!__all_sync(0xffffffffu, oz_wait(tfull, (uint32_t)chunk & 1u, abort_flag))) return false;
+      if (!__all_sync(0xffffffffu, oz_wait(tfull, (uint32_t)chunk & 1u, abort_flag, p.wait_ns))) return false;
       ++chunk;
       tc_fence_after();
       const bool end = b + 1 == p.kb || last;
@@ -708,8 +721,8 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
     for (int i = 0; i < total; ++i) {
       if (b == 0 || i == 0) e = en;
       const int s = i % OZ_BS, q = i % OZ_PH;
-      ok = __all_sync(0xffffffffu, oz_wait(pfull(q), (uint32_t)(i / OZ_PH) & 1u, abort_flag) &&
-                                       oz_wait(bempty(s), ((uint32_t)(i / OZ_BS) & 1u) ^ 1u, abort_flag));
+      ok = __all_sync(0xffffffffu, oz_wait(pfull(q), (uint32_t)(i / OZ_PH) & 1u, abort_flag, p.wait_ns) &&
+                                       oz_wait(bempty(s), ((uint32_t)(i / OZ_BS) & 1u) ^ 1u, abort_flag, p.wait_ns));
       if (!ok) break;
       oz_fix f[8];
 #pragma unroll
@@ -835,7 +848,7 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaFuncSetAttribute(oz_project, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_PSMEM) != cudaSuccess) {
     cudaGetLastError();
-    return BSE_ERR_CUDA;
+    return BSE_OK;
   }
   const size_t per = (size_t)kp / 2 * sizeof(double2);
   const int nkc = (int)std::min<size_t>({(size_t)nkt, std::max<size_t>(((size_t)256 << 20) / per, 1), (size_t)32768});
@@ -890,8 +903,9 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
   p.alpha = dv;
   p.out = (double*)a;
   p.err = word;
+  p.wait_ns = wait_limit();
   CUtensorMap ma;
-  if (!digit_map(&ma, (const __half*)A.digits, kp, A.rows, OZ_S, OZ_M, 1)) return BSE_ERR_CUDA;
+  if (!digit_map(&ma, (const __half*)A.digits, kp, A.rows, OZ_S, OZ_M, 1)) return BSE_OK;
   cudaMemsetAsync(word, 0, 2 * sizeof(int), st);
   // rows (Re f, Im f) and (-Im f, Re f): real and imaginary part of conj(f) times a column
   bse_status s = bse_oz_split_rows(f, np, nxt, nullptr, 1, 1, A, word + 1, st);
@@ -920,8 +934,7 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
     cudaStreamSynchronize(st);   // before the scratch goes
     return s;
   }
-  if (hw[0]) return BSE_ERR_TIMEOUT;
-  *done = hw[1] == 0;
+  *done = hw[0] == 0 && hw[1] == 0;
   return BSE_OK;
 }
 
@@ -930,7 +943,7 @@ bse_status bse_oz_gemm(const bse_oz_operand& a, const bse_oz_operand& b, int bat
   CUtensorMap ma, mb;
   if (!digit_map(&ma, (const __half*)a.digits, a.kp, a.rows, OZ_S * a.batches, OZ_M, 1) ||
       !digit_map(&mb, (const __half*)b.digits, b.kp, b.rows, OZ_S * b.batches, OZ_N, OZ_S))
-    return BSE_ERR_CUDA;
+    return BSE_ERR_UNSUPPORTED;
   OzParams p{};
   p.mt = (a.rows + OZ_M - 1) / OZ_M;
   p.nt = (b.rows + OZ_N - 1) / OZ_N;
@@ -949,12 +962,13 @@ bse_status bse_oz_gemm(const bse_oz_operand& a, const bse_oz_operand& b, int bat
   p.sr1 = sr1;
   p.sc = sc;
   p.err = err;
+  p.wait_ns = wait_limit();
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaFuncSetAttribute(oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM) != cudaSuccess) {
     cudaGetLastError();
-    return BSE_ERR_CUDA;
+    return BSE_ERR_UNSUPPORTED;
   }
   oz_gemm<<<std::min(p.ntiles, sms), OZ_THREADS, OZ_SMEM, st>>>(ma, mb, p);
   return cudaGetLastError() == cudaSuccess ? BSE_OK : BSE_ERR_CUDA;

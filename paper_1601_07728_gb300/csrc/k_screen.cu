@@ -101,8 +101,9 @@ struct Scratch {
 
 // G_j on the tensor cores (k_oz.cu): the rows psi(r, :) d_j against the row
 // pairs of psi(r', :), as many frequencies per pass as the scratch holds.
-// *done = false (and nothing but G written) where the scratch cannot be had or
-// psi d_j holds Inf/NaN or a magnitude outside 2^+-400.
+// *done = false (and nothing but G written) where the scratch or the kernel's
+// set-up cannot be had, psi d_j holds Inf/NaN or a magnitude outside 2^+-400, or
+// a bounded wait gave up.
 bse_status green_tensor(const double2* psi, const double* eps, int nr, int nkk, double mu, const double* t, int nt,
                         double2* G, cudaStream_t st, bool* done) {
   *done = false;
@@ -148,10 +149,9 @@ bse_status green_tensor(const double2* psi, const double* eps, int nr, int nkk, 
     s = BSE_ERR_CUDA;
   if (s != BSE_OK) {
     cudaStreamSynchronize(st);   // before the scratch goes
-    return s;
+    return s == BSE_ERR_UNSUPPORTED ? BSE_OK : s;
   }
-  if (hw[0]) return BSE_ERR_TIMEOUT;
-  *done = hw[1] == 0;
+  *done = hw[0] == 0 && hw[1] == 0;
   return BSE_OK;
 }
 

@@ -126,3 +126,32 @@ def test_every_call_over_h_reports_a_wait_that_gave_up(l23, precision):
     outs, sts = bse.haydock_batch([sysg], [psi], 4)
     assert list(sts) == [bse.BSE_OK] and outs[0][2][0] == 4
     sysg.close()
+
+
+def _projection():
+    rng = np.random.default_rng(4)
+    u, f = S.complex_normal(rng, (27, 1331, 64)), S.complex_normal(rng, (36, 1331))
+    args = (u, (3, 3, 3), (11, 11, 11), f, 0.3)
+    return lambda: bse.local_projection(*args), O.local_projection(*args)
+
+
+def _screening():
+    psi, eps = S.screening_grid_states(260, 900, seed=2)
+    args = (psi, eps, 0.1, np.array([0.4, 2.0]), np.array([1.0, 0.5]))
+    return lambda: bse.screening_chi0(*args), O.screening_chi0(*args)
+
+
+@pytest.mark.parametrize("case", [_projection, _screening])
+def test_set_up_calls_finish_where_a_wait_gives_up(monkeypatch, case):
+    """With 1 microsecond for each wait of the tensor-core kernel (a chunk of
+    products takes several) it gives up, and the FP64 kernel does the work."""
+    f, ref = case()
+    monkeypatch.delenv("BSE_SPLIT_WAIT_NS", raising=False)
+    split = f()
+    monkeypatch.setenv("BSE_SPLIT_WAIT_NS", "1000")
+    fp64 = f()
+    assert not np.array_equal(split, fp64)   # other sums: it did give up
+    monkeypatch.delenv("BSE_SPLIT_WAIT_NS")
+    assert np.array_equal(f(), split)        # and left nothing behind
+    for out in (split, fp64):
+        assert np.abs(out - ref).max() <= 1e-13 * np.abs(ref).max()
