@@ -300,7 +300,9 @@ bse_status bse_jacobi_diag(bse_handle* h, double* diag);
  * a [n_proj][Nk][Nb].  All complex128, host or device; FP64 accuracy (large
  * problems as exactly split tensor-core products, with scratch allocated for
  * the call; without it, for Inf/NaN and magnitudes outside 2^+-400, or where a
- * bounded wait of that kernel gives up, on the FP64 pipe).  Work runs on `stream` (NULL: legacy default) and the call returns
+ * bounded wait of that kernel gives up, on the FP64 pipe; so are elements whose
+ * error there could lift above about 2^-53 sum |f| |u|, and with more than one
+ * in 32 of those all).  Work runs on `stream` (NULL: legacy default) and the call returns
  * when a is written.  Allocates staging copies of host arrays.  Returns
  * BSE_ERR_INVALID_ARG (before any device work) for a NULL u, nk, nx, f or a,
  * n_bands < 1, n_proj outside 1..4096, nk[d] outside 1..16, nx[d] < 1 or

@@ -242,7 +242,7 @@ bse_status bse_oz_split_rows(const double2* x, int rows, int n, const double2* d
                              const bse_oz_operand& o, int* bad, cudaStream_t st);
 // the projection of bse_local_projection_device on the tensor cores; *done = false (a not to be
 // used) where the scratch or the kernel's set-up cannot be had, u or f hold Inf/NaN or magnitudes
-// outside 2^+-400, or a bounded wait gave up
+// outside 2^+-400, a bounded wait gave up, or too many elements are refused (oz_accept)
 bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb, const double* kshift,
                           const double2* f, int np, double dv, double2* a, cudaStream_t st, bool* done);
 // out = alpha A_b B_b^T for every batch (an operand with one batch serves all);

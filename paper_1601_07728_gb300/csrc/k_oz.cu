@@ -7,13 +7,17 @@
 // FP16 products, so that the 19 products of 128 x 128 x 16 which replace one
 // FP64 product of 128 x 64 x 16 still run some 50 times faster.  Measured:
 // Green's functions of 900 points, 4096 states and 16 frequencies 682 ms
-// (FP64 kernel) -> 13.5 ms (this one 12.4, writing the digits 0.97); the
+// (FP64 kernel) -> 13.3 ms (this one 12.2, writing the digits 0.97); the
 // projection of 8^3 k x 16^3 points x 64 bands onto 64 functions 102.6 ms ->
-// 5.4 ms with the Bloch functions' digits in memory -> 3.1 ms with the digits
-// made on the way into shared memory (oz_project 2.4, row scales 0.29).  The
-// error against 64 bits fell from 1.9e-15 to 1.3e-15 and from 1.4e-15 to
-// 1.2e-15.  What bounds oz_gemm now: operand tiles from L2 (35 bytes per SM and
+// 5.4 ms with the Bloch functions' digits in memory -> 3.0 ms with the digits
+// made on the way into shared memory (oz_project 2.55, scales and magnitudes
+// 0.38).  The error against 64 bits fell from 1.9e-15 to 1.4e-15 and from 1.4e-15
+// to 0.7e-15.  What bounds oz_gemm now: operand tiles from L2 (35 bytes per SM and
 // clock) beside the products' 64 clocks each.
+//
+// The digits hold an entry to 2^-56 of its row's largest.  Where that is not
+// FP64's accuracy (oz_accept) the projection's elements are formed again on the
+// FP64 pipe, and all of them if these are more than one in 32.
 #include "bse_internal.cuh"
 #include "oz_dev.cuh"
 #include "tc_ptx.cuh"
@@ -29,6 +33,8 @@ constexpr int OZ_A = OZ_M * 128;                   // bytes of one digit's A til
 constexpr int OZ_BD = OZ_N * 128;                  // bytes of one digit's B tile
 constexpr int OZ_B = OZ_S * OZ_BD;                 // ... and of the seven
 constexpr int OZ_AS = 5, OZ_BS = 2;               // ring slots: A per digit, B per K block
+constexpr int OZ_D = 8;                            // accumulators, s = 0..7
+constexpr int OZ_SF = 8;                           // digits of the local functions in the projection
 constexpr int OZ_THREADS = 320;
 // B slots lie between tiles of zeros: 0 B_0..B_6 0 B_0..B_6 0
 constexpr int OZ_BAREA = OZ_BS * (OZ_B + OZ_BD) + OZ_BD;
@@ -71,20 +77,26 @@ __device__ __forceinline__ bool oz_wait(uint32_t a, uint32_t parity, volatile in
   return true;
 }
 
-// Chunks of 128 K elements.  The accumulators s = 4..6 hold one chunk's sums
-// (at most 7 * 128 * 2^14 < 2^24), s = 2, 3 two and s = 0, 1 four (4 * 256 and
+// Chunks of 128 K elements.  The accumulators s = 4, 5 hold one chunk's sums
+// (at most 6 * 128 * 2^14 < 2^24), s = 2, 3 two and s = 0, 1 four (4 * 256 and
 // 2 * 512 times 2^14): c counts the chunks of a tile, `last` its last one.
-// Draining all of them after every chunk cost 12.9 instead of 12.4 ms and 2.6
-// instead of 2.4 (float to integer runs at 16 per SM and clock).  Issuing the
-// products of s < 4 first while the others drain holds four A slots of five and
-// was slower (14.5 ms).
+// s = 6, 7 are kept for 32: past 2^24 (random digits stay below) an addition of
+// 16 K elements is rounded by 2^-24 of the sum so far, which weighs 2^-48 of the
+// whole: all of them by less than 2^-49 of 7 sum |a| |b| even if every digit were
+// at its largest, and 7 * 4096 * 2^14 < 2^31 still converts to an integer.
+// Draining costs as much as converting u (float to integer runs at 16 per SM and
+// clock): all seven of s < 7 after every chunk 12.9 ms for the Green's functions
+// below, s >= 4 after every chunk 12.4 (with s = 7 13.0), as it is 12.2; oz_project
+// 2.6, 2.4 (2.7) and 2.55.
+// Issuing the products of s < 4 first while the others drain holds four A slots
+// of five and was slower (14.5 ms).
 __device__ __forceinline__ bool drains(int s, int c, bool last) {
-  return last || s >= 4 || (s >= 2 ? (c & 1) == 1 : (c & 3) == 3);
+  return last || (s >= 6 ? (c & 31) == 31 : s >= 4 || (s >= 2 ? (c & 1) == 1 : (c & 3) == 3));
 }
 
-// state of the issuing thread: A ring slot and phase, restarts of the accumulators s = 0, 1 / 2, 3 / 4..6
+// state of the issuing thread: A ring slot and phase, restarts of the accumulators s = 0, 1 / 2, 3 / 4, 5 / 6, 7
 struct oz_issue {
-  int sl = 0, r0 = 0, r1 = 0, r2 = 0;
+  int sl = 0, r0 = 0, r1 = 0, r2 = 0, r3 = 0;
   uint32_t ph = 0;
 };
 
@@ -95,8 +107,9 @@ struct oz_issue {
 // (about 64 clocks measured at N = 32 and 64), so two neighbouring B digits
 // form one operand of 128 rows and the accumulators of s = 2P, 2P + 1 one of
 // 128 columns: digit A_i meets (B_0, B_1), (B_2, B_3), ... for even i and (0,
-// B_0), (B_1, B_2), ... for odd i, 19 products instead of 28 per 16 K elements
-// and all of one shape (s = 7 is computed along and not used).
+// B_0), (B_1, B_2), ... for odd i: 19 products per 16 K elements for seven A
+// digits (34 pairs of digits), 20 for eight, and all of one shape.
+template <int SA>   // A digits
 __device__ __forceinline__ bool issue_block(uint32_t tmem, uint32_t sa, unsigned long long db, bool first, int c,
                                             oz_issue& z, uint32_t afull, uint32_t aempty, uint32_t tempty,
                                             volatile int* abort_flag, unsigned long long limit_ns) {
@@ -114,11 +127,11 @@ __device__ __forceinline__ bool issue_block(uint32_t tmem, uint32_t sa, unsigned
   };
   auto drained = [&](int s, int n) { return oz_wait(tempty + 8 * s, ((uint32_t)n & 1u) ^ 1u, abort_flag, limit_ns); };
 #pragma unroll
-  for (int i = 0; i < OZ_S; ++i) {
+  for (int i = 0; i < SA; ++i) {
     if (!oz_wait(afull + 8 * z.sl, z.ph, abort_flag, limit_ns)) return false;
     tc_fence_after();
     if (i == 0 && first) {
-      const bool n0 = (c & 3) == 0, n1 = (c & 1) == 0;
+      const bool n0 = (c & 3) == 0, n1 = (c & 1) == 0, n3 = (c & 31) == 0;
       if (n0 && !(drained(0, z.r0) && drained(1, z.r0))) return false;
       tc_fence_after();
       products(0, 0, 1, n0 ? 0u : 1u);
@@ -128,10 +141,10 @@ __device__ __forceinline__ bool issue_block(uint32_t tmem, uint32_t sa, unsigned
       if (!(drained(4, z.r2) && drained(5, z.r2))) return false;
       tc_fence_after();
       products(0, 2, 3, 0u);
-      if (!drained(6, z.r2)) return false;
+      if (n3 && !(drained(6, z.r3) && drained(7, z.r3))) return false;
       tc_fence_after();
-      products(0, 3, 4, 0u);
-      z.r0 += n0, z.r1 += n1, z.r2 += 1;
+      products(0, 3, 4, n3 ? 0u : 8u);
+      z.r0 += n0, z.r1 += n1, z.r2 += 1, z.r3 += n3;
     } else {
       products(i, i / 2, 4, 15u);   // consecutive products go to different accumulators
     }
@@ -151,14 +164,15 @@ __device__ __forceinline__ void add96(long long& hi, uint32_t& lo, int d, int sh
       : "r"(l), "r"(m), "r"(t));
 }
 
-// Accumulators of 32 TMEM lanes x C columns at ta into sums hi 2^-30 + lo 2^-62
-// (lo unsigned; s < 3 have the weights 2^-14, 2^-22, 2^-30, the rest 2^-38 ..
-// 2^-62).  Each is given back as soon as it is read.
+// Accumulators of 32 TMEM lanes x C columns at ta into sums hi 2^-38 + lo 2^-70
+// (lo unsigned; s < 4 have the weights 2^-14 .. 2^-38, the rest 2^-46 ..
+// 2^-70).  Each is given back as soon as it is read.  |hi| <= 2^48 per 512 K
+// elements: K <= 2^21.
 template <int C>
 __device__ __forceinline__ void drain_chunk(uint32_t ta, int c, bool last, uint32_t tempty, int lane, long long* hi,
                                             uint32_t* lo) {
 #pragma unroll
-  for (int s = 0; s < OZ_S; ++s) {
+  for (int s = 0; s < OZ_D; ++s) {
     if (!drains(s, c, last)) continue;
 #pragma unroll
     for (int h = 0; h < C / 16; ++h) {
@@ -172,18 +186,18 @@ __device__ __forceinline__ void drain_chunk(uint32_t ta, int c, bool last, uint3
 #pragma unroll
       for (int k = 0; k < 16; ++k) {
         const int d = __float2int_rn(v[k]), j = 16 * h + k;
-        if (s < 3) {
-          hi[j] += (long long)d * (1 << (8 * (2 - s)));
+        if (s < 4) {
+          hi[j] += (long long)d * (1 << (8 * (3 - s)));
         } else {
           // 96-bit addition; as 64-bit arithmetic lo would take a pair of registers
-          add96(hi[j], lo[j], d, 8 * (6 - s));
+          add96(hi[j], lo[j], d, 8 * (7 - s));
         }
       }
     }
   }
 }
 __device__ __forceinline__ double oz_value(long long hi, long long lo) {
-  return (double)hi * 0x1p-30 + (double)lo * 0x1p-62;
+  return (double)hi * 0x1p-38 + (double)lo * 0x1p-70;
 }
 
 // Persistent warp-specialised kernel, one CTA per SM: warp 0 streams digit
@@ -197,7 +211,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   extern __shared__ unsigned char oz_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)oz_raw + 1023) & ~(uintptr_t)1023);
   unsigned long long* bars = (unsigned long long*)(sm + OZ_AS * OZ_A + OZ_BAREA);
-  constexpr int NBAR = 2 * OZ_AS + 2 * OZ_BS + 1 + OZ_S + 1;
+  constexpr int NBAR = 2 * OZ_AS + 2 * OZ_BS + 1 + OZ_D + 1;
   uint32_t* tmem_slot = (uint32_t*)(bars + NBAR);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   volatile int* a_issued = (volatile int*)(tmem_slot + 2);
@@ -221,7 +235,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       mbar_init(bempty(s), 1);
     }
     mbar_init(tfull, 1);
-    for (int s = 0; s < OZ_S; ++s) mbar_init(tempty(s), 8);
+    for (int s = 0; s < OZ_D; ++s) mbar_init(tempty(s), 8);
     mbar_init(fin, 1);
     *abort_flag = 0;
     *a_issued = 0;
@@ -277,7 +291,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         if (!(ok = oz_wait(bfull(s), (uint32_t)(ib / OZ_BS) & 1u, abort_flag, p.wait_ns))) break;
         ++ib;
         const unsigned long long db = sdesc_sw128(sb + s * (OZ_B + OZ_BD));
-        if (!(ok = issue_block(tmem, sa, db, first, kb >> 1, z, afull(0), aempty(0), tempty(0), abort_flag, p.wait_ns))) break;
+        if (!(ok = issue_block<OZ_S>(tmem, sa, db, first, kb >> 1, z, afull(0), aempty(0), tempty(0), abort_flag, p.wait_ns))) break;
         mma_commit(bempty(s));
         if (last) mma_commit(tfull);
       }
@@ -410,37 +424,231 @@ __global__ void __launch_bounds__(256) oz_split_rows(const double2* __restrict__
   }
 }
 
-// Largest magnitude key of u[k][x][n] over x for every (k, n): blocks of 32
-// bands x 8 rows walk a part of the grid (coalesced along n).
-__global__ void __launch_bounds__(256) oz_col_keys(const double2* __restrict__ u, int nx, int nb, int per,
-                                                   unsigned* __restrict__ keys) {
-  __shared__ unsigned sk[8][32];
-  const int n = blockIdx.y * 32 + (threadIdx.x & 31), g = threadIdx.x >> 5, k = blockIdx.z;
-  const int x0 = blockIdx.x * per, x1 = min(nx, x0 + per);
-  unsigned key = 0;
-  if (n < nb) {
-    const double2* p = u + (size_t)k * nx * nb + n;
-#pragma unroll 4
-    for (int x = x0 + g; x < x1; x += 8) {
-      const double2 v = p[(size_t)x * nb];
-      key = max(key, max(oz_key(v.x), oz_key(v.y)));
-    }
-  }
-  sk[g][threadIdx.x & 31] = key;
-  __syncthreads();
-  if (g == 0 && n < nb) {
-#pragma unroll
-    for (int i = 1; i < 8; ++i) key = max(key, sk[i][threadIdx.x]);
-    atomicMax(keys + (size_t)k * nb + n, key);
-  }
-}
-
 // a load that stays where it stands: the compiler otherwise sinks the next
 // block's loads behind the waits, to their use
 __device__ __forceinline__ double2 load_in_place(const double2* p) {
   double2 v;
   asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
   return v;
+}
+
+// Digits of the local functions' rows f [np][n], eight each (a function that
+// falls off keeps FP64's digits to 2^-10 of its largest value, and what it loses
+// below is 2^-64 of that): rows (Re f, Im f) and (-Im f, Re f) as in
+// oz_split_rows with pair = 1, dig [8][2 np][kp]; with them its magnitudes max(|Re|,
+// |Im|) as BF16 in units of the row's scale, mag [np][kp / 2], the row's norm in
+// these units and 2^1/2 of its number of entries.  One block per function.
+struct __align__(8) OzNorm {
+  float norm, root;
+};
+__global__ void __launch_bounds__(256) oz_split_functions(const double2* __restrict__ f, int n, int np, int kp,
+                                                          __half* __restrict__ dig, unsigned short* __restrict__ mag,
+                                                          double* __restrict__ scale, OzNorm* __restrict__ norm,
+                                                          int* __restrict__ bad) {
+  __shared__ float ws[8];
+  __shared__ int wc[8];
+  const int row = blockIdx.x;
+  const double2* x = f + (size_t)row * n;
+  unsigned key = 0;
+  for (int k = threadIdx.x; k < n; k += blockDim.x) key = max(key, max(oz_key(x[k].x), oz_key(x[k].y)));
+  key = block_max(key);
+  int flag = 0;
+  const int e = oz_exponent(key, &flag);
+  uint32_t* out = reinterpret_cast<uint32_t*>(dig) + (size_t)2 * row * (kp / 2);
+  const size_t digit = (size_t)2 * np * (kp / 2);
+  float sq = 0.f;
+  int count = 0;
+  for (int k = threadIdx.x; k < kp / 2; k += blockDim.x) {
+    const double2 v = k < n ? x[k] : make_double2(0.0, 0.0);
+    int dr[OZ_SF], di[OZ_SF], dm[OZ_SF];
+    oz_digits8(v.x, e, dr);
+    oz_digits8(v.y, e, di);
+    oz_digits8(-v.y, e, dm);
+#pragma unroll
+    for (int i = 0; i < OZ_SF; ++i) {
+      const __half2 a = __floats2half2_rn((float)dr[i], (float)di[i]), b = __floats2half2_rn((float)dm[i], (float)dr[i]);
+      out[i * digit + k] = *reinterpret_cast<const uint32_t*>(&a);
+      out[i * digit + kp / 2 + k] = *reinterpret_cast<const uint32_t*>(&b);
+    }
+    const float ur = oz_unit(v.x, e), ui = oz_unit(v.y, e);
+    mag[(size_t)row * (kp / 2) + k] = (unsigned short)(__float_as_uint(fmaxf(ur, ui)) >> 16);
+    sq += ur * ur + ui * ui;
+    count += v.x != 0.0 || v.y != 0.0;
+  }
+  for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+  count = __reduce_add_sync(0xffffffffu, count);
+  if ((threadIdx.x & 31) == 0) {
+    ws[threadIdx.x >> 5] = sq;
+    wc[threadIdx.x >> 5] = count;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < 8; ++w) {
+    sq += ws[w];
+    count += wc[w];
+  }
+  const double s = scalbn(1.0, e);
+  scale[2 * row] = scale[2 * row + 1] = s;
+  norm[row] = OzNorm{sqrtf(sq), sqrtf(2.f * (float)count)};
+  if (flag) atomicOr(bad, 1);
+}
+
+// exponent that the magnitudes of column n are taken relative to: its first entry's
+__device__ __forceinline__ int first_exponent(double2 v) {
+  const unsigned key = max(oz_key(v.x), oz_key(v.y));
+  return key ? (int)(key >> 20) - 1022 : 0;
+}
+
+// One reading of u[k][x][n] for the row scales and for what oz_accept asks:
+//   keys[k][n]          largest magnitude key over x
+//   cover[part][k][p][n] sum over the part's grid points of |f_p(x)| |u_kn(x)|, of the
+//                       larger component's BF16 each, rounded down, in units of
+//                       f's scale and 2^first_exponent
+// Blocks of 64 bands x `per` grid points; a warp takes 8 bands, whose values it
+// loads as they stand in the product's registers, and 64 functions at a time
+// from shared memory (mma.sync m16n8k16).  Bound by HBM: 2.1 GB in 0.36 ms (the
+// keys alone 0.29).
+constexpr int CV_P = 64, CV_X = 256, CV_LD = CV_X + 8;
+__global__ void __launch_bounds__(256) oz_cover(const double2* __restrict__ u, int nx, int nb, int per,
+                                                const unsigned short* __restrict__ mag, int np, int xp,
+                                                unsigned* __restrict__ keys, float* __restrict__ cover) {
+  __shared__ __align__(16) unsigned short fs[CV_P * CV_LD];
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, k = blockIdx.z;
+  const int n0 = blockIdx.y * 64 + (threadIdx.x >> 5) * 8, n = n0 + g;
+  const int xa = blockIdx.x * per, xb = min(nx, xa + per);
+  const bool in = n < nb;
+  const double2* p = u + (size_t)k * nx * nb + (in ? n : 0);
+  const int shift = (first_exponent(p[0]) + (1023 - 127)) << 7;   // of the exponent, above BF16's 7 bits
+  unsigned key = 0;
+  auto bf16 = [&](double2 v) {
+    const int m = max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
+    return (uint32_t)min(max((m >> 13) - shift, 0), 0x7f7f);
+  };
+  double2 w[8];   // the next 32 points: of each 16, this lane's four
+  auto load = [&](int x0) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int x = x0 + 2 * t + (i & 1) + 8 * (i >> 1);
+      w[i] = make_double2(0.0, 0.0);
+      if (in && x < xb) w[i] = load_in_place(p + (size_t)x * nb);
+    }
+  };
+  for (int p0 = 0; p0 < np; p0 += CV_P) {
+    load(xa);
+    float c[CV_P / 16][4];
+#pragma unroll
+    for (int i = 0; i < CV_P / 4; ++i) c[i >> 2][i & 3] = 0.f;
+    for (int x0 = xa; x0 < xb; x0 += CV_X) {
+      __syncthreads();
+#pragma unroll
+      for (int i = threadIdx.x; i < CV_P * (CV_X / 8); i += 256) {
+        const int r = i / (CV_X / 8), x = i % (CV_X / 8) * 8;
+        *reinterpret_cast<uint4*>(&fs[r * CV_LD + x]) =
+            p0 + r < np && x0 + x < xp ? *reinterpret_cast<const uint4*>(&mag[(size_t)(p0 + r) * xp + x0 + x])
+                                       : make_uint4(0, 0, 0, 0);
+      }
+      __syncthreads();
+      for (int xs = 0; xs < CV_X && x0 + xs < xb; xs += 32) {
+        double2 v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = w[i];
+        if (x0 + xs + 32 < xb) load(x0 + xs + 32);   // across the barriers above too
+        if (p0 == 0)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) key = max(key, max(oz_key(v[i].x), oz_key(v[i].y)));
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const uint32_t b0 = bf16(v[4 * h]) | bf16(v[4 * h + 1]) << 16, b1 = bf16(v[4 * h + 2]) | bf16(v[4 * h + 3]) << 16;
+#pragma unroll
+          for (int mt = 0; mt < CV_P / 16; ++mt) {
+            uint32_t a[4];
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
+                         : "r"(smem_u32(&fs[(mt * 16 + (lane & 15)) * CV_LD + xs + 16 * h + (lane >> 4) * 8])));
+            asm volatile(
+                "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, "
+                "%1, %2, %3};"
+                : "+f"(c[mt][0]), "+f"(c[mt][1]), "+f"(c[mt][2]), "+f"(c[mt][3])
+                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+          }
+        }
+      }
+    }
+    float* o = cover + ((size_t)blockIdx.x * gridDim.z + k) * np * nb;
+#pragma unroll
+    for (int mt = 0; mt < CV_P / 16; ++mt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int q = p0 + mt * 16 + g + 8 * (i >> 1), m = n0 + 2 * t + (i & 1);
+        if (q < np && m < nb) o[(size_t)q * nb + m] = c[mt][i];
+      }
+  }
+  key = max(key, __shfl_xor_sync(0xffffffffu, key, 1));
+  key = max(key, __shfl_xor_sync(0xffffffffu, key, 2));
+  if (t == 0 && in) atomicMax(keys + (size_t)k * nb + n, key);
+}
+
+// Lists the elements [k][p][n] of a pass whose magnitudes do not cover the
+// digits' error.  u's rounding counts with f's norm; f's own is 2^-8 of u's.
+struct OzRepair {
+  const double2 *u, *f, *phase;   // u, phase: the pass's first k point
+  const float* cover;
+  const unsigned* keys;
+  const int* expo;
+  const OzNorm* norm;
+  int parts, nk, nx, xp, nb, np, nkt, k0;
+  double alpha;
+  double2* out;
+  unsigned* list;    // [cap]
+  unsigned cap;
+  unsigned* count;
+};
+__global__ void __launch_bounds__(256) oz_refused(const OzRepair p, int* __restrict__ bad) {
+  const size_t total = (size_t)p.nk * p.np * p.nb, i = blockIdx.x * (size_t)256 + threadIdx.x;
+  bool refused = false;
+  if (i < total) {
+    const int n = (int)(i % p.nb), q = (int)(i / p.nb % p.np), k = (int)(i / p.nb / p.np);
+    const OzNorm f = p.norm[q];
+    if (f.norm > 0.f && p.keys[(size_t)k * p.nb + n]) {
+      float s = 0.f;
+      for (int j = 0; j < p.parts; ++j) s += p.cover[j * total + i];
+      s = ldexpf(s, first_exponent(p.u[(size_t)k * p.nx * p.nb + n]) - p.expo[(size_t)k * p.nb + n]);
+      refused = !(isfinite(s) && oz_accept(s, f.norm, f.root * 0x1p-8f));
+    }
+  }
+  const unsigned w = __ballot_sync(0xffffffffu, refused), lane = threadIdx.x & 31;
+  if (!w) return;
+  unsigned at = 0;
+  if (lane == 0) {
+    at = atomicAdd(p.count, __popc(w));
+    if (at + __popc(w) > p.cap) *bad = 1;
+  }
+  at = __shfl_sync(0xffffffffu, at, 0) + __popc(w & ((1u << lane) - 1u));
+  if (refused && at < p.cap) p.list[at] = (unsigned)i;
+}
+
+// ... and forms them on the FP64 pipe, one warp each
+__global__ void __launch_bounds__(256) oz_repair(const OzRepair p) {
+  const unsigned m = min(*p.count, p.cap), lane = threadIdx.x & 31;
+  for (unsigned w = blockIdx.x * 8 + (threadIdx.x >> 5); w < m; w += gridDim.x * 8) {
+    const unsigned i = p.list[w];
+    const int n = (int)(i % p.nb), q = (int)(i / p.nb % p.np), k = (int)(i / p.nb / p.np);
+    const double2 *f = p.f + (size_t)q * p.nx, *ph = p.phase + (size_t)k * p.xp, *u = p.u + (size_t)k * p.nx * p.nb + n;
+    double2 s = make_double2(0.0, 0.0);
+    for (int x = lane; x < p.nx; x += 32) {
+      const double2 a = f[x];
+      if (a.x == 0.0 && a.y == 0.0) continue;
+      const double2 b = u[(size_t)x * p.nb], e = ph[x];
+      const double br = b.x * e.x - b.y * e.y, bi = b.x * e.y + b.y * e.x;
+      s.x = fma(a.x, br, fma(a.y, bi, s.x));
+      s.y = fma(a.x, bi, fma(-a.y, br, s.y));
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+    }
+    if (lane == 0) p.out[((size_t)q * p.nkt + p.k0 + k) * p.nb + n] = make_double2(p.alpha * s.x, p.alpha * s.y);
+  }
 }
 
 // e^{ik.x} per dimension: tab_d[m][j] = e^{2 pi i (m + s_d) j / (nk_d nx_d)}, the
@@ -547,7 +755,7 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
   unsigned char* const bs = sm + OZ_AS * OZ_A + OZ_BD;   // first B slot
   double2* phs = (double2*)(sm + OZ_AS * OZ_A + OZ_BAREA);
   unsigned long long* bars = (unsigned long long*)(phs + OZ_PH * (OZ_KB / 2));
-  constexpr int NBAR = 2 * OZ_AS + 2 * OZ_BS + 2 * OZ_PH + 1 + OZ_S + 1;
+  constexpr int NBAR = 2 * OZ_AS + 2 * OZ_BS + 2 * OZ_PH + 1 + OZ_D + 1;
   uint32_t* tmem_slot = (uint32_t*)(bars + NBAR);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   volatile int* a_issued = (volatile int*)(tmem_slot + 2);
@@ -575,7 +783,7 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
       mbar_init(pempty(s), OZ_W);
     }
     mbar_init(tfull, 1);
-    for (int s = 0; s < OZ_S; ++s) mbar_init(tempty + 8 * s, OZ_W);
+    for (int s = 0; s < OZ_D; ++s) mbar_init(tempty + 8 * s, OZ_W);
     mbar_init(fin, 1);
     *abort_flag = 0;
     *a_issued = 0;
@@ -618,7 +826,7 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
     for (int i = 0; i < total && ok; ++i) {
       while (ok && ip < total && ip < i + OZ_PH - 1) ok = phases();
       const int m = t % p.mt;
-      for (int j = 0; j < OZ_S && ok; ++j) {
+      for (int j = 0; j < OZ_SF && ok; ++j) {
         const int q = ia % OZ_AS;
         if (!(ok = oz_wait(aempty(q), ((uint32_t)(ia / OZ_AS) & 1u) ^ 1u, abort_flag, p.wait_ns))) break;
         mbar_expect_tx(afull(q), OZ_A);
@@ -639,7 +847,7 @@ __global__ void __launch_bounds__(OZ_PT, 1) oz_project(const __grid_constant__ C
       const int s = i % OZ_BS;
       if (!(ok = oz_wait(bfull(s), (uint32_t)(i / OZ_BS) & 1u, abort_flag, p.wait_ns))) break;
       const unsigned long long db = sdesc_sw128(sb + s * (OZ_B + OZ_BD));
-      if (!(ok = issue_block(tmem, sa, db, (b & 1) == 0, c, z, afull(0), aempty(0), tempty, abort_flag, p.wait_ns))) break;
+      if (!(ok = issue_block<OZ_SF>(tmem, sa, db, (b & 1) == 0, c, z, afull(0), aempty(0), tempty, abort_flag, p.wait_ns))) break;
       mma_commit(bempty(s));
       if ((b & 1) == 1 || b + 1 == p.kb) {
         mma_commit(tfull);
@@ -850,21 +1058,29 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
     cudaGetLastError();
     return BSE_OK;
   }
-  const size_t per = (size_t)kp / 2 * sizeof(double2);
-  const int nkc = (int)std::min<size_t>({(size_t)nkt, std::max<size_t>(((size_t)256 << 20) / per, 1), (size_t)32768});
+  // parts of the grid in oz_cover: of 1024 points, and enough to fill the SMs
+  const int nbt = (nb + 63) / 64, want = std::max((nxt + 1023) / 1024, (4 * sms + nkt * nbt - 1) / (nkt * nbt));
+  const int xpart = (nxt + CV_X * std::min(want, 64) - 1) / (CV_X * std::min(want, 64)) * CV_X;
+  const int parts = (nxt + xpart - 1) / xpart;
+  const size_t per = (size_t)kp / 2 * sizeof(double2), outs = (size_t)np * nb, pcov = (size_t)parts * outs * sizeof(float);
+  const int nkc = (int)std::min<size_t>({(size_t)nkt, std::max<size_t>(((size_t)256 << 20) / (per + pcov), 1), (size_t)32768,
+                                         std::max<size_t>(((size_t)1 << 31) / outs, 1)});
   auto pad = [](size_t n) { return (n + 255) / 256 * 256; };
   long long ntab = 0;
   for (int i = 0; i < 3; ++i) ntab += (long long)nk[i] * nx[i];
-  const size_t sd = bse_oz_digit_bytes(1, 2 * np, kp), sf = pad((size_t)2 * np * sizeof(double)), sph = pad(nkc * per);
+  const size_t sd = bse_oz_digit_bytes(1, 2 * np, kp) / OZ_S * OZ_SF, sf = pad((size_t)2 * np * sizeof(double)), sph = pad(nkc * per);
   const size_t stab = pad((size_t)ntab * sizeof(double2)), skey = pad((size_t)nkc * nb * sizeof(unsigned));
   const size_t ssc = pad((size_t)nkc * nb * sizeof(double)), npart = (size_t)2 * sms * OZ_M * OZ_N;
+  const size_t smag = pad((size_t)np * (kp / 2) * sizeof(short)), snrm = pad((size_t)np * sizeof(OzNorm));
+  const size_t scov = pad(nkc * pcov), cap = nkc * outs / 32 + 1024, slist = pad(cap * sizeof(unsigned));
   struct Scratch {
     void* p = nullptr;
     ~Scratch() {
       if (p) cudaFree(p);
     }
   } sc;
-  if (cudaMalloc(&sc.p, sd + sf + sph + stab + 2 * skey + ssc + npart * 12 + 256) != cudaSuccess) {
+  if (cudaMalloc(&sc.p, sd + sf + sph + stab + 2 * skey + ssc + npart * 12 + smag + snrm + scov + slist + 256) !=
+      cudaSuccess) {
     cudaGetLastError();
     sc.p = nullptr;
     return BSE_OK;
@@ -887,7 +1103,15 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
   q += ssc;
   p.part_hi = (long long*)q, q += npart * 8;
   p.part_lo = (uint32_t*)q, q += npart * 4;
-  int* word = (int*)q;   // {wait gave up, out of range}
+  unsigned short* mag = (unsigned short*)q;
+  q += smag;
+  OzNorm* norm = (OzNorm*)q;
+  q += snrm;
+  float* cover = (float*)q;
+  q += scov;
+  unsigned* list = (unsigned*)q;
+  q += slist;
+  int* word = (int*)q;   // {wait gave up, out of range or too many elements refused, elements refused}
   p.phase = phase;
   p.expo = expo;
   p.scale = scale;
@@ -905,25 +1129,39 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
   p.err = word;
   p.wait_ns = wait_limit();
   CUtensorMap ma;
-  if (!digit_map(&ma, (const __half*)A.digits, kp, A.rows, OZ_S, OZ_M, 1)) return BSE_OK;
+  if (!digit_map(&ma, (const __half*)A.digits, kp, A.rows, OZ_SF, OZ_M, 1)) return BSE_OK;
   cudaMemsetAsync(word, 0, 2 * sizeof(int), st);
   // rows (Re f, Im f) and (-Im f, Re f): real and imaginary part of conj(f) times a column
-  bse_status s = bse_oz_split_rows(f, np, nxt, nullptr, 1, 1, A, word + 1, st);
+  oz_split_functions<<<(unsigned)np, 256, 0, st>>>(f, nxt, np, kp, (__half*)A.digits, mag, A.scale, norm, word + 1);
+  bse_status s = BSE_OK;
+  OzRepair rp{};
+  rp.f = f, rp.phase = phase, rp.cover = cover, rp.keys = keys, rp.expo = expo, rp.norm = norm;
+  rp.parts = parts, rp.nx = nxt, rp.xp = kp / 2, rp.nb = nb, rp.np = np, rp.nkt = nkt;
+  rp.alpha = dv;
+  rp.out = a;
+  rp.list = list;
+  rp.cap = (unsigned)cap;
+  rp.count = (unsigned*)word + 2;
   oz_tables<<<(unsigned)((ntab + 255) / 256), 256, 0, st>>>(ms, tab);
-  const int xrows = nxt > 8192 ? 1024 : 512;   // grid points per block of the key kernel
   for (int k = 0; k < nkt && s == BSE_OK; k += nkc) {
     const int n = std::min(nkc, nkt - k);
     p.u = u + (size_t)k * nxt * nb;
     p.k0 = k;
     p.ntiles = p.mt * p.nt * n;
     cudaMemsetAsync(keys, 0, (size_t)n * nb * sizeof(unsigned), st);
-    oz_col_keys<<<dim3((unsigned)((nxt + xrows - 1) / xrows), (unsigned)((nb + 31) / 32), (unsigned)n), 256, 0, st>>>(
-        p.u, nxt, nb, xrows, keys);
+    cudaMemsetAsync(rp.count, 0, sizeof(unsigned), st);
+    oz_cover<<<dim3((unsigned)parts, (unsigned)nbt, (unsigned)n), 256, 0, st>>>(p.u, nxt, nb, xpart, mag, np, kp / 2, keys,
+                                                                                cover);
     oz_bloch_scales<<<(unsigned)(((long long)n * nb + 255) / 256), 256, 0, st>>>(keys, n * nb, expo, scale, word + 1);
     oz_phases<<<dim3((unsigned)((kp / 2 + 255) / 256), (unsigned)n), 256, 0, st>>>(ms, tab, k, kp / 2, phase);
     const int grid = (int)std::min<long long>(sms, (long long)p.ntiles * p.cpt);
     oz_project<<<grid, OZ_PT, OZ_PSMEM, st>>>(ma, p);
     oz_join<<<dim3((unsigned)p.ntiles, OZ_M / 16), 256, 0, st>>>(p, grid);
+    rp.u = p.u;
+    rp.nk = n;
+    rp.k0 = k;
+    oz_refused<<<(unsigned)((n * outs + 255) / 256), 256, 0, st>>>(rp, word + 1);
+    oz_repair<<<(unsigned)(4 * sms), 256, 0, st>>>(rp);
     if (cudaGetLastError() != cudaSuccess) s = BSE_ERR_CUDA;
   }
   int hw[2] = {0, 0};

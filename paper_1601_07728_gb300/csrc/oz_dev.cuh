@@ -5,13 +5,15 @@
 // A row of an operand is scaled by a power of two to |y| < 1 and written as
 // seven balanced base-256 digits, y = sum_i d_i 2^(-7-8i), |d_i| <= 128, i < 7:
 // 55 bits below the row's largest entry (the 53 of FP64 and two guard bits at
-// the top).  A digit is an integer that FP16 holds exactly, and a sum of fewer than 2^24 /
-// 2^14 products of two digits is exact in the FP32 accumulators.  Digit
-// products (i, j) of equal s = i + j < 7 share an accumulator; 128 K elements
+// the top; eight digits: 2^-64 of the largest).  A digit is an integer that FP16 holds
+// exactly, and a sum of fewer than 2^24 / 2^14 products of two digits is exact in
+// the FP32 accumulators.  Digit
+// products (i, j) of equal s = i + j share an accumulator; 128 K elements
 // of up to seven products reach at most 7 * 128 * 2^14 < 2^24 (fewer products:
-// more elements), after which the accumulators are drained into integers.  The only roundings are the
-// one of each operand entry at 2^-56 of its row's largest, the dropped
-// products s >= 7 (of the same size) and the final conversion.
+// more elements), after which the accumulators are drained into integers.
+// Products of s = 7 are formed as well: of the rest, 2^-8 of that, none.  The
+// only roundings are then the one of each operand entry at 2^-56 of its row's
+// largest and the final conversion.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -89,6 +91,22 @@ __device__ __forceinline__ float oz_unit(double x, int e) {
 // 0.1 sqrt(n) (1 / r_a + 1 / r_b), r = 3..8 their scale over their deviation.
 __device__ __forceinline__ bool oz_accept(float s, float norm_a, float norm_b) {
   return s >= 0.1f * (norm_a + norm_b);
+}
+
+// the same to 63 bits as eight digits, d[0] the leading one
+__device__ __forceinline__ void oz_digits8(double x, int e, int* d) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  // |x| 2^(63-e) = (mantissa << 10) >> r with the leading bit of the mantissa at 52
+  const int r = max(0, 1022 + e - (int)((b >> 52) & 0x7ff));
+  const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+  long long v = r <= 10 ? (long long)(m << (10 - r)) : r < 73 ? (long long)((m + (1ull << (r - 11))) >> (r - 10)) : 0;
+  if ((long long)b < 0) v = -v;
+#pragma unroll
+  for (int i = 7; i > 0; --i) {
+    d[i] = (int)(signed char)(v & 0xff);
+    v = (v - d[i]) >> 8;
+  }
+  d[0] = (int)v;
 }
 
 // digit i (0 = leading) of two entries as packed FP16: the bytes b become

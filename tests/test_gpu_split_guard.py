@@ -97,3 +97,62 @@ def test_non_finite_entries_reach_what_they_reached_in_fp64():
     assert not np.any(np.isfinite(out[1]))
     others = np.ix_([0, 2, 3, 4, 5], [n for n in range(32) if n != 3])   # 0 * inf of the spin-orbit term in band 3
     assert np.array_equal(out[others], ref[others])
+
+
+# ---------------------------------------------------------------------------
+# set-up projection (csrc/k_oz.cu)
+# ---------------------------------------------------------------------------
+def projection_bound(u, nk, f, dv):
+    """2 (n_x + 16) 2^-53 dv |f| |u|: the sum's products, and the phases' three factors in each."""
+    return 2 * (f.shape[1] + 16) * U64 * dv * np.einsum("px,kxn->pkn", np.abs(f), np.abs(u))
+
+
+# some elements of the call (listed and formed again), most of them (the FP64
+# kernel for all), a grid in several parts and one that ends inside a K block,
+# more functions than one pass of the magnitudes takes
+@pytest.mark.parametrize("decades", [10, 18])
+@pytest.mark.parametrize("shape", [((3, 3, 3), (11, 11, 11), 64, 36, 10, 6), ((3, 3, 3), (11, 11, 11), 64, 36, 64, 36),
+                                   ((2, 1, 1), (17, 16, 15), 130, 70, 6, 5), ((1, 1, 1), (24, 24, 24), 65, 16, 8, 1)])
+def test_projection_of_graded_functions_keeps_fp64_accuracy(shape, decades):
+    nk, nx, nb, npj, bands, functions = shape
+    n, m = int(np.prod(nk)), int(np.prod(nx))
+    rng = np.random.default_rng(m + bands)
+    u, f = S.complex_normal(rng, (n, m, nb)), S.complex_normal(rng, (npj, m))
+    rise = 10.0 ** (-decades * np.linspace(0, 1, m))
+    u[:, :, :bands] *= rise[None, :, None]
+    f[-functions:] *= rise[::-1]
+    a = bse.local_projection(u, nk, nx, f, 0.3, (0.0, 0.25, 0.5))
+    ref = O.local_projection(u, nk, nx, f, 0.3, (0.0, 0.25, 0.5))
+    assert np.all(np.abs(a - ref) <= 2 * projection_bound(u, nk, f, 0.3))
+
+
+def test_only_the_refused_elements_of_a_projection_leave_the_tensor_cores(monkeypatch):
+    nk, nx, nb, npj = (3, 3, 3), (11, 11, 11), 64, 36
+    rng = np.random.default_rng(3)
+    u, f = S.complex_normal(rng, (27, 1331, nb)), S.complex_normal(rng, (npj, 1331))
+    flat = bse.local_projection(u, nk, nx, f, 0.3)
+    rise = 10.0 ** (-12 * np.linspace(0, 1, 1331))
+    u[:, :, 5] *= rise[None, :]
+    f[7] *= rise[::-1]
+    f[9] = 0
+    f[11, 700:] = 0
+    u[:, :700, 40] = 0
+    a = bse.local_projection(u, nk, nx, f, 0.3)
+    monkeypatch.setenv("BSE_SPLIT_WAIT_NS", "1000")   # gives up: the FP64 kernel
+    fp64 = bse.local_projection(u, nk, nx, f, 0.3)
+    rows, cols = [p for p in range(npj) if p not in (7, 9, 11)], [n for n in range(nb) if n not in (5, 40)]
+    same = np.ix_(rows, range(27), cols)
+    assert np.array_equal(a[same], flat[same]) and np.mean(a[same] == fp64[same]) < 0.1
+    assert np.all(a[9] == 0) and np.all(a[11, :, 40] == 0)
+    bound = projection_bound(u, nk, f, 0.3)
+    assert np.all(np.abs(a - O.local_projection(u, nk, nx, f, 0.3)) <= 2 * bound)
+
+
+@pytest.mark.parametrize("power", [-390, -130, 130, 390])
+def test_projection_of_functions_of_any_scale(power):
+    """Magnitudes far outside FP32's range on either side, per column of u and row of f."""
+    nk, nx, nb, npj = (3, 3, 3), (11, 11, 11), 64, 36
+    rng = np.random.default_rng(power + 400)
+    u, f = S.complex_normal(rng, (27, 1331, nb)), S.complex_normal(rng, (npj, 1331))
+    a = bse.local_projection(u * 2.0 ** power, nk, nx, f * 2.0 ** -power, 0.3)
+    assert np.array_equal(a, bse.local_projection(u, nk, nx, f, 0.3))
