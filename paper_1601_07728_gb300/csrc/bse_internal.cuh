@@ -232,6 +232,7 @@ bse_status bse_local_projection_device(const double2* u, const int* nk, const in
 struct bse_oz_operand {
   void* digits = nullptr;
   double* scale = nullptr;
+  float2* norm = nullptr;   // of the complex rows: {norm in units of the scale, 2^1/2 of the number of entries}
   int batches = 1, rows = 0, kp = 0;
 };
 size_t bse_oz_digit_bytes(int batches, int rows, int kp);
@@ -250,6 +251,11 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
 // bounded wait gave up; BSE_ERR_UNSUPPORTED (nothing launched) where the set-up fails
 bse_status bse_oz_gemm(const bse_oz_operand& a, const bse_oz_operand& b, int batches, double alpha, double* out,
                        long long sb, long long sr2, long long sr1, long long sc, int* err, cudaStream_t st);
+// elements (batch << 32 | r << 16 | r') of the product of pair = 0 rows a and pair = 1 rows b of the
+// same vectors that the digits cannot stand for (oz_accept): count[0] of them in the list, or
+// count[1] where count[0] > cap; *bad = 1 where that is beyond `cap` too
+bse_status bse_oz_refused(const bse_oz_operand& a, const bse_oz_operand& b, int batches, unsigned long long* list,
+                          unsigned cap, unsigned* count, int* bad, cudaStream_t st);
 // screening: G_j = psi diag(1/(mu + i t_j - eps)) psi^H for all j, chi0 from them (k_screen.cu)
 bse_status bse_screening_device(const double2* psi, const double* eps, int nr, int nkk, double mu, const double* t,
                                 const double* w, int nt, double2* G, double2* chi, cudaStream_t st);

@@ -7,7 +7,7 @@
 // FP16 products, so that the 19 products of 128 x 128 x 16 which replace one
 // FP64 product of 128 x 64 x 16 still run some 50 times faster.  Measured:
 // Green's functions of 900 points, 4096 states and 16 frequencies 682 ms
-// (FP64 kernel) -> 13.3 ms (this one 12.2, writing the digits 0.97); the
+// (FP64 kernel) -> 13.6 ms (this one 12.2, writing the digits 0.97, magnitudes 0.29); the
 // projection of 8^3 k x 16^3 points x 64 bands onto 64 functions 102.6 ms ->
 // 5.4 ms with the Bloch functions' digits in memory -> 3.0 ms with the digits
 // made on the way into shared memory (oz_project 2.55, scales and magnitudes
@@ -16,8 +16,8 @@
 // clock) beside the products' 64 clocks each.
 //
 // The digits hold an entry to 2^-56 of its row's largest.  Where that is not
-// FP64's accuracy (oz_accept) the projection's elements are formed again on the
-// FP64 pipe, and all of them if these are more than one in 32.
+// FP64's accuracy (oz_accept) the elements are formed again on the FP64 pipe, and
+// all of them if these are more than one in 32.
 #include "bse_internal.cuh"
 #include "oz_dev.cuh"
 #include "tc_ptx.cuh"
@@ -374,15 +374,37 @@ __device__ unsigned block_max(unsigned v) {
   return m;
 }
 
+// {norm, 2^1/2 of the number of entries} of a row from every thread's sum of
+// squares and count (blockDim.x <= 256); for thread 0
+__device__ float2 block_norm(float sq, int count) {
+  __shared__ float ws[8];
+  __shared__ int wc[8];
+  for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+  count = __reduce_add_sync(0xffffffffu, count);
+  if ((threadIdx.x & 31) == 0) {
+    ws[threadIdx.x >> 5] = sq;
+    wc[threadIdx.x >> 5] = count;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
+      sq += ws[w];
+      count += wc[w];
+    }
+  return make_float2(sqrtf(sq), sqrtf(2.f * (float)count));
+}
+
 // Digits of the rows of X [rows][n] (complex), one block per row and batch j;
 // with d != nullptr entry K of batch j is first multiplied by d[j][K].
 //   pair = 0: one row (re, im) per complex row, K = 2n interleaved
 //   pair = 1: two rows, (re, im) and (-im, re): the products with a pair-0 row
 //             are the real and imaginary part of sum x_a conj(x_b)
-// dig [batch][7][rows (x2)][kp], zero beyond 2n; scale 2^e per row.
+// dig [batch][7][rows (x2)][kp], zero beyond 2n; scale 2^e per row; norm [batch][rows]
+// of the complex rows in units of that, with 2^1/2 of their number of entries.
 __global__ void __launch_bounds__(256) oz_split_rows(const double2* __restrict__ X, int n, const double2* __restrict__ d,
                                                      int rows, int kp, int pair, __half* __restrict__ dig,
-                                                     double* __restrict__ scale, int* __restrict__ bad) {
+                                                     double* __restrict__ scale, float2* __restrict__ norm,
+                                                     int* __restrict__ bad) {
   const int row = blockIdx.x, b = blockIdx.y;
   const double2* x = X + (size_t)row * n;
   const double2* db = d ? d + (size_t)b * n : nullptr;
@@ -411,8 +433,13 @@ __global__ void __launch_bounds__(256) oz_split_rows(const double2* __restrict__
   }
   uint32_t* out = reinterpret_cast<uint32_t*>(dig) + ((size_t)b * OZ_S * nr + r0) * (kp / 2);
   const size_t digit = (size_t)nr * (kp / 2);
+  float sq = 0.f;
+  int count = 0;
   for (int k = threadIdx.x; k < kp / 2; k += blockDim.x) {
     const double2 v = k < n ? entry(k) : make_double2(0.0, 0.0);
+    const float ur = oz_unit(v.x, e), ui = oz_unit(v.y, e);
+    sq += ur * ur + ui * ui;
+    count += (oz_key(v.x) | oz_key(v.y)) != 0;
     const oz_fix fr = oz_fixed(v.x, e), fi = oz_fixed(v.y, e);
 #pragma unroll
     for (int i = 0; i < OZ_S; ++i) out[i * digit + k] = oz_digit2(fr, fi, i);
@@ -422,6 +449,139 @@ __global__ void __launch_bounds__(256) oz_split_rows(const double2* __restrict__
       for (int i = 0; i < OZ_S; ++i) out[i * digit + kp / 2 + k] = oz_digit2(fm, fr, i);
     }
   }
+  const float2 v = block_norm(sq, count);
+  if (threadIdx.x == 0) norm[(size_t)b * rows + row] = v;
+}
+
+// two registers of interleaved (re, im) to one of two |re| + |im|
+__device__ __forceinline__ uint32_t abs_sum(uint32_t x, uint32_t y) {
+  const uint32_t re = __byte_perm(x, y, 0x5410) & 0x7fff7fffu, im = __byte_perm(x, y, 0x7632) & 0x7fff7fffu;
+  const __half2 s = __hadd2(*reinterpret_cast<const __half2*>(&re), *reinterpret_cast<const __half2*>(&im));
+  return *reinterpret_cast<const uint32_t*>(&s);
+}
+
+// Lists the elements (batch, r, r') of the product of rows A (pair = 0, batched)
+// and B (pair = 1, of the same vectors, so that the magnitudes' sum is the same
+// with r and r' exchanged: tiles on and below the diagonal only) whose magnitudes
+// do not cover the digits' error: sum |a| |b| from the leading digits on the
+// older tensor-core form (mma.sync m16n8k16 on |re| + |im|, K in any order as
+// long as both sides have it).  Tiles of 128 x 128, K blocks of 64 in three
+// buffers, a warp 64 x 32.  Part of the K blocks is enough for most: the first
+// launch takes every `step`-th, and only where that refuses more than the list
+// holds does a second one take them all (`after`: its count).  900 rows, 8192 K
+// elements, 16 batches: 0.29 ms with every fourth.
+constexpr int RF_T = 128, RF_S = 3, RF_BYTES = 2 * RF_T * 128;   // buffers, bytes of one: 128 rows of each operand
+struct OzRefused {
+  const __half *a, *b;              // digits [batch][7][nr][kp], [7][2 nr][kp]
+  const double *sa, *sb;            // scales [batch][nr], [2 nr]
+  const float2 *na, *nb;            // [batch][nr], [nr]
+  int nr, kp, mt;                   // rows, padded K, tiles per side
+  unsigned long long* list;
+  unsigned cap;
+  unsigned* count;
+  int step;
+  const unsigned* after;
+  int* bad;
+};
+__global__ void __launch_bounds__(256, 2) oz_gemm_refused(const OzRefused p) {
+  extern __shared__ __align__(128) unsigned char rf_sm[];
+  if (p.after && *p.after <= p.cap) return;
+  int m = (int)((sqrtf(8.f * blockIdx.x + 1.f) - 1.f) * 0.5f);   // row of the triangle
+  while ((m + 1) * (m + 2) / 2 <= (int)blockIdx.x) ++m;
+  while (m * (m + 1) / 2 > (int)blockIdx.x) --m;
+  const int q = blockIdx.x - m * (m + 1) / 2, bt = blockIdx.y;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wm = (warp & 1) * 64, wn = (warp >> 1) * 32;
+  const __half* a = p.a + (size_t)bt * OZ_S * p.nr * p.kp;
+  // 16-byte chunks: row of A or B, chunk of the K block, swizzled by the row
+  const int nkb = (p.kp / OZ_KB + p.step - 1) / p.step;
+  auto load = [&](int i0) {
+    const uint32_t base = smem_u32(rf_sm) + i0 % RF_S * RF_BYTES;
+#pragma unroll
+    for (int i = 0; i < 2 * RF_T * 8 / 256 && i0 < nkb; ++i) {
+      const int e = threadIdx.x + 256 * i, r = e >> 3, c = e & 7;
+      const __half* src = r < RF_T ? a + (size_t)min(m * RF_T + r, p.nr - 1) * p.kp
+                                   : p.b + (size_t)2 * min(q * RF_T + r - RF_T, p.nr - 1) * p.kp;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(base + r * 128 + ((c ^ (r & 7)) << 4)),
+                   "l"(src + (size_t)i0 * p.step * OZ_KB + c * 8)
+                   : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");   // empty past the end: the waits count groups
+  };
+  float c[4][4][4];
+#pragma unroll
+  for (int i = 0; i < 64; ++i) c[i >> 4][(i >> 2) & 3][i & 3] = 0.f;
+  load(0);
+  load(1);
+  for (int kb = 0; kb < nkb; ++kb) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();   // block kb is there, and every warp is done with kb - 1, whose buffer the next load takes
+    load(kb + 2);
+    const uint32_t base = smem_u32(rf_sm) + kb % RF_S * RF_BYTES;
+    auto ldm = [&](int row, int chunk, uint32_t* r) {
+      asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                   : "r"(base + row * 128 + ((chunk ^ (row & 7)) << 4)));
+    };
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {   // 32 K elements, 16 complex ones
+      uint32_t b[4][2];
+#pragma unroll
+      for (int nt = 0; nt < 4; nt += 2) {
+        const int row = RF_T + wn + nt * 8 + (lane & 7) + ((lane >> 4) << 3), ch = 4 * h + ((lane >> 3) & 1);
+        uint32_t x[4], y[4];
+        ldm(row, ch, x);
+        ldm(row, ch + 2, y);
+        b[nt][0] = abs_sum(x[0], x[1]), b[nt][1] = abs_sum(y[0], y[1]);
+        b[nt + 1][0] = abs_sum(x[2], x[3]), b[nt + 1][1] = abs_sum(y[2], y[3]);
+      }
+#pragma unroll
+      for (int mt = 0; mt < 4; ++mt) {
+        const int row = wm + mt * 16 + (lane & 15), ch = 4 * h + (lane >> 4);
+        uint32_t x[4], y[4];
+        ldm(row, ch, x);
+        ldm(row, ch + 2, y);
+        const uint32_t a0 = abs_sum(x[0], x[2]), a1 = abs_sum(x[1], x[3]), a2 = abs_sum(y[0], y[2]), a3 = abs_sum(y[1], y[3]);
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+          asm volatile(
+              "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, "
+              "%1, %2, %3};"
+              : "+f"(c[mt][nt][0]), "+f"(c[mt][nt][1]), "+f"(c[mt][nt][2]), "+f"(c[mt][nt][3])
+              : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b[nt][0]), "r"(b[nt][1]));
+      }
+    }
+  }
+  const double* sa = p.sa + (size_t)bt * p.nr;
+  const float2* na = p.na + (size_t)bt * p.nr;
+  // s: the sum in units of the scales of A's row r and B's row c
+  auto refused = [&](int r, int c2, float s) {
+    const float2 x = na[r], y = p.nb[c2];
+    return x.x != 0.f && y.x != 0.f && !oz_accept(s, fminf(x.x, y.y), fminf(y.x, x.y));
+  };
+  auto put = [&](int r, int c2) {
+    const unsigned at = atomicAdd(p.count, 1u);
+    if (at < p.cap)
+      p.list[at] = ((unsigned long long)bt << 32) | ((unsigned long long)r << 16) | (unsigned long long)c2;
+    else if (p.step == 1)
+      *p.bad = 1;
+  };
+#pragma unroll
+  for (int mt = 0; mt < 4; ++mt)
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = m * RF_T + wm + mt * 16 + (lane >> 2) + 8 * (i >> 1);
+        const int c2 = q * RF_T + wn + nt * 8 + 2 * (lane & 3) + (i & 1);
+        if (r >= p.nr || c2 >= p.nr) continue;
+        const float s = c[mt][nt][i] * 0x1p-14f;
+        if (refused(r, c2, s)) put(r, c2);
+        if (m != q) {   // the element across the diagonal: in other units, powers of two (FP64 divisions took 0.1 ms a launch)
+          auto ex = [](double v) { return __double2hiint(v) >> 20; };
+          const int u = ex(sa[r]) - ex(sa[c2]) + ex(p.sb[2 * c2]) - ex(p.sb[2 * r]);
+          if (refused(c2, r, s * __uint_as_float((uint32_t)(min(max(u, -126), 127) + 127) << 23))) put(c2, r);
+        }
+      }
 }
 
 // a load that stays where it stands: the compiler otherwise sinks the next
@@ -438,15 +598,10 @@ __device__ __forceinline__ double2 load_in_place(const double2* p) {
 // oz_split_rows with pair = 1, dig [8][2 np][kp]; with them its magnitudes max(|Re|,
 // |Im|) as BF16 in units of the row's scale, mag [np][kp / 2], the row's norm in
 // these units and 2^1/2 of its number of entries.  One block per function.
-struct __align__(8) OzNorm {
-  float norm, root;
-};
 __global__ void __launch_bounds__(256) oz_split_functions(const double2* __restrict__ f, int n, int np, int kp,
                                                           __half* __restrict__ dig, unsigned short* __restrict__ mag,
-                                                          double* __restrict__ scale, OzNorm* __restrict__ norm,
+                                                          double* __restrict__ scale, float2* __restrict__ norm,
                                                           int* __restrict__ bad) {
-  __shared__ float ws[8];
-  __shared__ int wc[8];
   const int row = blockIdx.x;
   const double2* x = f + (size_t)row * n;
   unsigned key = 0;
@@ -473,23 +628,13 @@ __global__ void __launch_bounds__(256) oz_split_functions(const double2* __restr
     const float ur = oz_unit(v.x, e), ui = oz_unit(v.y, e);
     mag[(size_t)row * (kp / 2) + k] = (unsigned short)(__float_as_uint(fmaxf(ur, ui)) >> 16);
     sq += ur * ur + ui * ui;
-    count += v.x != 0.0 || v.y != 0.0;
+    count += (oz_key(v.x) | oz_key(v.y)) != 0;
   }
-  for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
-  count = __reduce_add_sync(0xffffffffu, count);
-  if ((threadIdx.x & 31) == 0) {
-    ws[threadIdx.x >> 5] = sq;
-    wc[threadIdx.x >> 5] = count;
-  }
-  __syncthreads();
+  const float2 nr = block_norm(sq, count);
   if (threadIdx.x != 0) return;
-  for (int w = 1; w < 8; ++w) {
-    sq += ws[w];
-    count += wc[w];
-  }
   const double s = scalbn(1.0, e);
   scale[2 * row] = scale[2 * row + 1] = s;
-  norm[row] = OzNorm{sqrtf(sq), sqrtf(2.f * (float)count)};
+  norm[row] = nr;
   if (flag) atomicOr(bad, 1);
 }
 
@@ -595,7 +740,7 @@ struct OzRepair {
   const float* cover;
   const unsigned* keys;
   const int* expo;
-  const OzNorm* norm;
+  const float2* norm;   // of f's rows {norm, root}
   int parts, nk, nx, xp, nb, np, nkt, k0;
   double alpha;
   double2* out;
@@ -608,12 +753,12 @@ __global__ void __launch_bounds__(256) oz_refused(const OzRepair p, int* __restr
   bool refused = false;
   if (i < total) {
     const int n = (int)(i % p.nb), q = (int)(i / p.nb % p.np), k = (int)(i / p.nb / p.np);
-    const OzNorm f = p.norm[q];
-    if (f.norm > 0.f && p.keys[(size_t)k * p.nb + n]) {
+    const float2 f = p.norm[q];
+    if (f.x > 0.f && p.keys[(size_t)k * p.nb + n]) {
       float s = 0.f;
       for (int j = 0; j < p.parts; ++j) s += p.cover[j * total + i];
       s = ldexpf(s, first_exponent(p.u[(size_t)k * p.nx * p.nb + n]) - p.expo[(size_t)k * p.nb + n]);
-      refused = !(isfinite(s) && oz_accept(s, f.norm, f.root * 0x1p-8f));
+      refused = !(isfinite(s) && oz_accept(s, f.x, f.y * 0x1p-8f));
     }
   }
   const unsigned w = __ballot_sync(0xffffffffu, refused), lane = threadIdx.x & 31;
@@ -1034,7 +1179,7 @@ int bse_oz_kp(int k) { return (k + OZ_KB - 1) / OZ_KB * OZ_KB; }
 bse_status bse_oz_split_rows(const double2* x, int rows, int n, const double2* d, int batches, int pair,
                              const bse_oz_operand& o, int* bad, cudaStream_t st) {
   oz_split_rows<<<dim3((unsigned)rows, (unsigned)batches), 256, 0, st>>>(x, n, d, rows, o.kp, pair, (__half*)o.digits,
-                                                                          o.scale, bad);
+                                                                          o.scale, o.norm, bad);
   return cudaGetLastError() == cudaSuccess ? BSE_OK : BSE_ERR_CUDA;
 }
 
@@ -1071,7 +1216,7 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
   const size_t sd = bse_oz_digit_bytes(1, 2 * np, kp) / OZ_S * OZ_SF, sf = pad((size_t)2 * np * sizeof(double)), sph = pad(nkc * per);
   const size_t stab = pad((size_t)ntab * sizeof(double2)), skey = pad((size_t)nkc * nb * sizeof(unsigned));
   const size_t ssc = pad((size_t)nkc * nb * sizeof(double)), npart = (size_t)2 * sms * OZ_M * OZ_N;
-  const size_t smag = pad((size_t)np * (kp / 2) * sizeof(short)), snrm = pad((size_t)np * sizeof(OzNorm));
+  const size_t smag = pad((size_t)np * (kp / 2) * sizeof(short)), snrm = pad((size_t)np * sizeof(float2));
   const size_t scov = pad(nkc * pcov), cap = nkc * outs / 32 + 1024, slist = pad(cap * sizeof(unsigned));
   struct Scratch {
     void* p = nullptr;
@@ -1105,7 +1250,7 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
   p.part_lo = (uint32_t*)q, q += npart * 4;
   unsigned short* mag = (unsigned short*)q;
   q += smag;
-  OzNorm* norm = (OzNorm*)q;
+  float2* norm = (float2*)q;
   q += snrm;
   float* cover = (float*)q;
   q += scov;
@@ -1209,5 +1354,34 @@ bse_status bse_oz_gemm(const bse_oz_operand& a, const bse_oz_operand& b, int bat
     return BSE_ERR_UNSUPPORTED;
   }
   oz_gemm<<<std::min(p.ntiles, sms), OZ_THREADS, OZ_SMEM, st>>>(ma, mb, p);
+  return cudaGetLastError() == cudaSuccess ? BSE_OK : BSE_ERR_CUDA;
+}
+
+bse_status bse_oz_refused(const bse_oz_operand& a, const bse_oz_operand& b, int batches, unsigned long long* list,
+                          unsigned cap, unsigned* count, int* bad, cudaStream_t st) {
+  OzRefused p{};
+  p.a = (const __half*)a.digits, p.b = (const __half*)b.digits;
+  p.sa = a.scale, p.sb = b.scale;
+  p.na = a.norm, p.nb = b.norm;
+  p.nr = a.rows;
+  p.kp = a.kp;
+  p.mt = (a.rows + RF_T - 1) / RF_T;
+  p.list = list;
+  p.cap = cap;
+  p.bad = bad;
+  if (cudaFuncSetAttribute(oz_gemm_refused, cudaFuncAttributeMaxDynamicSharedMemorySize, RF_S * RF_BYTES) != cudaSuccess) {
+    cudaGetLastError();
+    return BSE_ERR_UNSUPPORTED;
+  }
+  // every fourth K block from 64 of them on (a random sum's magnitudes are then
+  // still some 20 times the limit)
+  cudaMemsetAsync(count, 0, 2 * sizeof(unsigned), st);
+  for (int all = 0; all < 2; ++all) {
+    p.step = all || a.kp < 64 * OZ_KB ? 1 : 4;
+    p.count = count + all;
+    p.after = all ? count : nullptr;
+    oz_gemm_refused<<<dim3((unsigned)(p.mt * (p.mt + 1) / 2), (unsigned)batches), 256, RF_S * RF_BYTES, st>>>(p);
+    if (p.step == 1) break;
+  }
   return cudaGetLastError() == cudaSuccess ? BSE_OK : BSE_ERR_CUDA;
 }

@@ -696,7 +696,7 @@ __device__ void record_column(bool fits, int e, float sq, int count, int* eb, HC
   cb->norm = fits ? sqrtf(sq) : -1.f;
   cb->root = sqrtf(2.f * (float)count);
 }
-__device__ __forceinline__ bool nonzero(double2 v) { return v.x != 0.0 || v.y != 0.0; }
+__device__ __forceinline__ bool nonzero(double2 v) { return (oz_key(v.x) | oz_key(v.y)) != 0; }   // FP64 compares: 2 per SM and clock
 
 // Digits of psi for band->grid, one block per (k, column): rows 2c = (psi_r,
 // -psi_i) and 2c + 1 = (psi_i, psi_r) along (n; re, im).  dig [k][7][H_J][kp]

@@ -9,6 +9,8 @@
 // memory, the diagonal applied while staging); chi0 is an element-wise pass.
 #include "bse_internal.cuh"
 
+#include <algorithm>
+
 namespace {
 
 constexpr int GT = 32, GK = 16;   // output tile GT x GT, K chunk GK; 256 threads, 4 outputs each
@@ -92,6 +94,29 @@ __global__ void green_weights(const double* __restrict__ eps, int nkk, double mu
   d[(size_t)blockIdx.y * nkk + K] = make_double2(x / den, -tj / den);
 }
 
+// G of the elements that bse_oz_refused lists (j << 32 | r << 16 | r'), one warp each
+__global__ void __launch_bounds__(256) green_repair(const double2* __restrict__ psi, const double2* __restrict__ d, int nr,
+                                                    int nkk, const unsigned long long* __restrict__ list, unsigned cap,
+                                                    const unsigned* __restrict__ count, double2* __restrict__ G) {
+  const unsigned m = count[0] <= cap ? count[0] : min(count[1], cap), lane = threadIdx.x & 31;
+  for (unsigned w = blockIdx.x * 8 + (threadIdx.x >> 5); w < m; w += gridDim.x * 8) {
+    const unsigned j = (unsigned)(list[w] >> 32), r = (unsigned)(list[w] >> 16) & 0xffffu, c = (unsigned)list[w] & 0xffffu;
+    const double2 *a = psi + (size_t)r * nkk, *b = psi + (size_t)c * nkk, *dj = d + (size_t)j * nkk;
+    double2 s = make_double2(0.0, 0.0);
+    for (int K = lane; K < nkk; K += 32) {
+      const double2 p = a[K], q = b[K], e = dj[K];
+      const double x = p.x * e.x - p.y * e.y, y = p.x * e.y + p.y * e.x;
+      s.x = fma(x, q.x, fma(y, q.y, s.x));
+      s.y = fma(y, q.x, fma(-x, q.y, s.y));
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+    }
+    if (lane == 0) G[((size_t)j * nr + r) * nr + c] = s;
+  }
+}
+
 struct Scratch {
   void* p = nullptr;
   ~Scratch() {
@@ -102,8 +127,9 @@ struct Scratch {
 // G_j on the tensor cores (k_oz.cu): the rows psi(r, :) d_j against the row
 // pairs of psi(r', :), as many frequencies per pass as the scratch holds.
 // *done = false (and nothing but G written) where the scratch or the kernel's
-// set-up cannot be had, psi d_j holds Inf/NaN or a magnitude outside 2^+-400, or
-// a bounded wait gave up.
+// set-up cannot be had, psi d_j holds Inf/NaN or a magnitude outside 2^+-400, a
+// bounded wait gave up, or more than one element in 32 of a pass is refused
+// (oz_accept; fewer are formed on the FP64 pipe).
 bse_status green_tensor(const double2* psi, const double* eps, int nr, int nkk, double mu, const double* t, int nt,
                         double2* G, cudaStream_t st, bool* done) {
   *done = false;
@@ -116,8 +142,11 @@ bse_status green_tensor(const double2* psi, const double* eps, int nr, int nkk, 
   const size_t tab = ((size_t)nt * nkk * sizeof(double2) + 255) / 256 * 256;
   const size_t sca = ((size_t)nj * nr * sizeof(double) + 255) / 256 * 256;
   const size_t scb = ((size_t)2 * nr * sizeof(double) + 255) / 256 * 256;
+  const size_t nma = ((size_t)nj * nr * sizeof(float2) + 255) / 256 * 256, nmb = ((size_t)nr * sizeof(float2) + 255) / 256 * 256;
+  const size_t cap = std::min<size_t>((size_t)nj * nr * nr / 32 + 1024, (size_t)1 << 22);
+  const size_t lst = (cap * sizeof(unsigned long long) + 255) / 256 * 256;
   Scratch sc;
-  if (cudaMalloc(&sc.p, bd + fixed + tab + sca + scb + 256) != cudaSuccess) {
+  if (cudaMalloc(&sc.p, bd + fixed + tab + sca + scb + nma + nmb + lst + 256) != cudaSuccess) {
     cudaGetLastError();
     sc.p = nullptr;
     return BSE_OK;
@@ -130,7 +159,11 @@ bse_status green_tensor(const double2* psi, const double* eps, int nr, int nkk, 
   q += tab;
   a.scale = (double*)q, q += sca;
   b.scale = (double*)q, q += scb;
-  int* word = (int*)q;   // {wait gave up, out of range}
+  a.norm = (float2*)q, q += nma;
+  b.norm = (float2*)q, q += nmb;
+  unsigned long long* list = (unsigned long long*)q;
+  q += lst;
+  int* word = (int*)q;   // {wait gave up, out of range or too many refused, elements refused (two)}
   a.rows = nr, b.rows = 2 * nr;
   a.kp = b.kp = kp;
   cudaMemsetAsync(word, 0, 2 * sizeof(int), st);
@@ -142,6 +175,10 @@ bse_status green_tensor(const double2* psi, const double* eps, int nr, int nkk, 
     s = bse_oz_split_rows(psi, nr, nkk, d + (size_t)j * nkk, n, 0, a, word + 1, st);
     if (s == BSE_OK)
       s = bse_oz_gemm(a, b, n, 1.0, (double*)(G + (size_t)j * nr * nr), 2ll * nr * nr, 4ll * nr, 2ll * nr, 1, word, st);
+    if (s == BSE_OK) s = bse_oz_refused(a, b, n, list, (unsigned)cap, (unsigned*)word + 2, word + 1, st);
+    if (s == BSE_OK)
+      green_repair<<<608, 256, 0, st>>>(psi, d + (size_t)j * nkk, nr, nkk, list, (unsigned)cap, (unsigned*)word + 2,
+                                        G + (size_t)j * nr * nr);
   }
   int hw[2] = {0, 0};
   if (s == BSE_OK && (cudaMemcpyAsync(hw, word, sizeof(hw), cudaMemcpyDeviceToHost, st) != cudaSuccess ||

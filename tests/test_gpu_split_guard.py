@@ -156,3 +156,61 @@ def test_projection_of_functions_of_any_scale(power):
     u, f = S.complex_normal(rng, (27, 1331, nb)), S.complex_normal(rng, (npj, 1331))
     a = bse.local_projection(u * 2.0 ** power, nk, nx, f * 2.0 ** -power, 0.3)
     assert np.array_equal(a, bse.local_projection(u, nk, nx, f, 0.3))
+
+
+# ---------------------------------------------------------------------------
+# Green's functions (csrc/k_oz.cu, csrc/k_screen.cu)
+# ---------------------------------------------------------------------------
+def green_case(nr, ns, nt, graded, decades, seed):
+    """`graded` points where psi falls off over the states, as many where it rises."""
+    psi, eps = S.screening_grid_states(nr, ns, seed=seed)
+    rise = 10.0 ** (-decades * np.linspace(0, 1, ns))
+    psi[:graded] *= rise
+    psi[-graded:] *= rise[::-1]
+    t = np.linspace(0.3, 5.0, nt)
+    return psi, eps, t, np.full(nt, 0.7)
+
+
+def green_bound(psi, eps, t):
+    d = 1 / np.abs(0.1234 + 1j * t[:, None] - eps[None])
+    return 2 * (psi.shape[1] + 16) * U64 * np.einsum("rs,js,qs->jrq", np.abs(psi), d, np.abs(psi), optimize=True)
+
+
+# few elements, more than one in 32, rows at and past the 128-row tile (both
+# sides of the diagonal), several K blocks and part of one
+@pytest.mark.parametrize("decades", [10, 18])
+@pytest.mark.parametrize("shape", [(129, 287, 3, 9), (256, 130, 1, 20), (300, 513, 2, 150), (140, 4001, 1, 5)])
+def test_green_functions_of_graded_states_keep_fp64_accuracy(shape, decades):
+    nr, ns, nt, graded = shape
+    psi, eps, t, w = green_case(nr, ns, nt, graded, decades, nr)
+    _, g = bse.screening_chi0(psi, eps, 0.1234, t, w, want_green=True)
+    assert np.all(np.abs(g - O.screening_green(psi, eps, 0.1234, t)) <= 2 * green_bound(psi, eps, t))
+
+
+def test_only_the_refused_green_functions_leave_the_tensor_cores(monkeypatch):
+    psi, eps, t, w = green_case(300, 513, 2, 3, 0, 11)
+    _, flat = bse.screening_chi0(psi, eps, 0.1234, t, w, want_green=True)
+    psi, eps, t, w = green_case(300, 513, 2, 3, 14, 11)
+    psi[50] = 0
+    psi[60, :300] = 0
+    psi[70, 300:] = 0
+    _, g = bse.screening_chi0(psi, eps, 0.1234, t, w, want_green=True)
+    monkeypatch.setenv("BSE_SPLIT_WAIT_NS", "1000")   # gives up: the FP64 kernel
+    _, fp64 = bse.screening_chi0(psi, eps, 0.1234, t, w, want_green=True)
+    rows = [r for r in range(3, 297) if r not in (50, 60, 70)]
+    same = np.ix_(range(2), rows, rows)
+    assert np.array_equal(g[same], flat[same]) and np.mean(g[same] == fp64[same]) < 0.1
+    assert np.all(g[:, 50] == 0) and np.all(g[:, :, 50] == 0) and np.all(g[:, 60, 70] == 0)
+    assert np.all(np.abs(g - O.screening_green(psi, eps, 0.1234, t)) <= 2 * green_bound(psi, eps, t))
+
+
+def test_green_functions_of_states_that_the_first_look_misses(monkeypatch):
+    """States with weight only where every fourth block of 32 is not: the look
+    at part of the magnitudes refuses everything, the one at all of them nothing."""
+    psi, eps, t, w = green_case(140, 2400, 1, 1, 0, 17)
+    psi[:, np.arange(2400) // 32 % 4 == 0] = 0
+    _, g = bse.screening_chi0(psi, eps, 0.1234, t, w, want_green=True)
+    monkeypatch.setenv("BSE_SPLIT_WAIT_NS", "1000")   # gives up: the FP64 kernel
+    _, fp64 = bse.screening_chi0(psi, eps, 0.1234, t, w, want_green=True)
+    assert np.mean(g == fp64) < 0.1
+    assert np.all(np.abs(g - O.screening_green(psi, eps, 0.1234, t)) <= 2 * green_bound(psi, eps, t))
