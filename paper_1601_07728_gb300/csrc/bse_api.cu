@@ -6,6 +6,8 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <map>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -44,6 +46,43 @@ bse_status bse_handle_malloc(bse_handle* h, void** p, size_t bytes, const char* 
   }
   h->dev_bytes += bytes;
   return BSE_OK;
+}
+
+namespace {
+std::mutex pool_mutex;
+std::map<int, cudaMemPool_t> pools;   // by device
+}  // namespace
+
+cudaMemPool_t bse_scratch_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  std::lock_guard<std::mutex> lock(pool_mutex);
+  auto it = pools.find(dev);
+  if (it != pools.end()) return it->second;
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  cudaMemPool_t pool = nullptr;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  // keep 256 MB; no stream is made to wait for another's release
+  unsigned long long keep = 256ull << 20;
+  int off = 0;
+  cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &off);
+  pools[dev] = pool;
+  return pool;
+}
+
+void bse_scratch_trim() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return;
+  std::lock_guard<std::mutex> lock(pool_mutex);
+  auto it = pools.find(dev);
+  if (it != pools.end()) cudaMemPoolTrimTo(it->second, 0);
 }
 
 bse_status bse_cuda_check(bse_handle* h, cudaError_t e, const char* what) {
@@ -237,6 +276,7 @@ bse_status bse_setup(bse_handle** out, const bse_system_desc* d) {
     free_handle(h);
     return BSE_ERR_CUDA;
   }
+  bse_scratch_trim();
   bse_status s = bse_setup_device(h, d);
   if (s != BSE_OK) {
     fprintf(stderr, "bse_setup: %s (%s)\n", h->err.c_str(), bse_status_string(s));

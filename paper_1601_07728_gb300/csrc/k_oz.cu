@@ -1183,9 +1183,9 @@ bse_status bse_oz_split_rows(const double2* x, int rows, int n, const double2* d
   return cudaGetLastError() == cudaSuccess ? BSE_OK : BSE_ERR_CUDA;
 }
 
-// The scratch holds the projectors' digits, the phases of as many k points per
-// pass as fit 256 MB, and the shared tiles' sums: 87 MB for 8^3 k x 16^3 points
-// (a gigabyte of Bloch digits took 1.0 ms to allocate and free).
+// The scratch holds the projectors' digits, the phases and magnitude sums of as
+// many k points per pass as fit 256 MB, and the shared tiles' sums: 128 MB for
+// 8^3 k x 16^3 points.
 bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb, const double* kshift,
                           const double2* f, int np, double dv, double2* a, cudaStream_t st, bool* done) {
   *done = false;
@@ -1218,18 +1218,8 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
   const size_t ssc = pad((size_t)nkc * nb * sizeof(double)), npart = (size_t)2 * sms * OZ_M * OZ_N;
   const size_t smag = pad((size_t)np * (kp / 2) * sizeof(short)), snrm = pad((size_t)np * sizeof(float2));
   const size_t scov = pad(nkc * pcov), cap = nkc * outs / 32 + 1024, slist = pad(cap * sizeof(unsigned));
-  struct Scratch {
-    void* p = nullptr;
-    ~Scratch() {
-      if (p) cudaFree(p);
-    }
-  } sc;
-  if (cudaMalloc(&sc.p, sd + sf + sph + stab + 2 * skey + ssc + npart * 12 + smag + snrm + scov + slist + 256) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    sc.p = nullptr;
-    return BSE_OK;
-  }
+  bse_scratch sc(st);
+  if (!sc.get(sd + sf + sph + stab + 2 * skey + ssc + npart * 12 + smag + snrm + scov + slist + 256)) return BSE_OK;
   char* q = (char*)sc.p;
   bse_oz_operand A;
   A.digits = q, q += sd;
@@ -1313,10 +1303,7 @@ bse_status bse_oz_project(const double2* u, const int* nk, const int* nx, int nb
   if (s == BSE_OK && (cudaMemcpyAsync(hw, word, sizeof(hw), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
                       cudaStreamSynchronize(st) != cudaSuccess))
     s = BSE_ERR_CUDA;
-  if (s != BSE_OK) {
-    cudaStreamSynchronize(st);   // before the scratch goes
-    return s;
-  }
+  if (s != BSE_OK) return s;
   *done = hw[0] == 0 && hw[1] == 0;
   return BSE_OK;
 }

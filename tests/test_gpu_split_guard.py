@@ -214,3 +214,25 @@ def test_green_functions_of_states_that_the_first_look_misses(monkeypatch):
     _, fp64 = bse.screening_chi0(psi, eps, 0.1234, t, w, want_green=True)
     assert np.mean(g == fp64) < 0.1
     assert np.all(np.abs(g - O.screening_green(psi, eps, 0.1234, t)) <= 2 * green_bound(psi, eps, t))
+
+
+def test_projection_of_device_arrays_waits_for_its_own_stream_only():
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(6)
+    u = torch.from_numpy(S.complex_normal(rng, (27, 1331, 64))).cuda()
+    f = torch.from_numpy(S.complex_normal(rng, (36, 1331))).cuda()
+    mine, other = torch.cuda.Stream(), torch.cuda.Stream()
+    done = torch.cuda.Event()
+
+    def call():
+        return bse.local_projection(u, (3, 3, 3), (11, 11, 11), f, 0.3, stream=mine.cuda_stream)
+
+    ref = call().clone()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(other):
+        torch.cuda._sleep(int(2e9))   # about a second
+        done.record()
+    out = call()
+    assert not done.query()
+    assert torch.equal(out, ref)
+    torch.cuda.synchronize()
