@@ -34,16 +34,25 @@ void bse_drop_graph(bse_handle* h) {
   for (auto& k : h->hay_key) k = 0;
 }
 
+bool bse_malloc(bse_handle* h, void** p, size_t bytes) {
+  if (bytes == 0) bytes = 16;
+  if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  bse_scratch_trim();
+  if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  if (h && bse_ozh_release(h) && cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  *p = nullptr;
+  return false;
+}
+
 bse_status bse_handle_malloc(bse_handle* h, void** p, size_t bytes, const char* what) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
   if (h->dev_cap && h->dev_bytes + bytes > h->dev_cap)
     return bse_fail(h, BSE_ERR_OOM, std::string("device memory cap reached allocating ") + what);
-  if (cudaMalloc(p, bytes) != cudaSuccess) {
-    *p = nullptr;
-    cudaGetLastError();
-    return bse_fail(h, BSE_ERR_OOM, std::string("cudaMalloc failed for ") + what);
-  }
+  if (!bse_malloc(h, p, bytes)) return bse_fail(h, BSE_ERR_OOM, std::string("cudaMalloc failed for ") + what);
   h->dev_bytes += bytes;
   return BSE_OK;
 }
@@ -132,11 +141,7 @@ bse_status stage_in(bse_handle* h, Staged& s, const void* p, size_t bytes, bool 
     s.dev = const_cast<void*>(p);
     return BSE_OK;
   }
-  if (cudaMalloc(&s.dev, bytes ? bytes : 16) != cudaSuccess) {
-    cudaGetLastError();
-    s.dev = nullptr;
-    return bse_fail(h, BSE_ERR_OOM, std::string("cudaMalloc failed staging ") + what);
-  }
+  if (!bse_malloc(h, &s.dev, bytes)) return bse_fail(h, BSE_ERR_OOM, std::string("cudaMalloc failed staging ") + what);
   s.owned = true;
   if (copy && bytes) return bse_cuda_check(h, cudaMemcpyAsync(s.dev, p, bytes, cudaMemcpyHostToDevice, h->stream), what);
   return BSE_OK;
@@ -298,6 +303,10 @@ bse_status bse_apply_h(bse_handle* h, const bse_c128* psi, bse_c128* hpsi, int n
   if (!psi || !hpsi || n_vec < 0) return bse_fail(h, BSE_ERR_INVALID_ARG, "apply_h: bad arguments");
   if (n_vec == 0) return BSE_OK;
   if ((const void*)psi == (void*)hpsi) return bse_fail(h, BSE_ERR_INVALID_ARG, "apply_h: psi and hpsi overlap");
+  if (h->ozh && !h->ozh_recorded) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (h->stream && cudaStreamIsCapturing(h->stream, &cs) == cudaSuccess) h->ozh_recorded = cs == cudaStreamCaptureStatusActive;
+  }
   const size_t bytes = (size_t)n_vec * h->N * sizeof(double2);
   const bool din = bse_is_device_ptr(psi), dout = bse_is_device_ptr(hpsi);
   if ((!din || !dout) && h->io_cap < bytes) {
@@ -305,10 +314,8 @@ bse_status bse_apply_h(bse_handle* h, const bse_c128* psi, bse_c128* hpsi, int n
     if (h->io_out) cudaFree(h->io_out);
     h->io_in = h->io_out = nullptr;
     h->io_cap = 0;
-    if (cudaMalloc(&h->io_in, bytes) != cudaSuccess || cudaMalloc(&h->io_out, bytes) != cudaSuccess) {
-      cudaGetLastError();
+    if (!bse_malloc(h, &h->io_in, bytes) || !bse_malloc(h, &h->io_out, bytes))
       return bse_fail(h, BSE_ERR_OOM, "apply_h: staging allocation failed");
-    }
     h->io_cap = bytes;
   }
   const double2* dp = din ? (const double2*)psi : (const double2*)h->io_in;

@@ -105,8 +105,12 @@ struct bse_handle {
   int op_max_vec = 0;          // one pass: largest n_vec it takes (0: none)
   bool concurrent = false;     // kernels of other handles may run beside this one's (many-site graph)
 
-  // tensor-core form of the FP64 contractions (k_ozh.cu), nullptr where not used
+  // tensor-core form of the FP64 contractions (k_ozh.cu), nullptr where not used;
+  // given back where another allocation fails (bse_malloc), unless a caller's own
+  // stream capture has recorded kernels that use it
   void* ozh = nullptr;
+  bool ozh_recorded = false;
+  bool gave_up = false;        // a bounded wait gave up in kernels whose error word is gone with it
 
   // grow-only device workspace of the Haydock driver (kept between calls)
   void* ws = nullptr;
@@ -151,7 +155,7 @@ bse_status bse_handle_malloc(bse_handle* h, void** p, size_t bytes, const char* 
 // its release does not wait for the work of other streams.  From a pool of the
 // library's own that keeps up to 256 MB between calls (mapping 128 MB anew took
 // 0.4 ms of a projection of 3.1) until bse_scratch_trim gives it back, at every
-// bse_setup.
+// bse_setup and where an allocation of the library fails.
 cudaMemPool_t bse_scratch_pool();   // of the current device; nullptr: none to be had
 void bse_scratch_trim();
 struct bse_scratch {
@@ -171,6 +175,11 @@ struct bse_scratch {
     return false;
   }
 };
+
+// cudaMalloc for a call over h (nullptr: over none): where the device is out of
+// memory, without the scratch pool's reserve and the handle's optional tables
+// before it fails.  Waits for the handle's stream in that case.
+bool bse_malloc(bse_handle* h, void** p, size_t bytes);
 
 // drop the cached Haydock graph (tiles, limits or buffers changed)
 void bse_drop_graph(bse_handle* h);
@@ -298,6 +307,7 @@ bool bse_apply_fuses_dot(const bse_handle* h);
 void bse_ozh_prepare(bse_handle* h);   // sets h->ozh where it applies
 bool bse_ozh_takes(const bse_handle* h, int nc);   // nc columns are worth its launches
 void bse_ozh_free(bse_handle* h);
+bool bse_ozh_release(bse_handle* h);   // free it before the handle goes; false where there is none, or it is recorded
 bse_status bse_ozh_band_to_grid(bse_handle* h, const double2* psi, int nc);
 bse_status bse_ozh_grid_to_band(bse_handle* h, const double2* psi, double2* hpsi, int nc);
 int* bse_ozh_word(const bse_handle* h);   // device error word of its kernels

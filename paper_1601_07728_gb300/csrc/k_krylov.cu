@@ -305,11 +305,7 @@ __global__ void copy_vecs(const double2* __restrict__ src, double2* __restrict__
 
 template <typename T>
 bse_status dalloc(bse_handle* h, T** p, size_t bytes, const char* what) {
-  if (cudaMalloc((void**)p, bytes ? bytes : 16) != cudaSuccess) {
-    cudaGetLastError();
-    *p = nullptr;
-    return bse_fail(h, BSE_ERR_OOM, std::string("cudaMalloc failed for ") + what);
-  }
+  if (!bse_malloc(h, (void**)p, bytes)) return bse_fail(h, BSE_ERR_OOM, std::string("cudaMalloc failed for ") + what);
   return BSE_OK;
 }
 

@@ -581,13 +581,8 @@ void bse_multi_dot(bse_handle* h, const double2* basis, long long vstride, long 
 namespace {
 
 template <typename T>
-bool dmalloc(T** p, size_t bytes) {
-  if (cudaMalloc((void**)p, bytes ? bytes : 16) != cudaSuccess) {
-    cudaGetLastError();
-    *p = nullptr;
-    return false;
-  }
-  return true;
+bool dmalloc(T** p, size_t bytes, bse_handle* h = nullptr) {
+  return bse_malloc(h, (void**)p, bytes);
 }
 
 void mlp_free(bse_mlp* m) {
@@ -608,7 +603,7 @@ bse_status ensure_rows(bse_handle* h, bse_mlp* m, size_t rows, Act* a) {
     if (m->act) cudaFree(m->act);
     m->act = nullptr;
     m->rows_cap = 0;
-    if (!dmalloc(&m->act, rows * per * sizeof(float))) return bse_fail(h, BSE_ERR_OOM, "mlp activations");
+    if (!dmalloc(&m->act, rows * per * sizeof(float), h)) return bse_fail(h, BSE_ERR_OOM, "mlp activations");
     m->rows_cap = rows;
   }
   float* p = m->act;
@@ -635,7 +630,7 @@ bse_status ensure_rows(bse_handle* h, bse_mlp* m, size_t rows, Act* a) {
 bse_status ensure_anorm(bse_handle* h) {
   if (h->mlp_anorm || h->np == 0) return BSE_OK;
   const int nkb = h->nk * h->nb;
-  if (!dmalloc(&h->mlp_anorm, (size_t)nkb * sizeof(float))) return bse_fail(h, BSE_ERR_OOM, "a_norm");
+  if (!dmalloc(&h->mlp_anorm, (size_t)nkb * sizeof(float), h)) return bse_fail(h, BSE_ERR_OOM, "a_norm");
   BSE_PROF(h, BSE_K_PREP, mlp_anorm<<<(nkb + 255) / 256, 256, 0, h->stream>>>(h->a_proj, h->np, nkb, h->mlp_anorm));
   return BSE_OK;
 }
@@ -748,15 +743,15 @@ bse_status ensure_probe(bse_handle* h, bse_mlp* m, size_t n) {
   if (m->probe) cudaFree(m->probe);
   m->probe = nullptr;
   m->probe_cap = 0;
-  if (!dmalloc(&m->probe, n * sizeof(double2))) return bse_fail(h, BSE_ERR_OOM, "probe buffers");
+  if (!dmalloc(&m->probe, n * sizeof(double2), h)) return bse_fail(h, BSE_ERR_OOM, "probe buffers");
   m->probe_cap = n;
   return BSE_OK;
 }
 
-bool grow(double2** buf, size_t* cap, size_t n) {
+bool grow(bse_handle* h, double2** buf, size_t* cap, size_t n) {
   if (*cap >= n) return true;
   double2* b = nullptr;
-  if (!dmalloc(&b, n * sizeof(double2))) return false;
+  if (!dmalloc(&b, n * sizeof(double2), h)) return false;
   cudaFree(*buf);
   *buf = b;
   *cap = n;
@@ -897,8 +892,8 @@ bse_status loss_grad_krylov(bse_handle* h, bse_mlp* m, double omega, double gamm
   const int per = (k + 1) * (k + 1);
   const int TT = k * T;
   cudaStreamSynchronize(st);   // the scratch below may be reallocated
-  if (!grow(&m->red, &m->red_cap, std::max((size_t)NRED * T * per, (size_t)NRED * TT * (RANK + 1))) ||
-      !grow(&m->stats, &m->stats_cap, (size_t)T * per + (size_t)T * KMAX + TT + 2 * (size_t)TT * (RANK + 1)))
+  if (!grow(h, &m->red, &m->red_cap, std::max((size_t)NRED * T * per, (size_t)NRED * TT * (RANK + 1))) ||
+      !grow(h, &m->stats, &m->stats_cap, (size_t)T * per + (size_t)T * KMAX + TT + 2 * (size_t)TT * (RANK + 1)))
     return bse_fail(h, BSE_ERR_OOM, "k-step loss scratch");
   double2* part = m->red;
   float2* pc = (float2*)a.dA;   // conj(p): the first N float2 of a scratch activation, free until backward
@@ -1119,8 +1114,8 @@ bse_status bse_mlp_loss_grad(bse_handle* h, bse_mlp* m, double omega, double gam
   const int n_pairs = n_probes;
   const long long N = h->N;
   float2 *p = nullptr, *u = nullptr, *v = nullptr;
-  if (!dmalloc(&p, (size_t)N * sizeof(float2)) || !dmalloc(&u, (size_t)N * RANK * sizeof(float2)) ||
-      !dmalloc(&v, (size_t)N * RANK * sizeof(float2))) {
+  if (!dmalloc(&p, (size_t)N * sizeof(float2), h) || !dmalloc(&u, (size_t)N * RANK * sizeof(float2), h) ||
+      !dmalloc(&v, (size_t)N * RANK * sizeof(float2), h)) {
     cudaFree(p);
     cudaFree(u);
     return bse_fail(h, BSE_ERR_OOM, "mlp_loss_grad scratch");
@@ -1130,10 +1125,10 @@ bse_status bse_mlp_loss_grad(bse_handle* h, bse_mlp* m, double omega, double gam
   if (s == BSE_OK)
     s = bse_cuda_check(h, cudaMemcpyAsync(grad, m->g, (size_t)NPARAM * sizeof(float), cudaMemcpyDefault, h->stream),
                        "grad copy");
-  if (s == BSE_OK) s = bse_cuda_check(h, cudaStreamSynchronize(h->stream), "grad sync");
   // the products with H may have given up a bounded wait: the gradient is then no result
   const bse_status t = bse_tc_status(h);
   if (t != BSE_OK) s = t;
+  if (s == BSE_OK) s = bse_cuda_check(h, cudaStreamSynchronize(h->stream), "grad sync");
   cudaMemsetAsync(m->g, 0, (size_t)NPARAM * sizeof(float), h->stream);
   cudaFree(p);
   cudaFree(u);
@@ -1206,10 +1201,10 @@ extern "C" bse_status bse_mlp_train(bse_handle* const* hs, const bse_c128* const
     double2 *bd = nullptr, *zd = nullptr, *x = nullptr, *hx = nullptr;
     int* it = nullptr;
     double* rr = nullptr;
-    if (!dmalloc(&bd, N * sizeof(double2)) || !dmalloc(&zd, n_z * sizeof(double2)) ||
-        !dmalloc(&x, (size_t)n_z * N * sizeof(double2)) || !dmalloc(&hx, (size_t)n_z * N * sizeof(double2)) ||
-        !dmalloc(&it, n_z * sizeof(int)) || !dmalloc(&rr, n_z * sizeof(double)) ||
-        !dmalloc(&R[s], (size_t)n_z * T * N * sizeof(double2))) {
+    if (!dmalloc(&bd, N * sizeof(double2), h) || !dmalloc(&zd, n_z * sizeof(double2), h) ||
+        !dmalloc(&x, (size_t)n_z * N * sizeof(double2), h) || !dmalloc(&hx, (size_t)n_z * N * sizeof(double2), h) ||
+        !dmalloc(&it, n_z * sizeof(int), h) || !dmalloc(&rr, n_z * sizeof(double), h) ||
+        !dmalloc(&R[s], (size_t)n_z * T * N * sizeof(double2), h)) {
       st = bse_fail(h, BSE_ERR_OOM, "training harvest");
     }
     if (st == BSE_OK) {

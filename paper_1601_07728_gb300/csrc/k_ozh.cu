@@ -940,6 +940,17 @@ void bse_ozh_free(bse_handle* h) {
   h->ozh = nullptr;
 }
 
+bool bse_ozh_release(bse_handle* h) {
+  if (!h->ozh || h->ozh_recorded) return false;
+  int e = 0;
+  cudaMemcpyAsync(&e, ((OzhState*)h->ozh)->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  if (cudaStreamSynchronize(h->stream) != cudaSuccess) return false;
+  h->gave_up = h->gave_up || e;
+  bse_drop_graph(h);   // its kernels use the tables
+  bse_ozh_free(h);
+  return true;
+}
+
 // phi[k][c][x] = sum_n U psi for every column
 bse_status bse_ozh_band_to_grid(bse_handle* h, const double2* psi, int nc) {
   OzhState* z = (OzhState*)h->ozh;

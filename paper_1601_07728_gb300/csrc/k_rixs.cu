@@ -93,11 +93,8 @@ extern "C" bse_status bse_rixs(bse_handle* core, bse_handle* val, const bse_c128
   const bool d_b = bse_is_device_ptr(b), d_z = bse_is_device_ptr(z_in), d_d = bse_is_device_ptr(d_em);
   DevBuf sb, sz, sd, sx, sy, sa, sbc, ss, si, sr;
   auto need = [&](DevBuf& buf, size_t bytes, const char* what) -> bse_status {
-    if (cudaMalloc(&buf.p, bytes ? bytes : 16) != cudaSuccess) {
-      cudaGetLastError();
-      buf.p = nullptr;
+    if (!bse_malloc(core, &buf.p, bytes) && !bse_malloc(val, &buf.p, bytes))
       return bse_fail(core, BSE_ERR_OOM, std::string("rixs: cudaMalloc failed for ") + what);
-    }
     return BSE_OK;
   };
   bse_status s = BSE_OK;

@@ -1528,6 +1528,10 @@ extern "C" bse_status bse_autotune(bse_handle* h, int n_vec, int reps, int* spli
 }
 
 bse_status bse_tc_status(bse_handle* h) {
+  if (h->gave_up) {
+    h->gave_up = false;
+    return bse_fail(h, BSE_ERR_TIMEOUT, "tensor-core pipeline wait timed out");
+  }
   int* word = nullptr;
   if (h->ozh)
     word = bse_ozh_word(h);

@@ -155,3 +155,60 @@ def test_set_up_calls_finish_where_a_wait_gives_up(monkeypatch, case):
     assert np.array_equal(f(), split)        # and left nothing behind
     for out in (split, fp64):
         assert np.abs(out - ref).max() <= 1e-13 * np.abs(ref).max()
+
+
+def _short_of_memory(torch, leave):
+    """All of the device's free memory but `leave` bytes, as an array that nothing touches."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.empty(torch.cuda.mem_get_info()[0] - leave, dtype=torch.uint8, device="cuda")
+
+
+def test_fp64_tables_make_room_for_a_krylov_basis():
+    """The FP64 form's tables (64 MB here) are optional: a basis (97 MB) that fits
+    the device's remaining 80 MB only without them is solved on the FP64 kernels."""
+    torch = pytest.importorskip("torch")
+    s = S.tiny_system(31, n_alpha=6, nk=(4, 4, 4), n_bands=64, nx=(16, 16, 16), n_proj=8)
+    b = S.make_start_vectors(s, 1)[0]
+    z = np.linspace(-3.0, 12.0, 8) + 1j
+    stream = torch.cuda.Stream()
+    h = bse.System(s, precision="fp64", max_vec=8, stream=stream.cuda_stream)
+    x, iters, rel_res, _ = h.gmres(b, z, rtol=1e-8, restart=30, max_iter=30, precond="jacobi")
+    a, bc, _, _ = h.haydock(b, 6)
+    hold = _short_of_memory(torch, 80 << 20)
+    try:
+        x2, iters2, _, _ = h.gmres(b, z, rtol=1e-8, restart=30, max_iter=30, precond="jacobi")
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert np.array_equal(iters, iters2) and np.abs(x2 - x).max() <= 1e-9 * np.abs(x).max()
+    assert rel(h.apply_h(b[None])[0], O.apply_h(s, b)) < 1e-14
+    a2, bc2, _, _ = h.haydock(b, 6)   # not the graph over the tables
+    np.testing.assert_allclose(a2, a, rtol=1e-11)
+    np.testing.assert_allclose(bc2, bc, rtol=1e-11)
+    h.close()
+
+
+def test_fp64_tables_of_a_callers_graph_stay():
+    torch = pytest.importorskip("torch")
+    s = S.tiny_system(31, n_alpha=6, nk=(4, 4, 4), n_bands=64, nx=(16, 16, 16), n_proj=8)
+    psi = torch.from_numpy(S.make_start_vectors(s, 1)).cuda()
+    stream = torch.cuda.Stream()
+    h = bse.System(s, precision="fp64", max_vec=8, stream=stream.cuda_stream)
+    ref, out = h.apply_h(psi, out=torch.empty_like(psi)), torch.empty_like(psi)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        h.apply_h(psi, out=out)
+    hold = _short_of_memory(torch, 80 << 20)
+    try:
+        with pytest.raises(bse.BSEError) as e:
+            h.gmres(psi[0].cpu().numpy(), np.linspace(-3.0, 12.0, 8) + 1j, rtol=1e-8, restart=30, max_iter=30)
+        assert e.value.status == bse.BSE_ERR_OOM
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref)
+    h.close()
