@@ -876,7 +876,10 @@ cudaError_t launch(const CUtensorMap& map, const HParams& p, int sms, cudaStream
 // Tables and buffers of the tensor-core contractions of an FP64 handle; without
 // them (small systems, U out of the scheme's range, no memory left for them)
 // the handle keeps the FP64 kernels.  Called last in the set-up.
+// The low part of a sum grows by at most 5.1 * 2^14 * 2^24 per K element: 2^22
+// points, and 2^21 bands, stay below 2^63.
 void bse_ozh_prepare(bse_handle* h) {
+  if (h->nx > (1 << 22) || h->nb > (1 << 21)) return;
   if (!split_is_faster(h, h->na) && !split_is_faster(h, h->na * h->max_vec)) return;
   OzhState* z = new (std::nothrow) OzhState();
   if (!z) return;
