@@ -73,16 +73,17 @@ bse_status bse_local_projection_device(const double2* u, const int* nk, const in
                                        const double2* f, int np, double dv, double2* a, cudaStream_t st) {
   const int nkt = nk[0] * nk[1] * nk[2];
   // Tensor-core form or FP64 kernel, from their times (us) as measured over 1 to
-  // 512 k, 512 to 13,824 points, 16 to 64 bands and 1 to 64 functions.  FP64: a
-  // block walks the grid, 152 of them at a time.  Tensor cores: scratch and
-  // launches, and 5.6 per K block of 32 points and SM.  (4^3 k, 8^3 points, 32
-  // bands, 9 functions: 344 us against 355; 2^3 k, 9^3, 27, 27: 475 against 325.)
-  // K is bounded by the 64-bit partial sums.
+  // 512 k, 125 to 13,824 points, 9 to 130 bands and 1 to 65 functions.  FP64: a
+  // block walks the grid, 152 of them at a time.  Tensor cores: launches, and 7.0
+  // per K block of 32 points and SM.  (4^3 k, 8^3 points, 32 bands, 9 functions:
+  // 343 us against 198; 8^3 k, 5^3, 9, 9: 289 against 265; 2^3 k, 9^3, 27, 27: 478
+  // against 167; 2^3 k, 16^3, 16, 16: 2440 against 218.)  K is bounded by the 64-bit
+  // partial sums.
   const double nxd = (double)nx[0] * nx[1] * nx[2];
   const double blocks = (double)nkt * ((nb + LN - 1) / LN) * ((np + LP - 1) / LP);
   const double tiles = (double)nkt * ((nb + 63) / 64) * ((2 * np + 127) / 128);
   const double fp64 = 50.0 + 0.585 * nxd * std::max(1.0, blocks / 152);
-  const double tensor = 320.0 + 5.6 * tiles * std::ceil(nxd / 32) / 152;
+  const double tensor = 165.0 + 7.0 * tiles * std::ceil(nxd / 32) / 152;
   if (tensor < fp64 && nxd <= 1048576.0) {
     bool done = false;
     const bse_status s = bse_oz_project(u, nk, nx, nb, kshift, f, np, dv, a, st, &done);

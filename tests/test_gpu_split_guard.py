@@ -236,3 +236,39 @@ def test_projection_of_device_arrays_waits_for_its_own_stream_only():
     assert not done.query()
     assert torch.equal(out, ref)
     torch.cuda.synchronize()
+
+
+# ---------------------------------------------------------------------------
+# the forms that calls take at the ends of the kernels' tiles
+# ---------------------------------------------------------------------------
+# grid rows at the 128-row tile, one short of it and one past it; enough k points
+# and bands for the tensor-core form
+@pytest.mark.parametrize("nx", [(127, 1, 1), (8, 4, 4), (3, 43, 1), (1, 5, 51), (4, 8, 8), (257, 1, 1)])
+def test_split_contractions_at_the_ends_of_a_row_tile(nx):
+    s = S.make_system_from(dict(id=972, n_alpha=6, nk=(5, 4, 4), n_bands=100, nx=nx, cell=7.4, eps=5.0, n_proj=4,
+                                so_split=5.7, m_scale=0.5, kshift=(0.1, 0.0, 0.2)), 1)
+    psi = S.make_start_vectors(s, 1)
+    h = bse.System(s, precision="fp64")
+    h.profile()
+    out = h.apply_h(psi)[0]
+    assert h.profile_read()["prep"][0] == 2   # digits of psi and phi: the split kernels
+    ref = O.apply_h(s, psi[0])
+    assert np.abs(out - ref).max() <= 1e-13 * np.abs(ref).max()
+    assert np.linalg.norm(out - ref) <= 1e-14 * np.linalg.norm(ref)
+
+
+# the shapes of test_gpu_split_products.py::test_projection_within_the_bound, and
+# CTAs that own several whole tiles of more than one band and function
+@pytest.mark.parametrize("shape", [((2, 2, 2), (9, 9, 9), 64, 64), ((3, 1, 2), (11, 8, 7), 65, 65),
+                                   ((5, 4, 4), (5, 7, 6), 33, 16), ((1, 1, 1), (16, 16, 16), 130, 9),
+                                   ((8, 8, 8), (5, 5, 5), 9, 9), ((8, 8, 8), (4, 5, 8), 17, 10)])
+def test_projections_that_take_the_split_kernel(monkeypatch, shape):
+    nk, nx, nb, npj = shape
+    n, m = int(np.prod(nk)), int(np.prod(nx))
+    rng = np.random.default_rng(npj * nb)
+    u, f = S.complex_normal(rng, (n, m, nb)), S.complex_normal(rng, (npj, m))
+    a = bse.local_projection(u, nk, nx, f, 0.37)
+    ref = O.local_projection(u, nk, nx, f, 0.37)
+    assert np.all(np.abs(a - ref) <= 2 * projection_bound(u, nk, f, 0.37))
+    monkeypatch.setenv("BSE_SPLIT_WAIT_NS", "1000")   # gives up: the FP64 kernel
+    assert np.mean(bse.local_projection(u, nk, nx, f, 0.37) == a) < 0.1
