@@ -362,38 +362,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   }
 }
 
-// block-wide maximum (blockDim.x <= 256); every thread returns it
-__device__ unsigned block_max(unsigned v) {
-  __shared__ unsigned wm[8];
-  v = __reduce_max_sync(0xffffffffu, v);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = v;
-  __syncthreads();
-  unsigned m = 0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, wm[w]);
-  return m;
-}
-
-// {norm, 2^1/2 of the number of entries} of a row from every thread's sum of
-// squares and count (blockDim.x <= 256); for thread 0
-__device__ float2 block_norm(float sq, int count) {
-  __shared__ float ws[8];
-  __shared__ int wc[8];
-  for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
-  count = __reduce_add_sync(0xffffffffu, count);
-  if ((threadIdx.x & 31) == 0) {
-    ws[threadIdx.x >> 5] = sq;
-    wc[threadIdx.x >> 5] = count;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-      sq += ws[w];
-      count += wc[w];
-    }
-  return make_float2(sqrtf(sq), sqrtf(2.f * (float)count));
-}
-
 // Digits of the rows of X [rows][n] (complex), one block per row and batch j;
 // with d != nullptr entry K of batch j is first multiplied by d[j][K].
 //   pair = 0: one row (re, im) per complex row, K = 2n interleaved
@@ -437,9 +405,8 @@ __global__ void __launch_bounds__(256) oz_split_rows(const double2* __restrict__
   int count = 0;
   for (int k = threadIdx.x; k < kp / 2; k += blockDim.x) {
     const double2 v = k < n ? entry(k) : make_double2(0.0, 0.0);
-    const float ur = oz_unit(v.x, e), ui = oz_unit(v.y, e);
-    sq += ur * ur + ui * ui;
-    count += (oz_key(v.x) | oz_key(v.y)) != 0;
+    sq += oz_unit_square(v, e);
+    count += oz_nonzero(v);
     const oz_fix fr = oz_fixed(v.x, e), fi = oz_fixed(v.y, e);
 #pragma unroll
     for (int i = 0; i < OZ_S; ++i) out[i * digit + k] = oz_digit2(fr, fi, i);
@@ -517,11 +484,7 @@ __global__ void __launch_bounds__(256, 2) oz_gemm_refused(const OzRefused p) {
     __syncthreads();   // block kb is there, and every warp is done with kb - 1, whose buffer the next load takes
     load(kb + 2);
     const uint32_t base = smem_u32(rf_sm) + kb % RF_S * RF_BYTES;
-    auto ldm = [&](int row, int chunk, uint32_t* r) {
-      asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                   : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                   : "r"(base + row * 128 + ((chunk ^ (row & 7)) << 4)));
-    };
+    auto ldm = [&](int row, int chunk, uint32_t* r) { ldmatrix_x4(base + row * 128 + ((chunk ^ (row & 7)) << 4), r); };
 #pragma unroll
     for (int h = 0; h < 2; ++h) {   // 32 K elements, 16 complex ones
       uint32_t b[4][2];
@@ -540,14 +503,9 @@ __global__ void __launch_bounds__(256, 2) oz_gemm_refused(const OzRefused p) {
         uint32_t x[4], y[4];
         ldm(row, ch, x);
         ldm(row, ch + 2, y);
-        const uint32_t a0 = abs_sum(x[0], x[2]), a1 = abs_sum(x[1], x[3]), a2 = abs_sum(y[0], y[2]), a3 = abs_sum(y[1], y[3]);
+        const uint32_t v[4] = {abs_sum(x[0], x[2]), abs_sum(x[1], x[3]), abs_sum(y[0], y[2]), abs_sum(y[1], y[3])};
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-          asm volatile(
-              "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, "
-              "%1, %2, %3};"
-              : "+f"(c[mt][nt][0]), "+f"(c[mt][nt][1]), "+f"(c[mt][nt][2]), "+f"(c[mt][nt][3])
-              : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b[nt][0]), "r"(b[nt][1]));
+        for (int nt = 0; nt < 4; ++nt) mma_16x8x16<false>(c[mt][nt], v, b[nt][0], b[nt][1]);
       }
     }
   }
@@ -582,14 +540,6 @@ __global__ void __launch_bounds__(256, 2) oz_gemm_refused(const OzRefused p) {
           if (refused(c2, r, s * __uint_as_float((uint32_t)(min(max(u, -126), 127) + 127) << 23))) put(c2, r);
         }
       }
-}
-
-// a load that stays where it stands: the compiler otherwise sinks the next
-// block's loads behind the waits, to their use
-__device__ __forceinline__ double2 load_in_place(const double2* p) {
-  double2 v;
-  asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
-  return v;
 }
 
 // Digits of the local functions' rows f [np][n], eight each (a function that
@@ -628,7 +578,7 @@ __global__ void __launch_bounds__(256) oz_split_functions(const double2* __restr
     const float ur = oz_unit(v.x, e), ui = oz_unit(v.y, e);
     mag[(size_t)row * (kp / 2) + k] = (unsigned short)(__float_as_uint(fmaxf(ur, ui)) >> 16);
     sq += ur * ur + ui * ui;
-    count += (oz_key(v.x) | oz_key(v.y)) != 0;
+    count += oz_nonzero(v);
   }
   const float2 nr = block_norm(sq, count);
   if (threadIdx.x != 0) return;
@@ -707,14 +657,8 @@ __global__ void __launch_bounds__(256) oz_cover(const double2* __restrict__ u, i
 #pragma unroll
           for (int mt = 0; mt < CV_P / 16; ++mt) {
             uint32_t a[4];
-            asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
-                         : "r"(smem_u32(&fs[(mt * 16 + (lane & 15)) * CV_LD + xs + 16 * h + (lane >> 4) * 8])));
-            asm volatile(
-                "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, "
-                "%1, %2, %3};"
-                : "+f"(c[mt][0]), "+f"(c[mt][1]), "+f"(c[mt][2]), "+f"(c[mt][3])
-                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+            ldmatrix_x4(smem_u32(&fs[(mt * 16 + (lane & 15)) * CV_LD + xs + 16 * h + (lane >> 4) * 8]), a);
+            mma_16x8x16<true>(c[mt], a, b0, b1);
           }
         }
       }

@@ -63,14 +63,6 @@ __device__ __forceinline__ unsigned long long sdesc_sw64(uint32_t saddr) {
   return d;
 }
 
-// a read-only load that stays where it is written: the compiler otherwise
-// sinks the next block's loads behind the waits, to their use
-__device__ __forceinline__ double2 load_in_place(const double2* p) {
-  double2 v;
-  asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
-  return v;
-}
-
 // (hi 2^32 + lo) 2^e: three FP64-pipe operations; the exponent is added to the
 // bits where the result stays a normal number
 __device__ __forceinline__ double h_value(long long hi, long long lo, int e) {
@@ -81,18 +73,10 @@ __device__ __forceinline__ double h_value(long long hi, long long lo, int e) {
   return __hiloint2double(h + (e << 20), __double2loint(v));
 }
 
-// a warp's 8 x 8 matrices of FP16 at the lanes' row addresses, as magnitudes
-__device__ __forceinline__ void ldmatrix4_abs(uint32_t a, uint32_t* r) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(a));
+__device__ __forceinline__ void ldmatrix4_abs(uint32_t a, uint32_t* r) {   // ... as magnitudes
+  ldmatrix_x4(a, r);
 #pragma unroll
   for (int i = 0; i < 4; ++i) r[i] &= 0x7fff7fffu;
-}
-__device__ __forceinline__ void mma_16x8x16(float* c, const uint32_t* a, const uint32_t* b) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
 // FP64 sums over i < n of u_i p_c,i for the H_C columns p_c = p + c cs (those
@@ -404,8 +388,8 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
             const int ar = w * 64 + mt * 16 + (lane & 15);
             uint32_t aq[4];
             ldmatrix4_abs(at + ar * 64 + (((2 * ks + (lane >> 4)) ^ ((ar >> 1) & 3)) << 4), aq);
-            mma_16x8x16(c[mt][0], aq, bq);
-            mma_16x8x16(c[mt][1], aq, bq + 2);
+            mma_16x8x16<false>(c[mt][0], aq, bq[0], bq[1]);
+            mma_16x8x16<false>(c[mt][1], aq, bq[2], bq[3]);
           }
         }
         __syncwarp();
@@ -592,11 +576,6 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
   }
 }
 
-// |v|^2 in units of 2^2e
-__device__ __forceinline__ float unit_square(double2 v, int e) {
-  const float x = oz_unit(v.x, e), y = oz_unit(v.y, e);
-  return x * x + y * y;
-}
 __device__ __forceinline__ float warp_sum(float v) {
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
   return v;
@@ -617,7 +596,7 @@ __global__ void __launch_bounds__(256) ozh_row_exponents(const double2* __restri
     int flag = 0;
     const int er = oz_exponent(key, &flag);
     float s = 0.f;
-    for (int n = lane; n < nb; n += 32) s += unit_square(u[(size_t)r * nb + n], er);
+    for (int n = lane; n < nb; n += 32) s += oz_unit_square(u[(size_t)r * nb + n], er);
     s = warp_sum(s);
     if (lane == 0) {
       e[r] = (short)er;
@@ -647,7 +626,7 @@ __global__ void __launch_bounds__(256) ozh_band_exponents(const double2* __restr
   const int en = oz_exponent(key, &flag);
   float s = 0.f;
   if (n < nb)
-    for (int x = g; x < nx; x += 8) s += unit_square(u[((size_t)k * nx + x) * nb + n], en);
+    for (int x = g; x < nx; x += 8) s += oz_unit_square(u[((size_t)k * nx + x) * nb + n], en);
   ss[g][threadIdx.x & 31] = s;
   __syncthreads();
   if (g == 0 && n < nb) {
@@ -667,37 +646,13 @@ __device__ __forceinline__ bool column_exponent(unsigned key, int* e) {
   *e = 0;
   return false;
 }
-__device__ unsigned block_key(unsigned v) {
-  __shared__ unsigned wm[8];
-  v = __reduce_max_sync(0xffffffffu, v);
-  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = v;
-  __syncthreads();
-  unsigned m = 0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, wm[w]);
-  return m;
-}
 // thread 0 records the column of exponent e from every thread's sum of squares and count of entries
 __device__ void record_column(bool fits, int e, float sq, int count, int* eb, HColumn* cb) {
-  __shared__ float ws[8];
-  __shared__ int wc[8];
-  sq = warp_sum(sq);
-  count = __reduce_add_sync(0xffffffffu, count);
-  if ((threadIdx.x & 31) == 0) {
-    ws[threadIdx.x >> 5] = sq;
-    wc[threadIdx.x >> 5] = count;
-  }
-  __syncthreads();
+  const float2 n = block_norm(sq, count);
   if (threadIdx.x != 0) return;
-  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-    sq += ws[w];
-    count += wc[w];
-  }
   *eb = e;
-  cb->norm = fits ? sqrtf(sq) : -1.f;
-  cb->root = sqrtf(2.f * (float)count);
+  *cb = HColumn{fits ? n.x : -1.f, n.y};
 }
-__device__ __forceinline__ bool nonzero(double2 v) { return (oz_key(v.x) | oz_key(v.y)) != 0; }   // FP64 compares: 2 per SM and clock
-
 // Digits of psi for band->grid, one block per (k, column): rows 2c = (psi_r,
 // -psi_i) and 2c + 1 = (psi_i, psi_r) along (n; re, im).  dig [k][7][H_J][kp]
 __global__ void __launch_bounds__(64) ozh_psi_digits(const double2* __restrict__ psi, int nk, int nb, int kp,
@@ -708,14 +663,14 @@ __global__ void __launch_bounds__(64) ozh_psi_digits(const double2* __restrict__
   unsigned key = 0;
   for (int n = threadIdx.x; n < nb; n += blockDim.x) key = max(key, max(oz_key(p[n].x), oz_key(p[n].y)));
   int e;
-  const bool fits = column_exponent(block_key(key), &e);
+  const bool fits = column_exponent(block_max(key), &e);
   float sq = 0.f;
   int count = 0;
   uint32_t* o = reinterpret_cast<uint32_t*>(dig) + ((size_t)k * OZ_S * H_J + 2 * c) * (kp / 2);
   for (int n = threadIdx.x; n < nb; n += blockDim.x) {
     const double2 v = p[n];
-    sq += unit_square(v, e);
-    count += nonzero(v);
+    sq += oz_unit_square(v, e);
+    count += oz_nonzero(v);
     const oz_fix fr = oz_fixed(v.x, e), fi = oz_fixed(v.y, e), fm = oz_fixed(-v.y, e);
 #pragma unroll
     for (int i = 0; i < OZ_S; ++i) {
@@ -740,14 +695,14 @@ __global__ void __launch_bounds__(256) ozh_phi_digits(const double2* __restrict_
     key = max(key, max(oz_key(v.x), oz_key(v.y)));
   }
   int e;
-  const bool fits = column_exponent(block_key(key), &e);
+  const bool fits = column_exponent(block_max(key), &e);
   float sq = 0.f;
   int count = 0;
   uint32_t* o = reinterpret_cast<uint32_t*>(dig) + ((size_t)k * OZ_S * H_J + 2 * c) * (kp / 2);
   for (int x = 2 * threadIdx.x; x < nx; x += 2 * blockDim.x) {
     const double2 v0 = p[x], v1 = x + 1 < nx ? p[x + 1] : make_double2(0.0, 0.0);
-    sq += unit_square(v0, e) + unit_square(v1, e);
-    count += nonzero(v0) + nonzero(v1);
+    sq += oz_unit_square(v0, e) + oz_unit_square(v1, e);
+    count += oz_nonzero(v0) + oz_nonzero(v1);
     const oz_fix r0 = oz_fixed(v0.x, e), r1 = oz_fixed(v1.x, e), i0 = oz_fixed(v0.y, e), i1 = oz_fixed(v1.y, e);
 #pragma unroll
     for (int i = 0; i < OZ_S; ++i) {

@@ -78,6 +78,13 @@ __device__ __forceinline__ float oz_unit(double x, int e) {
   return f <= 0 ? 0.f : __uint_as_float(((uint32_t)min(f, 254) << 23) | ((xh & 0xfffffu) << 3));
 }
 
+__device__ __forceinline__ float oz_unit_square(double2 v, int e) {   // |v|^2 in units of 2^2e
+  const float x = oz_unit(v.x, e), y = oz_unit(v.y, e);
+  return x * x + y * y;
+}
+// (FP64 compares would run at 2 per SM and clock)
+__device__ __forceinline__ bool oz_nonzero(double2 v) { return (oz_key(v.x) | oz_key(v.y)) != 0; }
+
 // Which sums the digits may stand for.  With every entry held to 2^-56 of its
 // row's scale, the error of a sum over k is about 0.58 * 2^-56 (|a|^2 + |b|^2)^1/2
 // in units of the two scales (|.| the norms of the two rows there), whatever the
@@ -123,6 +130,46 @@ __device__ __forceinline__ uint32_t oz_digit2(oz_fix f0, oz_fix f1, int i) {
   const uint32_t c = 0x64806480u;   // 1152 twice
   const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&w), *reinterpret_cast<const __half2*>(&c));
   return *reinterpret_cast<const uint32_t*>(&d);
+}
+
+// block-wide maximum (blockDim.x <= 256); every thread returns it
+__device__ unsigned block_max(unsigned v) {
+  __shared__ unsigned wm[8];
+  v = __reduce_max_sync(0xffffffffu, v);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = v;
+  __syncthreads();
+  unsigned m = 0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, wm[w]);
+  return m;
+}
+
+// {norm, 2^1/2 of the number of entries} of a row from every thread's sum of
+// squares and count (blockDim.x <= 256); for thread 0
+__device__ float2 block_norm(float sq, int count) {
+  __shared__ float ws[8];
+  __shared__ int wc[8];
+  for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+  count = __reduce_add_sync(0xffffffffu, count);
+  if ((threadIdx.x & 31) == 0) {
+    ws[threadIdx.x >> 5] = sq;
+    wc[threadIdx.x >> 5] = count;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
+      sq += ws[w];
+      count += wc[w];
+    }
+  return make_float2(sqrtf(sq), sqrtf(2.f * (float)count));
+}
+
+// a read-only load that stays where it is written: the compiler otherwise sinks
+// the next block's loads behind the waits, to their use
+__device__ __forceinline__ double2 load_in_place(const double2* p) {
+  double2 v;
+  asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
 }
 
 }  // namespace
