@@ -19,7 +19,7 @@
 // The digits hold an entry to 2^-56 of its row's largest, so every sum comes with
 // that of its magnitudes, and those for which this is not FP64 accuracy are
 // formed on the FP64 pipe (oz_accept; columns with Inf or NaN and columns below
-// 2^-960 wholly): band->grid's in the kernel, grid->band's in ozh_final.
+// 2^-960 wholly): band->grid's by ozh_repair, grid->band's in ozh_final.
 //
 // L2,3 workload (8^3 k, 16^3 grid, 64 bands, 6 columns): H psi 15.0 ms with the
 // FP64 kernels -> 2.88; of it band->grid 0.97, grid->band with the last sum 0.98,
@@ -81,7 +81,7 @@ __device__ __forceinline__ void ldmatrix4_abs(uint32_t a, uint32_t* r) {   // ..
 
 // FP64 sums over i < n of u_i p_c,i for the H_C columns p_c = p + c cs (those
 // from nc on repeat the first), by one warp: lane L returns part (L >> 1) & 1 of column L >> 2
-__device__ __noinline__ double warp_columns(const double2* __restrict__ u, const double2* __restrict__ p, size_t cs, int nc,
+__device__ double warp_columns(const double2* __restrict__ u, const double2* __restrict__ p, size_t cs, int nc,
                                             int n) {
   double v[2 * H_C];
 #pragma unroll
@@ -140,7 +140,8 @@ struct HParams {
   const float* na;        // mode 0: norm per grid row in units of its scale
   const int* eb;          // exponent per column: [nk][H_C]
   const HColumn* cb;      // mode 0: columns [nk][H_C]
-  const double2* psi;     // mode 0: this pass's columns of psi [c][nk][nb]
+  unsigned char* refused; // mode 0: [nk][nx], a bit per column whose sum is to come from the FP64 pipe
+  int* any;               // mode 0: set where there is one
   double2* out;           // mode 0: phi; mode 1: partial sums [split][nk][H_C][nb]
   float* sums;            // mode 1: sums of magnitudes, as out
   int nk, nx, nb, mt, nsplit, ntiles, kb, kb_per_split;
@@ -158,7 +159,7 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
   extern __shared__ unsigned char ozh_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)ozh_raw + 1023) & ~(uintptr_t)1023);
   unsigned long long* bars = (unsigned long long*)(sm + H_STAGES * OZ_S * H_A + H_BAREA);
-  uint32_t* tmem_slot = (uint32_t*)(bars + 3 * H_STAGES + 9);
+  uint32_t* tmem_slot = (uint32_t*)(bars + 3 * H_STAGES + 5);
   volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
   volatile int* issued = (volatile int*)(tmem_slot + 2);
   const uint32_t sbase = smem_u32(sm);
@@ -169,7 +170,6 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
   auto tfull = [&](int a) { return smem_u32(&bars[3 * H_STAGES + a]); };
   auto tempty = [&](int a) { return smem_u32(&bars[3 * H_STAGES + 2 + a]); };
   const uint32_t fin = smem_u32(&bars[3 * H_STAGES + 4]);
-  auto stored = [&](int a) { return smem_u32(&bars[3 * H_STAGES + 5 + a]); };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < H_STAGES; ++s) {
@@ -181,7 +181,6 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
       mbar_init(tfull(a), 1);
       mbar_init(tempty(a), 4);
     }
-    for (int a = 0; a < 4; ++a) mbar_init(stored(a), 4);
     mbar_init(fin, 1);
     *abort_flag = 0;
     *issued = 0;
@@ -274,9 +273,9 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
   } else if (warp < 6) {
     const int q = warp & 3, row = q * 32 + lane;
     const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16);
-    int chunk = 0, tiles = 0;
+    int chunk = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x, ++tiles) {
+    for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
       int k, m, sp, b0, b1;
       tile(t, k, m, sp, b0, b1);
       long long hi[H_J], lo[H_J];   // units 2^-38 (s <= 3) and 2^-70 (s = 4..7)
@@ -318,8 +317,6 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
                   make_double2(h_value(hi[2 * c], lo[2 * c], e), h_value(hi[2 * c + 1], lo[2 * c + 1], e));
             }
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(stored(tiles & 3));
       } else {
         double v[H_J];
         const int n = (m * H_M + row) >> 1;
@@ -351,9 +348,9 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
     // of 0.98 ms); their comparison with the norms there alone cost 0.23 ms.
     const int w = warp - (6 + H_CONV), br = (lane & 7) + ((lane >> 4) << 3);
     const int row0 = w * 64 + (lane >> 2);   // first of this lane's rows, 8 apart; its columns lane & 3 and 4 on
-    int it = 0, tiles = 0;
+    int it = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x, ++tiles) {
+    for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
       int k, m, sp, b0, b1;
       tile(t, k, m, sp, b0, b1);
       float c[4][2][4], na[8];
@@ -399,27 +396,22 @@ __global__ void __launch_bounds__(H_THREADS, 1) oz_contract(const __grid_constan
       // both parts of a complex column together, in units of the two scales
       auto sum = [&](int i, int nt) { return (c[i >> 1][nt][2 * (i & 1)] + c[i >> 1][nt][2 * (i & 1) + 1]) * 0x1p-14f; };
       if constexpr (MODE == 0) {
-        // bit i * 2 + nt: row row0 + 8 i, column (lane & 3) + 4 nt
-        unsigned refused = 0;
+        unsigned any = 0;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < 8; ++i) {
+          const int x = m * H_M + row0 + 8 * i;
+          unsigned f = 0;
 #pragma unroll
           for (int nt = 0; nt < 2; ++nt)
-            if (!column_accepts(cb[nt], na[i], sum(i, nt)) && m * H_M + row0 + 8 * i < p.nx) refused |= 1u << (2 * i + nt);
-        if (!__any_sync(0xffffffffu, refused)) continue;
-        // Those of FP64, over what the draining warps store.  They may be three
-        // tiles ahead (of one stage each), hence four barriers.
-        ok = __all_sync(0xffffffffu, mbar_wait(stored(tiles & 3), (uint32_t)(tiles >> 2) & 1u, abort_flag, p.wait_ns));
-        if (!ok) break;
-        for (int i = 0; i < 64; ++i) {
-          const unsigned f = __shfl_sync(0xffffffffu, refused, 4 * (i & 7) + ((lane >> 2) & 3)) >> (2 * (i >> 3) + (lane >> 4));
-          if (!__any_sync(0xffffffffu, f & 1u)) continue;
-          const int x = m * H_M + w * 64 + i, col = lane >> 2;
-          const double v = warp_columns(p.u + ((size_t)k * p.nx + x) * p.nb, p.psi + (size_t)k * p.nb, (size_t)p.nk * p.nb,
-                                        p.ncc, p.nb);
-          if ((lane & 1) == 0 && (f & 1u))
-            reinterpret_cast<double*>(p.out + ((size_t)k * p.nc + p.c0 + col) * p.nx + x)[(lane >> 1) & 1] = v;
+            if (!column_accepts(cb[nt], na[i], sum(i, nt))) f |= 1u << ((lane & 3) + 4 * nt);
+          f |= __shfl_xor_sync(0xffffffffu, f, 1);
+          f |= __shfl_xor_sync(0xffffffffu, f, 2);
+          if (x < p.nx) {
+            any |= f;
+            if ((lane & 3) == 0) p.refused[(size_t)k * p.nx + x] = (unsigned char)f;
+          }
         }
+        if (any) *p.any = 1;
       } else {
         // rows 2n and 2n + 1 (lanes 4 apart) are the parts of band n
         const size_t o = ((size_t)sp * p.nk + k) * H_C * p.nb;
@@ -581,6 +573,27 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// The sums of band->grid that oz_contract refuses, on the FP64 pipe: a warp looks
+// at 32 grid rows and forms all columns of one at a time.  3 us where there are
+// none; all 12.6 million of the L2,3 workload 9 ms (28 by the two warps of
+// oz_contract that sum the magnitudes).
+__global__ void __launch_bounds__(256) ozh_repair(const HParams p, const double2* __restrict__ psi) {
+  if (!*p.any) return;
+  const int lane = threadIdx.x & 31;
+  const long long rows = (long long)p.nk * p.nx;
+  for (long long r0 = 32ll * (blockIdx.x * 8 + (threadIdx.x >> 5)); r0 < rows; r0 += 32ll * 8 * gridDim.x) {
+    const unsigned mine = r0 + lane < rows ? p.refused[r0 + lane] : 0;
+    for (unsigned w = __ballot_sync(0xffffffffu, mine != 0); w; w &= w - 1) {
+      const long long r = r0 + __ffs(w) - 1;
+      const unsigned f = __shfl_sync(0xffffffffu, mine, __ffs(w) - 1);
+      const int k = (int)(r / p.nx), x = (int)(r % p.nx), c = lane >> 2;
+      const double v = warp_columns(p.u + r * p.nb, psi + (size_t)k * p.nb, (size_t)p.nk * p.nb, p.ncc, p.nb);
+      if ((lane & 1) == 0 && (f >> c & 1))
+        reinterpret_cast<double*>(p.out + ((size_t)k * p.nc + p.c0 + c) * p.nx + x)[(lane >> 1) & 1] = v;
+    }
+  }
+}
+
 // exponent and norm (in units of 2^exponent) of every grid row (k, x) over its bands: one warp per row
 __global__ void __launch_bounds__(256) ozh_row_exponents(const double2* __restrict__ u, long long rows, int nb,
                                                          short* __restrict__ e, float* __restrict__ norm,
@@ -657,8 +670,9 @@ __device__ void record_column(bool fits, int e, float sq, int count, int* eb, HC
 // -psi_i) and 2c + 1 = (psi_i, psi_r) along (n; re, im).  dig [k][7][H_J][kp]
 __global__ void __launch_bounds__(64) ozh_psi_digits(const double2* __restrict__ psi, int nk, int nb, int kp,
                                                      __half* __restrict__ dig, int* __restrict__ eb,
-                                                     HColumn* __restrict__ cb) {
+                                                     HColumn* __restrict__ cb, int* __restrict__ any) {
   const int k = blockIdx.x, c = blockIdx.y;
+  if (k == 0 && c == 0 && threadIdx.x == 0) *any = 0;   // refused sums of the pass that follows
   const double2* p = psi + ((size_t)c * nk + k) * nb;
   unsigned key = 0;
   for (int n = threadIdx.x; n < nb; n += blockDim.x) key = max(key, max(oz_key(p[n].x), oz_key(p[n].y)));
@@ -714,8 +728,7 @@ __global__ void __launch_bounds__(256) ozh_phi_digits(const double2* __restrict_
 }
 
 // out[c][k][n] = sum_split part + E psi - sum_b chi psi_b + short-range out, FP64.
-// Sums over the grid that the digits may not stand for are formed here again,
-// one warp each.
+// Sums over the grid that the digits may not stand for are formed here again.
 struct HFinal {
   const double2 *part, *psi;
   double2* out;
@@ -744,7 +757,22 @@ __global__ void __launch_bounds__(256) ozh_final(const HFinal p) {
       m += p.sums[o];
     }
     const bool good = column_accepts(p.cb[(size_t)k * H_C + cc], p.norm[kn], m);
-    for (unsigned w = __ballot_sync(0xffffffffu, in && !good); w; w &= w - 1) {
+    unsigned w = __ballot_sync(0xffffffffu, in && !good);
+    if (__popc(w) >= 8) {   // many of a warp's bands: each lane its own, u read along the bands
+      if (in && !good) {
+        const double2 *u = p.u + (size_t)k * p.nx * p.nb + n, *f = p.phi + ((size_t)k * p.nc + c) * p.nx;
+        lr = make_double2(0.0, 0.0);
+#pragma unroll 8
+        for (int x = 0; x < p.nx; ++x) {
+          const double2 q = u[(size_t)x * p.nb], b = f[x];
+          lr.x = fma(q.x, b.x, fma(q.y, b.y, lr.x));
+          lr.y = fma(q.x, b.y, fma(-q.y, b.x, lr.y));
+        }
+      }
+      w = 0;
+      __syncwarp();
+    }
+    for (; w; w &= w - 1) {   // else one at a time, lanes along the grid
       const int r = __ffs(w) - 1;
       const int kr = __shfl_sync(0xffffffffu, k, r), nr = __shfl_sync(0xffffffffu, n, r), cr = __shfl_sync(0xffffffffu, c, r);
       const double2 t = warp_dot(p.u + (size_t)kr * p.nx * p.nb + nr, p.nb, p.phi + ((size_t)kr * p.nc + cr) * p.nx, p.nx);
@@ -786,18 +814,19 @@ struct OzhState {
   short *ex = nullptr, *en = nullptr;           // exponents of U per grid row and per band
   int *epsi = nullptr, *ephi = nullptr;         // exponents of the columns, [nk][H_C]
   __half *dpsi = nullptr, *dphi = nullptr;      // digits, [nk][7][H_J][kp]
+  unsigned char* refused = nullptr;             // [nk][nx], band->grid
   float *nx = nullptr, *nn = nullptr;           // norms of U's rows and bands in units of their scales
   HColumn *cpsi = nullptr, *cphi = nullptr;     // the columns, [nk][H_C]
   double2* part = nullptr;                      // [nsplit][nk][H_C][nb]
   float* sums = nullptr;                        // their sums of magnitudes
-  int* err = nullptr;
+  int* err = nullptr;                           // {wait gave up, U out of range, sums refused}
   CUtensorMap mpsi, mphi;
   int kp = 0, kpx = 0, nsplit = 1, sms = 0;
 };
 
 void free_state(OzhState* z) {
   void* ptrs[] = {z->ex,   z->en,   z->epsi, z->ephi, z->dpsi, z->dphi, z->nx,
-                  z->nn, z->cpsi, z->cphi, z->part, z->sums, z->err};
+                  z->nn, z->cpsi, z->cphi, z->part, z->sums, z->refused, z->err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete z;
@@ -857,6 +886,7 @@ void bse_ozh_prepare(bse_handle* h) {
               {(void**)&z->ephi, nk * H_C * sizeof(int)},
               {(void**)&z->dpsi, bpsi},
               {(void**)&z->dphi, bphi},
+              {(void**)&z->refused, nk * h->nx},
               {(void**)&z->nx, nk * h->nx * sizeof(float)},
               {(void**)&z->nn, nk * h->nb * sizeof(float)},
               {(void**)&z->cpsi, nk * H_C * sizeof(HColumn)},
@@ -918,6 +948,8 @@ bse_status bse_ozh_band_to_grid(bse_handle* h, const double2* psi, int nc) {
   p.na = z->nx;
   p.eb = z->epsi;
   p.cb = z->cpsi;
+  p.refused = z->refused;
+  p.any = z->err + 2;
   p.out = (double2*)h->phi;
   p.nk = h->nk, p.nx = h->nx, p.nb = h->nb;
   p.mt = (h->nx + H_M - 1) / H_M;
@@ -931,13 +963,14 @@ bse_status bse_ozh_band_to_grid(bse_handle* h, const double2* psi, int nc) {
   for (int c0 = 0; c0 < nc && e == cudaSuccess; c0 += H_C) {
     p.c0 = c0;
     p.ncc = std::min(H_C, nc - c0);
-    p.psi = psi + (size_t)c0 * h->nk * h->nb;
+    const double2* pc = psi + (size_t)c0 * h->nk * h->nb;
     BSE_PROF(h, BSE_K_PREP,
              ozh_psi_digits<<<dim3((unsigned)h->nk, (unsigned)p.ncc), 64, 0, h->stream>>>(
-                 p.psi, h->nk, h->nb, z->kp, z->dpsi, z->epsi, z->cpsi));
+                 pc, h->nk, h->nb, z->kp, z->dpsi, z->epsi, z->cpsi, p.any));
     BSE_PROF(h, BSE_K_BAND_TO_GRID, e = launch<0>(z->mpsi, p, z->sms, h->stream));
+    BSE_PROF(h, BSE_K_BAND_TO_GRID, ozh_repair<<<(unsigned)(8 * z->sms), 256, 0, h->stream>>>(p, pc));
   }
-  return bse_cuda_check(h, e, "band->grid (split FP64)");
+  return bse_cuda_check(h, e == cudaSuccess ? cudaGetLastError() : e, "band->grid (split FP64)");
 }
 
 // out = grid->band of phi + diagonal, spin-orbit and short-range terms

@@ -16,15 +16,15 @@ pytestmark = pytest.mark.gpu
 U64 = 2.0 ** -53
 
 
-def graded_system(nk, nx, nb, na, npj, decades, ks=(0.0, 0.0, 0.0), seed=1):
-    """Two groups of bands, each `decades` smaller on the other's half of the grid."""
+def graded_system(nk, nx, nb, na, npj, decades, ks=(0.0, 0.0, 0.0), seed=1, every=2):
+    """Two groups of bands (each `every`-th one, the rest), each `decades` smaller on the other's half of the grid."""
     s = S.make_system_from(dict(id=971, n_alpha=na, nk=nk, n_bands=nb, nx=nx, cell=7.4, eps=5.0, n_proj=npj,
                                 so_split=5.7, m_scale=0.5, kshift=ks), seed)
     s.chi = np.zeros_like(s.chi)   # no coupling that would lift the small entries
     if npj:
         s.a_proj = s.a_proj * 0.0
     half = np.arange(s.n_x) < s.n_x // 2
-    group = np.arange(nb) % 2 == 0
+    group = np.arange(nb) % every == 0
     s.u = s.u * np.where(half[:, None] == group[None, :], 1.0, 10.0 ** -decades)
     return s, group
 
@@ -53,6 +53,16 @@ def test_graded_bands_keep_fp64_accuracy(case, decades):
     out = bse.System(s, precision="fp64", max_vec=nv).apply_h(psi)
     for v in range(nv):
         assert np.all(np.abs(out[v] - O.apply_h(s, psi[v])) <= 2 * apply_bound(s, psi[v]))
+
+
+def test_few_graded_bands_keep_fp64_accuracy():
+    """One band in 24: grid->band's sums are formed again one at a time, not by warps."""
+    s, group = graded_system((2, 2, 1), (13, 10, 10), 150, 6, 0, 12, every=24)
+    rng = np.random.default_rng(24)
+    for part in (group, ~group):
+        psi = (S.complex_normal(rng, (1, 6, s.n_k, 150)) * part).reshape(1, -1)
+        out = bse.System(s, precision="fp64").apply_h(psi)[0]
+        assert np.all(np.abs(out - O.apply_h(s, psi[0])) <= 2 * apply_bound(s, psi[0]))
 
 
 def test_sparse_real_and_empty_columns():
