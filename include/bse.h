@@ -128,8 +128,10 @@ long long bse_dim(const bse_handle* h);
 
 /* hpsi[v] = H psi[v] for v < n_vec, both [n_vec][N] complex128.  psi and hpsi
  * must not overlap.  Returns when the result is in hpsi (host) or enqueued on
- * the handle's stream (device output).  One call = n_vec matrix-vector
- * products (Eq. 9). */
+ * the handle's stream (device output: a bounded wait that gives up under it,
+ * see bse_set_wait_limit, is then reported by the handle's next call with host
+ * output or over a whole solve, whose own outputs are to be computed again).
+ * One call = n_vec matrix-vector products (Eq. 9). */
 bse_status bse_apply_h(bse_handle* h, const bse_c128* psi, bse_c128* hpsi, int n_vec);
 
 /* Haydock recursion (Sec. 3.2, Eq. 9) started from b[v] ([n_vec][N]):

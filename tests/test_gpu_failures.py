@@ -212,3 +212,20 @@ def test_fp64_tables_of_a_callers_graph_stay():
     torch.cuda.synchronize()
     assert torch.equal(out, ref)
     h.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "split_bf16"])
+def test_a_wait_that_gave_up_under_a_device_output_is_reported_by_the_next_call(l23, precision):
+    torch = pytest.importorskip("torch")
+    s, psi, ref = l23
+    stream = torch.cuda.Stream()
+    sysg = bse.System(s, precision=precision, stream=stream.cuda_stream)
+    p = torch.from_numpy(psi).cuda()
+    out = torch.empty_like(p)
+    torch.cuda.synchronize()
+    sysg.set_wait_limit(2e-6)
+    sysg.apply_h(p, out=out)
+    sysg.set_wait_limit(2.0)
+    _raises_timeout(sysg.haydock, psi[0], 2)
+    assert rel(sysg.apply_h(psi)[0], ref[0]) < (1e-13 if precision == "fp64" else 1e-5)
+    sysg.close()
