@@ -80,10 +80,13 @@ __device__ __forceinline__ bool oz_wait(uint32_t a, uint32_t parity, volatile in
 // Chunks of 128 K elements.  The accumulators s = 4, 5 hold one chunk's sums
 // (at most 6 * 128 * 2^14 < 2^24), s = 2, 3 two and s = 0, 1 four (4 * 256 and
 // 2 * 512 times 2^14): c counts the chunks of a tile, `last` its last one.
-// s = 6, 7 are kept for 32: past 2^24 (random digits stay below) an addition of
-// 16 K elements is rounded by 2^-24 of the sum so far, which weighs 2^-48 of the
-// whole: all of them by less than 2^-49 of 7 sum |a| |b| even if every digit were
-// at its largest, and 7 * 4096 * 2^14 < 2^31 still converts to an integer.
+// s = 6, 7 are kept for 32 (7 * 4096 * 2^14 < 2^31 still converts to an integer).
+// Past 2^24 an addition of 16 K elements is rounded, by up to 2^-23 of the sum so
+// far.  Digits of random signs stay below (2^20 after 4096 elements).  If all of
+// K elements' digits were at their largest with one sign, the 56 * 32 additions
+// until a drain, at half of 7 * 4096 * 2^14 on average, would add up to K 2^-58
+// in units of the two scales: at most K 2^-55 sum |a| |b| for an accepted sum (a
+// tenth and more), a quarter of what K roundings of an FP64 sum may add.
 // Draining costs as much as converting u (float to integer runs at 16 per SM and
 // clock): all seven of s < 7 after every chunk 12.9 ms for the Green's functions
 // below, s >= 4 after every chunk 12.4 (with s = 7 13.0), as it is 12.2; oz_project
