@@ -9,7 +9,7 @@
 // Green's functions of 900 points, 4096 states and 16 frequencies 682 ms
 // (FP64 kernel) -> 13.6 ms (this one 12.2, writing the digits 0.97, magnitudes 0.29); the
 // projection of 8^3 k x 16^3 points x 64 bands onto 64 functions 102.6 ms ->
-// 5.4 ms with the Bloch functions' digits in memory -> 3.0 ms with the digits
+// 5.4 ms with the Bloch functions' digits in memory -> 3.2 ms with the digits
 // made on the way into shared memory (oz_project 2.55, scales and magnitudes
 // 0.38).  The error against 64 bits fell from 1.9e-15 to 1.4e-15 and from 1.4e-15
 // to 0.7e-15.  What bounds oz_gemm now: operand tiles from L2 (35 bytes per SM and
@@ -835,9 +835,9 @@ __device__ __forceinline__ void oz_store(const OzProject& p, int t, int row, int
 // columns each).  A chunk is drained after the first block of the next one is
 // converted, so that the tensor core has that block while they drain.  The
 // phases' products (4 FP64 operations per complex entry: 4096 clocks a block at
-// two per SM and clock) run beside the digit products' 4864 clocks; a block
-// takes about 10,700, in which the 16 warps' FP64, integer and load phases
-// overlap only in part (FP64 pipe 41 %, tensor pipe 47 %).  With conversion and
+// two per SM and clock) run beside the digit products' 5120 clocks; a block
+// takes about 11,300, in which the 16 warps' FP64, integer and load phases
+// overlap only in part (FP64 pipe 39 %, tensor pipe 47 %).  With conversion and
 // draining on warps of their own (eight each) it was 12,300.
 // The CTAs take equal shares of all tiles' chunks; sums of a tile that two or more share
 // go to part_hi and part_lo, exact as they are, and oz_join adds them.

@@ -22,9 +22,11 @@
 // 2^-960 wholly): band->grid's by ozh_repair, grid->band's in ozh_final.
 //
 // L2,3 workload (8^3 k, 16^3 grid, 64 bands, 6 columns): H psi 15.0 ms with the
-// FP64 kernels -> 2.88; of it band->grid 0.97, grid->band with the last sum 0.98,
-// digits of psi and phi 0.13, k-transform 1.08 (with the magnitude sums left out
-// 0.98, 0.96 and 0.13; 2.85 in all).
+// FP64 kernels -> 2.86 in calls that follow one another on several streams (2.84
+// with the magnitude sums left out); 3.15 by itself, of it the k-transform 1.08,
+// oz_contract 0.92 and 0.90, digits of psi and phi 0.12, ozh_final 0.07.  What
+// bounds oz_contract: the integer instructions that make digits (ALU pipe 68 and
+// 78 % of active cycles, tensor pipe 24 and 29 %, DRAM 32 and 37 %).
 #include "bse_internal.cuh"
 #include "oz_dev.cuh"
 #include "tc_ptx.cuh"

@@ -105,7 +105,7 @@ __device__ __forceinline__ Tile decode(const TcParams& p, int t) {
 // six columns: 185 -> 171 and 185 -> 174 us (174 and 177 at the copy rate).
 // From N = 48 on the products are issued in a rolled loop: the longer ones hide
 // it, and the steadier release of the stages streams better (20 steps with 18
-// columns 14.43 -> 14.28 ms, the 48^3 supercell with 18 columns 2.47 -> 2.41; at
+// columns 14.43 -> 14.29 ms, the 48^3 supercell with 18 columns 2.47 -> 2.41; at
 // N = 16 and 32 the straight line wins, 9.69 -> 9.25 and 11.75 -> 11.55 ms).
 template <int MODE>   // 0: band->grid, 1: grid->band, 2: grid->band from the row-major U~
 __global__ void __launch_bounds__(TC_THREADS, 1)

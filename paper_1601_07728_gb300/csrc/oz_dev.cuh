@@ -93,7 +93,9 @@ __device__ __forceinline__ bool oz_nonzero(double2 v) { return (oz_key(v.x) | oz
 // S = sum |a_k| |b_k| is taken along from the leading digits (entries below
 // 2^-8 of their row's scale count as zero, so that S is rather too small), and
 // a sum is accepted where the error is below 2^-53 S, one rounding of it:
-// S >= 0.0725 (|a|^2 + |b|^2)^1/2.  The rest is summed on the FP64 pipe.  Rows
+// S >= 0.0725 (|a|^2 + |b|^2)^1/2.  (With all K roundings of one sign it is at
+// most K^1/2 2^-53 S, within the K 2^-53 S of an FP64 sum.)  The rest is summed
+// on the FP64 pipe.  Rows
 // of n normal random entries reach about 0.6 n / (r_a r_b) against a limit of
 // 0.1 sqrt(n) (1 / r_a + 1 / r_b), r = 3..8 their scale over their deviation.
 __device__ __forceinline__ bool oz_accept(float s, float norm_a, float norm_b) {
