@@ -326,7 +326,10 @@ bse_status bse_local_projection(const bse_c128* u, const int* nk, const int* nx,
  * legacy default), returns when the outputs are written.  Allocates staging
  * and the G_j scratch, and for large problems that of exactly split tensor-core
  * products (without it, for Inf/NaN and magnitudes outside 2^+-400, or where a
- * bounded wait of that kernel gives up, BSE_SPLIT_WAIT_NS as above: the FP64 pipe).  Returns BSE_ERR_INVALID_ARG (before any device work) for a NULL psi,
+ * bounded wait of that kernel gives up, BSE_SPLIT_WAIT_NS as above: the FP64
+ * pipe; so are elements of G whose error there could lift above about 2^-53
+ * sum |psi d| |psi'|, and with more than one in 32 of those all).  Returns
+ * BSE_ERR_INVALID_ARG (before any device work) for a NULL psi,
  * eps, t, w or chi0, n_r, n_states or n_t < 1, n_r > 65535 or n_t > 65535;
  * BSE_ERR_OOM or BSE_ERR_CUDA from staging or the launches.  A
  * node t_j = 0 with some eps[K] == mu sits on the integrand's pole and gives
